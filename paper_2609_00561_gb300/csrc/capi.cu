@@ -478,6 +478,9 @@ iccg_status iccg_setup(iccg_ctx **out, int32_t n, int64_t nnz, const int64_t *ro
     L.fac_lev0 = H.fac_lev0;
     L.fac_nlev = H.fac_nlev;
     L.fac_wide = H.fac_wide;
+    L.fac_unit_cap = 0;
+    if (P.fac_rec)
+      for (const WarpUnit &u : H.units) L.fac_unit_cap = std::max(L.fac_unit_cap, H.lrp[size_t(u.row0 + u.nrows)] - H.lrp[size_t(u.row0)]);
   }
   int32_t *d_cg;
   CK(dev_upload(ctx, &d_cg, H.color_group), "alloc groups");
@@ -617,20 +620,27 @@ iccg_status iccg_factor(iccg_ctx *ctx) {
   ctx->factored = false;
   if (ctx->H.n == 0) { ctx->factored = true; return ICCG_OK; }
   // the factorization's launches (one per in-block level of every color)
-  // are captured once into a graph and replayed: no host launch cost per level
+  // are captured once into a graph and replayed: no host launch cost per
+  // level.  Captured on a private stream (the legacy default stream cannot
+  // capture), launched on the context's stream.
   if (ctx->opts.no_graph == 0 && !ctx->fexec && !ctx->fgraph_failed) {
     cudaGraph_t fg = nullptr;
-    cudaError_t e = cudaStreamBeginCapture(ctx->stream, cudaStreamCaptureModeThreadLocal);
+    cudaStream_t cs = nullptr;
+    cudaError_t e = cudaStreamCreateWithFlags(&cs, cudaStreamNonBlocking);
+    if (e == cudaSuccess) e = cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal);
     if (e == cudaSuccess) {
-      cudaError_t e1 = cudaMemsetAsync(ctx->P.err_row, 0xff, sizeof(unsigned long long), ctx->stream);
-      if (e1 == cudaSuccess) e1 = launch_factor(ctx->P, ctx->plan, int(ctx->H.nL));
-      e = cudaStreamEndCapture(ctx->stream, &fg);
+      Plan Lc = ctx->plan;
+      Lc.stream = cs;
+      cudaError_t e1 = cudaMemsetAsync(ctx->P.err_row, 0xff, sizeof(unsigned long long), cs);
+      if (e1 == cudaSuccess) e1 = launch_factor(ctx->P, Lc, int(ctx->H.nL));
+      e = cudaStreamEndCapture(cs, &fg);
       if (e == cudaSuccess) e = e1;
     }
+    if (cs) cudaStreamDestroy(cs);
     if (e == cudaSuccess) e = cudaGraphInstantiate(&ctx->fexec, fg, 0);
     if (fg) cudaGraphDestroy(fg);
     if (e != cudaSuccess) {
-      // e.g. the legacy default stream, which cannot be captured
+      // a runtime that refuses the capture: plain launches
       cudaGetLastError();
       if (ctx->fexec) cudaGraphExecDestroy(ctx->fexec);
       ctx->fexec = nullptr;
@@ -1046,7 +1056,7 @@ iccg_status iccg_info(const iccg_ctx *ctx, int64_t out[18]) {
   const Plan &L = ctx->plan;
   int64_t fac = 1;    // factor_finish
   for (int c = 0; c < L.n_c; ++c)
-    fac += (L.tile1[c] > L.tile0[c] || L.unit1[c] > L.unit0[c]) ? L.fac_nlev[c] : 1;
+    fac += !fac_unit_color(L, c) && (L.tile1[c] > L.tile0[c] || L.unit1[c] > L.unit0[c]) ? L.fac_nlev[c] : 1;
   const int64_t sw = L.n_c == 0 ? 0 : (L.coop ? 1 : (L.tail_c > 0 ? 2 * int64_t(L.tail_c) + 1 : 2 * int64_t(L.n_c) - 1));
   out[15] = fac;
   out[16] = 2 + sw;

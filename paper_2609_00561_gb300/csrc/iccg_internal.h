@@ -351,6 +351,7 @@ struct Plan {
   int32_t cap_ws = 0;                   // steps per tile held in a warp's buffer
   std::vector<int32_t> off_rr, off_rz;  // slot regions of the color-c forward / backward launches
   std::vector<int32_t> fac_ptr, fac_lev0, fac_nlev, fac_wide;   // IC(0) level schedule (host copy)
+  int32_t fac_unit_cap = 0;             // most L entries of a warp unit (0: no update pairs, no one-launch IC(0))
   int32_t last_rr = 0, last_rz = 0;     // slots written before the final launch of an iteration
   int32_t grid_a = 0;                   // CTAs of the SpMV-shaped kernels
   int32_t grid_v = 0;                   // CTAs of the vector kernels
@@ -373,6 +374,7 @@ int wtile_resident_ctas(bool fp32, int threads, int smem);   // CTAs per SM of t
 int pair_resident_ctas(bool fp32, int threads);              // CTAs per SM of the pair kernels
 int unit_resident_ctas(bool fp32, int S, int threads);       // CTAs per SM of the warp-unit kernels
 int coop_sweep_resident_ctas(bool fp32);                     // CTAs per SM of the cooperative sweep (0: none)
+bool fac_unit_color(const Plan &L, int c);                   // color c's IC(0) is one launch
 cudaError_t launch_factor(const Params &P, const Plan &L, int nL);
 cudaError_t launch_solve_init(const Params &P, const Plan &L, bool fp32, PhaseHook h, void *u);
 cudaError_t launch_solve_body(const Params &P, const Plan &L, bool fp32, PhaseHook h, void *u);

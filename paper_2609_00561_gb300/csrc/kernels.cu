@@ -1792,10 +1792,34 @@ __global__ void __launch_bounds__(kVecThreads) widen_kernel(const float *src, do
 // ---------------------------------------------------------------------------
 // IC(0) (up-looking, rows of a group level by level, one row per lane)
 // ---------------------------------------------------------------------------
+// End of a factor row: the pivot's reciprocal, which later rows wait for
+// (one FP64 sequence instead of a square root and then a division), and its
+// square root.
+__device__ __forceinline__ double factor_check(const Params &P, int i, double d) {
+  if (!(d > 0.0) || !isfinite(d)) {
+    atomicMin(P.err_row, (unsigned long long)i);
+    d = 1.0;
+  }
+  return d;
+}
+__device__ __forceinline__ void factor_pivot(const Params &P, int i, double d) {
+  d = factor_check(P, i, d);
+  P.invd[i] = rsqrt(d);
+  P.ldiag[i] = sqrt(d);
+}
+// the same for a CTA's rows (d in sd, row in srow), warps 0 and 1 a part each
+__device__ __forceinline__ void factor_pivots(const Params &P, const double *sd, const int *srow, int rows, int w,
+                                              int lane) {
+  if (w == 0 && lane < rows) P.invd[srow[lane]] = rsqrt(factor_check(P, srow[lane], sd[lane]));
+  if (w == 1 && lane < rows) P.ldiag[srow[lane]] = sqrt(factor_check(P, srow[lane], sd[lane]));
+}
+
 // Row i of the up-looking IC(0): for every j < i in the pattern, ascending,
 //   L_ij = (a_ij - sum_{k < j, k in pat(i) and pat(j)} L_ik L_jk) / L_jj,
 // then L_ii = sqrt(a_ii - sum_j L_ij^2); rows j are final when row i runs.
-// A finished row also stores 1/L_ii, and later rows multiply by it.
+// A finished row also stores 1/L_ii, and later rows multiply by it, and its
+// entries times 1/L_jj (in uval, entry for entry: free until the finishing
+// pass writes U there), which is what a later row's terms use.
 // General form: the common columns by a merge of the two sorted rows (a
 // chain of dependent loads).
 __device__ __forceinline__ void factor_row_merge(const Params &P, int i) {
@@ -1812,17 +1836,12 @@ __device__ __forceinline__ void factor_row_merge(const Params &P, int i) {
       else if (ca < cb) ++a;
       else ++b;
     }
-    const double lij = s * __ldcg(P.invd + j);
+    const double iv = __ldcg(P.invd + j), lij = s * iv;
     P.lval[p] = lij;
+    P.uval[p] = lij * iv;
     d -= lij * lij;
   }
-  if (!(d > 0.0) || !isfinite(d)) {
-    atomicMin(P.err_row, (unsigned long long)i);
-    d = 1.0;
-  }
-  const double lii = sqrt(d);
-  P.ldiag[i] = lii;
-  P.invd[i] = 1.0 / lii;
+  factor_pivot(P, i, d);
 }
 
 // Rows of at most kFacRow strictly-lower entries whose referenced rows have
@@ -1878,171 +1897,409 @@ __device__ __forceinline__ void factor_row(const Params &P, int i, int32_t *sc, 
     sv[p] = lij;
     d -= lij * lij;
   }
-  for (int t = 0; t < ni; ++t) P.lval[rb + t] = sv[t];
-  if (!(d > 0.0) || !isfinite(d)) {
-    atomicMin(P.err_row, (unsigned long long)i);
-    d = 1.0;
+  for (int t = 0; t < ni; ++t) {
+    P.lval[rb + t] = sv[t];
+    P.uval[rb + t] = sv[t] * __ldcg(P.invd + sc[t]);
   }
-  const double lii = sqrt(d);
-  P.ldiag[i] = lii;
-  P.invd[i] = 1.0 / lii;
+  factor_pivot(P, i, d);
 }
 
-// Row i from its precomputed update pairs (per entry L_ij, the pairs
-// (position of k in row i, index of L_jk) for the common columns k < j,
-// ascending k).  A level has few rows, so each row's latency is the cost:
-// all pair indices and positions of a pass are copied into shared memory
-// with cp.async at once, then all pair values L_jk (rows j are final)
-// gathered the same way, then every entry takes its own terms from shared
-// memory, k ascending as in the general form.  Shared memory is
-// thread-interleaved (element q of thread t at q T + t: no bank conflicts).
-constexpr int kFacRowThreads = 32;
-constexpr int kFacStage = 160;   // pairs per pass
+// One in-block level of a lane-tile or warp-unit color, a warp per row (rows
+// of 9..32 strictly-lower entries with precomputed update pairs).
+// Lane p holds entry p of the row; the pairs' values L_jk / L_kk are gathered
+// by the whole warp into shared memory, then
+//   s_p = a_ip - sum_{k < p} s_k (L_pk / L_kk),   L_ip = s_p / L_pp
+// in steps: at each, every lane whose next term's s_k is final (lane k has no
+// term left) takes it from lane k by a shuffle, k ascending per entry as in
+// the general form.
+//
+// Bound by latency: a level has few rows (27-point, blocks of 32: about 1000
+// rows in each of 200 levels), so what counts is the chain of one row.  A
+// thread per row walked its 60 pairs one FP64 multiply-add after another
+// (64 cycles each) behind staged copies, 44 us a level; the warp's steps are
+// as many as the deepest chain of terms or the longest list (about 10) and
+// its loads are all in flight at once.  Static data (record, columns, a_ij, pair indices)
+// is read before griddepcontrol.wait, while the previous level runs.  Square
+// root and division are FP64 sequences that cost a whole warp however few
+// lanes run them, so one warp does them for the CTA's rows together.
+constexpr int kFacWarps = 8;
+constexpr int kFacPairs = kFacRow * (kFacRow - 1) / 2;   // most pairs of a row
+constexpr int kFacBatch = 4;                             // pair loads in flight per lane
+constexpr int kFacWarpBytes = kFacPairs * 8 + ((kFacPairs + 15) & ~15);
 
-template <typename T>
-struct Strided {
-  T *base;
-  __device__ __forceinline__ T &operator[](int q) const { return base[q * kFacRowThreads]; }
-};
-
-
-struct FacSmem {
-  Strided<double> sv, ivj, pv;
-  Strided<int32_t> qe, pb;
-  Strided<uint32_t> pw;   // fp_pos bytes, as the 4-byte words covering the pass
-};
-
-// STAGE: pairs per pass
-// The row's static data (its record, pair indices and positions, columns,
-// a_ij, pair ends) is read before griddepcontrol.wait, i.e. while the
-// previous level's launch still runs; 1/L_jj and the pair values L_jk after.
-template <int STAGE>
-__device__ __forceinline__ void factor_row_pairs(const Params &P, int4 rec, const FacSmem &m) {
-  const int i = rec.x, rb = rec.y, q0 = rec.z, ni = rec.w & 0xff, np = rec.w >> 8;
-  if (ni > kFacRow) {
-    pdl_wait();
-    factor_row_merge(P, i);
-    return;
-  }
-  // the first pass's pair indices and position words, before anything else
-  const uint32_t *posw = reinterpret_cast<const uint32_t *>(P.fp_pos);
-  {
-    const int nq = min(STAGE, np), w0 = q0 >> 2, w1 = (q0 + nq + 3) >> 2;
-    for (int q = 0; q < nq; ++q) cp_async4(&m.pb[q], P.fp_b + q0 + q);
-    for (int w = w0; w < w1; ++w) cp_async4(&m.pw[w - w0], posw + w);
-    cp_commit();
-  }
-  {
-    int col[kFacRow];
-#pragma unroll
-    for (int p = 0; p < kFacRow; ++p) col[p] = p < ni ? __ldg(P.lcol + rb + p) : 0;
-#pragma unroll
-    for (int p = 0; p < kFacRow; ++p)
-      if (p < ni) {
-        m.sv[p] = __ldg(P.ainit + rb + p);
-        m.qe[p] = __ldg(P.fp_ptr + rb + p + 1) - q0;
-      }
-    pdl_wait();
-#pragma unroll
-    for (int p = 0; p < kFacRow; ++p)
-      if (p < ni) m.ivj[p] = __ldcg(P.invd + col[p]);
-  }
-  double d = P.adiag[i];
-  int p = 0;
-  double s = 0.0;
-  // entries without terms before the first pair
-  while (p < ni && m.qe[p] == 0) {
-    const double lij = m.sv[p] * m.ivj[p];
-    m.sv[p] = lij;
-    d -= lij * lij;
-    ++p;
-  }
-  if (p < ni) s = m.sv[p];
-  for (int qa = 0; qa < np; qa += STAGE) {
-    const int nq = min(STAGE, np - qa);
-    // indices and the words holding the positions (the first pass's were
-    // issued at the start)
-    const int g0 = q0 + qa, w0 = g0 >> 2, w1 = (g0 + nq + 3) >> 2;
-    if (qa > 0) {
-      for (int q = 0; q < nq; ++q) cp_async4(&m.pb[q], P.fp_b + g0 + q);
-      for (int w = w0; w < w1; ++w) cp_async4(&m.pw[w - w0], posw + w);
-      cp_commit();
-    }
-    cp_wait_all();
-    // the pair values
-    for (int q = 0; q < nq; ++q) cp_async8(&m.pv[q], P.lval + m.pb[q]);
-    cp_commit();
-    cp_wait_all();
-    const int sh = g0 & 3;
-    for (int q = 0; q < nq; ++q) {
-      const int bq = q + sh;
-      const int pos = int((m.pw[bq >> 2] >> (8 * (bq & 3))) & 0xffu);
-      s -= m.sv[pos] * m.pv[q];
-      // the entry is complete after its last pair; then the following
-      // entries up to the next one with pairs left
-      while (p < ni && m.qe[p] == qa + q + 1) {
-        const double lij = s * m.ivj[p];
-        m.sv[p] = lij;
-        d -= lij * lij;
-        ++p;
-        s = p < ni ? m.sv[p] : 0.0;
+// the steps of one row: lane p's terms are pv / ps [c, ce)
+__device__ __forceinline__ double factor_steps(double s, int c, int ce, const double *pv, const uint8_t *ps, int lane) {
+  int src = c < ce ? int(ps[c]) : lane;
+  double nv = c < ce ? pv[c] : 0.0;
+  for (uint32_t left = __ballot_sync(0xffffffffu, c < ce); left;) {
+    const double sk = __shfl_sync(0xffffffffu, s, src);
+    if (c < ce && !((left >> src) & 1u)) {
+      s -= sk * nv;
+      ++c;
+      if (c < ce) {
+        src = int(ps[c]);
+        nv = pv[c];
       }
     }
+    left = __ballot_sync(0xffffffffu, c < ce);
   }
-  cp_wait_all();   // no copy of this row may land in the next row's buffers
-  for (int t = 0; t < ni; ++t) P.lval[rb + t] = m.sv[t];
-  if (!(d > 0.0) || !isfinite(d)) {
-    atomicMin(P.err_row, (unsigned long long)i);
-    d = 1.0;
-  }
-  const double lii = sqrt(d);
-  P.ldiag[i] = lii;
-  P.invd[i] = 1.0 / lii;
+  return s;
 }
 
-constexpr int kFacPosWords = kFacStage / 4 + 2;
-constexpr int kFacSmem = kFacRowThreads * (kFacRow * 20 + kFacStage * 12 + kFacPosWords * 4);
-
-// the rows of one in-block level of a lane-tile or warp-unit color, one row
-// per thread (dynamic shared memory, thread-interleaved)
-__global__ void __launch_bounds__(kFacRowThreads) factor_rows_kernel(Params P, int k0, int k1) {
+__global__ void __launch_bounds__(kFacWarps * kWarp) factor_warp_kernel(Params P, int k0, int k1) {
   pdl_trigger();
   extern __shared__ __align__(16) unsigned char fsm[];
-  const int t = threadIdx.x;
-  constexpr int T = kFacRowThreads;
-  unsigned char *q = fsm;
-  FacSmem m;
-  m.sv.base = reinterpret_cast<double *>(q) + t;
-  q += size_t(T) * kFacRow * 8;
-  m.ivj.base = reinterpret_cast<double *>(q) + t;
-  q += size_t(T) * kFacRow * 8;
-  m.pv.base = reinterpret_cast<double *>(q) + t;
-  q += size_t(T) * kFacStage * 8;
-  m.qe.base = reinterpret_cast<int32_t *>(q) + t;
-  q += size_t(T) * kFacRow * 4;
-  m.pb.base = reinterpret_cast<int32_t *>(q) + t;
-  q += size_t(T) * kFacStage * 4;
-  m.pw.base = reinterpret_cast<uint32_t *>(q) + t;
-  for (int k = k0 + int(blockIdx.x * blockDim.x + threadIdx.x); k < k1; k += int(gridDim.x * blockDim.x)) {
-    if (P.fac_rec) {
-      factor_row_pairs<kFacStage>(P, __ldg(P.fac_rec + k), m);
-    } else {
-      pdl_wait();
-      factor_row_merge(P, __ldg(P.fac_rows + k));
+  __shared__ double sd[kFacWarps];
+  __shared__ int srow[kFacWarps];
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  double *pv = reinterpret_cast<double *>(fsm + size_t(w) * kFacWarpBytes);
+  uint8_t *ps = reinterpret_cast<uint8_t *>(pv + kFacPairs);
+  bool waited = false;
+  for (int kb = k0 + int(blockIdx.x) * kFacWarps; kb < k1; kb += int(gridDim.x) * kFacWarps) {
+    const int k = kb + w;
+    const int4 rec = k < k1 ? __ldg(P.fac_rec + k) : make_int4(0, 0, 0, 0);
+    const int i = rec.x, rb = rec.y, q0 = rec.z, ni = rec.w & 0xff, np = rec.w >> 8;
+    const bool on = lane < ni;
+    const int col = on ? __ldg(P.lcol + rb + lane) : 0;
+    double s = on ? __ldg(P.ainit + rb + lane) : 0.0;
+    const int c = on ? __ldg(P.fp_ptr + rb + lane) - q0 : 0;
+    const int ce = on ? __ldg(P.fp_ptr + rb + lane + 1) - q0 : 0;
+    const double dg = k < k1 ? __ldg(P.adiag + i) : 1.0;
+    int fb[kFacBatch], fp[kFacBatch];
+#pragma unroll
+    for (int u = 0; u < kFacBatch; ++u) {
+      const int q = u * kWarp + lane;
+      fb[u] = q < np ? __ldg(P.fp_b + q0 + q) : 0;
+      fp[u] = q < np ? int(__ldg(P.fp_pos + q0 + q)) : 0;
     }
+    if (!waited) {
+      pdl_wait();
+      waited = true;
+    }
+    const double iv = on ? __ldcg(P.invd + col) : 0.0;
+    for (int qa = 0; qa < np; qa += kFacBatch * kWarp) {
+      if (qa > 0) {
+#pragma unroll
+        for (int u = 0; u < kFacBatch; ++u) {
+          const int q = qa + u * kWarp + lane;
+          fb[u] = q < np ? __ldg(P.fp_b + q0 + q) : 0;
+          fp[u] = q < np ? int(__ldg(P.fp_pos + q0 + q)) : 0;
+        }
+      }
+      double v[kFacBatch];
+#pragma unroll
+      for (int u = 0; u < kFacBatch; ++u) v[u] = qa + u * kWarp + lane < np ? __ldcg(P.uval + fb[u]) : 0.0;
+#pragma unroll
+      for (int u = 0; u < kFacBatch; ++u) {
+        const int q = qa + u * kWarp + lane;
+        if (q < np) {
+          pv[q] = v[u];
+          ps[q] = uint8_t(fp[u]);
+        }
+      }
+    }
+    __syncwarp();
+    s = factor_steps(s, c, ce, pv, ps, lane);
+    const double l = s * iv;
+    if (on) {
+      P.lval[rb + lane] = l;
+      P.uval[rb + lane] = l * iv;
+    }
+    const double ss = warp_sum(l * l);
+    if (lane == 0) {
+      sd[w] = dg - ss;
+      srow[w] = i;
+    }
+    __syncthreads();
+    factor_pivots(P, sd, srow, min(kFacWarps, k1 - kb), w, lane);
+    __syncthreads();
   }
 }
 
-// levels of short rows (at most kFacShort lower entries): one row per thread,
-// the general form (short merges), no staging, full CTAs
+// A warp-unit color in one launch, a CTA per unit (at most 32 rows of whole
+// blocks, their L entries one range), for rows above kFacShort.  Blocks of one color share no
+// edge, so a row waits only for rows of its own block: the CTA's warps take
+// the rows in turn (first rows of all blocks, second rows, ...), a warp per
+// row as above, and a finished row is announced through a flag in shared
+// memory, where its scaled entries and 1/L_ii also stay for the rows that
+// follow.  A warp loads its next row's indices and its entries of other
+// colors while the others work.
+//
+// Why: with a launch per level every level of a block cost a launch boundary
+// and a trip of its values through L2 (27-point 61x67x59, blocks of 32: 205
+// launches of 7-9 us, 1.86 ms in all); one launch per color takes 0.90 ms, half
+// of it the FP64 pipe (about 30 warp instructions a row).  IC(0) and one
+// application together there: 7.41 ms with a thread per row, 1.15 ms now.
+constexpr int kFacUnitWarps = 4;
+constexpr int kFacSpin = 1 << 22;   // polls of a row's flags before giving up
+
+inline int fac_unit_bytes(int cap) { return kFacUnitWarps * kFacWarpBytes + cap * 8; }
+
+__global__ void __launch_bounds__(kFacUnitWarps * kWarp) factor_unit_kernel(Params P, int u0, int S) {
+  pdl_trigger();
+  extern __shared__ __align__(16) unsigned char fsm[];
+  __shared__ double ivs[kWarp], ds[kWarp];
+  __shared__ volatile int ready[kWarp];
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  double *pv = reinterpret_cast<double *>(fsm + size_t(w) * kFacWarpBytes);
+  uint8_t *ps = reinterpret_cast<uint8_t *>(pv + kFacPairs);
+  double *us = reinterpret_cast<double *>(fsm + kFacUnitWarps * kFacWarpBytes);
+  const WarpUnit d = load_unit(P.units + u0 + int(blockIdx.x));
+  const int row0 = d.row0, row1 = d.row0 + d.nrows;
+  const int l0 = __ldg(P.lrp + row0), l1 = __ldg(P.lrp + row1);
+  if (threadIdx.x < kWarp) ready[threadIdx.x] = 0;
+  __syncthreads();
+  bool waited = false;
+  for (int t = w; t < S * d.nblk; t += kFacUnitWarps) {
+    const int b = d.blk0 + t % d.nblk, i = __ldg(P.bptr + b) + t / d.nblk;
+    if (i >= __ldg(P.bptr + b + 1)) continue;
+    const int rb = __ldg(P.lrp + i), ni = __ldg(P.lrp + i + 1) - rb;
+    const int q0 = __ldg(P.fp_ptr + rb), np = __ldg(P.fp_ptr + rb + ni) - q0;
+    const bool on = lane < ni;
+    const int col = on ? __ldg(P.lcol + rb + lane) : 0;
+    double s = on ? __ldg(P.ainit + rb + lane) : 0.0;
+    const int c = on ? __ldg(P.fp_ptr + rb + lane) - q0 : 0;
+    const int ce = on ? __ldg(P.fp_ptr + rb + lane + 1) - q0 : 0;
+    const double dg = __ldg(P.adiag + i);
+    int fb[kFacBatch], fp[kFacBatch];
+#pragma unroll
+    for (int u = 0; u < kFacBatch; ++u) {
+      const int q = u * kWarp + lane;
+      fb[u] = q < np ? __ldg(P.fp_b + q0 + q) : 0;
+      fp[u] = q < np ? int(__ldg(P.fp_pos + q0 + q)) : 0;
+    }
+    if (!waited) {
+      pdl_wait();
+      waited = true;
+    }
+    // values of other colors, before the wait for the block's own rows
+    const bool in = on && col >= row0;
+    double iv = on && !in ? __ldcg(P.invd + col) : 0.0;
+    double v[kFacBatch];
+#pragma unroll
+    for (int u = 0; u < kFacBatch; ++u) {
+      const int q = u * kWarp + lane;
+      v[u] = q < np && (fb[u] < l0 || fb[u] >= l1) ? __ldcg(P.uval + fb[u]) : 0.0;
+    }
+    for (int spin = 0; !__all_sync(0xffffffffu, !in || ready[col - row0] != 0); ++spin)
+      if (spin > kFacSpin) {
+        if (lane == 0) atomicMin(P.err_row, (unsigned long long)i);
+        break;
+      }
+    __threadfence_block();
+    if (in) iv = ivs[col - row0];
+#pragma unroll
+    for (int u = 0; u < kFacBatch; ++u) {
+      const int q = u * kWarp + lane;
+      if (q < np) {
+        pv[q] = fb[u] >= l0 && fb[u] < l1 ? us[fb[u] - l0] : v[u];
+        ps[q] = uint8_t(fp[u]);
+      }
+    }
+    for (int q = kFacBatch * kWarp + lane; q < np; q += kWarp) {
+      const int e = __ldg(P.fp_b + q0 + q);
+      pv[q] = e >= l0 && e < l1 ? us[e - l0] : __ldcg(P.uval + e);
+      ps[q] = __ldg(P.fp_pos + q0 + q);
+    }
+    __syncwarp();
+    s = factor_steps(s, c, ce, pv, ps, lane);
+    const double l = s * iv, lu = l * iv;
+    const double ss = warp_sum(l * l);
+    if (on) us[rb - l0 + lane] = lu;
+    if (lane == 0) {
+      const double dd = factor_check(P, i, dg - ss);
+      ds[i - row0] = dd;
+      ivs[i - row0] = rsqrt(dd);
+    }
+    __threadfence_block();
+    __syncwarp();
+    if (lane == 0) ready[i - row0] = 1;
+    if (on) {
+      P.lval[rb + lane] = l;
+      P.uval[rb + lane] = lu;
+    }
+  }
+  if (!waited) pdl_wait();
+  __syncthreads();
+  if (threadIdx.x < d.nrows) {
+    P.invd[row0 + threadIdx.x] = ivs[threadIdx.x];
+    P.ldiag[row0 + threadIdx.x] = sqrt(ds[threadIdx.x]);
+  }
+}
+
+// The same for rows of 9..64 strictly-lower entries without precomputed
+// pairs (a matrix with any row above 32): two entries per lane, and the
+// values L_pk / L_kk as the strictly-lower triangle of a dense matrix in the
+// warp's shared memory (column k: entries p = k + 1 .. ni - 1 consecutive, so
+// the lanes of a column read without bank conflicts).  The warp reads row j of
+// every entry (i, j) coalesced and finds its columns in row i by a binary
+// search in shared memory.  Bound by the FP64 pipe (about 2 warp instructions
+// per column of a row).  IC(0) and one application for a 3-unknown
+// 27-neighbour 33^3 network with one-row blocks: 3.24 ms with a thread per row
+// merging index lists, 0.96 ms so.
+constexpr int kFacWide = 64;
+constexpr int kFacWideWarps = 4;
+
+__host__ __device__ inline int fac_wide_bytes(int cap) { return r16b(cap * (cap - 1) / 2 * 8 + cap * 4); }
+
+__global__ void __launch_bounds__(kFacWideWarps * kWarp) factor_wide_kernel(Params P, int k0, int k1, int cap) {
+  pdl_trigger();
+  extern __shared__ __align__(16) unsigned char fsm[];
+  __shared__ double sd[kFacWideWarps];
+  __shared__ int srow[kFacWideWarps];
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const int bytes = fac_wide_bytes(cap);
+  double *M = reinterpret_cast<double *>(fsm + size_t(w) * bytes);
+  int32_t *cs = reinterpret_cast<int32_t *>(M + cap * (cap - 1) / 2);
+  bool waited = false;
+  for (int kb = k0 + int(blockIdx.x) * kFacWideWarps; kb < k1; kb += int(gridDim.x) * kFacWideWarps) {
+    const int k = kb + w;
+    const int i = k < k1 ? __ldg(P.fac_rows + k) : 0;
+    const int rb = k < k1 ? __ldg(P.lrp + i) : 0, ni = k < k1 ? __ldg(P.lrp + i + 1) - rb : 0;
+    const bool on0 = lane < ni, on1 = lane + kWarp < ni;
+    const int c0 = on0 ? __ldg(P.lcol + rb + lane) : 0, c1 = on1 ? __ldg(P.lcol + rb + kWarp + lane) : 0;
+    double s0 = on0 ? __ldg(P.ainit + rb + lane) : 0.0, s1 = on1 ? __ldg(P.ainit + rb + kWarp + lane) : 0.0;
+    const int b0 = on0 ? __ldg(P.lrp + c0) : 0, b1 = on1 ? __ldg(P.lrp + c1) : 0;
+    const int n0 = on0 ? __ldg(P.lrp + c0 + 1) - b0 : 0, n1 = on1 ? __ldg(P.lrp + c1 + 1) - b1 : 0;
+    const double dg = k < k1 ? __ldg(P.adiag + i) : 1.0;
+    const int tri = ni * (ni - 1) / 2;
+    for (int e = lane; e < tri; e += kWarp) M[e] = 0.0;
+    if (on0) cs[lane] = c0;
+    if (on1) cs[lane + kWarp] = c1;
+    if (!waited) {
+      pdl_wait();
+      waited = true;
+    }
+    const double iv0 = on0 ? __ldcg(P.invd + c0) : 0.0, iv1 = on1 ? __ldcg(P.invd + c1) : 0.0;
+    __syncwarp();
+    // entry p's row j against the columns before p
+    auto place = [&](int p, int cu, double v) {
+      int lo = 0, hi = p;
+      while (lo < hi) {
+        const int mid = (lo + hi) >> 1;
+        if (cs[mid] < cu) lo = mid + 1;
+        else hi = mid;
+      }
+      if (lo < p && cs[lo] == cu) M[lo * (ni - 1) - lo * (lo - 1) / 2 + (p - lo - 1)] = v;
+    };
+    for (int p0 = 1; p0 < ni; p0 += kFacBatch) {
+      int cu[kFacBatch], nj[kFacBatch], jb[kFacBatch];
+      double v[kFacBatch];
+#pragma unroll
+      for (int u = 0; u < kFacBatch; ++u) {
+        const int p = p0 + u;
+        jb[u] = __shfl_sync(0xffffffffu, p < kWarp ? b0 : b1, p & 31);
+        nj[u] = __shfl_sync(0xffffffffu, p < kWarp ? n0 : n1, p & 31);
+        if (p >= ni) nj[u] = 0;
+        cu[u] = lane < nj[u] ? __ldg(P.lcol + jb[u] + lane) : 0;
+        v[u] = lane < nj[u] ? __ldcg(P.uval + jb[u] + lane) : 0.0;
+      }
+#pragma unroll
+      for (int u = 0; u < kFacBatch; ++u) {
+        if (lane < nj[u]) place(p0 + u, cu[u], v[u]);
+        for (int q = kWarp + lane; q < nj[u]; q += kWarp)
+          place(p0 + u, __ldg(P.lcol + jb[u] + q), __ldcg(P.uval + jb[u] + q));
+      }
+    }
+    __syncwarp();
+    int off = -1;   // column kk's entry p at off + p - kk
+    for (int kk = 0; kk < ni - 1; ++kk) {
+      const double sk = __shfl_sync(0xffffffffu, kk < kWarp ? s0 : s1, kk & 31);
+      if (kk < kWarp - 1) {
+        const double m = lane > kk && on0 ? M[off + lane - kk] : 0.0;
+        if (__double_as_longlong(m) != 0) s0 -= sk * m;
+      }
+      if (ni > kWarp) {
+        const double m = lane + kWarp > kk && on1 ? M[off + lane + kWarp - kk] : 0.0;
+        if (__double_as_longlong(m) != 0) s1 -= sk * m;
+      }
+      off += ni - 1 - kk;
+    }
+    const double l0 = s0 * iv0, l1 = s1 * iv1;
+    if (on0) {
+      P.lval[rb + lane] = l0;
+      P.uval[rb + lane] = l0 * iv0;
+    }
+    if (on1) {
+      P.lval[rb + kWarp + lane] = l1;
+      P.uval[rb + kWarp + lane] = l1 * iv1;
+    }
+    double ss = l0 * l0;
+    if (ni > kWarp) ss += l1 * l1;
+    ss = warp_sum(ss);
+    if (lane == 0) {
+      sd[w] = dg - ss;
+      srow[w] = i;
+    }
+    __syncthreads();
+    factor_pivots(P, sd, srow, min(kFacWideWarps, k1 - kb), w, lane);
+    __syncthreads();
+  }
+}
+
+// Levels of short rows (at most kFacShort lower entries) with precomputed
+// pairs: one row per thread (a warp per row would leave 24 lanes idle in
+// every FP64 instruction).  Static data before griddepcontrol.wait; a stencil
+// without triangles (5- and 7-point) has no pairs at all.
 constexpr int kFacShort = 8;
 __global__ void __launch_bounds__(kVecThreads) factor_short_kernel(Params P, int k0, int k1) {
+  pdl_trigger();
+  bool waited = false;
+  for (int k = k0 + int(blockIdx.x * blockDim.x + threadIdx.x); k < k1; k += int(gridDim.x * blockDim.x)) {
+    const int4 rec = __ldg(P.fac_rec + k);
+    const int i = rec.x, rb = rec.y, q0 = rec.z, ni = rec.w & 0xff, np = rec.w >> 8;
+    int col[kFacShort], qe[kFacShort];
+    double l[kFacShort], iv[kFacShort];
+#pragma unroll
+    for (int p = 0; p < kFacShort; ++p) {
+      col[p] = p < ni ? __ldg(P.lcol + rb + p) : 0;
+      l[p] = p < ni ? __ldg(P.ainit + rb + p) : 0.0;
+      qe[p] = np > 0 && p < ni ? __ldg(P.fp_ptr + rb + p + 1) - q0 : 0;
+    }
+    double d = __ldg(P.adiag + i);
+    if (!waited) {
+      pdl_wait();
+      waited = true;
+    }
+#pragma unroll
+    for (int p = 0; p < kFacShort; ++p) iv[p] = p < ni ? __ldcg(P.invd + col[p]) : 0.0;
+    int q = 0;
+#pragma unroll
+    for (int p = 0; p < kFacShort; ++p) {
+      if (p < ni) {
+        double s = l[p];
+        for (; q < qe[p]; ++q) {
+          const int pos = int(__ldg(P.fp_pos + q0 + q));
+          const double v = __ldcg(P.lval + __ldg(P.fp_b + q0 + q));
+          double lk = 0.0;
+#pragma unroll
+          for (int t = 0; t < kFacShort; ++t)
+            if (t < p && t == pos) lk = l[t];
+          s -= lk * v;
+        }
+        l[p] = s * iv[p];
+        d -= l[p] * l[p];
+      }
+    }
+#pragma unroll
+    for (int p = 0; p < kFacShort; ++p)
+      if (p < ni) {
+        P.lval[rb + p] = l[p];
+        P.uval[rb + p] = l[p] * iv[p];
+      }
+    factor_pivot(P, i, d);
+  }
+  if (!waited) pdl_wait();
+}
+
+// levels without precomputed pairs of short rows (short merges) or of rows
+// above kFacWide: one row per thread, the general form
+__global__ void __launch_bounds__(kVecThreads) factor_merge_kernel(Params P, int k0, int k1) {
   pdl_trigger();
   pdl_wait();
   for (int k = k0 + int(blockIdx.x * blockDim.x + threadIdx.x); k < k1; k += int(gridDim.x * blockDim.x))
     factor_row_merge(P, __ldg(P.fac_rows + k));
 }
-
 
 // group colors: one CTA per group, its rows level by level of the in-group
 // schedule (dynamic shared memory: a kFacRow slice per thread)
@@ -2932,27 +3189,50 @@ cudaError_t launch_solve_persistent(const Params &P, const Plan &L, bool fp32) {
 cudaError_t configure_kernels() {
   cudaError_t e = cudaFuncSetAttribute(factor_color_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        kMaxWarpsPerCta * kWarp * kFacRow * 12);
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(factor_rows_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kFacSmem);
+  if (e == cudaSuccess) e = allow_smem(factor_wide_kernel);
+  if (e == cudaSuccess) e = allow_smem(factor_unit_kernel);
   if (e == cudaSuccess) e = configure_pt<double>();
   if (e == cudaSuccess) e = configure_pt<float>();
   return e;
 }
 
+// IC(0) of color c as one launch (factor_unit_kernel): warp units of several
+// levels with precomputed pairs and rows above kFacShort entries; shorter
+// rows would fill too few lanes of a warp (a launch per level, a thread per
+// row: 7-point 99x90x85 in blocks of 32 0.62 ms; a warp per row spends 32
+// lanes of the scarce FP64 pipe on 3 entries)
+bool fac_unit_color(const Plan &L, int c) {
+  if (L.unit1[c] <= L.unit0[c] || L.fac_unit_cap <= 0 || L.fac_nlev[c] < 2) return false;
+  int wide = 0;
+  for (int v = 0; v < L.fac_nlev[c]; ++v) wide = std::max(wide, L.fac_wide[size_t(L.fac_lev0[c] + v)]);
+  return wide > kFacShort;
+}
+
 cudaError_t launch_factor(const Params &P, const Plan &L, int nL) {
   for (int c = 0; c < L.n_c; ++c) {
-    if (L.tile1[c] > L.tile0[c] || L.unit1[c] > L.unit0[c]) {
-      // lane-tile and warp-unit colors: one launch per in-block level, a thread per row
+    if (fac_unit_color(L, c)) {
+      cudaError_t e = launch(factor_unit_kernel, L.unit1[c] - L.unit0[c], kFacUnitWarps * kWarp,
+                             fac_unit_bytes(L.fac_unit_cap), L, P, L.unit0[c], L.unit_S[c]);
+      if (e != cudaSuccess) return e;
+    } else if (L.tile1[c] > L.tile0[c] || L.unit1[c] > L.unit0[c]) {
+      // other lane-tile and warp-unit colors: one launch per in-block level
       for (int v = 0; v < L.fac_nlev[c]; ++v) {
         const int k0 = L.fac_ptr[size_t(L.fac_lev0[c] + v)], k1 = L.fac_ptr[size_t(L.fac_lev0[c] + v + 1)];
         // consecutive levels overlap through programmatic dependent launch:
         // a level's static loads run while the previous level finishes
         cudaError_t e;
-        if (L.fac_wide[size_t(L.fac_lev0[c] + v)] <= kFacShort) {
-          const int grid = std::max(1, std::min((k1 - k0 + kVecThreads - 1) / kVecThreads, L.grid_v));
-          e = launch(factor_short_kernel, grid, kVecThreads, 0, L, P, k0, k1);
+        const int rows = k1 - k0, wide = L.fac_wide[size_t(L.fac_lev0[c] + v)];
+        const bool pairs = P.fac_rec != nullptr;
+        if (pairs && wide > kFacShort) {
+          const int grid = std::max(1, std::min((rows + kFacWarps - 1) / kFacWarps, 4 * L.grid_v));
+          e = launch(factor_warp_kernel, grid, kFacWarps * kWarp, kFacWarps * kFacWarpBytes, L, P, k0, k1);
+        } else if (!pairs && wide > kFacShort && wide <= kFacWide) {
+          const int grid = std::max(1, std::min((rows + kFacWideWarps - 1) / kFacWideWarps, 4 * L.grid_v));
+          const int sm = kFacWideWarps * fac_wide_bytes(wide);
+          e = launch(factor_wide_kernel, grid, kFacWideWarps * kWarp, sm, L, P, k0, k1, wide);
         } else {
-          const int grid = std::max(1, std::min((k1 - k0 + kFacRowThreads - 1) / kFacRowThreads, 8 * L.grid_v));
-          e = launch(factor_rows_kernel, grid, kFacRowThreads, kFacSmem, L, P, k0, k1);
+          const int grid = std::max(1, std::min((rows + kVecThreads - 1) / kVecThreads, L.grid_v));
+          e = launch(pairs ? factor_short_kernel : factor_merge_kernel, grid, kVecThreads, 0, L, P, k0, k1);
         }
         if (e != cudaSuccess) return e;
       }
