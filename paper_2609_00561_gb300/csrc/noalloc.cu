@@ -21,6 +21,8 @@
 // cudaGetSymbolAddress (with that device current) and caches it.  The stream
 // must belong to the current device (the cached address is that device's
 // copy of the array).
+#include <algorithm>
+#include <cstddef>
 #include <mutex>
 
 #include "iccg_internal.h"
@@ -41,6 +43,7 @@ struct NaScratch {
 };
 
 static_assert(kNaMaxCtas * kNaRowsPerCta == ICCG_NOALLOC_MAX_ROWS, "row limit must split into CTAs");
+static_assert(offsetof(NaScratch, ticket) == offsetof(NaScratch, gticket) + sizeof(NaScratch::gticket), "cleared together");
 
 static __device__ __align__(256) unsigned char g_noalloc_scratch[sizeof(NaScratch)];
 
@@ -74,19 +77,98 @@ __device__ __forceinline__ bool na_last(unsigned int *ticket, unsigned int expec
   return *flag != 0;
 }
 
+// A warp takes slices of 32 rows, whose CSR entries are one range: it copies
+// their columns and values into shared memory coalesced, kNaChunk at a time, and
+// a lane then sums its own row from there, the gathers of kNaBatch entries in
+// flight (consecutive rows gather neighbouring elements of p).  The next
+// slice's row pointers and first chunk are loaded while the current slice is
+// summed.  Bound by memory traffic and, equally, by the FP64 rate: an FP64
+// instruction costs a warp the same for 1 lane as for 32, so the <p, q> sum
+// runs once per CTA over all its slices, not once per 256 rows.
+constexpr int kNaChunk = 256;
+constexpr int kNaBatch = 8;
+
+constexpr int kNaGrid = 4 * 152;   // CTAs of a launch at most: those a GB300 holds at once
+
+struct NaChunk {
+  int32_t c[kNaChunk / 32];
+  double v[kNaChunk / 32];
+};
+
+__device__ __forceinline__ void na_load(NaChunk &k, const int32_t *colind, const double *val, int64_t b, int cnt,
+                                        int lane) {
+#pragma unroll
+  for (int u = 0; u < kNaChunk / 32; ++u) {
+    const int e = u * 32 + lane;
+    k.c[u] = e < cnt ? __ldg(colind + b + e) : 0;
+    k.v[u] = e < cnt ? __ldg(val + b + e) : 0.0;
+  }
+}
+
+__device__ __forceinline__ int na_count(int64_t b, int64_t e1) { return int(e1 - b < kNaChunk ? e1 - b : kNaChunk); }
+
 __global__ void __launch_bounds__(kNaRowsPerCta)
 spmv_dot_noalloc_kernel(int n, const int64_t *__restrict__ rowptr, const int32_t *__restrict__ colind,
                         const double *__restrict__ val, const double *__restrict__ p, double *__restrict__ q,
                         double *__restrict__ pq, NaScratch *s) {
   __shared__ double red[kNaWarps];
   __shared__ int flag;
-  const int i = blockIdx.x * kNaRowsPerCta + threadIdx.x;
+  __shared__ double sval[kNaWarps][kNaChunk];
+  __shared__ int32_t scol[kNaWarps][kNaChunk];
+  const int lane = threadIdx.x & 31;
+  double *sv = sval[threadIdx.x >> 5];
+  int32_t *sc = scol[threadIdx.x >> 5];
   double acc = 0.0;
-  if (i < n) {
+  const int stride = int(gridDim.x) * kNaRowsPerCta;
+  int i = blockIdx.x * kNaRowsPerCta + threadIdx.x;
+  int64_t rs = 0, re = 0;
+  NaChunk nx;
+  if (i - lane < n) {
+    rs = rowptr[min(i, n)];
+    re = rowptr[min(i + 1, n)];
+    const int64_t e0 = __shfl_sync(0xffffffffu, rs, 0), e1 = __shfl_sync(0xffffffffu, re, 31);
+    na_load(nx, colind, val, e0, na_count(e0, e1), lane);
+  }
+  while (i - lane < n) {
+    const int in = i + stride;   // at most 2 * ICCG_NOALLOC_MAX_ROWS
+    const bool more = in - lane < n;
+    const int64_t rsn = more ? rowptr[min(in, n)] : 0, ren = more ? rowptr[min(in + 1, n)] : 0;
+    const int64_t e0 = __shfl_sync(0xffffffffu, rs, 0), e1 = __shfl_sync(0xffffffffu, re, 31);
+    const double pi = i < n ? p[i] : 0.0;
     double sum = 0.0;
-    for (int64_t e = rowptr[i]; e < rowptr[i + 1]; ++e) sum += val[e] * p[colind[e]];
-    q[i] = sum;
-    acc = p[i] * sum;
+    for (int64_t b = e0;; b += kNaChunk) {
+      const int cnt = na_count(b, e1);
+      if (b > e0) na_load(nx, colind, val, b, cnt, lane);
+      __syncwarp();   // every lane is done with the previous chunk
+#pragma unroll
+      for (int u = 0; u < kNaChunk / 32; ++u) {
+        sc[u * 32 + lane] = nx.c[u];
+        sv[u * 32 + lane] = nx.v[u];
+      }
+      __syncwarp();
+      if (b + kNaChunk >= e1 && more) {
+        const int64_t f0 = __shfl_sync(0xffffffffu, rsn, 0), f1 = __shfl_sync(0xffffffffu, ren, 31);
+        na_load(nx, colind, val, f0, na_count(f0, f1), lane);
+      }
+      const int lo = int(rs > b ? (rs - b < cnt ? rs - b : cnt) : 0);
+      const int hi = int(re > b ? (re - b < cnt ? re - b : cnt) : 0);
+      for (int k0 = lo; k0 < hi; k0 += kNaBatch) {
+        double x[kNaBatch];
+#pragma unroll
+        for (int u = 0; u < kNaBatch; ++u) x[u] = k0 + u < hi ? p[sc[k0 + u]] : 0.0;
+#pragma unroll
+        for (int u = 0; u < kNaBatch; ++u)
+          if (k0 + u < hi) sum += sv[k0 + u] * x[u];
+      }
+      if (b + kNaChunk >= e1) break;
+    }
+    if (i < n) {
+      q[i] = sum;
+      acc += pi * sum;
+    }
+    rs = rsn;
+    re = ren;
+    i = in;
   }
   const double cta = na_cta_sum(acc, red);
   const int g = blockIdx.x / kNaGroup;
@@ -133,13 +215,11 @@ extern "C" iccg_status iccg_spmv_dot_noalloc(int32_t n, const int64_t *rowptr, c
     s = g_na_ptr[dev];
   }
   if (n == 0) return cudaMemsetAsync(pq, 0, sizeof(double), st) == cudaSuccess ? ICCG_OK : ICCG_ERR_CUDA;
-  const int grid = (n + kNaRowsPerCta - 1) / kNaRowsPerCta;
-  const int ngroups = (grid + kNaGroup - 1) / kNaGroup;
+  const int grid = std::min((n + kNaRowsPerCta - 1) / kNaRowsPerCta, kNaGrid);
   // the arrival counters must start at zero; the previous call left them at
   // their final counts
-  if (cudaMemsetAsync(s->gticket, 0, sizeof(unsigned int) * size_t(ngroups), st) != cudaSuccess ||
-      cudaMemsetAsync(&s->ticket, 0, sizeof(unsigned int), st) != cudaSuccess)
-    return ICCG_ERR_CUDA;
+  // (one memset over both, adjacent: a second one cost 2 us per call)
+  if (cudaMemsetAsync(s->gticket, 0, sizeof(s->gticket) + sizeof(s->ticket), st) != cudaSuccess) return ICCG_ERR_CUDA;
   // the launch's own status (cudaGetLastError would also report, and clear,
   // an error that earlier unrelated work of the caller left pending)
   cudaLaunchConfig_t cfg = {};
