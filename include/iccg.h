@@ -268,11 +268,11 @@ void iccg_destroy(iccg_ctx *ctx);
  *                      a system whose wait runs out stops and its right-hand
  *                      sides report ICCG_ERR_TIMEOUT; the batch stays usable.
  *   iccg_batch_info    out[7]: warps per CTA, CTAs per SM, grid, padded nrhs,
- *                      largest block, 3 x the exponent e of the CTA split
- *                      (CTAs per system proportional to n^e; e = 1 or 4/3,
- *                      chosen by the tuner with the shape), rows per thread
- *                      (consecutive rows a chain of right-hand-side lanes takes
- *                      per pass of the SpMV and the p update).
+ *                      largest block, 3 x the CTA split (3: CTAs per system
+ *                      in proportion to its rows; 4, the default: to rows x
+ *                      estimated iterations; chosen by the tuner with the
+ *                      shape), rows per thread (rows a chain of
+ *                      right-hand-side lanes has in flight in the SpMV).
  * The paper has no batched solver; this serves many independent systems
  * (e.g. the learned-blocking sweep) and multiple right-hand sides.
  * ------------------------------------------------------------------------ */

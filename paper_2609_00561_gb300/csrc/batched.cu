@@ -11,16 +11,17 @@
 // rows; a matrix or factor entry is loaded once per chain and broadcast to
 // its lanes, and every vector access of the chain is one coalesced line.
 //
-// Schedule.  The grid is split into per-system CTA ranges (proportional to
-// the system's rows, at least one CTA each); a system's CTAs synchronise
+// Schedule.  The grid is split into per-system CTA ranges (assign_ctas, at
+// least one CTA each); a system's CTAs synchronise
 // only among themselves (a bounded-wait barrier per system), so systems
 // progress independently.  Per iteration and system: p update | SpMV and
-// <p,q> | forward colors (x / r update fused, the last color's backward
-// sweep fused) | backward colors | reduction, with a barrier after each
-// phase (2 n_c + 2).  A chain owns a whole block at a time: its rows are
-// resolved in order (Alg. 1), the block's earlier (later) results in the
-// chain's shared-memory scratch.  Reductions are per right-hand side, per
-// CTA, summed in a fixed order by every CTA of the system after a barrier.
+// <p,q> | x / r update | forward colors (the last color's backward sweep
+// fused) | backward colors | reduction, with a barrier after each
+// phase (2 n_c + 3).  A warp owns a whole block at a time (batch_precond):
+// everything but the in-block recurrence is done for all rows at once, the
+// recurrence itself (rows in order, Alg. 1) on shared memory only.  Reductions
+// are per right-hand side, per CTA, summed in a fixed order by every CTA of the
+// system after a barrier.
 // A right-hand side that converged (or met a non-finite value) is frozen.
 #include <algorithm>
 #include <chrono>
@@ -35,6 +36,7 @@ namespace iccg {
 namespace {
 
 constexpr int kBatchMaxBlock = 64;   // rows of a block (a chain's scratch in shared memory)
+constexpr int kBatchCap = 512;       // most entries a warp stages (6 KB)
 constexpr long long kBatchSpinLimit = 1ll << 27;
 
 struct BatchSys {
@@ -116,81 +118,279 @@ __device__ __forceinline__ bool sys_sync(GridBar *bar, unsigned nct, unsigned &g
   return *flag != 0;
 }
 
+// Exact float -> double by bit arithmetic (about 8 integer instructions, 3
+// cycles of an SM per warp against 16 for the conversion instruction, which
+// shares this GPU's scarce FP64 rate); subnormals, infinities and NaN take the
+// instruction.
+__device__ __forceinline__ double widen(float f) {
+  const unsigned b = __float_as_uint(f), m = b & 0x7fffffffu;
+  if (m - 0x00800000u >= 0x7f000000u && m != 0u) return double(f);
+  return __hiloint2double(int((b & 0x80000000u) | (m ? (m >> 3) + 0x38000000u : 0u)), int(b << 29));
+}
+__device__ __forceinline__ double widen(double d) { return d; }
+
 // Per-right-hand-side CTA sum: every lane holds v for its (chain, j); the
-// sums over the CTA's chains (fixed order) go to part[lc][slot][j].
-__device__ __forceinline__ void cta_rhs_sum(double v, double *red, int kp, int nchain, double *part_slot) {
-  const int j = threadIdx.x % kp, ch = threadIdx.x / kp;
+// sums over the CTA's chains (fixed order) go to part_slot[j]: over a warp's
+// chains by shuffles, then over the warps.
+__device__ __forceinline__ void cta_rhs_sum(double v, double *red, int kp, double *part_slot) {
+  for (int o = 16; o >= kp; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, W = blockDim.x >> 5;
   __syncthreads();
-  red[ch * kp + j] = v;
+  if (lane < kp) red[w * kp + lane] = v;
   __syncthreads();
   if (threadIdx.x < kp) {
     double s = 0.0;
-    for (int c = 0; c < nchain; ++c) s += red[c * kp + threadIdx.x];
+    for (int c = 0; c < W; ++c) s += red[c * kp + threadIdx.x];
     part_slot[threadIdx.x] = s;
   }
 }
 
-// Sum over the system's CTAs of part[.][slot][j] (fixed order) into
-// out[j], j < kp; every CTA computes the same values.
-__device__ __forceinline__ void sys_rhs_sum(const double *part, int nct, int kp, int slot, double *out) {
+// Sum over the system's CTAs of part[.][slot][j] (fixed order) into out[j],
+// j < kp; every CTA computes the same values.  The CTA's chains take the CTAs
+// in turn (their loads in flight together: one thread per j walking them took
+// 10 us for 100 CTAs), then one thread per j adds the chains' sums.
+__device__ __forceinline__ void sys_rhs_sum(const double *part, int nct, int kp, int slot, double *out, double *red) {
+  const int ch = threadIdx.x / kp, j = threadIdx.x % kp, nchain = blockDim.x / kp;
+  const int used = min(nchain, 16);
+  __syncthreads();
+  if (ch < used) {
+    double s = 0.0;
+#pragma unroll 8
+    for (int c = ch; c < nct; c += used) s += __ldcg(part + (size_t(c) * 4 + slot) * kp + j);
+    red[ch * kp + j] = s;
+  }
   __syncthreads();
   if (threadIdx.x < kp) {
     double s = 0.0;
-    for (int c = 0; c < nct; ++c) s += __ldcg(part + (size_t(c) * 4 + slot) * kp + threadIdx.x);
+    for (int c = 0; c < used; ++c) s += red[c * kp + threadIdx.x];
     out[threadIdx.x] = s;
   }
   __syncthreads();
 }
 
-// One substitution pass of a system (UPDATE: with the x / r update in front
-// of the forward sweep).  A chain owns a block at a time; w is the chain's
-// scratch (block rows x kp).
-template <typename PT, bool UPDATE>
-__device__ __forceinline__ bool batch_precond(const BatchSys &S, PT *w, int kp, int j, int gc, int total,
-                                              double alpha, bool act, double &rr, double &rz, unsigned nct,
-                                              unsigned &gen, int *flag) {
-  const PT *lv = b_lv<PT>(S), *uv = b_uv<PT>(S), *dv = b_dv<PT>(S);
-  PT *y = reinterpret_cast<PT *>(S.y);
-  PT *z = reinterpret_cast<PT *>(S.z);
+// A warp's shared memory: w (row values of the current block, one per
+// right-hand side), the block's 1/L_ii, row pointers and the in-block / other-
+// color boundary of every row, and its entries (col, val; val holds PT in the
+// substitutions, double in the SpMV), cap of them; a range with more entries
+// is read from global memory.
+constexpr int kSpmvRows = 16;   // rows of a warp's SpMV tile
+struct BatchSmem {
+  int o_dv, o_val, o_col, o_rp, o_sp, bytes;
+};
+__host__ __device__ inline BatchSmem batch_smem_plan(int smax, int kp, int cap, int elem) {
+  const int rows = smax > kSpmvRows ? smax : kSpmvRows;
+  BatchSmem m;
+  int o = r16b(smax * kp * elem);
+  m.o_dv = o; o += r16b(smax * elem);
+  m.o_val = o; o += r16b(cap * 8);
+  m.o_col = o; o += r16b(cap * 4);
+  m.o_rp = o; o += r16b((rows + 1) * 4);
+  m.o_sp = o; o += r16b(rows * 4);
+  m.bytes = o;
+  return m;
+}
+
+// The block (or SpMV tile) a warp works on: rows [r0, r0 + nr), entries from
+// e0; in shared memory when staged (index entry - e0).
+template <typename VT>
+struct BatchRows {
+  int r0, nr, e0;
+  bool staged;
+  const int32_t *gcol;
+  const VT *gval;
+  const int32_t *scol;
+  const VT *sval;
+  const int32_t *rp;   // rp[k]: first entry of row r0 + k, from e0
+  __device__ __forceinline__ int col(int e) const { return staged ? scol[e] : __ldg(gcol + e0 + e); }
+  __device__ __forceinline__ VT val(int e) const { return staged ? sval[e] : __ldg(gval + e0 + e); }
+};
+
+template <typename VT>
+__device__ __forceinline__ BatchRows<VT> stage_rows(const int32_t *rp, const int32_t *col, const VT *val, int r0,
+                                                    int r1, unsigned char *sm, const BatchSmem &m, int cap, int lane) {
+  BatchRows<VT> b;
+  b.r0 = r0;
+  b.nr = r1 - r0;
+  b.e0 = __ldg(rp + r0);
+  const int ne = __ldg(rp + r1) - b.e0;
+  b.staged = ne <= cap;
+  b.gcol = col;
+  b.gval = val;
+  int32_t *sc = reinterpret_cast<int32_t *>(sm + m.o_col), *srp = reinterpret_cast<int32_t *>(sm + m.o_rp);
+  VT *sv = reinterpret_cast<VT *>(sm + m.o_val);
+  for (int k = lane; k <= b.nr; k += kWarp) srp[k] = __ldg(rp + r0 + k) - b.e0;
+  if (b.staged) {
+#pragma unroll 4
+    for (int e = lane; e < ne; e += kWarp) {
+      sc[e] = __ldg(col + b.e0 + e);
+      sv[e] = __ldg(val + b.e0 + e);
+    }
+  }
+  b.scol = sc;
+  b.sval = sv;
+  b.rp = srp;
+  return b;
+}
+
+// block blk of a substitution: its rows staged with 1/L_ii and, per row, the
+// first entry past the other colors (L) or past the block (U)
+template <typename PT, bool UPPER>
+__device__ __forceinline__ BatchRows<PT> stage_block(const BatchSys &S, int blk, unsigned char *sm,
+                                                     const BatchSmem &m, int cap, int lane) {
+  __syncwarp();   // the previous block's readers are done
+  const int r0 = __ldg(S.bptr + blk), r1 = __ldg(S.bptr + blk + 1);
+  const BatchRows<PT> b = UPPER ? stage_rows<PT>(S.urp, S.ucol, b_uv<PT>(S), r0, r1, sm, m, cap, lane)
+                                : stage_rows<PT>(S.lrp, S.lcol, b_lv<PT>(S), r0, r1, sm, m, cap, lane);
+  PT *sdv = reinterpret_cast<PT *>(sm + m.o_dv);
+  int32_t *ssp = reinterpret_cast<int32_t *>(sm + m.o_sp);
+  for (int k = lane; k < b.nr; k += kWarp) sdv[k] = __ldg(b_dv<PT>(S) + r0 + k);
+  __syncwarp();
+  for (int k = lane; k < b.nr; k += kWarp) {
+    int e = b.rp[k];
+    const int e1 = b.rp[k + 1], bound = UPPER ? r1 : r0;
+    while (e < e1 && b.col(e) < bound) ++e;
+    ssp[k] = e;
+  }
+  __syncwarp();
+  return b;
+}
+
+constexpr int kBatchRowsU = 4;   // rows a chain has in flight
+
+// The rows' sources (r forward, y backward) minus their entries to other colors
+// into w.  A chain takes every NC-th row, kBatchRowsU of them in flight.
+template <typename PT, bool UPPER>
+__device__ __forceinline__ void block_other(const BatchSys &S, const BatchRows<PT> &b, PT *w, const int32_t *ssp, int kp,
+                                            int j, int ch, int NC) {
+  const PT *y = reinterpret_cast<const PT *>(S.y);
+  const PT *g = UPPER ? reinterpret_cast<const PT *>(S.z) : y;
+  for (int k0 = ch; k0 < b.nr; k0 += NC * kBatchRowsU) {
+    int e[kBatchRowsU], len[kBatchRowsU], most = 0;
+    PT acc[kBatchRowsU], x[kBatchRowsU][3];
+    double ri[kBatchRowsU];
+#pragma unroll
+    for (int u = 0; u < kBatchRowsU; ++u) {
+      const int k = k0 + u * NC;
+      const size_t at = size_t(b.r0 + k) * kp + j;
+      const bool ok = k < b.nr;
+      if (UPPER) acc[u] = ok ? __ldcg(y + at) : PT(0);
+      else ri[u] = ok ? __ldcg(S.r + at) : 0.0;
+      e[u] = ok ? (UPPER ? ssp[k] : b.rp[k]) : 0;
+      len[u] = ok ? (UPPER ? b.rp[k + 1] : ssp[k]) - e[u] : 0;
+      most = max(most, len[u]);
+    }
+#pragma unroll
+    for (int u = 0; u < kBatchRowsU; ++u)
+#pragma unroll
+      for (int i = 0; i < 3; ++i)
+        x[u][i] = i < len[u] ? __ldcg(g + size_t(b.col(e[u] + i)) * kp + j) : PT(0);
+#pragma unroll
+    for (int u = 0; u < kBatchRowsU; ++u) {
+      if (!UPPER) acc[u] = PT(ri[u]);
+#pragma unroll
+      for (int i = 0; i < 3; ++i)
+        if (i < len[u]) acc[u] -= b.val(e[u] + i) * x[u][i];
+    }
+    for (int t = 3; t < most; t += 3) {
+#pragma unroll
+      for (int u = 0; u < kBatchRowsU; ++u)
+#pragma unroll
+        for (int i = 0; i < 3; ++i)
+          x[u][i] = t + i < len[u] ? __ldcg(g + size_t(b.col(e[u] + t + i)) * kp + j) : PT(0);
+#pragma unroll
+      for (int u = 0; u < kBatchRowsU; ++u)
+#pragma unroll
+        for (int i = 0; i < 3; ++i)
+          if (t + i < len[u]) acc[u] -= b.val(e[u] + t + i) * x[u][i];
+    }
+#pragma unroll
+    for (int u = 0; u < kBatchRowsU; ++u)
+      if (k0 + u * NC < b.nr) w[(k0 + u * NC) * kp + j] = acc[u];
+  }
+}
+
+// The in-block recurrence, rows in order (forward) or in reverse (backward),
+// by one chain on shared memory; a lane reads only its own right-hand side.
+template <typename PT, bool UPPER>
+__device__ __forceinline__ void block_chain(const BatchRows<PT> &b, PT *w, const PT *sdv, const int32_t *ssp, int kp,
+                                            int j) {
+  for (int q = 0; q < b.nr; ++q) {
+    const int k = UPPER ? b.nr - 1 - q : q;
+    PT acc = w[k * kp + j];
+    const int e1 = UPPER ? ssp[k] : b.rp[k + 1];
+    for (int e = UPPER ? b.rp[k] : ssp[k]; e < e1; ++e) acc -= b.val(e) * w[(b.col(e) - b.r0) * kp + j];
+    w[k * kp + j] = acc * sdv[k];
+  }
+}
+
+// the block's results from w: y (stored when `store`) and its share of <y, y>
+// forward, z backward
+template <typename PT, bool UPPER>
+__device__ __forceinline__ void block_store(const BatchSys &S, const BatchRows<PT> &b, const PT *w, int kp, int j,
+                                            int ch, int NC, bool store, double &yy) {
+  PT *res = reinterpret_cast<PT *>(UPPER ? S.z : S.y);
+  for (int k = ch; k < b.nr; k += NC) {
+    const PT v = w[k * kp + j];
+    if (store) res[size_t(b.r0 + k) * kp + j] = v;
+    if (!UPPER) {
+      const double d = widen(v);
+      yy += d * d;
+    }
+  }
+}
+
+// One substitution pass of a system; yy receives the warp's share of <y, y>,
+// y = L^-1 r, which is <r, z> (z = L^-T y): the backward sweep need not read r.
+// A warp owns a block at a time and works in three parts: every row minus its entries to other colors (block_other: all chains
+// of the warp, several rows each in flight), the in-block recurrence
+// (block_chain: shared memory only), the results (block_store).  The block's
+// static data is staged ahead; the first block of the next color before the
+// barrier that ends the current one.
+//
+// Bound by latency: a chain that walked its block row by row paid two to three
+// dependent L2 loads for each of 32 rows, 60-120 us for a color phase; split
+// so, a phase costs a few such trips (8 systems of sides 16..64, 16 right-hand
+// sides, FP32: 155 ms with the walk, 85 ms so; 3 systems of sides 21..57, 4
+// right-hand sides, FP64: 102 against 19 ms).  What remains is still latency: a
+// color of one system has fewer blocks than its CTAs have warps.
+template <typename PT>
+__device__ __forceinline__ bool batch_precond(const BatchSys &S, unsigned char *sm, const BatchSmem &m, int cap, int kp,
+                                              int gw, int total, double &yy, unsigned nct, unsigned &gen, int *flag) {
+  const int lane = threadIdx.x & 31, j = lane % kp, ch = lane / kp, NC = kWarp / kp;
+  PT *w = reinterpret_cast<PT *>(sm);
+  const PT *sdv = reinterpret_cast<const PT *>(sm + m.o_dv);
+  const int32_t *ssp = reinterpret_cast<const int32_t *>(sm + m.o_sp);
   const int nc = S.nc;
+  BatchRows<PT> b;
+  int blk = __ldg(S.cblk) + gw;
+  bool have = blk < __ldg(S.cblk + 1);
+  if (have) b = stage_block<PT, false>(S, blk, sm, m, cap, lane);
   for (int c = 0; c < nc; ++c) {
     const bool last = c == nc - 1;
     const int b1 = __ldg(S.cblk + c + 1);
-    for (int blk = __ldg(S.cblk + c) + gc; blk < b1; blk += total) {
-      const int r0 = __ldg(S.bptr + blk), r1 = __ldg(S.bptr + blk + 1);
-      for (int i = r0; i < r1; ++i) {
-        double ri = __ldcg(S.r + size_t(i) * kp + j);
-        if (UPDATE && act) {
-          ri -= alpha * __ldcg(S.q + size_t(i) * kp + j);
-          S.r[size_t(i) * kp + j] = ri;
-          S.x[size_t(i) * kp + j] = __ldcg(S.x + size_t(i) * kp + j) + alpha * __ldcg(S.p + size_t(i) * kp + j);
-          rr += ri * ri;
-        }
-        PT acc = PT(ri);
-        const int e1 = __ldg(S.lrp + i + 1);
-        for (int e = __ldg(S.lrp + i); e < e1; ++e) {
-          const int col = __ldg(S.lcol + e);
-          const PT v = __ldg(lv + e);
-          const PT yc = col >= r0 ? w[(col - r0) * kp + j] : __ldcg(y + size_t(col) * kp + j);
-          acc -= v * yc;
-        }
-        const PT yi = acc * __ldg(dv + i);
-        w[(i - r0) * kp + j] = yi;
-        if (!last) y[size_t(i) * kp + j] = yi;
-      }
+    while (have) {
+      block_other<PT, false>(S, b, w, ssp, kp, j, ch, NC);
+      __syncwarp();
+      if (ch == 0) block_chain<PT, false>(b, w, sdv, ssp, kp, j);
+      __syncwarp();
+      block_store<PT, false>(S, b, w, kp, j, ch, NC, !last, yy);
       if (last) {
         // the last color: backward sweep of the same block at once (no
-        // later colors), y in the scratch
-        for (int i = r1 - 1; i >= r0; --i) {
-          PT acc = w[(i - r0) * kp + j];
-          const int e1 = __ldg(S.urp + i + 1);
-          for (int e = __ldg(S.urp + i); e < e1; ++e) acc -= __ldg(uv + e) * w[(__ldg(S.ucol + e) - r0) * kp + j];
-          const PT zi = acc * __ldg(dv + i);
-          w[(i - r0) * kp + j] = zi;
-          z[size_t(i) * kp + j] = zi;
-          rz += __ldcg(S.r + size_t(i) * kp + j) * double(zi);
-        }
+        // later colors), y in w
+        b = stage_block<PT, true>(S, blk, sm, m, cap, lane);
+        if (ch == 0) block_chain<PT, true>(b, w, sdv, ssp, kp, j);
+        __syncwarp();
+        block_store<PT, true>(S, b, w, kp, j, ch, NC, true, yy);
       }
+      blk += total;
+      have = blk < b1;
+      if (have) b = stage_block<PT, false>(S, blk, sm, m, cap, lane);
+    }
+    const int cn = last ? nc - 2 : c + 1;
+    if (cn >= 0) {
+      blk = __ldg(S.cblk + cn) + gw;
+      have = blk < __ldg(S.cblk + cn + 1);
+      if (have) b = last ? stage_block<PT, true>(S, blk, sm, m, cap, lane) : stage_block<PT, false>(S, blk, sm, m, cap, lane);
     }
     // every color's results (for the last color: its z) complete before the
     // next color reads them
@@ -198,31 +398,96 @@ __device__ __forceinline__ bool batch_precond(const BatchSys &S, PT *w, int kp, 
   }
   for (int c = nc - 2; c >= 0; --c) {
     const int b1 = __ldg(S.cblk + c + 1);
-    for (int blk = __ldg(S.cblk + c) + gc; blk < b1; blk += total) {
-      const int r0 = __ldg(S.bptr + blk), r1 = __ldg(S.bptr + blk + 1);
-      for (int i = r1 - 1; i >= r0; --i) {
-        PT acc = __ldcg(y + size_t(i) * kp + j);
-        const int e1 = __ldg(S.urp + i + 1);
-        for (int e = __ldg(S.urp + i); e < e1; ++e) {
-          const int col = __ldg(S.ucol + e);
-          const PT zc = col < r1 ? w[(col - r0) * kp + j] : __ldcg(z + size_t(col) * kp + j);
-          acc -= __ldg(uv + e) * zc;
-        }
-        const PT zi = acc * __ldg(dv + i);
-        w[(i - r0) * kp + j] = zi;
-        z[size_t(i) * kp + j] = zi;
-        rz += __ldcg(S.r + size_t(i) * kp + j) * double(zi);
-      }
+    while (have) {
+      block_other<PT, true>(S, b, w, ssp, kp, j, ch, NC);
+      __syncwarp();
+      if (ch == 0) block_chain<PT, true>(b, w, sdv, ssp, kp, j);
+      __syncwarp();
+      block_store<PT, true>(S, b, w, kp, j, ch, NC, true, yy);
+      blk += total;
+      have = blk < b1;
+      if (have) b = stage_block<PT, true>(S, blk, sm, m, cap, lane);
     }
-    if (c > 0 && !sys_sync(S.bar, nct, gen, flag, S.wait_ns)) return false;
+    if (c > 0) {
+      blk = __ldg(S.cblk + c - 1) + gw;
+      have = blk < __ldg(S.cblk + c);
+      if (have) b = stage_block<PT, true>(S, blk, sm, m, cap, lane);
+      if (!sys_sync(S.bar, nct, gen, flag, S.wait_ns)) return false;
+    }
   }
   return true;
 }
 
-// R: rows per chain and pass of the SpMV and the p update (1, 2 or 4)
+// A times a [n][kp] vector, a warp per tile of kSpmvRows rows whose entries are
+// staged coalesced, a chain per row, R rows of a chain in flight (8 entries each
+// at R = 1 or 2, 4 at R = 4).  INIT: r = r - A x (r holds b), returns the share of <r, r>;
+// else q = A p, the share of <p, q>.
+template <int R, bool INIT>
+__device__ __forceinline__ double batch_spmv(const BatchSys &S, unsigned char *sm, const BatchSmem &m, int cap, int kp,
+                                             int gw, int total, bool act) {
+  constexpr int E = R < 4 ? 8 : 4;
+  const int lane = threadIdx.x & 31, j = lane % kp, ch = lane / kp, NC = kWarp / kp;
+  const double *v = INIT ? S.x : S.p;
+  const int ntile = (S.n + kSpmvRows - 1) / kSpmvRows;
+  double acc = 0.0;
+  for (int t = gw; t < ntile; t += total) {
+    __syncwarp();
+    const int r0 = t * kSpmvRows, r1 = min(S.n, r0 + kSpmvRows);
+    const BatchRows<double> b = stage_rows<double>(S.arp, S.acol, S.aval, r0, r1, sm, m, cap, lane);
+    __syncwarp();
+    if (!act) continue;
+    for (int k0 = ch; k0 < b.nr; k0 += NC * R) {
+      int e[R], len[R], most = 0;
+      double s[R], own[R], rb[R];
+#pragma unroll
+      for (int u = 0; u < R; ++u) {
+        const int k = k0 + u * NC;
+        const bool ok = k < b.nr;
+        e[u] = ok ? b.rp[k] : 0;
+        len[u] = ok ? b.rp[k + 1] - e[u] : 0;
+        most = max(most, len[u]);
+        s[u] = 0.0;
+        const size_t at = size_t(b.r0 + k) * kp + j;
+        own[u] = ok && !INIT ? __ldcg(v + at) : 0.0;
+        rb[u] = ok && INIT ? __ldcg(S.r + at) : 0.0;
+      }
+      for (int t0 = 0; t0 < most; t0 += E) {
+        double x[R][E];
+#pragma unroll
+        for (int u = 0; u < R; ++u)
+#pragma unroll
+          for (int i = 0; i < E; ++i)
+            x[u][i] = t0 + i < len[u] ? __ldcg(v + size_t(b.col(e[u] + t0 + i)) * kp + j) : 0.0;
+#pragma unroll
+        for (int u = 0; u < R; ++u)
+#pragma unroll
+          for (int i = 0; i < E; ++i)
+            if (t0 + i < len[u]) s[u] += b.val(e[u] + t0 + i) * x[u][i];
+      }
+#pragma unroll
+      for (int u = 0; u < R; ++u) {
+        const int k = k0 + u * NC;
+        if (k >= b.nr) continue;
+        const size_t at = size_t(b.r0 + k) * kp + j;
+        if (INIT) {
+          const double ri = rb[u] - s[u];
+          S.r[at] = ri;
+          acc += ri * ri;
+        } else {
+          S.q[at] = s[u];
+          acc += own[u] * s[u];
+        }
+      }
+    }
+  }
+  return acc;
+}
+
+// R: rows of a chain in flight in the SpMV (1, 2 or 4)
 template <typename PT, int R>
 __global__ void __launch_bounds__(kMaxWarpsPerCta * kWarp, 1)
-batch_kernel(const BatchSys *sys, const int32_t *cta_sys, int k, int kp, int smax, int maxit, double tol) {
+batch_kernel(const BatchSys *sys, const int32_t *cta_sys, int k, int kp, BatchSmem plan, int cap, int maxit,
+             double tol) {
   extern __shared__ __align__(16) unsigned char smem[];
   __shared__ BatchSys S;
   __shared__ int flag;
@@ -237,8 +502,10 @@ batch_kernel(const BatchSys *sys, const int32_t *cta_sys, int k, int kp, int sma
   const int lc = blockIdx.x - S.cta0;
   const unsigned nct = unsigned(S.cta1 - S.cta0);
   const int gc = lc * nchain + ch, total = int(nct) * nchain;
-  PT *w = reinterpret_cast<PT *>(smem) + size_t(ch) * smax * kp;
-  double *red = reinterpret_cast<double *>(smem + size_t(nchain) * smax * kp * sizeof(PT));
+  const int W = blockDim.x / kWarp, warp = threadIdx.x / kWarp;
+  const int gw = lc * W + warp, totalw = int(nct) * W;
+  unsigned char *wsm = smem + size_t(warp) * plan.bytes;
+  double *red = reinterpret_cast<double *>(smem + size_t(W) * plan.bytes);
   double *mypart = S.part + size_t(lc) * 4 * kp;
   const int n = S.n;
   unsigned gen = 0;
@@ -255,35 +522,26 @@ batch_kernel(const BatchSys *sys, const int32_t *cta_sys, int k, int kp, int sma
     S.p[size_t(i) * kp + j] = 0.0;
     acc += bi * bi;
   }
-  cta_rhs_sum(acc, red, kp, nchain, mypart + 0 * kp);
+  cta_rhs_sum(acc, red, kp, mypart + 0 * kp);
   ok = sys_sync(S.bar, nct, gen, &flag, S.wait_ns);
   // r0 = b - A x0, <r0, r0> (a row's b is read and r written by its own lane)
   if (ok) {
-    acc = 0.0;
-    for (int i = gc; i < n; i += total) {
-      double s = 0.0;
-      const int e1 = __ldg(S.arp + i + 1);
-      for (int e = __ldg(S.arp + i); e < e1; ++e)
-        s += __ldg(S.aval + e) * __ldcg(S.x + size_t(__ldg(S.acol + e)) * kp + j);
-      const double ri = __ldcg(S.r + size_t(i) * kp + j) - s;
-      S.r[size_t(i) * kp + j] = ri;
-      acc += ri * ri;
-    }
-    cta_rhs_sum(acc, red, kp, nchain, mypart + 1 * kp);
+    acc = batch_spmv<R, true>(S, wsm, plan, cap, kp, gw, totalw, true);
+    cta_rhs_sum(acc, red, kp, mypart + 1 * kp);
     ok = sys_sync(S.bar, nct, gen, &flag, S.wait_ns);
   }
   // z0 = M^-1 r0, <r0, z0>
   double rr = 0.0, rz = 0.0;
-  if (ok) ok = batch_precond<PT, false>(S, w, kp, j, gc, total, 0.0, false, rr, rz, nct, gen, &flag);
+  if (ok) ok = batch_precond<PT>(S, wsm, plan, cap, kp, gw, totalw, rz, nct, gen, &flag);
   if (ok) {
-    cta_rhs_sum(rz, red, kp, nchain, mypart + 3 * kp);
+    cta_rhs_sum(rz, red, kp, mypart + 3 * kp);
     ok = sys_sync(S.bar, nct, gen, &flag, S.wait_ns);
   }
   int it = 0;
   if (ok) {
-    sys_rhs_sum(S.part, int(nct), kp, 0, sv[0]);
-    sys_rhs_sum(S.part, int(nct), kp, 1, sv[1]);
-    sys_rhs_sum(S.part, int(nct), kp, 3, sv[3]);
+    sys_rhs_sum(S.part, int(nct), kp, 0, sv[0], red);
+    sys_rhs_sum(S.part, int(nct), kp, 1, sv[1], red);
+    sys_rhs_sum(S.part, int(nct), kp, 3, sv[3], red);
     if (threadIdx.x < kp) {
       const int t = threadIdx.x;
       const double bn = sqrt(sv[0][t]);
@@ -318,77 +576,65 @@ batch_kernel(const BatchSys *sys, const int32_t *cta_sys, int k, int kp, int sma
     const double beta = st_beta[j];
     // p = z + beta p
     const PT *z = reinterpret_cast<const PT *>(S.z);
-    // R consecutive rows per chain and pass: their loads are issued together
-    if (act && R == 1) {
-      for (int i = gc; i < n; i += total)
-        S.p[size_t(i) * kp + j] = double(__ldcg(z + size_t(i) * kp + j)) + beta * __ldcg(S.p + size_t(i) * kp + j);
-    } else if (act) {
-      for (int i0 = gc * R; i0 < n; i0 += total * R) {
-        double zz[R], pp[R];
+    // (kBatchRowsU rows of a chain in flight)
+    if (act) {
+      for (int i0 = gc; i0 < n; i0 += total * kBatchRowsU) {
+        double zz[kBatchRowsU], pp[kBatchRowsU];
 #pragma unroll
-        for (int u = 0; u < R; ++u)
-          if (i0 + u < n) {
-            zz[u] = double(__ldcg(z + size_t(i0 + u) * kp + j));
-            pp[u] = __ldcg(S.p + size_t(i0 + u) * kp + j);
-          }
+        for (int u = 0; u < kBatchRowsU; ++u) {
+          const int i = i0 + u * total;
+          zz[u] = i < n ? widen(__ldcg(z + size_t(i) * kp + j)) : 0.0;
+          pp[u] = i < n ? __ldcg(S.p + size_t(i) * kp + j) : 0.0;
+        }
 #pragma unroll
-        for (int u = 0; u < R; ++u)
-          if (i0 + u < n) S.p[size_t(i0 + u) * kp + j] = zz[u] + beta * pp[u];
+        for (int u = 0; u < kBatchRowsU; ++u)
+          if (i0 + u * total < n) S.p[size_t(i0 + u * total) * kp + j] = zz[u] + beta * pp[u];
       }
     }
     if (!(ok = sys_sync(S.bar, nct, gen, &flag, S.wait_ns))) break;
     // q = A p, <p, q>
-    acc = 0.0;
-    if (act && R == 1) {
-      for (int i = gc; i < n; i += total) {
-        double s = 0.0;
-        const int e1 = __ldg(S.arp + i + 1);
-        for (int e = __ldg(S.arp + i); e < e1; ++e)
-          s += __ldg(S.aval + e) * __ldcg(S.p + size_t(__ldg(S.acol + e)) * kp + j);
-        S.q[size_t(i) * kp + j] = s;
-        acc += __ldcg(S.p + size_t(i) * kp + j) * s;
-      }
-    } else if (act) {
-      for (int i0 = gc * R; i0 < n; i0 += total * R) {
-        int e0[R], e1[R];
-        double sq[R];
-        int len = 0;
+    acc = batch_spmv<R, false>(S, wsm, plan, cap, kp, gw, totalw, act);
+    cta_rhs_sum(acc, red, kp, mypart + 2 * kp);
+    if (!(ok = sys_sync(S.bar, nct, gen, &flag, S.wait_ns))) break;
+    sys_rhs_sum(S.part, int(nct), kp, 2, sv[2], red);
+    const double alpha = act ? st_rz[j] / sv[2][j] : 0.0;
+    // x / r update and <r,r> over all rows at once (in front of each color's
+    // forward sweep, where only that color's blocks are at work, it took twice
+    // as long), then z = M^-1 r and <r,z>
+    rr = 0.0;
+    if (act) {
+      for (int i0 = gc; i0 < n; i0 += total * kBatchRowsU) {
+        double ri[kBatchRowsU], qi[kBatchRowsU], xi[kBatchRowsU], pi[kBatchRowsU];
 #pragma unroll
-        for (int u = 0; u < R; ++u) {
-          const bool v = i0 + u < n;
-          e0[u] = v ? __ldg(S.arp + i0 + u) : 0;
-          e1[u] = v ? __ldg(S.arp + i0 + u + 1) : 0;
-          sq[u] = 0.0;
-          len = max(len, e1[u] - e0[u]);
-        }
-        // the rows' t-th entries together (each row's sum in entry order)
-        for (int t = 0; t < len; ++t) {
-#pragma unroll
-          for (int u = 0; u < R; ++u)
-            if (e0[u] + t < e1[u])
-              sq[u] += __ldg(S.aval + e0[u] + t) * __ldcg(S.p + size_t(__ldg(S.acol + e0[u] + t)) * kp + j);
+        for (int u = 0; u < kBatchRowsU; ++u) {
+          const int i = i0 + u * total;
+          const size_t at = size_t(i) * kp + j;
+          ri[u] = i < n ? __ldcg(S.r + at) : 0.0;
+          qi[u] = i < n ? __ldcg(S.q + at) : 0.0;
+          xi[u] = i < n ? __ldcg(S.x + at) : 0.0;
+          pi[u] = i < n ? __ldcg(S.p + at) : 0.0;
         }
 #pragma unroll
-        for (int u = 0; u < R; ++u)
-          if (i0 + u < n) {
-            S.q[size_t(i0 + u) * kp + j] = sq[u];
-            acc += __ldcg(S.p + size_t(i0 + u) * kp + j) * sq[u];
+        for (int u = 0; u < kBatchRowsU; ++u) {
+          const int i = i0 + u * total;
+          if (i < n) {
+            const size_t at = size_t(i) * kp + j;
+            ri[u] -= alpha * qi[u];
+            S.r[at] = ri[u];
+            S.x[at] = xi[u] + alpha * pi[u];
+            rr += ri[u] * ri[u];
           }
+        }
       }
     }
-    cta_rhs_sum(acc, red, kp, nchain, mypart + 2 * kp);
     if (!(ok = sys_sync(S.bar, nct, gen, &flag, S.wait_ns))) break;
-    sys_rhs_sum(S.part, int(nct), kp, 2, sv[2]);
-    const double alpha = act ? st_rz[j] / sv[2][j] : 0.0;
-    // x / r update, z = M^-1 r, <r,r>, <r,z>
-    rr = 0.0;
     rz = 0.0;
-    if (!(ok = batch_precond<PT, true>(S, w, kp, j, gc, total, alpha, act, rr, rz, nct, gen, &flag))) break;
-    cta_rhs_sum(rr, red, kp, nchain, mypart + 1 * kp);
-    cta_rhs_sum(rz, red, kp, nchain, mypart + 3 * kp);
+    if (!(ok = batch_precond<PT>(S, wsm, plan, cap, kp, gw, totalw, rz, nct, gen, &flag))) break;
+    cta_rhs_sum(rr, red, kp, mypart + 1 * kp);
+    cta_rhs_sum(rz, red, kp, mypart + 3 * kp);
     if (!(ok = sys_sync(S.bar, nct, gen, &flag, S.wait_ns))) break;
-    sys_rhs_sum(S.part, int(nct), kp, 1, sv[1]);
-    sys_rhs_sum(S.part, int(nct), kp, 3, sv[3]);
+    sys_rhs_sum(S.part, int(nct), kp, 1, sv[1], red);
+    sys_rhs_sum(S.part, int(nct), kp, 3, sv[3], red);
     ++it;
     if (threadIdx.x < kp) {
       const int t = threadIdx.x;
@@ -446,7 +692,7 @@ cudaError_t allow_smem_b(K kernel) {
                               optin - int(fa.sharedSizeBytes) - 256);
 }
 
-using BatchKernel = void (*)(const BatchSys *, const int32_t *, int, int, int, int, double);
+using BatchKernel = void (*)(const BatchSys *, const int32_t *, int, int, BatchSmem, int, int, double);
 
 template <typename PT>
 BatchKernel batch_kernel_of(int R) {
@@ -462,6 +708,7 @@ struct iccg_batch {
   int device = 0;
   cudaStream_t stream = nullptr;
   int nsys = 0, k = 0, kp = 0, smax = 1;
+  int cap = 0;           // entries of a block or SpMV tile staged per warp
   bool fp32 = false;
   std::vector<iccg_ctx *> ctxs;
   std::vector<int32_t> n;
@@ -477,7 +724,8 @@ struct iccg_batch {
   // launch shape
   int W = 8, cps = 1, grid = 0, smem = 0, max_part_ctas = 0;
   int R = 1;             // rows per chain and pass (SpMV, p update)
-  double wexp = 1.0;     // CTAs per system proportional to n^wexp
+  double wexp = 4.0 / 3.0;     // CTAs per system: 1 by rows, 4/3 by rows x estimated iterations
+  std::vector<double> work;    // rows x estimated iterations of each system
   std::vector<int32_t> cta0;
   cudaGraph_t graph = nullptr;
   cudaGraphExec_t gexec = nullptr;
@@ -497,11 +745,9 @@ cudaError_t b_alloc(iccg_batch *b, void **p, size_t bytes) {
   return cudaMemsetAsync(*p, 0, bytes + 64, b->stream);
 }
 
-int batch_smem(const iccg_batch *b, int W) {
-  const int nchain = W * kWarp / b->kp;
-  const int elem = b->fp32 ? 4 : 8;
-  return nchain * b->smax * b->kp * elem + nchain * b->kp * 8;
-}
+BatchSmem batch_plan(const iccg_batch *b) { return batch_smem_plan(b->smax, b->kp, b->cap, b->fp32 ? 4 : 8); }
+
+int batch_smem(const iccg_batch *b, int W) { return W * batch_plan(b).bytes + W * kWarp * 8; }
 
 int batch_occupancy(const iccg_batch *b, int W, int smem) {
   int nb = 0;
@@ -522,17 +768,37 @@ void destroy_batch_graph(iccg_batch *b) {
   b->graph = nullptr;
 }
 
-// CTA ranges per system (>= 1 each) for a grid of G CTAs, proportional to
-// n^wexp: wexp = 1 spreads rows evenly, wexp = 4/3 weights rows by an
-// iteration count that grows with the grid side (CG on a discretised
-// elliptic operator needs O(sqrt kappa) = O(side) iterations); returns false
-// when G < nsys.
+// Rows times an estimate of the iterations: CG takes O(sqrt(kappa)) of them,
+// and for a discretised elliptic operator lambda_min / lambda_max is about
+// n^(-2/3) (times a constant all systems share) plus the diagonal dominance
+// delta = min_i (a_ii - sum_j |a_ij|) / a_ii that a shift adds (0.2 delta in the
+// same unit: 7-point rows give 2.5 / side^2 + delta / 2).  Only the ratio
+// between systems matters: a system's CTAs work on it alone, so the batch ends
+// when the slowest system does.
+double system_work(const HostLayout &H) {
+  double delta = 1.0;
+  for (int32_t i = 0; i < H.n; ++i) {
+    double off = 0.0, d = 0.0;
+    for (int32_t e = H.arp[i]; e < H.arp[i + 1]; ++e) {
+      if (H.acol[e] == i) d = H.aval[e];
+      else off += std::fabs(H.aval[e]);
+    }
+    delta = std::min(delta, d > 0.0 ? (d - off) / d : 0.0);
+  }
+  const double n = double(H.n);
+  return n / std::sqrt(std::pow(n, -2.0 / 3.0) + 0.2 * std::max(delta, 0.0));
+}
+
+// CTA ranges per system (>= 1 each) for a grid of G CTAs: wexp = 1 in
+// proportion to the rows, wexp = 4/3 to rows x estimated iterations (rows^(4/3)
+// without diagonal dominance); returns false when G < nsys.  8 systems of sides
+// 16..64 with shifts in [1e-4, 1e-1] need 24 to 79 iterations.
 bool assign_ctas(iccg_batch *b, int G) {
   if (G < b->nsys) return false;
   double tot = 0.0;
   std::vector<double> wt(b->nsys);
   for (int s = 0; s < b->nsys; ++s) {
-    wt[s] = std::pow(double(b->n[s]), b->wexp);
+    wt[s] = b->wexp > 1.0 ? b->work[s] : double(b->n[s]);
     tot += wt[s];
   }
   std::vector<int32_t> c(b->nsys, 1);
@@ -624,8 +890,8 @@ cudaError_t batch_launch(iccg_batch *b, cudaStream_t s, int maxit, double tol) {
   cfg.numAttrs = 1;
   const BatchSys *sys = b->d_sys;
   const int32_t *cts = b->d_cta_sys;
-  if (b->fp32) return cudaLaunchKernelEx(&cfg, batch_kernel_of<float>(b->R), sys, cts, b->k, b->kp, b->smax, maxit, tol);
-  return cudaLaunchKernelEx(&cfg, batch_kernel_of<double>(b->R), sys, cts, b->k, b->kp, b->smax, maxit, tol);
+  if (b->fp32) return cudaLaunchKernelEx(&cfg, batch_kernel_of<float>(b->R), sys, cts, b->k, b->kp, batch_plan(b), b->cap, maxit, tol);
+  return cudaLaunchKernelEx(&cfg, batch_kernel_of<double>(b->R), sys, cts, b->k, b->kp, batch_plan(b), b->cap, maxit, tol);
 }
 
 iccg_status set_shape(iccg_batch *b, int W, int cps, int sms) {
@@ -767,7 +1033,16 @@ iccg_status iccg_batch_create(iccg_batch **out, iccg_ctx *const *ctxs, int32_t n
     const iccg_ctx *c = ctxs[s];
     const size_t n = size_t(c->H.n), kp = size_t(b->kp);
     b->n.push_back(c->H.n);
-    for (int j = 0; j < c->H.n_b; ++j) b->smax = std::max(b->smax, c->H.block_ptr[j + 1] - c->H.block_ptr[j]);
+    const HostLayout &H = c->H;
+    b->work.push_back(system_work(H));
+    for (int j = 0; j < H.n_b; ++j) {
+      const int r0 = H.block_ptr[j], r1 = H.block_ptr[j + 1];
+      b->smax = std::max(b->smax, r1 - r0);
+      b->cap = std::max(b->cap, std::max(H.lrp[r1] - H.lrp[r0], H.urp[r1] - H.urp[r0]));
+    }
+    for (int r0 = 0; r0 < H.n; r0 += kSpmvRows)
+      b->cap = std::max(b->cap, H.arp[std::min(H.n, r0 + kSpmvRows)] - H.arp[r0]);
+    b->cap = std::min(b->cap, kBatchCap);
     void *v = nullptr;
     if (e == cudaSuccess && (e = b_alloc(b, &v, 8 * n * kp)) == cudaSuccess) b->x[s] = static_cast<double *>(v);
     if (e == cudaSuccess && (e = b_alloc(b, &v, 8 * n * kp)) == cudaSuccess) b->r[s] = static_cast<double *>(v);
