@@ -289,8 +289,10 @@ iccg_status iccg_setup(iccg_ctx **out, int32_t n, int64_t nnz, const int64_t *ro
   L.unit0.assign(n_c, 0);
   L.unit1.assign(n_c, 0);
   L.unit_S.assign(n_c, 0);
+  L.unit_T.assign(n_c, 0);
   L.Wu = 8;
   int32_t gbig = 1;
+  bool lane_tiles = false;
   for (int c = 0; c < n_c; ++c) {
     L.task0[c] = H.color_group[c];
     L.task1[c] = H.color_group[c + 1];
@@ -323,10 +325,13 @@ iccg_status iccg_setup(iccg_ctx **out, int32_t n, int64_t nnz, const int64_t *ro
     const int nu = L.unit1[c] - L.unit0[c];
     if (nu > 0) {
       L.wtile[c] = 3;
-      const int full = sms * unit_resident_ctas(ctx->fp32, L.unit_S[c], L.Wu * kWarp);
+      for (int u = L.unit0[c]; u < L.unit1[c]; ++u)
+        L.unit_T[c] = std::max(L.unit_T[c], std::max(H.units[size_t(u)].lt, H.units[size_t(u)].ut));
+      const int full = sms * unit_resident_ctas(ctx->fp32, L.unit_S[c], L.unit_T[c], L.Wu * kWarp);
       L.grid_c[c] = std::max(1, std::min((nu + L.Wu - 1) / L.Wu, full));
-    } else if (L.wtile[c] == 1) L.grid_c[c] = std::min((nt + L.Ww - 1) / L.Ww, wt_full);
-    else if (L.wtile[c] == 2) {
+    } else if (L.wtile[c] == 1) {
+      L.grid_c[c] = std::min((nt + L.Ww - 1) / L.Ww, wt_full);
+    } else if (L.wtile[c] == 2) {
       L.grid_c[c] = std::min((nt + L.Wp - 1) / L.Wp, pr_full);
       // a sweep stages its entries to other colors ahead of the gathers when
       // its tiles have on average at least two (over both steps), and always
@@ -343,10 +348,25 @@ iccg_status iccg_setup(iccg_ctx **out, int32_t n, int64_t nnz, const int64_t *ro
       L.pstage_f[c] = ctx->fp32 || wf >= 2 * int64_t(nt);
       L.pstage_b[c] = ctx->fp32 || wb >= 2 * int64_t(nt);
     }
-    else L.grid_c[c] = nt > 0 ? std::min(nt, L.stage_ext[c] ? tile_full_x : tile_full)
-                              : std::max(1, L.task1[c] - L.task0[c]);
+    else if (nt > 0) {
+      L.grid_c[c] = std::min(nt, L.stage_ext[c] ? tile_full_x : tile_full);
+    } else {
+      L.grid_c[c] = std::max(1, L.task1[c] - L.task0[c]);
+    }
     gbig = std::max(gbig, L.grid_c[c]);
+    lane_tiles = lane_tiles || L.wtile[c] == 0 || L.wtile[c] == 1;
   }
+  // Lane-tile kernels take more shared memory than the others, and launches
+  // with different L1 / shared-memory splits cannot share an SM.  Colors of few
+  // rows are launch bound: one split for all launches lets each start beside the
+  // previous one (18 colors of 9,000 rows: 223 against 252 us an iteration; 8
+  // colors of 7,500: 99 against 103).  Colors of many rows need the larger L1
+  // more (2 colors of 485,000 rows: 118 against 124 us), and then several
+  // iterations per pass lose what they save (FP32, 4 colors of 266,000 rows, the
+  // last one lane tiles: 110 us with one, 116 with four).  Other layouts: default
+  // splits, four iterations (n = 4096 46 against 48.5 us, 128^3 170 against 174).
+  if (lane_tiles && n / n_c < 100000) L.carve = 60;
+  else if (lane_tiles) L.body = 1;
   // one cooperative launch per sweep when every color is pair tiles (blocks
   // of one or two rows) and every CTA of that launch can be resident
   {
@@ -384,19 +404,12 @@ iccg_status iccg_setup(iccg_ctx **out, int32_t n, int64_t nnz, const int64_t *ro
       }
     }
   }
-  // slot regions: forward launches in color order (<r,r>), then the fused
-  // launch and the backward launches in launch order (<r,z>); the final
-  // launch (backward color 0, or the fused launch of a one-color ordering)
-  // sums everything written before its own region
-  L.off_rr.assign(n_c, 0);
-  L.off_rz.assign(n_c, 0);
-  int32_t nslot = 0;
-  for (int c = 0; c < n_c; ++c) { L.off_rr[c] = nslot; nslot += L.grid_c[c]; }
-  int32_t orz = 0;
-  if (n_c > 0) { L.off_rz[n_c - 1] = orz; orz += L.grid_c[n_c - 1]; }
-  for (int c = n_c - 2; c >= 0; --c) { L.off_rz[c] = orz; orz += L.grid_c[c]; }
-  L.last_rr = n_c > 1 ? nslot : 0;
-  L.last_rz = n_c > 1 ? L.off_rz[0] : 0;
+  // slot regions in launch order: the fused launch, then the backward
+  // launches; the final launch (backward color 0, or the fused launch of a
+  // one-color ordering) sums everything before its own region
+  L.off.assign(n_c, 0);
+  L.nslot = 0;
+  for (int c = n_c - 1; c >= 0; --c) { L.off[c] = L.nslot; L.nslot += L.grid_c[c]; }
   const int ntile_a = (n + 31) / 32;
   const int a_full = sms * spmv_resident_ctas(Wa, L.smem_a);
   L.grid_a = std::max(1, std::min(a_full, (ntile_a + Wa - 1) / Wa));
@@ -589,10 +602,7 @@ iccg_status iccg_setup(iccg_ctx **out, int32_t n, int64_t nnz, const int64_t *ro
   CK(dev_alloc(ctx, &ctx->xin, nn), "alloc vectors");
   CK(dev_alloc(ctx, &ctx->xout, nn), "alloc vectors");
   P.bin = ctx->bin; P.xin = ctx->xin; P.xout = ctx->xout;
-  // reduction slots: one per CTA of the widest launch, doubled so the solve
-  // start can keep <b,b> and <r0,r0> partials side by side; kept even for
-  // 16-byte loads
-  P.nslot = std::max(nslot, 1);
+  P.nslot = std::max(std::max(L.nslot, L.grid_coop), 1);
   P.npart = std::max(gbig, L.grid_p);
   P.ngroup = (gbig + kGroup - 1) / kGroup;
   P.npart_a = L.grid_a;
@@ -603,9 +613,9 @@ iccg_status iccg_setup(iccg_ctx **out, int32_t n, int64_t nnz, const int64_t *ro
   CK(dev_alloc(ctx, &P.part1, size_t(P.npart)), "alloc reductions");
   CK(dev_alloc(ctx, &P.gsum0, size_t(P.ngroup)), "alloc reductions");
   CK(dev_alloc(ctx, &P.gsum1, size_t(P.ngroup)), "alloc reductions");
+  CK(dev_alloc(ctx, &P.gticket, size_t(P.ngroup)), "alloc reductions");
   CK(dev_alloc(ctx, &P.part_a, size_t(P.npart_a)), "alloc reductions");
   CK(dev_alloc(ctx, &P.init_bb, size_t(P.nbb)), "alloc reductions");
-  CK(dev_alloc(ctx, &P.gticket, size_t(P.ngroup)), "alloc reductions");
   CK(dev_alloc(ctx, &P.sc, 1), "alloc scalars");
   CK(dev_alloc(ctx, &P.err_row, 1), "alloc scalars");
   CK(cudaMallocHost(&ctx->sc_host, sizeof(Scalars)), "pinned");
@@ -619,6 +629,8 @@ iccg_status iccg_factor(iccg_ctx *ctx) {
   DeviceGuard g(ctx->device);
   ctx->factored = false;
   if (ctx->H.n == 0) { ctx->factored = true; return ICCG_OK; }
+  Plan Lc = ctx->plan;
+  Lc.carve = -1;   // (the split chosen for the solve's kernels)
   // the factorization's launches (one per in-block level of every color)
   // are captured once into a graph and replayed: no host launch cost per
   // level.  Captured on a private stream (the legacy default stream cannot
@@ -629,7 +641,6 @@ iccg_status iccg_factor(iccg_ctx *ctx) {
     cudaError_t e = cudaStreamCreateWithFlags(&cs, cudaStreamNonBlocking);
     if (e == cudaSuccess) e = cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal);
     if (e == cudaSuccess) {
-      Plan Lc = ctx->plan;
       Lc.stream = cs;
       cudaError_t e1 = cudaMemsetAsync(ctx->P.err_row, 0xff, sizeof(unsigned long long), cs);
       if (e1 == cudaSuccess) e1 = launch_factor(ctx->P, Lc, int(ctx->H.nL));
@@ -651,7 +662,7 @@ iccg_status iccg_factor(iccg_ctx *ctx) {
     CK(cudaGraphLaunch(ctx->fexec, ctx->stream), "factor graph launch");
   } else {
     CK(cudaMemsetAsync(ctx->P.err_row, 0xff, sizeof(unsigned long long), ctx->stream), "factor");
-    CK(launch_factor(ctx->P, ctx->plan, int(ctx->H.nL)), "factor launch");
+    CK(launch_factor(ctx->P, Lc, int(ctx->H.nL)), "factor launch");
   }
   unsigned long long row = 0;
   CK(cudaMemcpyAsync(&row, ctx->P.err_row, sizeof(row), cudaMemcpyDeviceToHost, ctx->stream), "factor");
@@ -724,7 +735,8 @@ static iccg_status build_graph(iccg_ctx *ctx) {
   if (e2 != cudaSuccess) return cuda_fail(ctx, e2, "end capture");
   cudaGraph_t body = cp.conditional.phGraph_out[0];
   CK(cudaStreamBeginCaptureToGraph(s, body, nullptr, nullptr, 0, cudaStreamCaptureModeThreadLocal), "capture body");
-  e = launch_solve_body(ctx->P, Lc, ctx->fp32, nullptr, nullptr);
+  for (int k = solve_body_iterations(Lc); k > 0 && e == cudaSuccess; --k)
+    e = launch_solve_body(ctx->P, Lc, ctx->fp32, nullptr, nullptr);
   e2 = cudaStreamEndCapture(s, &body);
   if (e != cudaSuccess) return cuda_fail(ctx, e, "capture body");
   if (e2 != cudaSuccess) return cuda_fail(ctx, e2, "end capture body");
@@ -937,8 +949,10 @@ iccg_status iccg_time_spmv_phase(iccg_ctx *ctx, int32_t reps, double *ms) {
   *ms = 0.0;
   if (ctx->H.n == 0) return ICCG_OK;
   cudaStream_t s = ctx->stream;
-  // beta = 0: every repetition computes p = z (no growth of p across them)
+  // beta = 0: every repetition computes p = z (no growth of p across them);
+  // done = 0: the kernels skip their work once a solve has ended
   static const double zero = 0.0;
+  CK(cudaMemsetAsync(&ctx->P.sc->done, 0, sizeof(int32_t), s), "scalars");
   CK(cudaMemcpyAsync(&ctx->P.sc->beta, &zero, sizeof(double), cudaMemcpyHostToDevice, s), "scalars");
   CK(cudaStreamSynchronize(s), "sync");
   cudaEvent_t a0, a1;

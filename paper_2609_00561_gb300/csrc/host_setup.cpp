@@ -561,8 +561,8 @@ iccg_status build_layout(int32_t n, int64_t nnz, const int64_t *rowptr, const in
             }
             mk.push_back(mask);
           }
-          if (pass == 0) { u.li = co; u.lm = M; u.ls = so; }
-          else { u.ui = co; u.um = M; u.us = so; }
+          if (pass == 0) { u.li = co; u.lm = M; u.ls = so; u.lt = int32_t(T); }
+          else { u.ui = co; u.um = M; u.us = so; u.ut = int32_t(T); }
         }
         H.units.push_back(u);
       }
@@ -912,6 +912,8 @@ extern "C" iccg_status iccg_check_layout(int32_t n, int64_t nnz, const int64_t *
               want.push_back(pass ? H.umap[size_t(e)] : e);
           std::vector<int32_t> got;
           int32_t j = 0;
+          ck((pass ? u.ut : u.lt) >= __builtin_popcount(m) && size_t(off) + size_t(pass ? u.ut : u.lt) * kWarp <= mp.size(), t,
+             "chain term depth");
           for (int k = 0; k < M; ++k) {
             const uint32_t src = (swd[size_t(so) + size_t(k / 4) * kWarp + size_t(l)] >> (8 * (k % 4))) & 0xffu;
             if (!((m >> k) & 1u)) continue;

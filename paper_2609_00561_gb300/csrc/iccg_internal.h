@@ -89,11 +89,12 @@ struct __align__(16) PairDesc {
 // off + 32 j + l; L at (lo, lw), U at (uo, uw)).  Its in-block recurrence runs
 // as lm (forward) / um (backward) chain steps: at step m a lane subtracts at
 // most one in-block term, coefficient x the final value of the source lane;
-// coefficient m of lane l at li + 32 m + l (ui for U), the source lanes as
-// bytes, four steps per word, word w of lane l at ls + 32 w + l (us for U),
-// and bit m of the lane's mask (wl_mask / wu_mask) marks a step with a term.
+// the coefficient of the j-th term (in step order) of lane l at li + 32 j + l,
+// lt terms deep (ui, ut for U), the source lanes as bytes, four steps per word,
+// word w of lane l at ls + 32 w + l (us for U), and bit m of the lane's mask
+// (wl_mask / wu_mask) marks a step with a term.
 struct __align__(16) WarpUnit {
-  int32_t blk0, nblk, lo, lw, uo, uw, li, lm, ui, um, row0, nrows, ls, us, pad0, pad1;
+  int32_t blk0, nblk, lo, lw, uo, uw, li, lm, ui, um, row0, nrows, ls, us, lt, ut;
 };
 constexpr int32_t kPadCol = 0x7fffffff;   // padding entry of a sliced-ELL step
 constexpr int kTileSmemBudget = 96 * 1024;      // lane-tile CTA with two buffers, bytes
@@ -161,8 +162,9 @@ struct GridBar {
 };
 
 // Device-resident scalars of one solve.
-struct Scalars {
-  double bb, bnorm, rr, rz, pq, alpha, beta, tol;
+struct __align__(16) Scalars {
+  double alpha, skip;    // read together (16 bytes); skip: 1.0 once the solve has ended
+  double bb, bnorm, rr, rz, pq, beta, tol;
   int32_t iter, maxit, done, status;
   uint32_t ticket;       // arrival counter for "last CTA reduces" epilogues
   int32_t use_cond;      // 1 when a graph conditional handle is live
@@ -196,14 +198,14 @@ struct Params {
   const double *bin, *xin;      // original-order inputs
   double *xout;                 // original-order output
   const int32_t *perm;
-  // reductions.  Every color launch stores one <r,r> and/or <r,z> partial
-  // per CTA into slot_rr / slot_rz (its own region, plain stores); the last
-  // launch of an iteration sums all slots: each of its CTAs sums a fixed chunk
-  // of the earlier launches' slots plus its own partial into part0 / part1,
-  // the last CTA of each group of kGroup CTAs sums its group into gsum0 /
-  // gsum1, and the last group runs the epilogue.  The SpMV stores one <p,q>
-  // partial per CTA in part_a; its last CTA sums them.  init_bb / part_a hold
-  // <b,b> and <r0,r0> partials at the solve start.
+  // reductions.  Every launch with a backward sweep stores one <r,r> and one
+  // <r,z> partial per CTA into slot_rr / slot_rz (its own region, plain
+  // stores); the last launch of an iteration sums all slots: each of its CTAs
+  // sums a fixed chunk of the earlier launches' slots plus its own partial into
+  // part0 / part1, the last CTA of each group of kGroup CTAs sums its group
+  // into gsum0 / gsum1, and the last group runs the epilogue.  The SpMV stores
+  // one <p,q> partial per CTA in part_a; its last CTA sums them.  init_bb /
+  // part_a hold <b,b> and <r0,r0> partials at the solve start.
   double *slot_rr, *slot_rz;    // [nslot]
   double *part0, *part1;        // [npart]
   double *gsum0, *gsum1;        // [ngroup]
@@ -324,6 +326,8 @@ iccg_status build_layout(int32_t n, int64_t nnz, const int64_t *rowptr, const in
 struct Plan {
   cudaStream_t stream = nullptr;
   bool pdl = true;                      // programmatic dependent launch
+  int32_t carve = -1;                   // shared-memory share of the L1 (percent) of every launch (-1: each its default)
+  int32_t body = 4;                     // iterations per pass of the graph's WHILE loop at most
   int32_t W = 8, R = 1, n_c = 0, n = 0;
   int32_t Wa = 4;                       // warps per CTA of the SpMV
   std::vector<int32_t> task0, task1;    // group range of each color
@@ -339,6 +343,7 @@ struct Plan {
   std::vector<char> stage_ext;          // color c's lane-tile launches stage those entries (tiles of <= 2 steps)
   std::vector<char> wtile;              // color c: 0 CTA per tile, 1 warp-tile kernels, 2 pair kernels, 3 warp units
   std::vector<int32_t> unit0, unit1, unit_S;   // warp-unit range and segment size of each color
+  std::vector<int32_t> unit_T;          // most chain coefficients of a lane in the color's units
   int32_t Wu = 8;                       // warps per CTA of the warp-unit kernels
   bool coop = false;                    // every sweep as one cooperative launch (pair-tile layouts)
   int32_t grid_coop = 0;                // CTAs of that launch (all resident)
@@ -349,10 +354,10 @@ struct Plan {
   std::vector<char> pstage_f, pstage_b; // pair color c's forward / backward launches stage their entries
   int32_t smem_wt = 0;                  // bytes per CTA of the warp-tile kernels
   int32_t cap_ws = 0;                   // steps per tile held in a warp's buffer
-  std::vector<int32_t> off_rr, off_rz;  // slot regions of the color-c forward / backward launches
+  std::vector<int32_t> off;             // slot regions of the color-c fused / backward launches
+  int32_t nslot = 0;                    // their slots in all
   std::vector<int32_t> fac_ptr, fac_lev0, fac_nlev, fac_wide;   // IC(0) level schedule (host copy)
   int32_t fac_unit_cap = 0;             // most L entries of a warp unit (0: no update pairs, no one-launch IC(0))
-  int32_t last_rr = 0, last_rz = 0;     // slots written before the final launch of an iteration
   int32_t grid_a = 0;                   // CTAs of the SpMV-shaped kernels
   int32_t grid_v = 0;                   // CTAs of the vector kernels
   int32_t smem_fwd = 0, smem_bwd = 0, smem_fused = 0, smem_a = 0;  // bytes per CTA
@@ -372,12 +377,17 @@ int spmv_resident_ctas(int Wa, int smem);                    // CTAs per SM of t
 int tile_resident_ctas(bool fp32, int threads, int smem);    // CTAs per SM of the lane-tile kernels
 int wtile_resident_ctas(bool fp32, int threads, int smem);   // CTAs per SM of the warp-tile kernels
 int pair_resident_ctas(bool fp32, int threads);              // CTAs per SM of the pair kernels
-int unit_resident_ctas(bool fp32, int S, int threads);       // CTAs per SM of the warp-unit kernels
+int unit_resident_ctas(bool fp32, int S, int T, int threads);   // CTAs per SM of the warp-unit kernels
 int coop_sweep_resident_ctas(bool fp32);                     // CTAs per SM of the cooperative sweep (0: none)
 bool fac_unit_color(const Plan &L, int c);                   // color c's IC(0) is one launch
 cudaError_t launch_factor(const Params &P, const Plan &L, int nL);
 cudaError_t launch_solve_init(const Params &P, const Plan &L, bool fp32, PhaseHook h, void *u);
 cudaError_t launch_solve_body(const Params &P, const Plan &L, bool fp32, PhaseHook h, void *u);
+// Iterations per pass of the graph's WHILE loop: the way from a pass's last
+// kernel to the next pass's first costs 3 to 4 us more than a launch, so up to
+// Plan::body iterations share one, within 160 launches (graph instantiation);
+// the launches after the last iteration return at once (Scalars::skip, done)
+int solve_body_iterations(const Plan &L);
 // the SpMV phase of a PCG iteration: p = z + beta p, then q = A p and <p,q>
 cudaError_t launch_spmv_phase(const Params &P, const Plan &L, bool fp32);
 cudaError_t launch_solve_final(const Params &P, const Plan &L);

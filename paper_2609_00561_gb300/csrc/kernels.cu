@@ -9,12 +9,16 @@
 //                        parallel, rows of a block in order)
 //   fused color n_c-1    the same, followed at once by the backward sweep of
 //                        the last color (its rows have no later-color
-//                        dependencies), <r,z>
+//                        dependencies), <r,z> and <r,r>
 //   bwd color n_c-2..0   backward substitution L^T z = y (the reverse sweep
-//                        described after Alg. 1), <r,z>; the last group of the
-//                        color-0 launch reduces <r,r>, <r,z>, records the
+//                        described after Alg. 1), <r,z> and <r,r>; the last
+//                        group of the color-0 launch sums them, records the
 //                        residual history, tests ||r||/||b|| <= tol and sets
 //                        the CUDA-graph WHILE condition.
+// Both sums are formed where the backward sweep reads r anyway, in one
+// reduction per launch, and the forward launches reduce nothing.  (<r,z> is not
+// taken as <y,y>, y = L^-1 r, although that needs no r: on ill-conditioned
+// systems the two differ by more than a sum's rounding.)
 //
 // Substitution work mapping.  One warp owns a group: consecutive whole blocks
 // of one color (at most 32R rows), or one block larger than that.  Blocks of
@@ -56,10 +60,18 @@ namespace {
 
 constexpr int kVecThreads = 256;
 constexpr int kChunk = 4;    // row entries processed per predicated batch
+constexpr int kRed = 6 * kMaxWarpsPerCta;   // reduction scratch of a CTA (doubles)
 enum StepMode { M_FWD = 0, M_BWD = 1, M_FUSED = 2 };
 
-__device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
-__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+// Programmatic dependent launch: everything before this call runs while the
+// previous launch finishes.  The next launch may start once every CTA of this
+// one is past it, i.e. at most one launch waits beside the working one.  (Let
+// off at the kernels' first instruction, five to ten launches piled up waiting
+// and held the slots that the working launch's grid counts on.)
+__device__ __forceinline__ void pdl_wait() {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
 
 __device__ __forceinline__ void cp_async16(void *smem, const void *gmem) {
   const unsigned s = static_cast<unsigned>(__cvta_generic_to_shared(smem));
@@ -87,39 +99,60 @@ __device__ __forceinline__ void cp_wait_all() { asm volatile("cp.async.wait_grou
 // all but the most recently committed group
 __device__ __forceinline__ void cp_wait_prev() { asm volatile("cp.async.wait_group 1;" ::: "memory"); }
 
-// sum over the warp, valid in lane 0: each step adds on the lower half of
-// the lanes still in play (16, 8, 4, 2, 1), since FP64 adds are the scarce
-// resource on this GPU
-__device__ __forceinline__ double warp_sum(double v) {
-  const int lane = threadIdx.x & 31;
+// Sums of a and b over the warp together: a's in lane 0, b's in lane 16.  An
+// FP64 instruction costs a warp 64 cycles however many of its lanes it serves,
+// so after one exchange the half warps carry one sum each: 5 additions for both.
+__device__ __forceinline__ double warp_sum2(double a, double b) {
+  const bool hi = (threadIdx.x & 16) != 0;
+  const double u = __shfl_xor_sync(0xffffffffu, hi ? a : b, 16);
+  double v = (hi ? b : a) + u;
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    const double u = __shfl_down_sync(0xffffffffu, v, o);
-    // a predicated add (the compiler would otherwise add on every lane and select)
-    asm("{\n\t.reg .pred p;\n\tsetp.lt.s32 p, %1, %2;\n\t@p add.rn.f64 %0, %0, %3;\n\t}"
-        : "+d"(v)
-        : "r"(lane), "r"(o), "d"(u));
+  for (int o = 8; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o, 16);
+  return v;
+}
+// Exact float -> double by bit arithmetic (about 8 integer instructions, 3
+// cycles of an SM per warp against 16 for the conversion instruction, which
+// shares this GPU's scarce FP64 rate); subnormals, infinities and NaN take the
+// instruction.
+__device__ __forceinline__ double widen(float f) {
+  const unsigned b = __float_as_uint(f), m = b & 0x7fffffffu;
+  if (m - 0x00800000u >= 0x7f000000u && m != 0u) return double(f);
+  return __hiloint2double(int((b & 0x80000000u) | (m ? (m >> 3) + 0x38000000u : 0u)), int(b << 29));
+}
+
+// sum over the warp, valid in lane 0
+__device__ __forceinline__ double warp_sum(double v) {
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
+  return v;
+}
+
+// Sums of a and b over the CTA in a fixed order (red: 2 kMaxWarpsPerCta
+// doubles): the warps' sums one after another.  In warp 0, lane 0 returns a's
+// and lane 16 b's (both in the same instructions).
+__device__ __forceinline__ double cta_sum2(double a, double b, double *red) {
+  double v = warp_sum2(a, b);
+  const int w = threadIdx.x >> 5, l = threadIdx.x & 31, nw = blockDim.x >> 5;
+  if (nw == 1) return v;
+  __syncthreads();
+  if ((l & 15) == 0) red[(l >> 4) * kMaxWarpsPerCta + w] = v;
+  __syncthreads();
+  if (w == 0) {
+    const double *p = red + (l >> 4) * kMaxWarpsPerCta;
+    v = p[0];
+    for (int k = 1; k < nw; ++k) v += p[k];
   }
   return v;
 }
 
 // Sum of one value per thread; result valid in thread 0.  Fixed order.
-__device__ __forceinline__ double cta_sum(double v, double *red) {
-  v = warp_sum(v);
-  const int w = threadIdx.x >> 5, l = threadIdx.x & 31, nw = blockDim.x >> 5;
-  __syncthreads();
-  if (l == 0) red[w] = v;
-  __syncthreads();
-  double s = 0.0;
-  if (threadIdx.x == 0)
-    for (int k = 0; k < nw; ++k) s += red[k];
-  return s;
-}
+__device__ __forceinline__ double cta_sum(double v, double *red) { return cta_sum2(v, 0.0, red); }
 
 // Deterministic sum of p[0..count) by the whole CTA (result in thread 0);
 // optionally clears the entries.
 __device__ __forceinline__ double cta_sum_array(double *p, int count, double *red, bool clear) {
   double s = 0.0;
+#pragma unroll 4
   for (int k = threadIdx.x; k < count; k += blockDim.x) {
     s += __ldcg(p + k);
     if (clear) p[k] = 0.0;
@@ -128,41 +161,33 @@ __device__ __forceinline__ double cta_sum_array(double *p, int count, double *re
 }
 
 // Arrival on a counter by thread 0 after a fence; true (for the whole CTA)
-// for the last of `expected` arrivals, which also resets the counter.
+// for the last of `expected` arrivals, with which the counter wraps to 0.
 __device__ __forceinline__ bool arrive_last(uint32_t *ticket, uint32_t expected, int *flag) {
   __syncthreads();
   if (threadIdx.x == 0) {
     __threadfence();
-    const uint32_t t = atomicAdd(ticket, 1u);
-    *flag = (t == expected - 1) ? 1 : 0;
-    if (*flag) {
-      *ticket = 0;
-      __threadfence();
-    }
+    const int last = atomicInc(ticket, expected - 1) == expected - 1 ? 1 : 0;
+    if (last) __threadfence();
+    *flag = last;
   }
   __syncthreads();
   return *flag != 0;
 }
 
-// First level: each CTA publishes (a, b); the last CTA of the group returns
-// true with the group sums in thread 0's ga / gb.
-__device__ __forceinline__ bool group_reduce(const Params &P, double a, double b, bool two, double *red, int *flag,
-                                             double &ga, double &gb) {
+// First level: each CTA publishes (a, b), valid in lanes 0 and 16 of its first
+// warp; the last CTA of the group returns true with the group's sums there.
+__device__ __forceinline__ bool group_reduce(const Params &P, double v, double *red, int *flag, double &gv) {
   const int g = blockIdx.x / kGroup;
   const int g0 = g * kGroup;
   const int gs = min(kGroup, int(gridDim.x) - g0);
-  if (threadIdx.x == 0) {
-    P.part0[blockIdx.x] = a;
-    if (two) P.part1[blockIdx.x] = b;
+  if (threadIdx.x == 0) P.part0[blockIdx.x] = v;
+  if (threadIdx.x == 16) {
+    P.part1[blockIdx.x] = v;
+    __threadfence();
   }
   if (!arrive_last(P.gticket + g, uint32_t(gs), flag)) return false;
-  const double va = threadIdx.x < gs ? __ldcg(P.part0 + g0 + threadIdx.x) : 0.0;
-  ga = cta_sum(va, red);
-  gb = 0.0;
-  if (two) {
-    const double vb = threadIdx.x < gs ? __ldcg(P.part1 + g0 + threadIdx.x) : 0.0;
-    gb = cta_sum(vb, red);
-  }
+  const bool in = threadIdx.x < unsigned(gs);
+  gv = cta_sum2(in ? __ldcg(P.part0 + g0 + threadIdx.x) : 0.0, in ? __ldcg(P.part1 + g0 + threadIdx.x) : 0.0, red);
   return true;
 }
 
@@ -239,6 +264,15 @@ template <> __device__ __forceinline__ const float *uvals<float>(const Params &P
 template <typename PT> __device__ __forceinline__ const PT *invds(const Params &P);
 template <> __device__ __forceinline__ const double *invds<double>(const Params &P) { return P.invd; }
 template <> __device__ __forceinline__ const float *invds<float>(const Params &P) { return P.invd32; }
+
+// alpha of this iteration, with the flag that the solve has ended: the graph
+// loop runs several iterations per pass, and the launches of the iterations
+// after the last one change nothing (false).
+__device__ __forceinline__ bool load_alpha(const Params &P, double &alpha) {
+  const double2 v = __ldcg(reinterpret_cast<const double2 *>(&P.sc->alpha));
+  alpha = v.x;
+  return v.y == 0.0;
+}
 
 // ---------------------------------------------------------------------------
 // per-CTA shared memory of the substitution kernels (one CTA per group)
@@ -371,12 +405,19 @@ __device__ __forceinline__ Sweep<PT> sweep_static(const Params &P, const GroupDe
   return sweep_desc<PT>(P, d, upper, m);
 }
 
+// a row's shares of <r,r> and <r,z> (FP32 z widened exactly)
+__device__ __forceinline__ void rz_add(double r, double z, double &rr, double &rz) {
+  rr += r * r;
+  rz += r * z;
+}
+__device__ __forceinline__ void rz_add(double r, float z, double &rr, double &rz) { rz_add(r, widen(z), rr, rz); }
+
 // One sweep over a group.  UPPER = false: forward, L rows (entries to earlier
 // colors are a prefix of each row, in-block entries the rest); the source is
 // r (with the x / r update when UPDATE) and the result y.  UPPER = true:
 // backward, U rows (in-block entries a prefix, later colors the rest); the
-// source is y (from `ysrc`: shared memory when the fused kernel keeps y of a
-// fitting group there) and the result z, with <r, z>.
+// source is y (shared memory when the fused kernel keeps y of a fitting group
+// there) and the result z, with <r, z> and <r, r>.
 // Fitting groups keep t / y / z in m.w; other groups work in place in the
 // global result vector.
 template <typename PT, bool UPPER, bool UPDATE>
@@ -403,7 +444,6 @@ __device__ __forceinline__ void group_sweep(const Params &P, const GroupDesc &d,
         ri -= alpha * __ldcg(P.q + i);
         P.r[i] = ri;
         P.xh[i] = __ldcg(P.xh + i) + alpha * __ldcg(pn + i);
-        rr_acc += ri * ri;
       }
       src = PT(ri);
     }
@@ -451,7 +491,7 @@ __device__ __forceinline__ void group_sweep(const Params &P, const GroupDesc &d,
     const int i = r0 + l;
     const PT v = fit ? m.w[l] : __ldcg(res + i);
     if (fit && store_result) res[i] = v;
-    if (UPPER) rz_acc += __ldcg(P.r + i) * double(v);
+    if (UPPER) rz_add(__ldcg(P.r + i), v, rr_acc, rz_acc);
   }
   __syncthreads();
 }
@@ -463,25 +503,47 @@ __device__ void set_condition(const Scalars *s, int keep_going) {
   if (s->use_cond) cudaGraphSetConditional((cudaGraphConditionalHandle)s->cond_handle, keep_going ? 1u : 0u);
 }
 
-// After the backward sweep of iteration k: residual history, stop test, beta.
-// rr, rz valid in thread 0.
-__device__ void finish_iteration(const Params &P, double rr, double rz) {
-  if (threadIdx.x == 0) {
+// What finish_iteration reads, loaded while the sums are still being formed.
+struct IterScalars {
+  double bnorm, tol, rz;
+  int iter, maxit, status;
+};
+__device__ __forceinline__ IterScalars load_iter(const Scalars *s) {
+  IterScalars v;
+  v.bnorm = __ldcg(&s->bnorm);
+  v.tol = __ldcg(&s->tol);
+  v.rz = __ldcg(&s->rz);
+  v.iter = __ldcg(&s->iter);
+  v.maxit = __ldcg(&s->maxit);
+  v.status = __ldcg(&s->status);
+  return v;
+}
+
+// After the backward sweep of iteration k: residual history, stop test, beta;
+// by warp 0, sum = rr in lane 0, rz in lane 16.  The two quotients (a division
+// is a sequence of FP64 instructions) run side by side in the two lanes.
+__device__ void finish_iteration(const Params &P, double sum, const IterScalars &v) {
+  if (threadIdx.x >= kWarp) return;
+  const bool l0 = threadIdx.x == 0;
+  const double quot = (l0 ? sqrt(sum) : sum) / (l0 ? v.bnorm : v.rz);
+  const double rz = __shfl_sync(0xffffffffu, sum, 16), beta = __shfl_sync(0xffffffffu, quot, 16);
+  if (l0) {
     Scalars *s = P.sc;
-    const int k = s->iter;
-    const double rn = sqrt(rr) / s->bnorm;
-    P.hist[k + 1] = rn;
-    s->iter = k + 1;
-    s->rr = rr;
+    const int k = v.iter;
+    const double rn = quot;
     int done = 0;
     // a bounded wait of this iteration gave up (a cooperative launch of the
     // sweep): the solve stops with that status
-    if (s->status == ICCG_ERR_TIMEOUT) done = 1;
+    if (v.status == ICCG_ERR_TIMEOUT) done = 1;
     else if (!isfinite(rn) || !isfinite(rz)) { s->status = ICCG_ERR_NONFINITE; done = 1; }
-    else if (rn <= s->tol) { s->status = ICCG_OK; done = 1; }
-    else if (k + 1 >= s->maxit) { s->status = ICCG_NOT_CONVERGED; done = 1; }
-    else { s->beta = rz / s->rz; s->rz = rz; }
+    else if (rn <= v.tol) { s->status = ICCG_OK; done = 1; }
+    else if (k + 1 >= v.maxit) { s->status = ICCG_NOT_CONVERGED; done = 1; }
+    else { s->beta = beta; s->rz = rz; }
+    P.hist[k + 1] = rn;
+    s->iter = k + 1;
+    s->rr = sum;
     s->done = done;
+    if (done) s->skip = 1.0;
     set_condition(s, !done);
   }
 }
@@ -513,6 +575,7 @@ __device__ void finish_init(const Params &P, double rz, double *red) {
       else s->status = ICCG_NOT_CONVERGED;
     }
     s->done = done;
+    s->skip = done ? 1.0 : 0.0;
     set_condition(s, !done);
   }
 }
@@ -523,76 +586,89 @@ enum Fin { FIN_NONE = 0, FIN_ITER = 1, FIN_INIT = 2 };
 // color kernel: MODE = forward sweep of one color, backward sweep of one
 // color, or both for the last color (fused); one CTA per group
 // ---------------------------------------------------------------------------
+// groups a warp of the final launch's last CTA sums itself at most, instead of
+// the groups' own last CTAs (that level costs an atomic and a trip to L2, about
+// 1 us); the same sums in the same order
+constexpr int kOneLevel = 2;
+
 struct SlotArgs {
-  int off_rr, off_rz;     // this launch's slot regions
-  int last_rr, last_rz;   // slots of earlier launches (final launch only)
+  int off;      // this launch's first slot (-1: no sums wanted)
+  int last;     // final launch: slots of the sweep's earlier launches
 };
 
-// End of a color launch: this CTA's <r,r> / <r,z> partials.  A non-final
-// launch stores one partial per CTA in its slot region (plain stores: the
-// iteration's last launch sums them).  The last launch of the iteration:
-// every CTA sums a fixed chunk of the earlier launches' slots (complete:
-// griddepcontrol.wait before) plus its own partial; then groups of CTAs, then
-// the last group runs the epilogue.
-__device__ __forceinline__ void launch_epilogue(const Params &P, int fin, const SlotArgs &sa, bool has_rr,
-                                                bool has_rz, double rr_acc, double rz_acc, double *red, int *flag) {
-  if (!has_rr && !has_rz) return;
+// End of a launch with a backward sweep: this CTA's <r,r> / <r,z> partials.  A
+// non-final launch stores them in its slot region (plain stores: the sweep's
+// last launch sums them).  In the last launch every CTA adds a fixed chunk of
+// the earlier launches' slots (complete: griddepcontrol.wait before) to its own
+// partials; then groups of CTAs, then the last group runs the epilogue.
+__device__ __forceinline__ void launch_epilogue(const Params &P, int fin, const SlotArgs &sa, double rr_acc,
+                                                double rz_acc, double *red, int *flag) {
+  if (sa.off < 0) return;
+  if (fin == FIN_ITER && __ldcg(&P.sc->done)) return;   // an iteration after the last one
   if (fin == FIN_NONE) {
-    const double rr_c = has_rr ? cta_sum(rr_acc, red) : 0.0;
-    const double rz_c = has_rz ? cta_sum(rz_acc, red) : 0.0;
-    if (threadIdx.x == 0) {
-      if (has_rr) P.slot_rr[sa.off_rr + blockIdx.x] = rr_c;
-      if (has_rz) P.slot_rz[sa.off_rz + blockIdx.x] = rz_c;
-    }
+    const double v = cta_sum2(rr_acc, rz_acc, red);
+    if (threadIdx.x == 0) P.slot_rr[sa.off + blockIdx.x] = v;
+    if (threadIdx.x == 16) P.slot_rz[sa.off + blockIdx.x] = v;
     return;
   }
-  // the final launch: this CTA's share of the earlier launches' slots joins
-  // the threads' own partial sums, then one CTA sum per quantity
-  const int nb = gridDim.x;
-  const int crr = (sa.last_rr + nb - 1) / nb, crz = (sa.last_rz + nb - 1) / nb;
-  double a = has_rr ? rr_acc : 0.0, b = has_rz ? rz_acc : 0.0;
-  for (int k = threadIdx.x; k < crr; k += blockDim.x) {
-    const int idx = blockIdx.x * crr + k;
-    if (idx < sa.last_rr) a += __ldcg(P.slot_rr + idx);
-  }
-  for (int k = threadIdx.x; k < crz; k += blockDim.x) {
-    const int idx = blockIdx.x * crz + k;
-    if (idx < sa.last_rz) b += __ldcg(P.slot_rz + idx);
-  }
-  // a quantity that only the first warp holds (slots alone, at most 32 per
-  // CTA) is summed by that warp
-  if (!has_rr && crr <= kWarp) {
-    if (threadIdx.x < kWarp) a = warp_sum(a);
-  } else {
-    a = cta_sum(a, red);
-  }
-  if (!has_rz && crz <= kWarp) {
-    if (threadIdx.x < kWarp) b = warp_sum(b);
-  } else {
-    b = cta_sum(b, red);
-  }
-  double ga, gb;
-  if (group_reduce(P, a, b, true, red, flag, ga, gb)) {
-    if (threadIdx.x == 0) {
-      P.gsum0[blockIdx.x / kGroup] = ga;
-      P.gsum1[blockIdx.x / kGroup] = gb;
+  const int nb = gridDim.x, chunk = (sa.last + nb - 1) / nb;
+  for (int k = threadIdx.x; k < chunk; k += blockDim.x) {
+    const int idx = blockIdx.x * chunk + k;
+    if (idx < sa.last) {
+      rr_acc += __ldcg(P.slot_rr + idx);
+      rz_acc += __ldcg(P.slot_rz + idx);
     }
-    if (launch_last(P, flag)) {
-      const int ng = (nb + kGroup - 1) / kGroup;
-      const double rr = cta_sum_array(P.gsum0, ng, red, false);
-      const double rz = cta_sum_array(P.gsum1, ng, red, false);
-      if (fin == FIN_ITER) finish_iteration(P, rr, rz);
-      else finish_init(P, rz, red);
+  }
+  double v = cta_sum2(rr_acc, rz_acc, red);
+  const int ng = (nb + kGroup - 1) / kGroup;
+  const double *p0 = P.gsum0, *p1 = P.gsum1;
+  if (ng <= kOneLevel * int(blockDim.x >> 5)) {
+    // few CTAs: the last of them forms the groups' sums itself, a warp a group
+    if (threadIdx.x == 0) P.part0[blockIdx.x] = v;
+    if (threadIdx.x == 16) {
+      P.part1[blockIdx.x] = v;
+      __threadfence();
     }
+    if (!arrive_last(&P.sc->ticket, uint32_t(nb), flag)) return;
+    double *gs = red + 2 * kMaxWarpsPerCta;
+    for (int g = threadIdx.x >> 5; g < ng; g += int(blockDim.x >> 5)) {
+      const int k = g * kGroup + int(threadIdx.x & 31);
+      v = warp_sum2(k < nb ? __ldcg(P.part0 + k) : 0.0, k < nb ? __ldcg(P.part1 + k) : 0.0);
+      if ((threadIdx.x & 15) == 0) gs[((threadIdx.x >> 4) & 1) * 2 * kMaxWarpsPerCta + g] = v;
+    }
+    __syncthreads();
+    p0 = gs;
+    p1 = gs + 2 * kMaxWarpsPerCta;
+  } else {
+    double gv;
+    if (!group_reduce(P, v, red, flag, gv)) return;
+    if (threadIdx.x == 0) P.gsum0[blockIdx.x / kGroup] = gv;
+    if (threadIdx.x == 16) {
+      P.gsum1[blockIdx.x / kGroup] = gv;
+      __threadfence();
+    }
+    if (!launch_last(P, flag)) return;
+  }
+  const IterScalars is = load_iter(P.sc);
+  double a = 0.0, b = 0.0;
+  for (int k = threadIdx.x; k < ng; k += blockDim.x) {
+    a += p0 == P.gsum0 ? __ldcg(p0 + k) : p0[k];
+    b += p0 == P.gsum0 ? __ldcg(p1 + k) : p1[k];
+  }
+  v = cta_sum2(a, b, red);
+  if (fin == FIN_ITER) {
+    finish_iteration(P, v, is);
+  } else {
+    const double rz = threadIdx.x < kWarp ? __shfl_sync(0xffffffffu, v, 16) : 0.0;
+    finish_init(P, rz, red);
   }
 }
 
 template <typename PT, int MODE, bool UPDATE>
 __global__ void __launch_bounds__(kMaxWarpsPerCta * kWarp)
 color_kernel(Params P, int g0, int g1, GroupSmemPlan plan, int fin, SlotArgs sa) {
-  pdl_trigger();
   extern __shared__ __align__(16) unsigned char smem[];
-  __shared__ double red[kMaxWarpsPerCta];
+  __shared__ double red[kRed];
   __shared__ int flag;
   const int tid = threadIdx.x, nthr = blockDim.x;
   const GroupSmem<PT> m = group_smem<PT>(smem, plan);
@@ -609,7 +685,7 @@ color_kernel(Params P, int g0, int g1, GroupSmemPlan plan, int fin, SlotArgs sa)
     } else {
       double alpha = 0.0;
       const double *pn = P.p0;
-      if (UPDATE) alpha = __ldcg(&P.sc->alpha);
+      if (UPDATE && !load_alpha(P, alpha)) return;
       group_sweep<PT, false, UPDATE>(P, d, sw, m, tid, nthr, alpha, pn, false, MODE == M_FWD || !sw.fit,
                                      rr_acc, rz_acc);
       if (MODE == M_FUSED) {
@@ -626,7 +702,7 @@ color_kernel(Params P, int g0, int g1, GroupSmemPlan plan, int fin, SlotArgs sa)
   } else {
     pdl_wait();
   }
-  launch_epilogue(P, fin, sa, MODE != M_BWD && UPDATE, MODE != M_FWD, rr_acc, rz_acc, red, &flag);
+  if (MODE != M_FWD) launch_epilogue(P, fin, sa, rr_acc, rz_acc, red, &flag);
 }
 
 // ---------------------------------------------------------------------------
@@ -810,7 +886,7 @@ __device__ __forceinline__ PT ext_sub(const int32_t *col, const PT *val, int e, 
 template <typename PT, bool UPPER, bool UPDATE>
 __device__ __forceinline__ void tile_phase_a(const Params &P, const TileDesc &t, const TileBuf<PT> &tb, PT *w,
                                              double alpha, const double *pn, bool y_in_smem, bool staged,
-                                             double &rr_acc, int warp, int W) {
+                                             int warp, int W) {
   const int lane = threadIdx.x & 31;
   PT *yv = reinterpret_cast<PT *>(P.y);
   const PT *zv = reinterpret_cast<const PT *>(P.z);
@@ -843,7 +919,6 @@ __device__ __forceinline__ void tile_phase_a(const Params &P, const TileDesc &t,
             ri -= alpha * v0[vs + i];
             P.r[i] = ri;
             P.xh[i] = v0[2 * vs + i] + alpha * v0[3 * vs + i];
-            rr_acc += ri * ri;
           }
           acc = ext_sub<PT, false>(oc_s, ov_s, s.lo + lane, cnt, s.lw, PT(ri), yv);
         } else {
@@ -852,7 +927,6 @@ __device__ __forceinline__ void tile_phase_a(const Params &P, const TileDesc &t,
             ri -= alpha * __ldcg(P.q + i);
             P.r[i] = ri;
             P.xh[i] = __ldcg(P.xh + i) + alpha * __ldcg(pn + i);
-            rr_acc += ri * ri;
           }
           acc = ext_sub<PT>(oc_g, ov_g, s.lo + lane, cnt, s.lw, PT(ri), yv);
         }
@@ -880,10 +954,11 @@ __device__ __forceinline__ void tile_phase_b(const TileDesc &t, const StepDesc *
   }
 }
 
-// Phase C: the tile's results to global memory (y or z), <r,z> (backward)
+// Phase C: the tile's results to global memory (y or z), <r,z> and <r,r>
+// (backward; rs: the staged r)
 template <typename PT, bool UPPER>
 __device__ __forceinline__ void tile_phase_c(const Params &P, const TileDesc &t, const StepDesc *st, const PT *w,
-                                             bool store, const double *rs, double &rz_acc, int warp, int W) {
+                                             const double *rs, double &rr_acc, double &rz_acc, int warp, int W) {
   const int lane = threadIdx.x & 31;
   PT *res = reinterpret_cast<PT *>(UPPER ? P.z : P.y);
   for (int k = warp; k < t.nsteps; k += W) {
@@ -891,12 +966,14 @@ __device__ __forceinline__ void tile_phase_c(const Params &P, const TileDesc &t,
     if (lane < s.cnt) {
       const int i = s.row + lane;
       const PT v = w[k * kWarp + lane];
-      if (store) res[i] = v;
       if (UPPER) {
         double ri;
         if (rs) ri = rs[i];
         else ri = __ldcg(P.r + i);
-        rz_acc += ri * double(v);
+        res[i] = v;
+        rz_add(ri, v, rr_acc, rz_acc);
+      } else {
+        res[i] = v;
       }
     }
   }
@@ -909,9 +986,8 @@ __device__ __forceinline__ void tile_phase_c(const Params &P, const TileDesc &t,
 template <typename PT, int MODE, bool UPDATE>
 __global__ void __launch_bounds__(kMaxWarpsPerCta * kWarp)
 tile_kernel(Params P, int t0, int t1, TilePlan pl, int fin, SlotArgs sa) {
-  pdl_trigger();
   extern __shared__ __align__(16) unsigned char smem[];
-  __shared__ double red[kMaxWarpsPerCta];
+  __shared__ double red[kRed];
   __shared__ int flag;
   constexpr bool FU = MODE == M_BWD, TWO = MODE == M_FUSED;
   const int bsize = TWO && pl.cap_i2 > 0 ? pl.buf2 : pl.buf1;
@@ -925,7 +1001,11 @@ tile_kernel(Params P, int t0, int t1, TilePlan pl, int fin, SlotArgs sa) {
   pdl_wait();
   if (t < t1) tile_stage_vec<PT, FU, UPDATE>(P, td, tile_buf<PT>(smem, pl, bsize, 0), pl, threadIdx.x, blockDim.x);
   cp_commit();
-  const double alpha = UPDATE ? __ldcg(&P.sc->alpha) : 0.0;
+  double alpha = 0.0;
+  if (UPDATE && !load_alpha(P, alpha)) {
+    cp_wait_all();
+    return;
+  }
   for (; t < t1; t += gridDim.x) {
     const int tn = t + int(gridDim.x);
     TileDesc tdn = td;
@@ -943,28 +1023,28 @@ tile_kernel(Params P, int t0, int t1, TilePlan pl, int fin, SlotArgs sa) {
     const InBlock<PT> ll = in_block<PT>(tb.ic, tb.iv, P.si_col, siv<PT>(P), td.li0, td.li1, pl.cap_i);
     const bool stg = ext_staged(pl, td, MODE == M_BWD);
     if (MODE == M_BWD) {
-      tile_phase_a<PT, true, false>(P, td, tb, w, 0.0, nullptr, false, stg, rr_acc, wid, nw);
+      tile_phase_a<PT, true, false>(P, td, tb, w, 0.0, nullptr, false, stg, wid, nw);
       __syncthreads();
       if (wid == 0) tile_phase_b<PT, true>(td, tb.st, dv, ul.ic, ul.iv, w, threadIdx.x);
       __syncthreads();
-      tile_phase_c<PT, true>(P, td, tb.st, w, true, stg ? tb.vec + tb.vstride - cover_base<double>(td.row0) : nullptr,
-                             rz_acc, wid, nw);
+      tile_phase_c<PT, true>(P, td, tb.st, w, stg ? tb.vec + tb.vstride - cover_base<double>(td.row0) : nullptr,
+                             rr_acc, rz_acc, wid, nw);
     } else {
-      tile_phase_a<PT, false, UPDATE>(P, td, tb, w, alpha, P.p0, false, stg, rr_acc, wid, nw);
+      tile_phase_a<PT, false, UPDATE>(P, td, tb, w, alpha, P.p0, false, stg, wid, nw);
       __syncthreads();
       if (wid == 0) tile_phase_b<PT, false>(td, tb.st, dv, ll.ic, ll.iv, w, threadIdx.x);
       __syncthreads();
       if (MODE == M_FWD) {
-        tile_phase_c<PT, false>(P, td, tb.st, w, true, nullptr, rz_acc, wid, nw);
+        tile_phase_c<PT, false>(P, td, tb.st, w, nullptr, rr_acc, rz_acc, wid, nw);
       } else {
         // the last color: y stays in shared memory for the backward sweep
         // (its entries to other colors from global memory: the staged set is L's)
         const InBlock<PT> u2 = in_block<PT>(tb.ic2, tb.iv2, P.ui_col, uiv<PT>(P), td.ui0, td.ui1, pl.cap_i2);
-        tile_phase_a<PT, true, false>(P, td, tb, w, 0.0, nullptr, true, false, rr_acc, wid, nw);
+        tile_phase_a<PT, true, false>(P, td, tb, w, 0.0, nullptr, true, false, wid, nw);
         __syncthreads();
         if (wid == 0) tile_phase_b<PT, true>(td, tb.st, dv, u2.ic, u2.iv, w, threadIdx.x);
         __syncthreads();
-        tile_phase_c<PT, true>(P, td, tb.st, w, true, nullptr, rz_acc, wid, nw);
+        tile_phase_c<PT, true>(P, td, tb.st, w, nullptr, rr_acc, rz_acc, wid, nw);
       }
     }
     __syncthreads();   // buffer buf and w are reused by the next tile
@@ -982,7 +1062,7 @@ tile_kernel(Params P, int t0, int t1, TilePlan pl, int fin, SlotArgs sa) {
     td = tdn;
   }
   cp_wait_all();
-  launch_epilogue(P, fin, sa, MODE != M_BWD && UPDATE, MODE != M_FWD, rr_acc, rz_acc, red, &flag);
+  if (MODE != M_FWD) launch_epilogue(P, fin, sa, rr_acc, rz_acc, red, &flag);
 }
 
 // ---------------------------------------------------------------------------
@@ -1006,7 +1086,7 @@ __device__ __forceinline__ StepDesc load_step_g(const StepDesc *s) {
 // One sweep over tile t by one warp.  Forward (UPPER = false): source r (with
 // the x / r update when UPDATE), entries to earlier colors gathered from y,
 // in-block entries from wv; result y.  Backward: source y (from wv when
-// y_in_smem, the fused last color), gathers of z, result z and <r,z>.
+// y_in_smem, the fused last color), gathers of z, result z, <r,z> and <r,r>.
 // wv[step * 32 + lane] keeps the lane's own values of the tile.
 template <typename PT, bool UPPER, bool UPDATE>
 __device__ __forceinline__ void wtile_sweep(const Params &P, const TileDesc &t, PT *wv, double alpha,
@@ -1045,7 +1125,6 @@ __device__ __forceinline__ void wtile_sweep(const Params &P, const TileDesc &t, 
           ri -= alpha * __ldcg(P.q + i);
           P.r[i] = ri;
           P.xh[i] = __ldcg(P.xh + i) + alpha * __ldcg(P.p0 + i);
-          rr_acc += ri * ri;
         }
         acc = ext_sub<PT>(P.sl_col, slv<PT>(P), s.lo + lane, s.cnt, s.lw, PT(ri), ext);
       }
@@ -1054,7 +1133,7 @@ __device__ __forceinline__ void wtile_sweep(const Params &P, const TileDesc &t, 
       const PT v = acc * __ldg(dvg + i);
       wv[k * kWarp + lane] = v;
       if (store) res[i] = v;
-      if (UPPER) rz_acc += __ldcg(P.r + i) * double(v);
+      if (UPPER) rz_add(__ldcg(P.r + i), v, rr_acc, rz_acc);
     }
   }
 }
@@ -1069,9 +1148,8 @@ __device__ __forceinline__ void wtile_sweep(const Params &P, const TileDesc &t, 
 template <typename PT, int MODE, bool UPDATE>
 __global__ void __maxnreg__(ICCG_TILE_MAXNREG)
 wtile_kernel(Params P, int t0, int t1, int cap_s, int fin, SlotArgs sa) {
-  pdl_trigger();
   extern __shared__ __align__(16) unsigned char smem[];
-  __shared__ double red[kMaxWarpsPerCta];
+  __shared__ double red[kRed];
   __shared__ int flag;
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
   PT *wv = reinterpret_cast<PT *>(smem) + size_t(wid) * cap_s * kWarp;
@@ -1079,7 +1157,8 @@ wtile_kernel(Params P, int t0, int t1, int cap_s, int fin, SlotArgs sa) {
   int t = t0 + int(blockIdx.x) * nw + wid;
   TileDesc td = load_tile(P.tiles + min(t, t1 - 1));
   pdl_wait();
-  const double alpha = UPDATE ? __ldcg(&P.sc->alpha) : 0.0;
+  double alpha = 0.0;
+  if (UPDATE && !load_alpha(P, alpha)) return;
   for (; t < t1; t += int(gridDim.x) * nw) {
     const int tn = t + int(gridDim.x) * nw;
     const TileDesc tdn = tn < t1 ? load_tile(P.tiles + tn) : td;
@@ -1093,7 +1172,7 @@ wtile_kernel(Params P, int t0, int t1, int cap_s, int fin, SlotArgs sa) {
     __syncwarp();
     td = tdn;
   }
-  launch_epilogue(P, fin, sa, MODE != M_BWD && UPDATE, MODE != M_FWD, rr_acc, rz_acc, red, &flag);
+  if (MODE != M_FWD) launch_epilogue(P, fin, sa, rr_acc, rz_acc, red, &flag);
 }
 
 // ---------------------------------------------------------------------------
@@ -1137,9 +1216,11 @@ __device__ __forceinline__ PT pair_sub(const int32_t *col, const PT *val, int e,
 }
 
 // backward over one tile from y0 (and y1 when a1): stores z, adds <r,z>
+// and <r,r>
 template <typename PT>
 __device__ __forceinline__ void pair_bwd(const Params &P, const PairDesc &d, int lane, bool a1, PT y0, PT y1,
-                                         PT dv0, PT dv1, double r0, double r1, double &rz_acc) {
+                                         PT dv0, PT dv1, double r0, double r1, double &rr_acc,
+                                         double &rz_acc) {
   PT *zv = reinterpret_cast<PT *>(P.z);
   const int i0 = d.row0 + lane, i1 = d.row0 + d.c0 + lane;
   // both steps' gathers before any store (a store to z would order the
@@ -1150,11 +1231,9 @@ __device__ __forceinline__ void pair_bwd(const Params &P, const PairDesc &d, int
   for (int j = 0; j < d.uiw0; ++j) acc0 -= __ldg(uiv<PT>(P) + d.ui + j * d.c0 + lane) * z1;
   const PT z0 = acc0 * dv0;
   zv[i0] = z0;
-  rz_acc += r0 * double(z0);
-  if (a1) {
-    zv[i1] = z1;
-    rz_acc += r1 * double(z1);
-  }
+  if (a1) zv[i1] = z1;
+  rz_add(r0, z0, rr_acc, rz_acc);
+  if (a1) rz_add(r1, z1, rr_acc, rz_acc);
 }
 
 // one tile of a pair color, warp-wide (lanes beyond the tile's blocks idle)
@@ -1171,19 +1250,17 @@ __device__ __forceinline__ void pair_tile_h(const Params &P, int t, int4 head, i
   if (MODE == M_BWD) {
     const PT y0 = __ldcg(yv + i0), y1 = a1 ? __ldcg(yv + i1) : PT(0);
     const double r0 = __ldcg(P.r + i0), r1 = a1 ? __ldcg(P.r + i1) : 0.0;
-    pair_bwd<PT>(P, d, lane, a1, y0, y1, dv0, dv1, r0, r1, rz_acc);
+    pair_bwd<PT>(P, d, lane, a1, y0, y1, dv0, dv1, r0, r1, rr_acc, rz_acc);
   } else {
     double r0 = __ldcg(P.r + i0), r1 = a1 ? __ldcg(P.r + i1) : 0.0;
     if (UPDATE) {
       r0 -= alpha * __ldcg(P.q + i0);
       P.r[i0] = r0;
       P.xh[i0] = __ldcg(P.xh + i0) + alpha * __ldcg(P.p0 + i0);
-      rr_acc += r0 * r0;
       if (a1) {
         r1 -= alpha * __ldcg(P.q + i1);
         P.r[i1] = r1;
         P.xh[i1] = __ldcg(P.xh + i1) + alpha * __ldcg(P.p0 + i1);
-        rr_acc += r1 * r1;
       }
     }
     const PT y0 = pair_sub<PT>(P.sl_col, slv<PT>(P), d.lo + lane, d.c0, d.lw0, PT(r0), yv, 0) * dv0;
@@ -1197,7 +1274,7 @@ __device__ __forceinline__ void pair_tile_h(const Params &P, int t, int4 head, i
       yv[i0] = y0;
       if (a1) yv[i1] = y1;
     } else {
-      pair_bwd<PT>(P, d, lane, a1, y0, y1, dv0, dv1, r0, r1, rz_acc);
+      pair_bwd<PT>(P, d, lane, a1, y0, y1, dv0, dv1, r0, r1, rr_acc, rz_acc);
     }
   }
 }
@@ -1335,11 +1412,9 @@ __device__ __forceinline__ void pair_tile_staged(const Params &P, const PairPre<
     const PT z0 = acc0 * q.dv0;
     PT *zv = reinterpret_cast<PT *>(P.z);
     zv[i0] = z0;
-    rz_acc += r0 * double(z0);
-    if (a1) {
-      zv[i1] = z1;
-      rz_acc += r1 * double(z1);
-    }
+    if (a1) zv[i1] = z1;
+    rz_add(r0, z0, rr_acc, rz_acc);
+    if (a1) rz_add(r1, z1, rr_acc, rz_acc);
   } else {
     PT acc0, acc1 = PT(0);
     double r0 = __ldcg(P.r + i0), r1 = a1 ? __ldcg(P.r + i1) : 0.0;
@@ -1352,11 +1427,7 @@ __device__ __forceinline__ void pair_tile_staged(const Params &P, const PairPre<
         p1 = __ldcg(P.p0 + i1);
       }
       r0 -= alpha * q0;
-      rr_acc += r0 * r0;
-      if (a1) {
-        r1 -= alpha * q1;
-        rr_acc += r1 * r1;
-      }
+      if (a1) r1 -= alpha * q1;
       acc0 = PT(r0);
       acc1 = PT(r1);
       pair_staged_sums<PT, false>(P, d, s, lane, a1, acc0, acc1);
@@ -1383,7 +1454,7 @@ __device__ __forceinline__ void pair_tile_staged(const Params &P, const PairPre<
       yv[i0] = y0;
       if (a1) yv[i1] = y1;
     } else {
-      pair_bwd<PT>(P, d, lane, a1, y0, y1, q.dv0, q.dv1, r0, r1, rz_acc);
+      pair_bwd<PT>(P, d, lane, a1, y0, y1, q.dv0, q.dv1, r0, r1, rr_acc, rz_acc);
     }
   }
 }
@@ -1394,9 +1465,8 @@ constexpr int pair_stage_bytes() { return int(sizeof(PairStage<PT>)); }
 template <typename PT, int MODE, bool UPDATE, bool STAGE>
 __global__ void __launch_bounds__(kMaxWarpsPerCta * kWarp)
 pair_kernel(Params P, int t0, int t1, int fin, SlotArgs sa) {
-  pdl_trigger();
   extern __shared__ __align__(16) unsigned char smem[];
-  __shared__ double red[kMaxWarpsPerCta];
+  __shared__ double red[kRed];
   __shared__ int flag;
   const int lane = threadIdx.x & 31, wid = int(threadIdx.x >> 5);
   const int nw = int(blockDim.x >> 5), stride = int(gridDim.x) * nw;
@@ -1407,7 +1477,11 @@ pair_kernel(Params P, int t0, int t1, int fin, SlotArgs sa) {
     PairPre<PT> q;
     if (t < t1) q = pair_stage<PT, MODE == M_BWD>(P, t, lane, st);
     pdl_wait();
-    const double alpha = UPDATE ? __ldcg(&P.sc->alpha) : 0.0;
+    double alpha = 0.0;
+    if (UPDATE && !load_alpha(P, alpha)) {
+      cp_wait_all();
+      return;
+    }
     while (t < t1) {
       pair_tile_staged<PT, MODE, UPDATE>(P, q, st, lane, alpha, rr_acc, rz_acc);
       t += stride;
@@ -1420,14 +1494,15 @@ pair_kernel(Params P, int t0, int t1, int fin, SlotArgs sa) {
     int4 hn = make_int4(0, 0, 0, 0);
     if (t < t1) hn = pair_head(P.pairs + t);
     pdl_wait();
-    const double alpha = UPDATE ? __ldcg(&P.sc->alpha) : 0.0;
+    double alpha = 0.0;
+    if (UPDATE && !load_alpha(P, alpha)) return;
     for (; t < t1; t += stride) {
       const int4 h = hn;
       if (t + stride < t1) hn = pair_head(P.pairs + t + stride);
       pair_tile_h<PT, MODE, UPDATE>(P, t, h, lane, alpha, rr_acc, rz_acc);
     }
   }
-  launch_epilogue(P, fin, sa, MODE != M_BWD && UPDATE, MODE != M_FWD, rr_acc, rz_acc, red, &flag);
+  if (MODE != M_FWD) launch_epilogue(P, fin, sa, rr_acc, rz_acc, red, &flag);
 }
 
 // ---------------------------------------------------------------------------
@@ -1445,9 +1520,11 @@ pair_kernel(Params P, int t0, int t1, int fin, SlotArgs sa) {
 //      become final, so independent terms of different rows share a step:
 //      the chain is about as long as the in-block dependency depth or the
 //      widest row, not the block size;
-//   C  y = t / L_ii (times 1/L_ii), stored; <r,z> for the backward sweep.
-// Every static datum of a unit (descriptor, masks, coefficients, 1/L_ii) is
-// loaded before the first dependent access (griddepcontrol.wait).  A step at
+//   C  y = t / L_ii (times 1/L_ii), stored; <r,z> and <r,r> for the backward
+//      sweep.
+// Every static datum of a unit (descriptor, masks, coefficients, 1/L_ii, the
+// first entries to other colors) is loaded before the first dependent access
+// (griddepcontrol.wait).  A step at
 // which no lane of the warp has a coefficient issues no FP64 instruction.
 // ---------------------------------------------------------------------------
 template <typename PT> __device__ __forceinline__ const PT *wlv(const Params &P);
@@ -1464,131 +1541,125 @@ __device__ __forceinline__ WarpUnit load_unit(const WarpUnit *u) {
   r.blk0 = a.x; r.nblk = a.y; r.lo = a.z; r.lw = a.w;
   r.uo = b.x; r.uw = b.y; r.li = b.z; r.lm = b.w;
   r.ui = c.x; r.um = c.y; r.row0 = c.z; r.nrows = c.w;
-  r.ls = e.x; r.us = e.y; r.pad0 = r.pad1 = 0;
+  r.ls = e.x; r.us = e.y; r.lt = e.z; r.ut = e.w;
   return r;
 }
 
 constexpr int kUnitChunk = 8;   // entries to other colors per batch of loads
 
-// acc -= sum over the lane's entries to other colors (width w, stride 32)
+// The first kUnitChunk of a lane's entries to other colors (static: loaded
+// before griddepcontrol.wait), their gathers, and the subtraction of all w
+// entries (stride 32), the first chunk from x.
 template <typename PT>
-__device__ __forceinline__ PT unit_ext(const int32_t *col, const PT *val, int e, int w, PT acc, const PT *g) {
-  for (int j0 = 0; j0 < w; j0 += kUnitChunk) {
-    const int nj = min(kUnitChunk, w - j0);
-    int cc[kUnitChunk];
-    PT vv[kUnitChunk], xx[kUnitChunk];
+struct UnitExt {
+  int c[kUnitChunk];
+  PT v[kUnitChunk];
+};
+template <typename PT>
+__device__ __forceinline__ void unit_ext_load(UnitExt<PT> &q, const int32_t *col, const PT *val, int e, int w) {
 #pragma unroll
-    for (int j = 0; j < kUnitChunk; ++j) {
-      cc[j] = j < nj ? __ldg(col + e + (j0 + j) * kWarp) : kPadCol;
-      vv[j] = j < nj ? __ldg(val + e + (j0 + j) * kWarp) : PT(0);
-    }
+  for (int j = 0; j < kUnitChunk; ++j) {
+    q.c[j] = j < w ? __ldg(col + e + j * kWarp) : kPadCol;
+    q.v[j] = j < w ? __ldg(val + e + j * kWarp) : PT(0);
+  }
+}
+template <typename PT>
+__device__ __forceinline__ void unit_ext_gather(const UnitExt<PT> &q, PT (&x)[kUnitChunk], const PT *g) {
 #pragma unroll
-    for (int j = 0; j < kUnitChunk; ++j) xx[j] = cc[j] == kPadCol ? PT(0) : __ldcg(g + cc[j]);
+  for (int j = 0; j < kUnitChunk; ++j) x[j] = q.c[j] == kPadCol ? PT(0) : __ldcg(g + q.c[j]);
+}
+template <typename PT>
+__device__ __forceinline__ PT unit_ext_sub(UnitExt<PT> &q, PT (&x)[kUnitChunk], const int32_t *col, const PT *val,
+                                           int e, int w, PT acc, const PT *g) {
+  for (int j0 = 0;;) {
+    const int nj = w - j0;
 #pragma unroll
     for (int j = 0; j < kUnitChunk; ++j)
-      if (j < nj) acc -= vv[j] * xx[j];
+      if (j < nj) acc -= q.v[j] * x[j];
+    j0 += kUnitChunk;
+    if (j0 >= w) return acc;
+    unit_ext_load(q, col, val, e + j0 * kWarp, w - j0);
+    unit_ext_gather(q, x, g);
   }
-  return acc;
 }
 
-// the lane's chain coefficients by step (0 where its mask has no bit) and the
-// source lanes (four bytes a word)
+constexpr int kUnitWarps = 8;   // warps (units in flight) per CTA of the warp-unit kernels
+
+// A unit's chain coefficients into the warp's shared memory as they lie in
+// memory (term-major: lane l's j-th term at j * 32 + l, T terms deep; 16-byte
+// cp.async, no registers held while the copies fly) and the lane's source
+// lanes into registers.  Compact, the buffer is as deep as the lane with most
+// terms (3 for 7-point, 13 for 27-point blocks) and not as the chain (up to 32
+// steps, 8 KB a warp in FP64), so that the next launch's CTAs fit beside this
+// one's and load their static data early, and the copy is T / 2 instructions
+// instead of a test and an address for each of 32 steps.
 template <typename PT, int S>
-__device__ __forceinline__ void unit_coef(const PT *v, const uint32_t *sw, int off, int soff, int M, uint32_t mask,
-                                          int lane, PT (&cf)[S], uint32_t (&src)[(S + 3) / 4]) {
-  // the lane's terms are stored term-major (its j-th term at off + j * 32 +
-  // lane): the term of step k is number popc(mask below k)
-#pragma unroll
-  for (int k = 0; k < S; ++k)
-    cf[k] = ((mask >> k) & 1u) ? __ldg(v + off + __popc(mask & ((1u << k) - 1u)) * kWarp + lane) : PT(0);
+__device__ __forceinline__ void unit_coef(const PT *v, const uint32_t *sw, int off, int T, int soff, int M, int lane,
+                                          PT *cfs, uint32_t (&src)[(S + 3) / 4]) {
+  constexpr int EV = 16 / sizeof(PT);
+  __syncwarp();   // the previous coefficients' readers are done
+  for (int k = lane; k < T * (kWarp / EV); k += kWarp) cp_async16(cfs + k * EV, v + off + k * EV);
+  cp_commit();
 #pragma unroll
   for (int w = 0; w < (S + 3) / 4; ++w) src[w] = 4 * w < M ? __ldg(sw + soff + w * kWarp + lane) : 0u;
-}
-
-// the lane's chain coefficients into its column of the warp's shared-memory
-// buffer (cp.async, only the steps its mask has: no registers held while the
-// copies fly) and its source lanes into registers
-
-template <typename PT, int S>
-__device__ __forceinline__ void unit_coef_smem(const PT *v, const uint32_t *sw, int off, int soff, int M,
-                                               uint32_t mask, int lane, PT *cfs, uint32_t (&src)[(S + 3) / 4]) {
-#pragma unroll
-  for (int k = 0; k < S; ++k)
-    if ((mask >> k) & 1u)
-      cp_async_elem<PT>(cfs + k * kWarp + lane, v + off + __popc(mask & ((1u << k) - 1u)) * kWarp + lane);
-  asm volatile("cp.async.commit_group;" ::: "memory");
-#pragma unroll
-  for (int w = 0; w < (S + 3) / 4; ++w) src[w] = 4 * w < M ? __ldg(sw + soff + w * kWarp + lane) : 0u;
-}
-
-// phase B with the coefficients in shared memory (the lane's own column)
-template <typename PT, int S>
-__device__ __forceinline__ PT unit_chain_smem(PT t, int M, uint32_t mask, uint32_t wmask, const PT *cfs, int lane,
-                                              const uint32_t (&src)[(S + 3) / 4]) {
-  asm volatile("cp.async.wait_group 0;" ::: "memory");
-#pragma unroll
-  for (int k = 0; k < S; ++k) {
-    if (k < M) {
-      const int sl = int((src[k / 4] >> (8 * (k % 4))) & 0xffu);
-      const PT tk = __shfl_sync(0xffffffffu, t, sl);
-      if ((wmask >> k) & 1u) {
-        if ((mask >> k) & 1u) t -= cfs[k * kWarp + lane] * tk;
-      }
-    }
-  }
-  return t;
 }
 
 // phase B of a unit: M chain steps; at step k every lane with a term
 // subtracts coefficient x the (final) value of its source lane; wmask = OR
 // of the warp's lane masks (a step no lane uses issues no FP64 instruction)
 template <typename PT, int S>
-__device__ __forceinline__ PT unit_chain(PT t, int M, uint32_t mask, uint32_t wmask, const PT (&cf)[S],
+__device__ __forceinline__ PT unit_chain(PT t, int M, uint32_t mask, uint32_t wmask, const PT *cfs, int lane,
                                          const uint32_t (&src)[(S + 3) / 4]) {
+  cp_wait_all();
+  __syncwarp();
+  const PT *p = cfs + lane;
+  PT c = *p;   // the next term's coefficient (one row of padding after the last)
 #pragma unroll
   for (int k = 0; k < S; ++k) {
     if (k < M) {
       const int sl = int((src[k / 4] >> (8 * (k % 4))) & 0xffu);
       const PT tk = __shfl_sync(0xffffffffu, t, sl);
       if ((wmask >> k) & 1u) {
-        if ((mask >> k) & 1u) t -= cf[k] * tk;
+        if ((mask >> k) & 1u) {
+          t -= c * tk;
+          p += kWarp;
+          c = *p;
+        }
       }
     }
   }
   return t;
 }
 
-constexpr int kUnitWarps = 8;   // warps (units in flight) per CTA of the warp-unit kernels
-
-// chain coefficients of segments of at least kUnitSmemS steps sit in shared
-// memory (S x 32 values per warp) instead of registers
-constexpr int kUnitSmemS = 16;
-
-inline int unit_smem_bytes(int S, int elem) { return S >= kUnitSmemS ? kUnitWarps * S * kWarp * elem : 0; }
+// shared memory of a warp-unit CTA, coefficients at most T terms deep
+inline int unit_smem_bytes(int T, int elem) { return kUnitWarps * (T + 1) * kWarp * elem; }
 
 template <typename PT, int MODE, bool UPDATE, int S>
 __global__ void __launch_bounds__(kUnitWarps * kWarp)
-unit_kernel(Params P, int u0, int u1, int fin, SlotArgs sa) {
-  pdl_trigger();
-  __shared__ double red[kMaxWarpsPerCta];
-  __shared__ int flag;
+unit_kernel(Params P, int u0, int u1, int T, int fin, SlotArgs sa) {
+  __shared__ double red[kRed];
   extern __shared__ __align__(16) unsigned char usm[];
-  constexpr bool SM = S >= kUnitSmemS;
+  __shared__ int flag;
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
-  PT *cfs = reinterpret_cast<PT *>(usm) + (SM ? wid * S * kWarp : 0);
+  PT *cfs = reinterpret_cast<PT *>(usm) + wid * (T + 1) * kWarp;
   const int step = lane & (S - 1);
   constexpr bool FWD = MODE != M_BWD;
   PT *yv = reinterpret_cast<PT *>(P.y);
   PT *zv = reinterpret_cast<PT *>(P.z);
   const PT *dvg = invds<PT>(P);
   double rr_acc = 0.0, rz_acc = 0.0;
-  bool waited = false;
+  bool waited = false, live = true;
   double alpha = 0.0;
   for (int u = u0 + int(blockIdx.x) * nw + wid; u < u1; u += int(gridDim.x) * nw) {
     // static data of the unit
     const WarpUnit d = load_unit(P.units + u);
+    UnitExt<PT> ext;
+    if (FWD) unit_ext_load(ext, P.sl_col, slv<PT>(P), d.lo + lane, d.lw);
+    else unit_ext_load(ext, P.su_col, suv<PT>(P), d.uo + lane, d.uw);
     int row = -1;
-    if (lane / S < d.nblk) {
+    if (S == kWarp) {   // one block: its rows are the unit's
+      if (lane < d.nrows) row = d.row0 + lane;
+    } else if (lane / S < d.nblk) {
       const int b = d.blk0 + lane / S;
       const int r = __ldg(P.bptr + b) + step;
       if (r < __ldg(P.bptr + b + 1)) row = r;
@@ -1596,61 +1667,63 @@ unit_kernel(Params P, int u0, int u1, int fin, SlotArgs sa) {
     const bool on = row >= 0;
     const uint32_t mf = FWD ? __ldg(P.wl_mask + size_t(u) * kWarp + lane) : 0u;
     const uint32_t mb = MODE != M_FWD ? __ldg(P.wu_mask + size_t(u) * kWarp + lane) : 0u;
-    PT cf[SM ? 1 : S];
     uint32_t src[(S + 3) / 4];
-    if constexpr (SM) {
-      if (FWD) unit_coef_smem<PT, S>(wlv<PT>(P), P.wl_src, d.li, d.ls, d.lm, mf, lane, cfs, src);
-      else unit_coef_smem<PT, S>(wuv<PT>(P), P.wu_src, d.ui, d.us, d.um, mb, lane, cfs, src);
-    } else {
-      if (FWD) unit_coef<PT, S>(wlv<PT>(P), P.wl_src, d.li, d.ls, d.lm, mf, lane, cf, src);
-      else unit_coef<PT, S>(wuv<PT>(P), P.wu_src, d.ui, d.us, d.um, mb, lane, cf, src);
-    }
+    if (FWD) unit_coef<PT, S>(wlv<PT>(P), P.wl_src, d.li, d.lt, d.ls, d.lm, lane, cfs, src);
+    else unit_coef<PT, S>(wuv<PT>(P), P.wu_src, d.ui, d.ut, d.us, d.um, lane, cfs, src);
     const PT dv = on ? __ldg(dvg + row) : PT(0);
     if (!waited) {
       pdl_wait();
       waited = true;
-      if (UPDATE) alpha = __ldcg(&P.sc->alpha);
+      if (UPDATE && !(live = load_alpha(P, alpha))) break;
     }
-    PT t = PT(0);
+    PT t = PT(0), x[kUnitChunk];
+    double ri = 0.0;
     if (FWD) {
-      // A: source r (with the x / r update), entries to earlier colors
-      if (on) {
-        double ri = __ldcg(P.r + row);
-        if (UPDATE) {
-          ri -= alpha * __ldcg(P.q + row);
+      // A: source r (with the x / r update), entries to earlier colors (their
+      // gathers before the update's stores)
+      ri = on ? __ldcg(P.r + row) : 0.0;
+      if (UPDATE) {
+        const double qi = on ? __ldcg(P.q + row) : 0.0, xi = on ? __ldcg(P.xh + row) : 0.0;
+        const double pi = on ? __ldcg(P.p0 + row) : 0.0;
+        unit_ext_gather(ext, x, yv);
+        ri -= alpha * qi;
+        if (on) {
           P.r[row] = ri;
-          P.xh[row] = __ldcg(P.xh + row) + alpha * __ldcg(P.p0 + row);
-          rr_acc += ri * ri;
+          P.xh[row] = xi + alpha * pi;
         }
-        t = PT(ri);
+      } else {
+        unit_ext_gather(ext, x, yv);
       }
-      t = unit_ext<PT>(P.sl_col, slv<PT>(P), d.lo + lane, d.lw, t, yv);
+      t = unit_ext_sub(ext, x, P.sl_col, slv<PT>(P), d.lo + lane, d.lw, PT(ri), yv);
       // B, C
-      if constexpr (SM) t = unit_chain_smem<PT, S>(t, d.lm, mf, __reduce_or_sync(0xffffffffu, mf), cfs, lane, src);
-      else t = unit_chain<PT, S>(t, d.lm, mf, __reduce_or_sync(0xffffffffu, mf), cf, src);
-      const PT y = t * dv;
-      if (MODE == M_FWD) {
-        if (on) yv[row] = y;
-        continue;
-      }
+      t = unit_chain<PT, S>(t, d.lm, mf, __reduce_or_sync(0xffffffffu, mf), cfs, lane, src);
+      const PT y = t * dv;   // 0 in an idle lane
+      if (MODE == M_FWD && on) yv[row] = y;
+      if (MODE == M_FWD) continue;
       // the last color: its backward sweep at once (y stays in registers)
-      if constexpr (SM) unit_coef_smem<PT, S>(wuv<PT>(P), P.wu_src, d.ui, d.us, d.um, mb, lane, cfs, src);
-      else unit_coef<PT, S>(wuv<PT>(P), P.wu_src, d.ui, d.us, d.um, mb, lane, cf, src);
+      unit_ext_load(ext, P.su_col, suv<PT>(P), d.uo + lane, d.uw);
+      unit_coef<PT, S>(wuv<PT>(P), P.wu_src, d.ui, d.ut, d.us, d.um, lane, cfs, src);
       t = y;
     } else {
-      if (on) t = __ldcg(yv + row);
+      if (on) {
+        t = __ldcg(yv + row);
+        if (sa.off >= 0) ri = __ldcg(P.r + row);
+      }
     }
-    t = unit_ext<PT>(P.su_col, suv<PT>(P), d.uo + lane, d.uw, t, zv);
-    if constexpr (SM) t = unit_chain_smem<PT, S>(t, d.um, mb, __reduce_or_sync(0xffffffffu, mb), cfs, lane, src);
-    else t = unit_chain<PT, S>(t, d.um, mb, __reduce_or_sync(0xffffffffu, mb), cf, src);
-    const PT z = t * dv;
-    if (on) {
-      zv[row] = z;
-      rz_acc += __ldcg(P.r + row) * double(z);
-    }
+    unit_ext_gather(ext, x, zv);
+    t = unit_ext_sub(ext, x, P.su_col, suv<PT>(P), d.uo + lane, d.uw, t, zv);
+    t = unit_chain<PT, S>(t, d.um, mb, __reduce_or_sync(0xffffffffu, mb), cfs, lane, src);
+    const PT z = t * dv;   // 0 in an idle lane
+    if (on) zv[row] = z;
+    if (sa.off >= 0) rz_add(ri, z, rr_acc, rz_acc);
   }
-  if (!waited) pdl_wait();
-  launch_epilogue(P, fin, sa, MODE != M_BWD && UPDATE, MODE != M_FWD, rr_acc, rz_acc, red, &flag);
+  if (!waited) {
+    pdl_wait();
+    if (UPDATE) live = load_alpha(P, alpha);
+  }
+  cp_wait_all();
+  if (!live) return;   // (the whole CTA)
+  if (MODE != M_FWD) launch_epilogue(P, fin, sa, rr_acc, rz_acc, red, &flag);
 }
 
 // ---------------------------------------------------------------------------
@@ -1659,9 +1732,9 @@ unit_kernel(Params P, int u0, int u1, int fin, SlotArgs sa) {
 // (two rows per thread per pass: 16-byte loads of p and, for FP64 z, of z)
 template <typename ZT>
 __global__ void __launch_bounds__(kVecThreads) pupdate_kernel(Params P) {
-  pdl_trigger();
   pdl_wait();
   const double beta = __ldcg(&P.sc->beta);
+  if (__ldcg(&P.sc->done)) return;
   const ZT *z = reinterpret_cast<const ZT *>(P.z);
   const int n2 = P.n / 2;
   const int stride = gridDim.x * blockDim.x;
@@ -1674,7 +1747,7 @@ __global__ void __launch_bounds__(kVecThreads) pupdate_kernel(Params P) {
       z0 = zv.x; z1 = zv.y;
     } else {
       const float2 zv = __ldcg(reinterpret_cast<const float2 *>(z) + k);
-      z0 = double(zv.x); z1 = double(zv.y);
+      z0 = widen(zv.x); z1 = widen(zv.y);
     }
     p2[k] = make_double2(z0 + beta * pv.x, z1 + beta * pv.y);
   }
@@ -1699,14 +1772,14 @@ constexpr int kSpmvChunk = 6;   // entries per predicated batch of the SpMV
 template <int MODE>
 __global__ void __launch_bounds__(kSpmvWarps * kWarp, 6)
 spmv_kernel(Params P) {
-  pdl_trigger();
-  __shared__ double red[kMaxWarpsPerCta];
+  __shared__ double red[kRed];
   __shared__ int flag;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, W = blockDim.x >> 5;
   const int nsl = (P.n + kWarp - 1) / kWarp;
   const double *xin = MODE == 0 ? P.p0 : P.xh;
   double acc = 0.0;
   pdl_wait();
+  if (MODE == 0 && __ldcg(&P.sc->done)) return;
   for (int sl = blockIdx.x * W + warp; sl < nsl; sl += gridDim.x * W) {
     const int e0 = __ldg(P.sa_ptr + sl), w = (__ldg(P.sa_ptr + sl + 1) - e0) >> 5;
     const int i = sl * kWarp + lane;
@@ -1747,17 +1820,18 @@ spmv_kernel(Params P) {
   const double tot = cta_sum(acc, red);
   if (threadIdx.x == 0) P.part_a[blockIdx.x] = tot;
   if (MODE == 0 && arrive_last(&P.sc->ticket, gridDim.x, &flag)) {
+    const double rz = __ldcg(&P.sc->rz);
     const double pq = cta_sum_array(P.part_a, gridDim.x, red, false);
     if (threadIdx.x == 0) {
+      P.sc->alpha = rz / pq;
       P.sc->pq = pq;
-      P.sc->alpha = __ldcg(&P.sc->rz) / pq;
     }
   }
 }
 
 // b_hat = b[perm], x_hat = x0[perm], <b, b> partials into init_bb
 __global__ void __launch_bounds__(kVecThreads) perm_in_kernel(Params P) {
-  __shared__ double red[kMaxWarpsPerCta];
+  __shared__ double red[kRed];
   double acc = 0.0;
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < P.n; i += gridDim.x * blockDim.x) {
     const int o = P.perm[i];
@@ -1947,7 +2021,6 @@ __device__ __forceinline__ double factor_steps(double s, int c, int ce, const do
 }
 
 __global__ void __launch_bounds__(kFacWarps * kWarp) factor_warp_kernel(Params P, int k0, int k1) {
-  pdl_trigger();
   extern __shared__ __align__(16) unsigned char fsm[];
   __shared__ double sd[kFacWarps];
   __shared__ int srow[kFacWarps];
@@ -2036,7 +2109,6 @@ constexpr int kFacSpin = 1 << 22;   // polls of a row's flags before giving up
 inline int fac_unit_bytes(int cap) { return kFacUnitWarps * kFacWarpBytes + cap * 8; }
 
 __global__ void __launch_bounds__(kFacUnitWarps * kWarp) factor_unit_kernel(Params P, int u0, int S) {
-  pdl_trigger();
   extern __shared__ __align__(16) unsigned char fsm[];
   __shared__ double ivs[kWarp], ds[kWarp];
   __shared__ volatile int ready[kWarp];
@@ -2143,7 +2215,6 @@ constexpr int kFacWideWarps = 4;
 __host__ __device__ inline int fac_wide_bytes(int cap) { return r16b(cap * (cap - 1) / 2 * 8 + cap * 4); }
 
 __global__ void __launch_bounds__(kFacWideWarps * kWarp) factor_wide_kernel(Params P, int k0, int k1, int cap) {
-  pdl_trigger();
   extern __shared__ __align__(16) unsigned char fsm[];
   __shared__ double sd[kFacWideWarps];
   __shared__ int srow[kFacWideWarps];
@@ -2243,7 +2314,6 @@ __global__ void __launch_bounds__(kFacWideWarps * kWarp) factor_wide_kernel(Para
 // without triangles (5- and 7-point) has no pairs at all.
 constexpr int kFacShort = 8;
 __global__ void __launch_bounds__(kVecThreads) factor_short_kernel(Params P, int k0, int k1) {
-  pdl_trigger();
   bool waited = false;
   for (int k = k0 + int(blockIdx.x * blockDim.x + threadIdx.x); k < k1; k += int(gridDim.x * blockDim.x)) {
     const int4 rec = __ldg(P.fac_rec + k);
@@ -2295,7 +2365,6 @@ __global__ void __launch_bounds__(kVecThreads) factor_short_kernel(Params P, int
 // levels without precomputed pairs of short rows (short merges) or of rows
 // above kFacWide: one row per thread, the general form
 __global__ void __launch_bounds__(kVecThreads) factor_merge_kernel(Params P, int k0, int k1) {
-  pdl_trigger();
   pdl_wait();
   for (int k = k0 + int(blockIdx.x * blockDim.x + threadIdx.x); k < k1; k += int(gridDim.x * blockDim.x))
     factor_row_merge(P, __ldg(P.fac_rows + k));
@@ -2618,7 +2687,7 @@ template <typename PT>
 __global__ void __launch_bounds__(kMaxWarpsPerCta * kWarp, ICCG_PERSIST_MIN_CTAS)
 persistent_kernel(Params P, GroupSmemPlan plan, int cap_a) {
   extern __shared__ __align__(16) unsigned char smem[];
-  __shared__ double red[kMaxWarpsPerCta];
+  __shared__ double red[kRed];
   __shared__ double bc;
   __shared__ int flag;
   const int tid = threadIdx.x, nthr = blockDim.x, nb = gridDim.x, b = blockIdx.x;
@@ -2743,21 +2812,21 @@ persistent_kernel(Params P, GroupSmemPlan plan, int cap_a) {
 constexpr int kCoopWarps = 8;
 
 // c_lo > 0: the tail of a sweep (forward colors c_lo .. n_c - 2, the fused
-// last color, backward colors n_c - 2 .. c_lo), between per-color launches;
-// its <r,r> / <r,z> partials go to the slot regions of those colors (one per
-// CTA in the first region of each, zeros in the others), which the
-// iteration's last launch sums.
+// last color, backward colors n_c - 2 .. c_lo), between per-color launches.
+// The <r,r> / <r,z> partials of a tail go to the slot regions of its colors
+// (from rr0; one per CTA in the first of the ntail regions, zeros in the others).
 template <typename PT, bool UPDATE>
 __global__ void __launch_bounds__(kCoopWarps * kWarp)
 coop_sweep_kernel(Params P, int c_lo, int fin, int rr0, int ntail) {
-  __shared__ double red[kMaxWarpsPerCta];
+  __shared__ double red[kRed];
   __shared__ int flag;
   const int lane = threadIdx.x & 31;
   const int nw = int(blockDim.x >> 5), gw = int(blockIdx.x) * nw + int(threadIdx.x >> 5);
   const int NW = int(gridDim.x) * nw, nc = P.n_c;
   double rr_acc = 0.0, rz_acc = 0.0;
   pdl_wait();
-  const double alpha = UPDATE ? __ldcg(&P.sc->alpha) : 0.0;
+  double alpha = 0.0;
+  if (UPDATE && !load_alpha(P, alpha)) return;
   GridSync gs{P.bar, 0u, &flag, nullptr, 0, 0, P.wait_ns};
   bool ok = true;
   for (int c = c_lo; c < nc - 1 && ok; ++c) {
@@ -2780,24 +2849,16 @@ coop_sweep_kernel(Params P, int c_lo, int fin, int rr0, int ntail) {
     if (threadIdx.x == 0) {
       P.sc->status = ICCG_ERR_TIMEOUT;
       P.sc->done = 1;
+      P.sc->skip = 1.0;
       set_condition(P.sc, 0);
     }
     return;
   }
-  if (c_lo > 0) {
-    const double rr_c = UPDATE ? cta_sum(rr_acc, red) : 0.0;
-    const double rz_c = cta_sum(rz_acc, red);
-    if (threadIdx.x == 0) {
-      const int G = int(gridDim.x), b = int(blockIdx.x);
-      for (int k = 0; k < ntail; ++k) {
-        if (UPDATE) P.slot_rr[rr0 + k * G + b] = k == 0 ? rr_c : 0.0;
-        P.slot_rz[k * G + b] = k == 0 ? rz_c : 0.0;
-      }
-    }
-    return;
-  }
-  if (fin == FIN_NONE) return;
-  launch_epilogue(P, fin, SlotArgs{0, 0, 0, 0}, UPDATE, true, rr_acc, rz_acc, red, &flag);
+  if (rr0 < 0) return;   // no sums wanted
+  launch_epilogue(P, fin, SlotArgs{rr0, 0}, rr_acc, rz_acc, red, &flag);
+  const int G = int(gridDim.x), b = int(blockIdx.x);
+  if (threadIdx.x == 0)
+    for (int k = 1; k < ntail; ++k) P.slot_rr[rr0 + k * G + b] = P.slot_rz[rr0 + k * G + b] = 0.0;
 }
 
 // ---------------------------------------------------------------------------
@@ -2825,11 +2886,18 @@ cudaError_t launch(void (*kernel)(KArgs...), int grid, int threads, int smem, co
   cfg.blockDim = dim3(unsigned(threads));
   cfg.dynamicSmemBytes = size_t(smem);
   cfg.stream = L.stream;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchAttribute attr[2];
+  int na = 0;
+  if (L.carve >= 0) {
+    attr[na].id = cudaLaunchAttributePreferredSharedMemoryCarveout;
+    attr[na++].val.sharedMemCarveout = unsigned(L.carve);
+  }
+  if (L.pdl) {
+    attr[na].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[na++].val.programmaticStreamSerializationAllowed = 1;
+  }
   cfg.attrs = attr;
-  cfg.numAttrs = L.pdl ? 1 : 0;
+  cfg.numAttrs = unsigned(na);
   return cudaLaunchKernelEx(&cfg, kernel, args...);
 }
 
@@ -2897,14 +2965,14 @@ cudaError_t launch_pair(const Params &P, const Plan &L, int c, int mode, bool up
 template <typename PT, int S>
 cudaError_t launch_unit_s(const Params &P, const Plan &L, int c, int mode, bool update, int fin, const SlotArgs &sa) {
   const int g = L.grid_c[c], t0 = L.unit0[c], t1 = L.unit1[c], th = kUnitWarps * kWarp;
-  const int sm = unit_smem_bytes(S, int(sizeof(PT)));
-  if (mode == M_BWD) return launch(unit_kernel<PT, M_BWD, false, S>, g, th, sm, L, P, t0, t1, fin, sa);
+  const int T = L.unit_T[c], sm = unit_smem_bytes(T, int(sizeof(PT)));
+  if (mode == M_BWD) return launch(unit_kernel<PT, M_BWD, false, S>, g, th, sm, L, P, t0, t1, T, fin, sa);
   if (update) {
-    if (mode == M_FUSED) return launch(unit_kernel<PT, M_FUSED, true, S>, g, th, sm, L, P, t0, t1, fin, sa);
-    return launch(unit_kernel<PT, M_FWD, true, S>, g, th, sm, L, P, t0, t1, fin, sa);
+    if (mode == M_FUSED) return launch(unit_kernel<PT, M_FUSED, true, S>, g, th, sm, L, P, t0, t1, T, fin, sa);
+    return launch(unit_kernel<PT, M_FWD, true, S>, g, th, sm, L, P, t0, t1, T, fin, sa);
   }
-  if (mode == M_FUSED) return launch(unit_kernel<PT, M_FUSED, false, S>, g, th, sm, L, P, t0, t1, fin, sa);
-  return launch(unit_kernel<PT, M_FWD, false, S>, g, th, sm, L, P, t0, t1, fin, sa);
+  if (mode == M_FUSED) return launch(unit_kernel<PT, M_FUSED, false, S>, g, th, sm, L, P, t0, t1, T, fin, sa);
+  return launch(unit_kernel<PT, M_FWD, false, S>, g, th, sm, L, P, t0, t1, T, fin, sa);
 }
 
 template <typename PT>
@@ -2919,22 +2987,20 @@ cudaError_t launch_unit(const Params &P, const Plan &L, int c, int mode, bool up
   }
 }
 
+// Forward launch of color c, with its backward sweep when fused; sums: <r,r> and
+// <r,z> are wanted.
 template <typename PT>
-cudaError_t launch_fwd(const Params &P, const Plan &L, int c, bool update, bool fused, int fin) {
-  if (L.unit1[c] > L.unit0[c])
-    return launch_unit<PT>(P, L, c, fused ? M_FUSED : M_FWD, update, fin, SlotArgs{L.off_rr[c], L.off_rz[c], 0, 0});
-  if (L.tile1[c] > L.tile0[c] && L.wtile[c] == 2)
-    return launch_pair<PT>(P, L, c, fused ? M_FUSED : M_FWD, update, fin, SlotArgs{L.off_rr[c], L.off_rz[c], 0, 0});
-  if (L.tile1[c] > L.tile0[c] && L.wtile[c])
-    return launch_wtile<PT>(P, L, c, fused ? M_FUSED : M_FWD, update, fin, SlotArgs{L.off_rr[c], L.off_rz[c], 0, 0});
-  if (L.tile1[c] > L.tile0[c])
-    return launch_tile<PT>(P, L, c, fused ? M_FUSED : M_FWD, update, fin, SlotArgs{L.off_rr[c], L.off_rz[c], 0, 0});
+cudaError_t launch_fwd(const Params &P, const Plan &L, int c, bool update, bool fused, bool sums, int fin) {
+  const SlotArgs sa{sums ? L.off[c] : -1, 0};   // a final fused launch (one color) has no earlier slots
+  const int mode = fused ? M_FUSED : M_FWD;
+  if (L.unit1[c] > L.unit0[c]) return launch_unit<PT>(P, L, c, mode, update, fin, sa);
+  if (L.tile1[c] > L.tile0[c] && L.wtile[c] == 2) return launch_pair<PT>(P, L, c, mode, update, fin, sa);
+  if (L.tile1[c] > L.tile0[c] && L.wtile[c]) return launch_wtile<PT>(P, L, c, mode, update, fin, sa);
+  if (L.tile1[c] > L.tile0[c]) return launch_tile<PT>(P, L, c, mode, update, fin, sa);
   const int threads = L.W * kWarp;
   const GroupSmemPlan pl = plan_of<PT>(P, fused, false);
   const int smem = pl.total;
   const int g = L.grid_c[c], t0 = L.task0[c], t1 = L.task1[c];
-  // a final fused launch (one color) has no earlier slots
-  const SlotArgs sa{L.off_rr[c], L.off_rz[c], 0, 0};
   if (update) {
     if (fused) return launch(color_kernel<PT, M_FUSED, true>, g, threads, smem, L, P, t0, t1, pl, fin, sa);
     return launch(color_kernel<PT, M_FWD, true>, g, threads, smem, L, P, t0, t1, pl, fin, sa);
@@ -2944,17 +3010,15 @@ cudaError_t launch_fwd(const Params &P, const Plan &L, int c, bool update, bool 
 }
 
 template <typename PT>
-cudaError_t launch_bwd(const Params &P, const Plan &L, int c, int fin) {
+cudaError_t launch_bwd(const Params &P, const Plan &L, int c, bool sums, int fin) {
   const GroupSmemPlan pl = plan_of<PT>(P, false, true);
-  // the final backward launch sums the <r,r> slots only in an iteration (the
-  // solve start has no x / r update)
-  const SlotArgs sa{0, L.off_rz[c], fin == FIN_ITER ? L.last_rr : 0, L.last_rz};
+  const SlotArgs sa{sums ? L.off[c] : -1, L.off[c]};
   if (L.unit1[c] > L.unit0[c]) return launch_unit<PT>(P, L, c, M_BWD, false, fin, sa);
   if (L.tile1[c] > L.tile0[c] && L.wtile[c] == 2) return launch_pair<PT>(P, L, c, M_BWD, false, fin, sa);
   if (L.tile1[c] > L.tile0[c] && L.wtile[c]) return launch_wtile<PT>(P, L, c, M_BWD, false, fin, sa);
   if (L.tile1[c] > L.tile0[c]) return launch_tile<PT>(P, L, c, M_BWD, false, fin, sa);
-  return launch(color_kernel<PT, M_BWD, false>, L.grid_c[c], L.W * kWarp, pl.total, L, P, L.task0[c],
-                L.task1[c], pl, fin, sa);
+  return launch(color_kernel<PT, M_BWD, false>, L.grid_c[c], L.W * kWarp, pl.total, L, P, L.task0[c], L.task1[c], pl,
+                fin, sa);
 }
 
 // Forward sweep (with or without the x/r update), fused last color, backward
@@ -2963,62 +3027,46 @@ template <typename PT>
 cudaError_t launch_coop_sweep(const Params &P, const Plan &L, bool update, int fin) {
   cudaError_t e = cudaMemsetAsync(P.bar, 0, sizeof(GridBar), L.stream);
   if (e != cudaSuccess) return e;
-  if (update) return launch_coop(coop_sweep_kernel<PT, true>, L.grid_coop, kCoopWarps * kWarp, 0, L.stream, P, 0, fin, 0, 0);
-  return launch_coop(coop_sweep_kernel<PT, false>, L.grid_coop, kCoopWarps * kWarp, 0, L.stream, P, 0, fin, 0, 0);
+  const int rr0 = fin == FIN_NONE ? -1 : 0;
+  if (update) return launch_coop(coop_sweep_kernel<PT, true>, L.grid_coop, kCoopWarps * kWarp, 0, L.stream, P, 0, fin, rr0, 1);
+  return launch_coop(coop_sweep_kernel<PT, false>, L.grid_coop, kCoopWarps * kWarp, 0, L.stream, P, 0, fin, rr0, 1);
 }
 
 // the sweep's tail colors (tail_c .. n_c - 1) in one cooperative launch
 template <typename PT>
-cudaError_t launch_coop_tail(const Params &P, const Plan &L, bool update) {
+cudaError_t launch_coop_tail(const Params &P, const Plan &L, bool update, bool sums) {
   cudaError_t e = cudaMemsetAsync(P.bar, 0, sizeof(GridBar), L.stream);
   if (e != cudaSuccess) return e;
-  const int ct = L.tail_c, nt = L.n_c - ct, rr0 = L.off_rr[ct];
+  const int ct = L.tail_c, nt = L.n_c - ct, rr0 = sums ? L.off[L.n_c - 1] : -1;
   if (update)
-    return launch_coop(coop_sweep_kernel<PT, true>, L.grid_tail, kCoopWarps * kWarp, 0, L.stream, P, ct, int(FIN_NONE),
-                       rr0, nt);
-  return launch_coop(coop_sweep_kernel<PT, false>, L.grid_tail, kCoopWarps * kWarp, 0, L.stream, P, ct, int(FIN_NONE),
-                     rr0, nt);
+    return launch_coop(coop_sweep_kernel<PT, true>, L.grid_tail, kCoopWarps * kWarp, 0, L.stream, P, ct, int(FIN_NONE), rr0, nt);
+  return launch_coop(coop_sweep_kernel<PT, false>, L.grid_tail, kCoopWarps * kWarp, 0, L.stream, P, ct, int(FIN_NONE), rr0, nt);
 }
 
 template <typename PT>
 cudaError_t sweep(const Params &P, const Plan &L, bool update, int fin_last, PhaseHook h, void *u) {
   cudaError_t e = cudaSuccess;
-  const int nc = L.n_c;
+  const int nc = L.n_c, ct = L.tail_c > 0 ? L.tail_c : nc - 1;   // forward launches of their own
+  const bool sums = fin_last != FIN_NONE;
   if (L.coop) {
     if (h) h(u, PH_FWD, 1);
     e = launch_coop_sweep<PT>(P, L, update, fin_last);
     if (h) h(u, PH_FWD, 0);
     return e;
   }
-  if (L.tail_c > 0) {
-    for (int c = 0; c < L.tail_c && e == cudaSuccess; ++c) {
-      if (h) h(u, PH_FWD, 1);
-      e = launch_fwd<PT>(P, L, c, update, false, FIN_NONE);
-      if (h) h(u, PH_FWD, 0);
-    }
-    if (e != cudaSuccess) return e;
-    if (h) h(u, PH_FUSED, 1);
-    e = launch_coop_tail<PT>(P, L, update);
-    if (h) h(u, PH_FUSED, 0);
-    for (int c = L.tail_c - 1; c >= 0 && e == cudaSuccess; --c) {
-      if (h) h(u, PH_BWD, 1);
-      e = launch_bwd<PT>(P, L, c, c == 0 ? fin_last : FIN_NONE);
-      if (h) h(u, PH_BWD, 0);
-    }
-    return e;
-  }
-  for (int c = 0; c < nc - 1 && e == cudaSuccess; ++c) {
+  for (int c = 0; c < ct && e == cudaSuccess; ++c) {
     if (h) h(u, PH_FWD, 1);
-    e = launch_fwd<PT>(P, L, c, update, false, FIN_NONE);
+    e = launch_fwd<PT>(P, L, c, update, false, false, FIN_NONE);
     if (h) h(u, PH_FWD, 0);
   }
   if (e != cudaSuccess) return e;
   if (h) h(u, PH_FUSED, 1);
-  e = launch_fwd<PT>(P, L, nc - 1, update, true, nc == 1 ? fin_last : FIN_NONE);
+  e = L.tail_c > 0 ? launch_coop_tail<PT>(P, L, update, sums)
+                   : launch_fwd<PT>(P, L, nc - 1, update, true, sums, nc == 1 ? fin_last : FIN_NONE);
   if (h) h(u, PH_FUSED, 0);
-  for (int c = nc - 2; c >= 0 && e == cudaSuccess; --c) {
+  for (int c = ct - 1; c >= 0 && e == cudaSuccess; --c) {
     if (h) h(u, PH_BWD, 1);
-    e = launch_bwd<PT>(P, L, c, c == 0 ? fin_last : FIN_NONE);
+    e = launch_bwd<PT>(P, L, c, sums, c == 0 ? fin_last : FIN_NONE);
     if (h) h(u, PH_BWD, 0);
   }
   return e;
@@ -3035,6 +3083,16 @@ cudaError_t allow_smem(K kernel) {
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
   return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, optin - 1024);
+}
+
+template <typename PT, int S>
+cudaError_t allow_unit() {
+  cudaError_t e = allow_smem(unit_kernel<PT, M_FWD, true, S>);
+  if (e == cudaSuccess) e = allow_smem(unit_kernel<PT, M_FWD, false, S>);
+  if (e == cudaSuccess) e = allow_smem(unit_kernel<PT, M_FUSED, true, S>);
+  if (e == cudaSuccess) e = allow_smem(unit_kernel<PT, M_FUSED, false, S>);
+  if (e == cudaSuccess) e = allow_smem(unit_kernel<PT, M_BWD, false, S>);
+  return e;
 }
 
 template <typename PT>
@@ -3061,11 +3119,12 @@ cudaError_t configure_pt() {
   if (e == cudaSuccess) e = allow_smem(wtile_kernel<PT, M_FUSED, false>);
   if (e == cudaSuccess) e = allow_smem(wtile_kernel<PT, M_FWD, false>);
   if (e == cudaSuccess) e = allow_smem(wtile_kernel<PT, M_BWD, false>);
-  if (e == cudaSuccess) e = allow_smem(unit_kernel<PT, M_FWD, true, 32>);
-  if (e == cudaSuccess) e = allow_smem(unit_kernel<PT, M_FWD, false, 32>);
-  if (e == cudaSuccess) e = allow_smem(unit_kernel<PT, M_FUSED, true, 32>);
-  if (e == cudaSuccess) e = allow_smem(unit_kernel<PT, M_FUSED, false, 32>);
-  if (e == cudaSuccess) e = allow_smem(unit_kernel<PT, M_BWD, false, 32>);
+  if (e == cudaSuccess) e = allow_unit<PT, 1>();
+  if (e == cudaSuccess) e = allow_unit<PT, 2>();
+  if (e == cudaSuccess) e = allow_unit<PT, 4>();
+  if (e == cudaSuccess) e = allow_unit<PT, 8>();
+  if (e == cudaSuccess) e = allow_unit<PT, 16>();
+  if (e == cudaSuccess) e = allow_unit<PT, 32>();
   return e;
 }
 
@@ -3124,10 +3183,10 @@ int coop_sweep_resident_ctas(bool fp32) {
   return nb;
 }
 
-int unit_resident_ctas(bool fp32, int S, int threads) {
+int unit_resident_ctas(bool fp32, int S, int T, int threads) {
   int nb = 0;
   cudaError_t e;
-  const size_t sm = size_t(unit_smem_bytes(S <= 8 ? 8 : 32, fp32 ? 4 : 8));
+  const size_t sm = size_t(unit_smem_bytes(T, fp32 ? 4 : 8));
   if (fp32) {
     e = S <= 8 ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, unit_kernel<float, M_FWD, true, 8>, threads, sm)
                : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, unit_kernel<float, M_FWD, true, 32>, threads, sm);
@@ -3149,6 +3208,11 @@ int spmv_resident_ctas(int Wa, int smem) {
     return 1;
   }
   return nb > 0 ? nb : 1;
+}
+
+int solve_body_iterations(const Plan &L) {
+  const int64_t launches = 2 + (L.coop ? 1 : 2 * int64_t(L.n_c) - 1);
+  return int(std::max<int64_t>(1, std::min<int64_t>(L.body, 160 / std::max<int64_t>(launches, 1))));
 }
 
 int persistent_smem_bytes(const Params &P, bool fp32, int W, int budget, int *cap_spmv) {
