@@ -8,7 +8,8 @@
 //
 // Building blocks: an exclusive scan, a stable LSD radix sort of 64-bit keys
 // (4-bit digits; each thread ranks 8 consecutive keys, so equal digits keep
-// their order), and compaction by flags.  The greedy coloring is exact in
+// their order), a bucket form of pairs -> CSR for short rows, and compaction by
+// flags.  The greedy coloring is exact in
 // parallel: block b's color depends only on the colors of its neighbours
 // with a smaller index, so b is colored in the wave after the last of those
 // (Jones-Plassmann with index priorities), and every wave gives exactly the
@@ -257,10 +258,120 @@ __global__ void unique_emit(const uint64_t *key, const int64_t *flag, const int6
     }
 }
 
+// The same for rows of at most kRowMax pairs: the pairs are put into their
+// rows' buckets (counted first), and a warp sorts and de-duplicates a row in
+// registers.  Three passes over the pairs instead of the radix sort's two per
+// 4 key bits (20 for a million rows).
+constexpr int kRowMax = 64;
+
+__global__ void bucket_count(const uint64_t *key, int64_t n, uint64_t none, uint64_t ncol, int64_t *rowcnt) {
+  for (int64_t k = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; k < n; k += int64_t(gridDim.x) * blockDim.x)
+    if (key[k] != none) atomicAdd(reinterpret_cast<unsigned long long *>(rowcnt + key[k] / ncol), 1ull);
+}
+
+__global__ void row_max(const int64_t *rowcnt, int64_t nrow, int *most) {
+  int v = 0;
+  for (int64_t r = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; r < nrow; r += int64_t(gridDim.x) * blockDim.x)
+    v = max(v, int(min(rowcnt[r], int64_t(1 << 30))));
+  v = __reduce_max_sync(0xffffffffu, v);
+  if ((threadIdx.x & 31) == 0 && v > 0) atomicMax(most, v);
+}
+
+__global__ void bucket_fill(const uint64_t *key, int64_t n, uint64_t none, uint64_t ncol, const int64_t *start,
+                            int32_t *fill, int32_t *col) {
+  for (int64_t k = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; k < n; k += int64_t(gridDim.x) * blockDim.x)
+    if (key[k] != none) {
+      const uint64_t r = key[k] / ncol;
+      col[start[r] + atomicAdd(fill + r, 1)] = int32_t(key[k] % ncol);
+    }
+}
+
+// a warp per row: ranks its distinct columns among themselves, two per lane
+__global__ void bucket_sort(const int64_t *start, int64_t nrow, int32_t *col, int64_t *ucnt) {
+  const int lane = threadIdx.x & 31;
+  const int64_t nw = int64_t(gridDim.x) * (blockDim.x >> 5);
+  for (int64_t r = (int64_t(blockIdx.x) * blockDim.x + threadIdx.x) >> 5; r < nrow; r += nw) {
+    const int64_t b = start[r];
+    const int c = int(start[r + 1] - b);
+    const int32_t none = 0x7fffffff;
+    const int32_t v0 = lane < c ? col[b + lane] : none, v1 = lane + 32 < c ? col[b + lane + 32] : none;
+    bool k0 = lane < c, k1 = lane + 32 < c;   // no equal column before it
+    for (int j = 0; j < c; ++j) {
+      const int32_t u = __shfl_sync(0xffffffffu, j < 32 ? v0 : v1, j & 31);
+      if (j < lane && u == v0) k0 = false;
+      if (j < lane + 32 && u == v1) k1 = false;
+    }
+    const unsigned m0 = __ballot_sync(0xffffffffu, k0), m1 = __ballot_sync(0xffffffffu, k1);
+    int p0 = 0, p1 = 0;                       // kept columns below it
+    for (int j = 0; j < c; ++j) {
+      const int32_t u = __shfl_sync(0xffffffffu, j < 32 ? v0 : v1, j & 31);
+      if (((j < 32 ? m0 : m1) >> (j & 31)) & 1u) {
+        p0 += u < v0 ? 1 : 0;
+        p1 += u < v1 ? 1 : 0;
+      }
+    }
+    if (k0) col[b + p0] = v0;
+    if (k1) col[b + p1] = v1;
+    if (lane == 0) ucnt[r] = __popc(m0) + __popc(m1);
+  }
+}
+
+// eight lanes a row: the rows without the gaps that duplicates left
+__global__ void bucket_emit(const int64_t *start, const int64_t *ptr, int64_t nrow, const int32_t *col, int32_t *adj) {
+  const int l = threadIdx.x & 7;
+  const int64_t ng = int64_t(gridDim.x) * (blockDim.x >> 3);
+  for (int64_t r = (int64_t(blockIdx.x) * blockDim.x + threadIdx.x) >> 3; r < nrow; r += ng) {
+    const int64_t b = start[r], o = ptr[r], c = ptr[r + 1] - o;
+    for (int64_t k = l; k < c; k += 8) adj[o + k] = col[b + k];
+  }
+}
+
+// *short_rows = false (and nothing written) when a row has more than kRowMax pairs
+cudaError_t pairs_to_csr_short(const uint64_t *key, int64_t n, uint64_t nrow, uint64_t ncol, int64_t *ptr,
+                               int32_t *adj, int64_t *m, Scratch &S, bool *short_rows) {
+  const uint64_t none = nrow * ncol;
+  *short_rows = false;
+  int64_t *start = S.get<int64_t>(size_t(nrow) + 1), *ucnt = S.get<int64_t>(size_t(nrow) + 1);
+  int32_t *fill = S.get<int32_t>(size_t(nrow) + 1), *col = S.get<int32_t>(size_t(n));
+  int *most = S.get<int>(1);
+  if (S.err != cudaSuccess) return S.err;
+  const int64_t nr = int64_t(nrow);
+  cudaError_t e = cudaMemsetAsync(start, 0, (size_t(nrow) + 1) * sizeof(int64_t), S.s);
+  if (e == cudaSuccess) e = cudaMemsetAsync(fill, 0, (size_t(nrow) + 1) * sizeof(int32_t), S.s);
+  if (e == cudaSuccess) e = cudaMemsetAsync(ucnt, 0, (size_t(nrow) + 1) * sizeof(int64_t), S.s);
+  if (e == cudaSuccess) e = cudaMemsetAsync(most, 0, sizeof(int), S.s);
+  if (e != cudaSuccess) return e;
+  bucket_count<<<grid_for(n), kT, 0, S.s>>>(key, n, none, ncol, start);
+  row_max<<<std::min(grid_for(nr), 1216), kT, 0, S.s>>>(start, nr, most);
+  int h = 0;
+  e = cudaGetLastError();
+  if (e == cudaSuccess) e = cudaMemcpyAsync(&h, most, sizeof(int), cudaMemcpyDeviceToHost, S.s);
+  if (e == cudaSuccess) e = cudaStreamSynchronize(S.s);
+  if (e != cudaSuccess || h > kRowMax) return e;
+  *short_rows = true;
+  e = scan(start, start, nr + 1, S);
+  if (e != cudaSuccess) return e;
+  bucket_fill<<<grid_for(n), kT, 0, S.s>>>(key, n, none, ncol, start, fill, col);
+  bucket_sort<<<grid_for(nr, kT / 32), kT, 0, S.s>>>(start, nr, col, ucnt);
+  e = cudaGetLastError();
+  if (e == cudaSuccess) e = scan(ucnt, ptr, nr + 1, S);
+  if (e != cudaSuccess) return e;
+  bucket_emit<<<grid_for(nr, kT / 8), kT, 0, S.s>>>(start, ptr, nr, col, adj);
+  e = cudaGetLastError();
+  if (e == cudaSuccess) e = cudaMemcpyAsync(m, ptr + nr, sizeof(int64_t), cudaMemcpyDeviceToHost, S.s);
+  if (e == cudaSuccess) e = cudaStreamSynchronize(S.s);
+  return e;
+}
+
 // sorts keys, writes ptr[nrow+1] and adj (capacity n), *m = entries (host)
 cudaError_t pairs_to_csr(uint64_t *key, int64_t n, uint64_t nrow, uint64_t ncol, int64_t *ptr, int32_t *adj,
                          int64_t *m, Scratch &S) {
   const uint64_t none = nrow * ncol;
+  if (n > 0 && nrow > 0) {
+    bool short_rows = false;
+    const cudaError_t es = pairs_to_csr_short(key, n, nrow, ncol, ptr, adj, m, S, &short_rows);
+    if (es != cudaSuccess || short_rows) return es;
+  }
   cudaError_t e = radix_sort(key, nullptr, n, bits_for(none), S);
   int64_t *flag = S.get<int64_t>(size_t(n) + 1);
   int64_t *rowcnt = S.get<int64_t>(size_t(nrow) + 1);
@@ -374,29 +485,59 @@ __global__ void lower_counts(int32_t n_b, const int64_t *bptr, const int32_t *ba
   }
 }
 
-// One wave: every listed block has all smaller neighbours colored; its color
-// is the smallest one none of them has.  Then each larger neighbour loses one
+// Wave k: every listed block has all smaller neighbours colored; its color is
+// the smallest one none of them has.  Then each larger neighbour loses one
 // pending smaller neighbour and joins the next wave when none is left.
-__global__ void color_wave(const int32_t *wave, int32_t nw, const int64_t *bptr, const int32_t *badj, int32_t *lower,
-                           int32_t *color, int32_t *next, int32_t *next_n, int32_t *ncolor) {
-  for (int64_t k = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; k < nw; k += int64_t(gridDim.x) * blockDim.x) {
-    const int32_t b = wave[k];
+// cnt[k % 3]: this wave's blocks, cnt[(k + 1) % 3]: the next one's (the third is
+// cleared for the wave after it), cnt[3]: colors used, cnt[4]: blocks colored.
+//
+// Bound by latency: hundreds of waves of a few thousand blocks follow one
+// another, so eight lanes share a block (its neighbours' loads in flight
+// together; a thread per block walked them one after another, 36 us a wave), and
+// the counts stay on the device, so that kWavesPerSync waves are launched
+// before the host looks (an empty wave costs 2 us, a look at the host 10).
+constexpr int kWaveLanes = 8;
+constexpr int kWavesPerSync = 16;
+constexpr int kWaveGrid = 304;   // CTAs of a wave
+
+__global__ void color_wave(int k, int32_t n_b, int32_t *waves, const int64_t *bptr, const int32_t *badj,
+                           int32_t *lower, int32_t *color, int32_t *cnt) {
+  const int32_t nw = cnt[k % 3], *wave = waves + size_t(k & 1) * size_t(n_b);
+  int32_t *next = waves + size_t((k + 1) & 1) * size_t(n_b), *next_n = cnt + (k + 1) % 3;
+  const int l = threadIdx.x & (kWaveLanes - 1);
+  const unsigned mask = ((1u << kWaveLanes) - 1u) << (threadIdx.x & 31 & ~(kWaveLanes - 1));
+  if (blockIdx.x == 0 && threadIdx.x == 0) {
+    cnt[(k + 2) % 3] = 0;
+    cnt[4] += nw;
+  }
+  const int64_t stride = int64_t(gridDim.x) * blockDim.x / kWaveLanes;
+  for (int64_t g = (int64_t(blockIdx.x) * blockDim.x + threadIdx.x) / kWaveLanes; g < nw; g += stride) {
+    const int32_t b = wave[g];
     const int64_t e0 = bptr[b], e1 = bptr[b + 1];
     int32_t c = 0;
     for (int base = 0;; base += 64) {
-      uint64_t used = 0;
-      for (int64_t e = e0; e < e1 && badj[e] < b; ++e) {
-        const int32_t q = color[badj[e]] - base;
-        if (q >= 0 && q < 64) used |= 1ull << q;
+      unsigned lo = 0, hi = 0;
+      for (int64_t e = e0 + l; e < e1; e += kWaveLanes) {
+        const int32_t u = badj[e];
+        if (u < b) {
+          const int32_t q = color[u] - base;
+          if (q >= 0 && q < 32) lo |= 1u << q;
+          else if (q >= 32 && q < 64) hi |= 1u << (q - 32);
+        }
       }
+      lo = __reduce_or_sync(mask, lo);
+      hi = __reduce_or_sync(mask, hi);
+      const uint64_t used = (uint64_t(hi) << 32) | lo;
       if (~used != 0) {
         c = base + __ffsll(static_cast<long long>(~used)) - 1;
         break;
       }
     }
-    color[b] = c;
-    atomicMax(ncolor, c + 1);
-    for (int64_t e = e0; e < e1; ++e) {
+    if (l == 0) {
+      color[b] = c;
+      if (c >= cnt[3]) atomicMax(cnt + 3, c + 1);
+    }
+    for (int64_t e = e0 + l; e < e1; e += kWaveLanes) {
       const int32_t u = badj[e];
       if (u > b && atomicSub(lower + u, 1) == 1) next[atomicAdd(next_n, 1)] = u;
     }
@@ -410,11 +551,15 @@ __global__ void keys_from(int64_t n, const int32_t *a, uint64_t *key, int32_t *v
   }
 }
 
-__global__ void block_rank_size(int32_t n_b, const int32_t *order, int32_t *rank, const int32_t *color,
-                                int32_t *color_cnt) {
+// ranks of the blocks in (color, index) order, and where each color starts
+// (every color has a block)
+__global__ void block_rank(int32_t n_b, const int32_t *order, int32_t *rank, const int32_t *color, int32_t ncol,
+                           int32_t *color_ptr) {
   for (int64_t k = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; k < n_b; k += int64_t(gridDim.x) * blockDim.x) {
-    rank[order[k]] = int32_t(k);
-    atomicAdd(color_cnt + color[order[k]], 1);
+    const int32_t b = order[k], c = color[b];
+    rank[b] = int32_t(k);
+    if (k == 0 || color[order[k - 1]] != c) color_ptr[c] = int32_t(k);
+    if (k == n_b - 1) color_ptr[ncol] = n_b;
   }
 }
 
@@ -574,8 +719,8 @@ __global__ void lm_decide(DGraph g, const int32_t *comm, const int64_t *W, const
 // a proposed move happens when it is the best proposal into its target (at
 // most one node joins a community per sub-round) and no node joins the
 // mover's own community; a move to a new community always happens
-__global__ void lm_apply(int32_t n, const int32_t *comm, const int32_t *newc, const int32_t *cnt,
-                         const unsigned long long *join, int32_t *out, int32_t *moved) {
+__global__ void lm_apply(int32_t n, int32_t *comm, const int32_t *newc, const int32_t *cnt,
+                         const unsigned long long *join, int32_t *moved) {
   for (int64_t vv = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; vv < n; vv += int64_t(gridDim.x) * blockDim.x) {
     const int32_t v = int32_t(vv), C = comm[v], D = newc[v];
     int32_t r = C;
@@ -583,8 +728,10 @@ __global__ void lm_apply(int32_t n, const int32_t *comm, const int32_t *newc, co
       if (D == v && cnt[v] == 0) r = D;
       else if (join[C] == 0 && (join[D] & 0xffffffffull) == 0xffffffffull - uint32_t(v)) r = D;
     }
-    out[v] = r;
-    if (r != C) atomicAdd(moved, 1);
+    if (r != C) {
+      comm[v] = r;   // read by this thread alone
+      *moved = 1;
+    }
   }
 }
 
@@ -645,14 +792,16 @@ __global__ void refine_decide(DGraph g, const int32_t *comm, const int64_t *W, c
   }
 }
 
-__global__ void refine_apply(int32_t n, const int32_t *sub, const int32_t *newsub, const unsigned long long *join,
-                             int32_t *out, int32_t *moved) {
+__global__ void refine_apply(int32_t n, int32_t *sub, const int32_t *newsub, const unsigned long long *join,
+                             int32_t *moved) {
   for (int64_t vv = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; vv < n; vv += int64_t(gridDim.x) * blockDim.x) {
     const int32_t v = int32_t(vv), s0 = sub[v], t = newsub[v];
     int32_t r = s0;
     if (t != s0 && join[v] == 0 && (join[t] & 0xffffffffull) == 0xffffffffull - uint32_t(v)) r = t;
-    out[v] = r;
-    if (r != s0) atomicAdd(moved, 1);
+    if (r != s0) {
+      sub[v] = r;   // read by this thread alone
+      *moved = 1;
+    }
   }
 }
 
@@ -785,7 +934,6 @@ struct LeidenRun {
 
   void move_nodes(const DGraph &g, int32_t *comm, int64_t *W, int32_t *cnt, int32_t *tmp) {
     unsigned long long *join = S.get<unsigned long long>(size_t(g.n));
-    int32_t *out = S.get<int32_t>(size_t(g.n));
     if (S.err != cudaSuccess) { e = S.err; return; }
     int idle = 0;
     for (int r = 0; r < kSubRounds && idle < 2 && e == cudaSuccess; ++r) {
@@ -793,8 +941,7 @@ struct LeidenRun {
       if (e == cudaSuccess) e = cudaMemsetAsync(dmoved, 0, sizeof(int32_t), s);
       if (e == cudaSuccess) e = cudaMemsetAsync(join, 0, size_t(g.n) * sizeof(unsigned long long), s);
       go(lm_decide, g.n, g, comm, W, cnt, gp, r & 1, tmp, join);
-      go(lm_apply, g.n, g.n, comm, tmp, cnt, join, out, dmoved);
-      if (e == cudaSuccess) e = cudaMemcpyAsync(comm, out, size_t(g.n) * sizeof(int32_t), cudaMemcpyDeviceToDevice, s);
+      go(lm_apply, g.n, g.n, comm, static_cast<const int32_t *>(tmp), cnt, join, dmoved);
       idle = read_i32(dmoved) == 0 ? idle + 1 : 0;
     }
     weights(g, comm, W, cnt);
@@ -804,7 +951,6 @@ struct LeidenRun {
               int64_t *subE, int32_t *tmp) {
     go(iota_i32, g.n, int64_t(g.n), sub);
     unsigned long long *join = S.get<unsigned long long>(size_t(g.n));
-    int32_t *out = S.get<int32_t>(size_t(g.n));
     if (S.err != cudaSuccess) { e = S.err; return; }
     int idle = 0;
     for (int r = 0; r < kSubRounds && idle < 2 && e == cudaSuccess; ++r) {
@@ -814,8 +960,7 @@ struct LeidenRun {
       if (e == cudaSuccess) e = cudaMemsetAsync(dmoved, 0, sizeof(int32_t), s);
       if (e == cudaSuccess) e = cudaMemsetAsync(join, 0, size_t(g.n) * sizeof(unsigned long long), s);
       go(refine_decide, g.n, g, comm, W, sub, SW, subN, subE, gp, r & 1, tmp, join);
-      go(refine_apply, g.n, g.n, sub, tmp, join, out, dmoved);
-      if (e == cudaSuccess) e = cudaMemcpyAsync(sub, out, size_t(g.n) * sizeof(int32_t), cudaMemcpyDeviceToDevice, s);
+      go(refine_apply, g.n, g.n, sub, static_cast<const int32_t *>(tmp), join, dmoved);
       idle = read_i32(dmoved) == 0 ? idle + 1 : 0;
     }
   }
@@ -966,7 +1111,7 @@ extern "C" iccg_status iccg_dev_color_order(int32_t n, const int64_t *gptr, cons
   int32_t *badj = S.get<int32_t>(size_t(m));
   int32_t *lower = S.get<int32_t>(size_t(n_b));
   int32_t *waves = S.get<int32_t>(2 * size_t(n_b));
-  int32_t *cnts = S.get<int32_t>(4);   // wave sizes (2), number of colors
+  int32_t *cnts = S.get<int32_t>(5);   // wave sizes (3), number of colors, blocks colored
   if (S.err != cudaSuccess) return ICCG_ERR_CUDA;
   cudaError_t e = cudaMemsetAsync(bad, 0, sizeof(int), s);
   if (e == cudaSuccess && n > 0) {
@@ -988,40 +1133,28 @@ extern "C" iccg_status iccg_dev_color_order(int32_t n, const int64_t *gptr, cons
   int64_t mb = 0;
   e = pairs_to_csr(key, m, uint64_t(n_b), uint64_t(n_b), bptr, badj, &mb, S);
   // waves of the exact greedy coloring
-  if (e == cudaSuccess) e = cudaMemsetAsync(cnts, 0, 4 * sizeof(int32_t), s);
+  if (e == cudaSuccess) e = cudaMemsetAsync(cnts, 0, 5 * sizeof(int32_t), s);
   if (e == cudaSuccess && n_b > 0) {
     lower_counts<<<grid_for(n_b), kT, 0, s>>>(n_b, bptr, badj, lower, waves, cnts, color_of);
     e = cudaGetLastError();
   }
-  int32_t h[4] = {0, 0, 0, 0};
-  if (e == cudaSuccess) e = cudaMemcpyAsync(h, cnts, 4 * sizeof(int32_t), cudaMemcpyDeviceToHost, s);
-  if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-  int cur = 0, done = 0;
-  int32_t nw = h[0];
-  while (e == cudaSuccess && nw > 0) {
-    const int nx = cur ^ 1;
-    e = cudaMemsetAsync(cnts + nx, 0, sizeof(int32_t), s);
-    if (e != cudaSuccess) break;
-    color_wave<<<grid_for(nw), kT, 0, s>>>(waves + size_t(cur) * size_t(n_b), nw, bptr, badj, lower, color_of,
-                                           waves + size_t(nx) * size_t(n_b), cnts + nx, cnts + 2);
-    e = cudaGetLastError();
-    if (e == cudaSuccess) e = cudaMemcpyAsync(&h[nx], cnts + nx, sizeof(int32_t), cudaMemcpyDeviceToHost, s);
+  int32_t h[5] = {0, 0, 0, 0, 0};
+  int k = 0;
+  do {
+    for (int w = 0; w < kWavesPerSync && e == cudaSuccess && n_b > 0; ++w, ++k) {
+      color_wave<<<kWaveGrid, kT, 0, s>>>(k, n_b, waves, bptr, badj, lower, color_of, cnts);
+      e = cudaGetLastError();
+    }
+    if (e == cudaSuccess) e = cudaMemcpyAsync(h, cnts, sizeof(h), cudaMemcpyDeviceToHost, s);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-    done += nw;
-    nw = h[nx];
-    cur = nx;
-  }
-  if (e == cudaSuccess && done != n_b) return ICCG_ERR_CUDA;   // every block is colored exactly once
-  if (e == cudaSuccess) e = cudaMemcpyAsync(&h[2], cnts + 2, sizeof(int32_t), cudaMemcpyDeviceToHost, s);
-  if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+  } while (e == cudaSuccess && h[k % 3] > 0);
   if (e != cudaSuccess) return ICCG_ERR_CUDA;
-  const int32_t ncol = h[2];
+  if (h[4] != n_b) return ICCG_ERR_CUDA;   // every block is colored exactly once
+  const int32_t ncol = h[3];
   *n_c = ncol;
   // blocks ordered by (color, index): a stable sort by color
   int32_t *order = S.get<int32_t>(size_t(n_b));
   int32_t *rank = S.get<int32_t>(size_t(n_b));
-  int32_t *ccnt = S.get<int32_t>(size_t(ncol) + 1);
-  int64_t *c64 = S.get<int64_t>(size_t(ncol) + 1);
   int64_t *bsz = S.get<int64_t>(size_t(n_b) + 1);
   int32_t *rv = S.get<int32_t>(size_t(n));
   if (S.err != cudaSuccess) return ICCG_ERR_CUDA;
@@ -1030,21 +1163,11 @@ extern "C" iccg_status iccg_dev_color_order(int32_t n, const int64_t *gptr, cons
     e = cudaGetLastError();
   }
   if (e == cudaSuccess) e = radix_sort(key, order, n_b, bits_for(uint64_t(ncol)), S);
-  if (e == cudaSuccess) e = cudaMemsetAsync(ccnt, 0, (size_t(ncol) + 1) * sizeof(int32_t), s);
   if (e == cudaSuccess && n_b > 0) {
-    block_rank_size<<<grid_for(n_b), kT, 0, s>>>(n_b, order, rank, color_of, ccnt);
+    block_rank<<<grid_for(n_b), kT, 0, s>>>(n_b, order, rank, color_of, ncol, color_ptr);
     e = cudaGetLastError();
   }
-  // color_ptr = scan of the per-color block counts
-  if (e == cudaSuccess) {
-    i32_to_i64<<<grid_for(ncol + 1), kT, 0, s>>>(ncol + 1, ccnt, c64);
-    e = cudaGetLastError();
-  }
-  if (e == cudaSuccess) e = scan(c64, c64, int64_t(ncol) + 1, S);
-  if (e == cudaSuccess) {
-    to_i32<<<grid_for(ncol + 1), kT, 0, s>>>(ncol + 1, c64, color_ptr);
-    e = cudaGetLastError();
-  }
+  if (e == cudaSuccess && n_b == 0) e = cudaMemsetAsync(color_ptr, 0, sizeof(int32_t), s);
   // rows ordered by (block rank, row): a stable sort by rank; block sizes
   if (e == cudaSuccess) e = cudaMemsetAsync(bsz, 0, (size_t(n_b) + 1) * sizeof(int64_t), s);
   if (e == cudaSuccess && n > 0) {
