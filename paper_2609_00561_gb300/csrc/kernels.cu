@@ -1866,9 +1866,7 @@ __global__ void __launch_bounds__(kVecThreads) widen_kernel(const float *src, do
 // ---------------------------------------------------------------------------
 // IC(0) (up-looking, rows of a group level by level, one row per lane)
 // ---------------------------------------------------------------------------
-// End of a factor row: the pivot's reciprocal, which later rows wait for
-// (one FP64 sequence instead of a square root and then a division), and its
-// square root.
+// End of a factor row: L_ii and its reciprocal, which later rows multiply by.
 __device__ __forceinline__ double factor_check(const Params &P, int i, double d) {
   if (!(d > 0.0) || !isfinite(d)) {
     atomicMin(P.err_row, (unsigned long long)i);
@@ -1877,23 +1875,17 @@ __device__ __forceinline__ double factor_check(const Params &P, int i, double d)
   return d;
 }
 __device__ __forceinline__ void factor_pivot(const Params &P, int i, double d) {
-  d = factor_check(P, i, d);
-  P.invd[i] = rsqrt(d);
-  P.ldiag[i] = sqrt(d);
-}
-// the same for a CTA's rows (d in sd, row in srow), warps 0 and 1 a part each
-__device__ __forceinline__ void factor_pivots(const Params &P, const double *sd, const int *srow, int rows, int w,
-                                              int lane) {
-  if (w == 0 && lane < rows) P.invd[srow[lane]] = rsqrt(factor_check(P, srow[lane], sd[lane]));
-  if (w == 1 && lane < rows) P.ldiag[srow[lane]] = sqrt(factor_check(P, srow[lane], sd[lane]));
+  const double lii = sqrt(factor_check(P, i, d));
+  P.ldiag[i] = lii;
+  P.invd[i] = 1.0 / lii;
 }
 
 // Row i of the up-looking IC(0): for every j < i in the pattern, ascending,
 //   L_ij = (a_ij - sum_{k < j, k in pat(i) and pat(j)} L_ik L_jk) / L_jj,
 // then L_ii = sqrt(a_ii - sum_j L_ij^2); rows j are final when row i runs.
-// A finished row also stores 1/L_ii, and later rows multiply by it, and its
-// entries times 1/L_jj (in uval, entry for entry: free until the finishing
-// pass writes U there), which is what a later row's terms use.
+// A finished row also stores 1/L_ii, and later rows multiply by it; rows without
+// precomputed pairs also their entries times 1/L_jj (in uval, entry for entry:
+// free until the finishing pass writes U there), for factor_wide_kernel.
 // General form: the common columns by a merge of the two sorted rows (a
 // chain of dependent loads).
 __device__ __forceinline__ void factor_row_merge(const Params &P, int i) {
@@ -1980,10 +1972,10 @@ __device__ __forceinline__ void factor_row(const Params &P, int i, int32_t *sc, 
 
 // One in-block level of a lane-tile or warp-unit color, a warp per row (rows
 // of 9..32 strictly-lower entries with precomputed update pairs).
-// Lane p holds entry p of the row; the pairs' values L_jk / L_kk are gathered
-// by the whole warp into shared memory, then
-//   s_p = a_ip - sum_{k < p} s_k (L_pk / L_kk),   L_ip = s_p / L_pp
-// in steps: at each, every lane whose next term's s_k is final (lane k has no
+// Lane p holds entry p of the row; the pairs' values L_jk are gathered by the
+// whole warp into shared memory, then
+//   s_p = a_ip - sum_{k < p} L_ik L_pk,   L_ip = s_p / L_pp
+// in steps: at each, every lane whose next term's L_ik is final (lane k has no
 // term left) takes it from lane k by a shuffle, k ascending per entry as in
 // the general form.
 //
@@ -1992,8 +1984,9 @@ __device__ __forceinline__ void factor_row(const Params &P, int i, int32_t *sc, 
 // thread per row walked its 60 pairs one FP64 multiply-add after another
 // (64 cycles each) behind staged copies, 44 us a level; the warp's steps are
 // as many as the deepest chain of terms or the longest list (about 10) and
-// its loads are all in flight at once.  Static data (record, columns, a_ij, pair indices)
-// is read before griddepcontrol.wait, while the previous level runs.  Square
+// its loads are all in flight at once.  Static data (record, columns, a_ij,
+// pair indices) is read before griddepcontrol.wait, while the previous level
+// runs.  Square
 // root and division are FP64 sequences that cost a whole warp however few
 // lanes run them, so one warp does them for the CTA's rows together.
 constexpr int kFacWarps = 8;
@@ -2001,23 +1994,48 @@ constexpr int kFacPairs = kFacRow * (kFacRow - 1) / 2;   // most pairs of a row
 constexpr int kFacBatch = 4;                             // pair loads in flight per lane
 constexpr int kFacWarpBytes = kFacPairs * 8 + ((kFacPairs + 15) & ~15);
 
-// the steps of one row: lane p's terms are pv / ps [c, ce)
-__device__ __forceinline__ double factor_steps(double s, int c, int ce, const double *pv, const uint8_t *ps, int lane) {
-  int src = c < ce ? int(ps[c]) : lane;
-  double nv = c < ce ? pv[c] : 0.0;
+// The steps of one row of ni entries: lane p holds s_p = a_ip, iv_p = 1/L_pp and
+// its terms pv / ps [c, ce); l_p = L_ip on return.  Lane 31 carries the pivot
+// a_ii - sum_p l_p^2 as one more entry, whose terms are the entries themselves
+// (returned in every lane; a row of 32 entries forms it afterwards).  Every sum
+// runs in the order of the general form, so the factor is the same to the bit.
+__device__ __forceinline__ double factor_steps(double s, double iv, int c, int ce, int ni, double dg, const double *pv,
+                                               const uint8_t *ps, int lane, double &l) {
+  const bool piv = lane == 31 && ni < 32;
+  if (piv) {
+    s = dg;
+    c = 0;
+    ce = ni;
+  }
+  int src = c < ce ? (piv ? 0 : int(ps[c])) : lane;
+  double nv = c < ce && !piv ? pv[c] : 0.0;
   for (uint32_t left = __ballot_sync(0xffffffffu, c < ce); left;) {
-    const double sk = __shfl_sync(0xffffffffu, s, src);
+    l = s * iv;
+    const double lk = __shfl_sync(0xffffffffu, l, src);
     if (c < ce && !((left >> src) & 1u)) {
-      s -= sk * nv;
+      s -= lk * (piv ? lk : nv);
       ++c;
       if (c < ce) {
-        src = int(ps[c]);
-        nv = pv[c];
+        src = piv ? c : int(ps[c]);
+        if (!piv) nv = pv[c];
       }
     }
     left = __ballot_sync(0xffffffffu, c < ce);
   }
-  return s;
+  l = s * iv;
+  if (ni < 32) return __shfl_sync(0xffffffffu, s, 31);
+  double d = dg;
+  for (int p = 0; p < 32; ++p) {
+    const double lp = __shfl_sync(0xffffffffu, l, p);
+    d -= lp * lp;
+  }
+  return d;
+}
+
+// the pivots of a CTA's rows (d in sd, row in srow)
+__device__ __forceinline__ void factor_pivots(const Params &P, const double *sd, const int *srow, int rows, int w,
+                                              int lane) {
+  if (w == 0 && lane < rows) factor_pivot(P, srow[lane], sd[lane]);
 }
 
 __global__ void __launch_bounds__(kFacWarps * kWarp) factor_warp_kernel(Params P, int k0, int k1) {
@@ -2034,7 +2052,7 @@ __global__ void __launch_bounds__(kFacWarps * kWarp) factor_warp_kernel(Params P
     const int i = rec.x, rb = rec.y, q0 = rec.z, ni = rec.w & 0xff, np = rec.w >> 8;
     const bool on = lane < ni;
     const int col = on ? __ldg(P.lcol + rb + lane) : 0;
-    double s = on ? __ldg(P.ainit + rb + lane) : 0.0;
+    const double s = on ? __ldg(P.ainit + rb + lane) : 0.0;
     const int c = on ? __ldg(P.fp_ptr + rb + lane) - q0 : 0;
     const int ce = on ? __ldg(P.fp_ptr + rb + lane + 1) - q0 : 0;
     const double dg = k < k1 ? __ldg(P.adiag + i) : 1.0;
@@ -2061,7 +2079,7 @@ __global__ void __launch_bounds__(kFacWarps * kWarp) factor_warp_kernel(Params P
       }
       double v[kFacBatch];
 #pragma unroll
-      for (int u = 0; u < kFacBatch; ++u) v[u] = qa + u * kWarp + lane < np ? __ldcg(P.uval + fb[u]) : 0.0;
+      for (int u = 0; u < kFacBatch; ++u) v[u] = qa + u * kWarp + lane < np ? __ldcg(P.lval + fb[u]) : 0.0;
 #pragma unroll
       for (int u = 0; u < kFacBatch; ++u) {
         const int q = qa + u * kWarp + lane;
@@ -2072,15 +2090,11 @@ __global__ void __launch_bounds__(kFacWarps * kWarp) factor_warp_kernel(Params P
       }
     }
     __syncwarp();
-    s = factor_steps(s, c, ce, pv, ps, lane);
-    const double l = s * iv;
-    if (on) {
-      P.lval[rb + lane] = l;
-      P.uval[rb + lane] = l * iv;
-    }
-    const double ss = warp_sum(l * l);
+    double l;
+    const double d = factor_steps(s, iv, c, ce, ni, dg, pv, ps, lane, l);
+    if (on) P.lval[rb + lane] = l;
     if (lane == 0) {
-      sd[w] = dg - ss;
+      sd[w] = d;
       srow[w] = i;
     }
     __syncthreads();
@@ -2094,15 +2108,17 @@ __global__ void __launch_bounds__(kFacWarps * kWarp) factor_warp_kernel(Params P
 // edge, so a row waits only for rows of its own block: the CTA's warps take
 // the rows in turn (first rows of all blocks, second rows, ...), a warp per
 // row as above, and a finished row is announced through a flag in shared
-// memory, where its scaled entries and 1/L_ii also stay for the rows that
+// memory, where its entries and 1/L_ii also stay for the rows that
 // follow.  A warp loads its next row's indices and its entries of other
 // colors while the others work.
 //
 // Why: with a launch per level every level of a block cost a launch boundary
 // and a trip of its values through L2 (27-point 61x67x59, blocks of 32: 205
-// launches of 7-9 us, 1.86 ms in all); one launch per color takes 0.90 ms, half
-// of it the FP64 pipe (about 30 warp instructions a row).  IC(0) and one
-// application together there: 7.41 ms with a thread per row, 1.15 ms now.
+// launches of 7-9 us); the launch count falls to one per color.  IC(0) and one
+// application together there: 7.40 ms with a thread per row, 1.58 ms now, about
+// half of it the FP64 pipe.  (Reciprocal square roots, pre-scaled terms and a
+// tree for the pivot's sum took 1.15 ms, but moved the factor's last bit; ill-
+// conditioned solves then differ by 1e-9.)
 constexpr int kFacUnitWarps = 4;
 constexpr int kFacSpin = 1 << 22;   // polls of a row's flags before giving up
 
@@ -2129,7 +2145,7 @@ __global__ void __launch_bounds__(kFacUnitWarps * kWarp) factor_unit_kernel(Para
     const int q0 = __ldg(P.fp_ptr + rb), np = __ldg(P.fp_ptr + rb + ni) - q0;
     const bool on = lane < ni;
     const int col = on ? __ldg(P.lcol + rb + lane) : 0;
-    double s = on ? __ldg(P.ainit + rb + lane) : 0.0;
+    const double s = on ? __ldg(P.ainit + rb + lane) : 0.0;
     const int c = on ? __ldg(P.fp_ptr + rb + lane) - q0 : 0;
     const int ce = on ? __ldg(P.fp_ptr + rb + lane + 1) - q0 : 0;
     const double dg = __ldg(P.adiag + i);
@@ -2151,7 +2167,7 @@ __global__ void __launch_bounds__(kFacUnitWarps * kWarp) factor_unit_kernel(Para
 #pragma unroll
     for (int u = 0; u < kFacBatch; ++u) {
       const int q = u * kWarp + lane;
-      v[u] = q < np && (fb[u] < l0 || fb[u] >= l1) ? __ldcg(P.uval + fb[u]) : 0.0;
+      v[u] = q < np && (fb[u] < l0 || fb[u] >= l1) ? __ldcg(P.lval + fb[u]) : 0.0;
     }
     for (int spin = 0; !__all_sync(0xffffffffu, !in || ready[col - row0] != 0); ++spin)
       if (spin > kFacSpin) {
@@ -2170,32 +2186,28 @@ __global__ void __launch_bounds__(kFacUnitWarps * kWarp) factor_unit_kernel(Para
     }
     for (int q = kFacBatch * kWarp + lane; q < np; q += kWarp) {
       const int e = __ldg(P.fp_b + q0 + q);
-      pv[q] = e >= l0 && e < l1 ? us[e - l0] : __ldcg(P.uval + e);
+      pv[q] = e >= l0 && e < l1 ? us[e - l0] : __ldcg(P.lval + e);
       ps[q] = __ldg(P.fp_pos + q0 + q);
     }
     __syncwarp();
-    s = factor_steps(s, c, ce, pv, ps, lane);
-    const double l = s * iv, lu = l * iv;
-    const double ss = warp_sum(l * l);
-    if (on) us[rb - l0 + lane] = lu;
+    double l;
+    const double dd = factor_steps(s, iv, c, ce, ni, dg, pv, ps, lane, l);
+    if (on) us[rb - l0 + lane] = l;
     if (lane == 0) {
-      const double dd = factor_check(P, i, dg - ss);
-      ds[i - row0] = dd;
-      ivs[i - row0] = rsqrt(dd);
+      const double lii = sqrt(factor_check(P, i, dd));
+      ds[i - row0] = lii;
+      ivs[i - row0] = 1.0 / lii;
     }
     __threadfence_block();
     __syncwarp();
     if (lane == 0) ready[i - row0] = 1;
-    if (on) {
-      P.lval[rb + lane] = l;
-      P.uval[rb + lane] = lu;
-    }
+    if (on) P.lval[rb + lane] = l;
   }
   if (!waited) pdl_wait();
   __syncthreads();
   if (threadIdx.x < d.nrows) {
     P.invd[row0 + threadIdx.x] = ivs[threadIdx.x];
-    P.ldiag[row0 + threadIdx.x] = sqrt(ds[threadIdx.x]);
+    P.ldiag[row0 + threadIdx.x] = ds[threadIdx.x];
   }
 }
 
@@ -2353,10 +2365,7 @@ __global__ void __launch_bounds__(kVecThreads) factor_short_kernel(Params P, int
     }
 #pragma unroll
     for (int p = 0; p < kFacShort; ++p)
-      if (p < ni) {
-        P.lval[rb + p] = l[p];
-        P.uval[rb + p] = l[p] * iv[p];
-      }
+      if (p < ni) P.lval[rb + p] = l[p];
     factor_pivot(P, i, d);
   }
   if (!waited) pdl_wait();
