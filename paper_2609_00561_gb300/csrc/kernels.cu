@@ -1883,9 +1883,7 @@ __device__ __forceinline__ void factor_pivot(const Params &P, int i, double d) {
 // Row i of the up-looking IC(0): for every j < i in the pattern, ascending,
 //   L_ij = (a_ij - sum_{k < j, k in pat(i) and pat(j)} L_ik L_jk) / L_jj,
 // then L_ii = sqrt(a_ii - sum_j L_ij^2); rows j are final when row i runs.
-// A finished row also stores 1/L_ii, and later rows multiply by it; rows without
-// precomputed pairs also their entries times 1/L_jj (in uval, entry for entry:
-// free until the finishing pass writes U there), for factor_wide_kernel.
+// A finished row also stores 1/L_ii, and later rows multiply by it.
 // General form: the common columns by a merge of the two sorted rows (a
 // chain of dependent loads).
 __device__ __forceinline__ void factor_row_merge(const Params &P, int i) {
@@ -1902,9 +1900,8 @@ __device__ __forceinline__ void factor_row_merge(const Params &P, int i) {
       else if (ca < cb) ++a;
       else ++b;
     }
-    const double iv = __ldcg(P.invd + j), lij = s * iv;
+    const double lij = s * __ldcg(P.invd + j);
     P.lval[p] = lij;
-    P.uval[p] = lij * iv;
     d -= lij * lij;
   }
   factor_pivot(P, i, d);
@@ -1963,10 +1960,7 @@ __device__ __forceinline__ void factor_row(const Params &P, int i, int32_t *sc, 
     sv[p] = lij;
     d -= lij * lij;
   }
-  for (int t = 0; t < ni; ++t) {
-    P.lval[rb + t] = sv[t];
-    P.uval[rb + t] = sv[t] * __ldcg(P.invd + sc[t]);
-  }
+  for (int t = 0; t < ni; ++t) P.lval[rb + t] = sv[t];
   factor_pivot(P, i, d);
 }
 
@@ -2213,14 +2207,15 @@ __global__ void __launch_bounds__(kFacUnitWarps * kWarp) factor_unit_kernel(Para
 
 // The same for rows of 9..64 strictly-lower entries without precomputed
 // pairs (a matrix with any row above 32): two entries per lane, and the
-// values L_pk / L_kk as the strictly-lower triangle of a dense matrix in the
-// warp's shared memory (column k: entries p = k + 1 .. ni - 1 consecutive, so
-// the lanes of a column read without bank conflicts).  The warp reads row j of
+// values L_pk as the strictly-lower triangle of a dense matrix in the warp's
+// shared memory (column k: entries p = k + 1 .. ni - 1 consecutive, so the
+// lanes of a column read without bank conflicts).  The warp reads row j of
 // every entry (i, j) coalesced and finds its columns in row i by a binary
-// search in shared memory.  Bound by the FP64 pipe (about 2 warp instructions
-// per column of a row).  IC(0) and one application for a 3-unknown
-// 27-neighbour 33^3 network with one-row blocks: 3.24 ms with a thread per row
-// merging index lists, 0.96 ms so.
+// search in shared memory, then resolves the row column by column, every sum in
+// the order of the general form (the same bits).  Bound by the FP64 pipe (about
+// 3 warp instructions per column of a row).  IC(0) and one application for a
+// 3-unknown 27-neighbour 33^3 network with one-row blocks: 3.24 ms with a thread
+// per row merging index lists, 1.22 ms so.
 constexpr int kFacWide = 64;
 constexpr int kFacWideWarps = 4;
 
@@ -2275,43 +2270,47 @@ __global__ void __launch_bounds__(kFacWideWarps * kWarp) factor_wide_kernel(Para
         nj[u] = __shfl_sync(0xffffffffu, p < kWarp ? n0 : n1, p & 31);
         if (p >= ni) nj[u] = 0;
         cu[u] = lane < nj[u] ? __ldg(P.lcol + jb[u] + lane) : 0;
-        v[u] = lane < nj[u] ? __ldcg(P.uval + jb[u] + lane) : 0.0;
+        v[u] = lane < nj[u] ? __ldcg(P.lval + jb[u] + lane) : 0.0;
       }
 #pragma unroll
       for (int u = 0; u < kFacBatch; ++u) {
         if (lane < nj[u]) place(p0 + u, cu[u], v[u]);
         for (int q = kWarp + lane; q < nj[u]; q += kWarp)
-          place(p0 + u, __ldg(P.lcol + jb[u] + q), __ldcg(P.uval + jb[u] + q));
+          place(p0 + u, __ldg(P.lcol + jb[u] + q), __ldcg(P.lval + jb[u] + q));
       }
     }
     __syncwarp();
+    // lane 31's spare entry carries the pivot a_ii - sum_p l_p^2 (a row of 64
+    // entries forms it afterwards)
+    const bool piv0 = lane == 31 && ni < kWarp, piv1 = lane == 31 && ni >= kWarp && ni < kFacWide;
+    if (piv0) s0 = dg;
+    if (piv1) s1 = dg;
     int off = -1;   // column kk's entry p at off + p - kk
-    for (int kk = 0; kk < ni - 1; ++kk) {
-      const double sk = __shfl_sync(0xffffffffu, kk < kWarp ? s0 : s1, kk & 31);
+    for (int kk = 0; kk < ni; ++kk) {
+      const double lk = __shfl_sync(0xffffffffu, kk < kWarp ? s0 * iv0 : s1 * iv1, kk & 31);
       if (kk < kWarp - 1) {
-        const double m = lane > kk && on0 ? M[off + lane - kk] : 0.0;
-        if (__double_as_longlong(m) != 0) s0 -= sk * m;
+        const double m = piv0 ? lk : (lane > kk && on0 ? M[off + lane - kk] : 0.0);
+        if (__double_as_longlong(m) != 0) s0 -= lk * m;
       }
-      if (ni > kWarp) {
-        const double m = lane + kWarp > kk && on1 ? M[off + lane + kWarp - kk] : 0.0;
-        if (__double_as_longlong(m) != 0) s1 -= sk * m;
+      if (ni >= kWarp) {
+        const double m = piv1 ? lk : (lane + kWarp > kk && on1 ? M[off + lane + kWarp - kk] : 0.0);
+        if (__double_as_longlong(m) != 0) s1 -= lk * m;
       }
       off += ni - 1 - kk;
     }
     const double l0 = s0 * iv0, l1 = s1 * iv1;
-    if (on0) {
-      P.lval[rb + lane] = l0;
-      P.uval[rb + lane] = l0 * iv0;
+    if (on0) P.lval[rb + lane] = l0;
+    if (on1) P.lval[rb + kWarp + lane] = l1;
+    double d = __shfl_sync(0xffffffffu, ni < kWarp ? s0 : s1, 31);
+    if (ni == kFacWide) {
+      d = dg;
+      for (int p = 0; p < kFacWide; ++p) {
+        const double lp = __shfl_sync(0xffffffffu, p < kWarp ? l0 : l1, p & 31);
+        d -= lp * lp;
+      }
     }
-    if (on1) {
-      P.lval[rb + kWarp + lane] = l1;
-      P.uval[rb + kWarp + lane] = l1 * iv1;
-    }
-    double ss = l0 * l0;
-    if (ni > kWarp) ss += l1 * l1;
-    ss = warp_sum(ss);
     if (lane == 0) {
-      sd[w] = dg - ss;
+      sd[w] = d;
       srow[w] = i;
     }
     __syncthreads();
