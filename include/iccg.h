@@ -91,7 +91,11 @@ typedef struct {
                                  ICCG_TILES_AUTO (0): warp units for colors whose
                                  largest block has 5..32 rows, pair kernels for the
                                  colors whose blocks all have two rows, one CTA per
-                                 tile otherwise */
+                                 tile otherwise; with at most 7 entries a row on
+                                 average, warp units also for blocks of 3 and 4
+                                 rows, for colors of one- and two-row blocks, and
+                                 (FP32 preconditioner) of one-row blocks, one warp
+                                 per tile for one-row blocks in FP64 */
   int32_t fuse_sweep;         /* layouts whose colors are all lane tiles of blocks of
                                  one or two rows: 1 runs each preconditioner sweep
                                  (every color forward and backward) as one

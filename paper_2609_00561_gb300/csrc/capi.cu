@@ -164,14 +164,23 @@ iccg_status iccg_setup(iccg_ctx **out, int32_t n, int64_t nnz, const int64_t *ro
   // lane tiles for colors of small blocks; the persistent kernel runs groups only
   const int lane_max = o.solver == ICCG_SOLVER_PERSISTENT || o.lane_block_max < 0 ? 0
                        : (o.lane_block_max == 0 ? 32 : o.lane_block_max);
-  // warp units (one warp per block, a lane per row): automatically for colors
-  // of blocks of 5..32 rows (on a GB300 12% faster than lane tiles at 8 rows,
-  // 2.7x at 32, 2.5% slower at 4), explicitly for every color of at most 32
-  const int32_t unit_min = lane_max <= 0 ? 0
-                           : o.tile_mapping == ICCG_TILES_UNITS ? 1
-                           : o.tile_mapping == ICCG_TILES_AUTO ? 5 : 0;
+  // Warp units (a lane per row): automatically for colors of blocks of 5..32
+  // rows, explicitly for every color of at most 32.  Where rows are narrow (at
+  // most 7 entries on average: 5- and 7-point) also for blocks of 3 and 4 rows
+  // (60^3, blocks of 4, an iteration: 113 us as lane tiles, 86 as units), for
+  // colors mixing one- and two-row blocks (127x101x83 CPM, one such color of 4:
+  // 108 against 95 us in FP32, 128 against 119 in FP64), and with the FP32
+  // preconditioner for one-row blocks (100^3: 96 against 82 us; in FP64 one
+  // warp per lane tile is quicker still, 116 against 100, units 113).  With wide
+  // rows lane tiles keep their lead (geometric graph, degree 16, 18 colors: 224
+  // us, units 238).
+  // (A requested cooperative sweep runs on lane tiles.)
+  const bool autom = o.tile_mapping == ICCG_TILES_AUTO;
+  const bool narrow = nnz <= 7 * int64_t(n) && o.fuse_sweep <= 0;
+  const UnitRule units{lane_max <= 0 ? 0 : (o.tile_mapping == ICCG_TILES_UNITS ? 1 : (autom ? (narrow ? 3 : 5) : 0)),
+                       autom && narrow && ctx->fp32, autom && narrow};
   iccg_status st = build_layout(n, nnz, hrp.data(), hci.data(), hval.data(), hperm.data(), hbp.data(),
-                                hcp.data(), n_b, n_c, G, lane_max, unit_min, ctx->H, ctx->err_index, ctx->err_msg);
+                                hcp.data(), n_b, n_c, G, lane_max, units, ctx->H, ctx->err_index, ctx->err_msg);
   if (st != ICCG_OK) return st;
   if (cudaGetDevice(&ctx->device) != cudaSuccess) return cuda_fail(ctx, cudaGetLastError(), "cudaGetDevice");
   {
@@ -307,12 +316,12 @@ iccg_status iccg_setup(iccg_ctx **out, int32_t n, int64_t nnz, const int64_t *ro
       steps = std::max(steps, td.nsteps);
       if (td.nsteps != 2 || H.steps[size_t(td.step0) + 1].cnt != H.steps[size_t(td.step0)].cnt) pairs = false;
     }
-    // automatic: colors of two-row blocks only as pair kernels, one CTA per
-    // tile otherwise (on a GB300 the pair kernels measured 7% faster for
+    // automatic: colors of two-row blocks only as pair kernels, one-row blocks
+    // of narrow rows as warp tiles, one CTA per tile otherwise (on a GB300 the pair kernels measured 7% faster for
     // ABMC with blocks of 2 rows, slower where one-row blocks share a tile
     // with two-row ones, and no better for one-row blocks alone)
     L.wtile[c] = 0;
-    if (nt > 0 && o.tile_mapping == ICCG_TILES_WARP) L.wtile[c] = 1;
+    if (nt > 0 && (o.tile_mapping == ICCG_TILES_WARP || (autom && narrow && steps == 1))) L.wtile[c] = 1;
     if (nt > 0 && steps <= 2 && ((pairs && o.tile_mapping == ICCG_TILES_AUTO) || o.tile_mapping == ICCG_TILES_PAIR))
       L.wtile[c] = 2;
     // one-CTA-per-tile colors of short tiles also stage their entries to
@@ -354,7 +363,7 @@ iccg_status iccg_setup(iccg_ctx **out, int32_t n, int64_t nnz, const int64_t *ro
       L.grid_c[c] = std::max(1, L.task1[c] - L.task0[c]);
     }
     gbig = std::max(gbig, L.grid_c[c]);
-    lane_tiles = lane_tiles || L.wtile[c] == 0 || L.wtile[c] == 1;
+    lane_tiles = lane_tiles || (nt > 0 && L.wtile[c] == 0);
   }
   // Lane-tile kernels take more shared memory than the others, and launches
   // with different L1 / shared-memory splits cannot share an SM.  Colors of few
@@ -362,8 +371,7 @@ iccg_status iccg_setup(iccg_ctx **out, int32_t n, int64_t nnz, const int64_t *ro
   // previous one (18 colors of 9,000 rows: 223 against 252 us an iteration; 8
   // colors of 7,500: 99 against 103).  Colors of many rows need the larger L1
   // more (2 colors of 485,000 rows: 118 against 124 us), and then several
-  // iterations per pass lose what they save (FP32, 4 colors of 266,000 rows, the
-  // last one lane tiles: 110 us with one, 116 with four).  Other layouts: default
+  // iterations per pass lose what they save (118 us with four, 117 with one).  Other layouts: default
   // splits, four iterations (n = 4096 46 against 48.5 us, 128^3 170 against 174).
   if (lane_tiles && n / n_c < 100000) L.carve = 60;
   else if (lane_tiles) L.body = 1;

@@ -26,7 +26,7 @@ iccg_status fail(iccg_status st, int64_t idx, const char *what, int64_t &bad, st
 iccg_status build_layout(int32_t n, int64_t nnz, const int64_t *rowptr, const int32_t *colind,
                          const double *val, const int32_t *perm, const int32_t *block_ptr,
                          const int32_t *color_ptr, int32_t n_b, int32_t n_c, int32_t group_rows,
-                         int32_t lane_max, int32_t unit_min, HostLayout &H, int64_t &bad, std::string &msg) {
+                         int32_t lane_max, UnitRule units, HostLayout &H, int64_t &bad, std::string &msg) {
   bad = -1;
   if (n < 0 || nnz < 0 || nnz >= (int64_t(1) << 31)) return fail(ICCG_ERR_ARG, -1, "n or nnz out of range", bad, msg);
   if (n > 0 && (n_b < 1 || n_c < 1 || n_b > n || n_c > n_b)) return fail(ICCG_ERR_ARG, -1, "n_b / n_c out of range", bad, msg);
@@ -126,14 +126,16 @@ iccg_status build_layout(int32_t n, int64_t nnz, const int64_t *rowptr, const in
   // active at a step are a prefix), its rows stored step-major per tile
   lane_max = std::max(0, std::min(lane_max, 32));
   std::vector<char> tcol(n_c > 0 ? n_c : 1, 0);
-  // warp units: colors whose largest block has unit_min..32 rows (when
-  // enabled, unit_min >= 1); they keep the caller's row order
+  // warp units: the colors that the rule names; they keep the caller's row order
   std::vector<char> wcol(n_c > 0 ? n_c : 1, 0);
   H.unit_colors = 0;
-  for (int32_t c = 0; c < n_c && unit_min > 0; ++c) {
-    int32_t mb = 0;
-    for (int32_t j = color_ptr[c]; j < color_ptr[c + 1]; ++j) mb = std::max(mb, block_ptr[j + 1] - block_ptr[j]);
-    if (mb >= unit_min && mb <= kWarp) {
+  for (int32_t c = 0; c < n_c && units.min_rows > 0; ++c) {
+    int32_t mb = 0, least = INT32_MAX;
+    for (int32_t j = color_ptr[c]; j < color_ptr[c + 1]; ++j) {
+      mb = std::max(mb, block_ptr[j + 1] - block_ptr[j]);
+      least = std::min(least, block_ptr[j + 1] - block_ptr[j]);
+    }
+    if ((mb >= units.min_rows && mb <= kWarp) || (units.one && mb == 1) || (units.mixed && mb == 2 && least == 1)) {
       wcol[c] = 1;
       H.unit_colors++;
     }
@@ -442,8 +444,27 @@ iccg_status build_layout(int32_t n, int64_t nnz, const int64_t *rowptr, const in
   H.units.clear();
   H.wl_mask.clear(); H.wu_mask.clear(); H.wl_src.clear(); H.wu_src.clear();
   H.wl_map.clear(); H.wl_srow.clear(); H.wu_map.clear(); H.wu_srow.clear();
+  // (units are independent: built in parallel, each thread a run of them, then
+  // put together in order)
   {
-    std::vector<std::vector<int32_t>> se(kWarp), sw(kWarp);
+    struct UnitRun {
+      std::vector<int32_t> sl_col, sl_map, su_col, su_map, wl_map, wl_srow, wu_map, wu_srow;
+      std::vector<uint32_t> wl_mask, wu_mask, wl_src, wu_src;
+      std::vector<WarpUnit> units;
+      int32_t bad = -1;
+    };
+    std::vector<std::pair<int32_t, int32_t>> list;   // (color, first block)
+    for (int32_t c = 0; c < n_c; ++c) {
+      H.color_unit[c] = int32_t(list.size());
+      if (!wcol[c]) continue;
+      int32_t mb = 0;
+      for (int32_t j = color_ptr[c]; j < color_ptr[c + 1]; ++j) mb = std::max(mb, block_ptr[j + 1] - block_ptr[j]);
+      int32_t S = 1;
+      while (S < mb) S <<= 1;
+      H.unit_S[c] = S;
+      for (int32_t j = color_ptr[c]; j < color_ptr[c + 1]; j += kWarp / S) list.push_back({c, j});
+    }
+    H.color_unit[n_c] = int32_t(list.size());
     // appends the per-lane lists sliced-ELL over 32 lanes, padding (pad, -1)
     auto slab = [&](std::vector<std::vector<int32_t>> &a, std::vector<std::vector<int32_t>> &b,
                     std::vector<int32_t> &oa, std::vector<int32_t> &ob, int32_t pad) {
@@ -457,117 +478,141 @@ iccg_status build_layout(int32_t n, int64_t nnz, const int64_t *rowptr, const in
         }
       return w;
     };
-    for (int32_t c = 0; c < n_c; ++c) {
-      H.color_unit[c] = int32_t(H.units.size());
-      if (!wcol[c]) continue;
-      int32_t mb = 0;
-      for (int32_t j = color_ptr[c]; j < color_ptr[c + 1]; ++j) mb = std::max(mb, block_ptr[j + 1] - block_ptr[j]);
-      int32_t S = 1;
-      while (S < mb) S <<= 1;
-      H.unit_S[c] = S;
-      const int32_t per = kWarp / S;
-      for (int32_t j = color_ptr[c]; j < color_ptr[c + 1]; j += per) {
-        WarpUnit u{};
-        u.blk0 = j;
-        u.nblk = std::min(per, color_ptr[c + 1] - j);
-        u.row0 = block_ptr[j];
-        u.nrows = block_ptr[j + u.nblk] - u.row0;
-        std::vector<int32_t> lrow(kWarp, -1);
-        for (int l = 0; l < kWarp; ++l) {
-          const int32_t b = j + l / S;
-          if (l / S < u.nblk && block_ptr[b] + l % S < block_ptr[b + 1]) lrow[size_t(l)] = block_ptr[b] + l % S;
-        }
-        for (int pass = 0; pass < 2; ++pass) {
-          const std::vector<int32_t> &rp = pass ? H.urp : H.lrp, &cols = pass ? H.ucol : H.lcol;
-          // entries to other colors
-          for (int l = 0; l < kWarp; ++l) {
-            se[size_t(l)].clear();
-            sw[size_t(l)].clear();
-            const int32_t i = lrow[size_t(l)];
-            if (i < 0) continue;
-            for (int32_t e = rp[size_t(i)]; e < rp[size_t(i) + 1]; ++e)
-              if (iblk[cols[size_t(e)]] != iblk[i]) {
-                se[size_t(l)].push_back(cols[size_t(e)]);
-                sw[size_t(l)].push_back(pass ? H.umap[size_t(e)] : e);
-              }
-          }
-          if (pass == 0) { u.lo = int32_t(H.sl_col.size()); u.lw = slab(se, sw, H.sl_col, H.sl_map, kPadCol); }
-          else { u.uo = int32_t(H.su_col.size()); u.uw = slab(se, sw, H.su_col, H.su_map, kPadCol); }
-          // in-block terms as a chain schedule: lane l's terms (source row
-          // k, coefficient) in the order their sources become final, one per
-          // step (a source is final the step after its own last term; rows
-          // are visited in dependency order: ascending forward, descending
-          // backward), each at the earliest step both it and the lane allow
-          std::vector<int32_t> ready(size_t(kWarp), 0);
-          std::vector<std::vector<std::pair<int32_t, int32_t>>> sched(kWarp);   // (step, term index)
-          std::vector<std::vector<int32_t>> tsrc(kWarp), tmap(kWarp), trow(kWarp);
-          for (int l = 0; l < kWarp; ++l) {
-            const int32_t i = lrow[size_t(l)];
-            if (i < 0) continue;
-            for (int32_t e = rp[size_t(i)]; e < rp[size_t(i) + 1]; ++e) {
-              const int32_t k = cols[size_t(e)];
-              if (iblk[k] != iblk[i]) continue;
-              tsrc[size_t(l)].push_back((l / S) * S + (k - block_ptr[iblk[i]]));
-              tmap[size_t(l)].push_back(pass ? H.umap[size_t(e)] : e);
-              trow[size_t(l)].push_back(k);
-            }
-          }
-          int32_t M = 0;
-          for (int q = 0; q < kWarp; ++q) {
-            const int l = pass ? kWarp - 1 - q : q;   // sources before their targets within a block
-            const size_t nt = tsrc[size_t(l)].size();
-            std::vector<int32_t> ord(nt);
-            for (size_t x = 0; x < nt; ++x) ord[x] = int32_t(x);
-            std::stable_sort(ord.begin(), ord.end(), [&](int32_t a, int32_t b) {
-              return ready[size_t(tsrc[size_t(l)][size_t(a)])] < ready[size_t(tsrc[size_t(l)][size_t(b)])];
-            });
-            int32_t t = 0;
-            for (int32_t x : ord) {
-              const int32_t st = std::max(t, ready[size_t(tsrc[size_t(l)][size_t(x)])]);
-              sched[size_t(l)].push_back({st, x});
-              t = st + 1;
-            }
-            ready[size_t(l)] = t;
-            M = std::max(M, t);
-          }
-          if (M > kWarp) return fail(ICCG_ERR_ARG, u.blk0, "warp-unit chain longer than 32 steps", bad, msg);
-          const int32_t co = int32_t((pass ? H.wu_map : H.wl_map).size());
-          const int32_t so = int32_t((pass ? H.wu_src : H.wl_src).size());
-          std::vector<int32_t> &mp = pass ? H.wu_map : H.wl_map, &sr = pass ? H.wu_srow : H.wl_srow;
-          std::vector<uint32_t> &swd = pass ? H.wu_src : H.wl_src, &mk = pass ? H.wu_mask : H.wl_mask;
-          // coefficients term-major: lane l's j-th term (in step order) at
-          // co + j * 32 + l, the block as deep as the lane with most terms
-          size_t T = 0;
-          for (int l = 0; l < kWarp; ++l) T = std::max(T, sched[size_t(l)].size());
-          mp.resize(size_t(co) + T * kWarp, -1);
-          sr.resize(size_t(co) + T * kWarp, -1);
-          const int32_t nw = (M + 3) / 4;
-          swd.resize(size_t(so) + size_t(nw) * kWarp, 0u);
-          for (int l = 0; l < kWarp; ++l) {
-            uint32_t mask = 0;
-            for (int m = 0; m < nw * 4; ++m) {   // idle steps read the lane itself
-              const size_t w = size_t(so) + size_t(m / 4) * kWarp + size_t(l);
-              swd[w] |= uint32_t(l) << (8 * (m % 4));
-            }
-            size_t j = 0;
-            for (const auto &pr : sched[size_t(l)]) {
-              const int32_t m = pr.first, x = pr.second;
-              mask |= 1u << m;
-              mp[size_t(co) + j * kWarp + size_t(l)] = tmap[size_t(l)][size_t(x)];
-              sr[size_t(co) + j * kWarp + size_t(l)] = trow[size_t(l)][size_t(x)];
-              ++j;
-              const size_t w = size_t(so) + size_t(m / 4) * kWarp + size_t(l);
-              swd[w] = (swd[w] & ~(0xffu << (8 * (m % 4)))) | (uint32_t(tsrc[size_t(l)][size_t(x)]) << (8 * (m % 4)));
-            }
-            mk.push_back(mask);
-          }
-          if (pass == 0) { u.li = co; u.lm = M; u.ls = so; u.lt = int32_t(T); }
-          else { u.ui = co; u.um = M; u.us = so; u.ut = int32_t(T); }
-        }
-        H.units.push_back(u);
+    // appends the unit of blocks j .. of color c; its first block when a chain
+    // would be longer than 32 steps, else -1
+    auto add_unit = [&](UnitRun &o, std::vector<std::vector<int32_t>> &se, std::vector<std::vector<int32_t>> &sw,
+                        int32_t c, int32_t j) -> int32_t {
+      const int32_t S = H.unit_S[c], per = kWarp / S;
+      WarpUnit u{};
+      u.blk0 = j;
+      u.nblk = std::min(per, color_ptr[c + 1] - j);
+      u.row0 = block_ptr[j];
+      u.nrows = block_ptr[j + u.nblk] - u.row0;
+      std::vector<int32_t> lrow(kWarp, -1);
+      for (int l = 0; l < kWarp; ++l) {
+        const int32_t b = j + l / S;
+        if (l / S < u.nblk && block_ptr[b] + l % S < block_ptr[b + 1]) lrow[size_t(l)] = block_ptr[b] + l % S;
       }
+      for (int pass = 0; pass < 2; ++pass) {
+        const std::vector<int32_t> &rp = pass ? H.urp : H.lrp, &cols = pass ? H.ucol : H.lcol;
+        // entries to other colors
+        for (int l = 0; l < kWarp; ++l) {
+          se[size_t(l)].clear();
+          sw[size_t(l)].clear();
+          const int32_t i = lrow[size_t(l)];
+          if (i < 0) continue;
+          for (int32_t e = rp[size_t(i)]; e < rp[size_t(i) + 1]; ++e)
+            if (iblk[cols[size_t(e)]] != iblk[i]) {
+              se[size_t(l)].push_back(cols[size_t(e)]);
+              sw[size_t(l)].push_back(pass ? H.umap[size_t(e)] : e);
+            }
+        }
+        if (pass == 0) { u.lo = int32_t(o.sl_col.size()); u.lw = slab(se, sw, o.sl_col, o.sl_map, kPadCol); }
+        else { u.uo = int32_t(o.su_col.size()); u.uw = slab(se, sw, o.su_col, o.su_map, kPadCol); }
+        // in-block terms as a chain schedule: lane l's terms (source row
+        // k, coefficient) in the order their sources become final, one per
+        // step (a source is final the step after its own last term; rows
+        // are visited in dependency order: ascending forward, descending
+        // backward), each at the earliest step both it and the lane allow
+        std::vector<int32_t> ready(size_t(kWarp), 0);
+        std::vector<std::vector<std::pair<int32_t, int32_t>>> sched(kWarp);   // (step, term index)
+        std::vector<std::vector<int32_t>> tsrc(kWarp), tmap(kWarp), trow(kWarp);
+        for (int l = 0; l < kWarp; ++l) {
+          const int32_t i = lrow[size_t(l)];
+          if (i < 0) continue;
+          for (int32_t e = rp[size_t(i)]; e < rp[size_t(i) + 1]; ++e) {
+            const int32_t k = cols[size_t(e)];
+            if (iblk[k] != iblk[i]) continue;
+            tsrc[size_t(l)].push_back((l / S) * S + (k - block_ptr[iblk[i]]));
+            tmap[size_t(l)].push_back(pass ? H.umap[size_t(e)] : e);
+            trow[size_t(l)].push_back(k);
+          }
+        }
+        int32_t M = 0;
+        for (int q = 0; q < kWarp; ++q) {
+          const int l = pass ? kWarp - 1 - q : q;   // sources before their targets within a block
+          const size_t nt = tsrc[size_t(l)].size();
+          std::vector<int32_t> ord(nt);
+          for (size_t x = 0; x < nt; ++x) ord[x] = int32_t(x);
+          std::stable_sort(ord.begin(), ord.end(), [&](int32_t a, int32_t b) {
+            return ready[size_t(tsrc[size_t(l)][size_t(a)])] < ready[size_t(tsrc[size_t(l)][size_t(b)])];
+          });
+          int32_t t = 0;
+          for (int32_t x : ord) {
+            const int32_t st = std::max(t, ready[size_t(tsrc[size_t(l)][size_t(x)])]);
+            sched[size_t(l)].push_back({st, x});
+            t = st + 1;
+          }
+          ready[size_t(l)] = t;
+          M = std::max(M, t);
+        }
+        if (M > kWarp) return u.blk0;
+        const int32_t co = int32_t((pass ? o.wu_map : o.wl_map).size());
+        const int32_t so = int32_t((pass ? o.wu_src : o.wl_src).size());
+        std::vector<int32_t> &mp = pass ? o.wu_map : o.wl_map, &sr = pass ? o.wu_srow : o.wl_srow;
+        std::vector<uint32_t> &swd = pass ? o.wu_src : o.wl_src, &mk = pass ? o.wu_mask : o.wl_mask;
+        // coefficients term-major: lane l's j-th term (in step order) at
+        // co + j * 32 + l, the block as deep as the lane with most terms
+        size_t T = 0;
+        for (int l = 0; l < kWarp; ++l) T = std::max(T, sched[size_t(l)].size());
+        mp.resize(size_t(co) + T * kWarp, -1);
+        sr.resize(size_t(co) + T * kWarp, -1);
+        const int32_t nw = (M + 3) / 4;
+        swd.resize(size_t(so) + size_t(nw) * kWarp, 0u);
+        for (int l = 0; l < kWarp; ++l) {
+          uint32_t mask = 0;
+          for (int m = 0; m < nw * 4; ++m) {   // idle steps read the lane itself
+            const size_t w = size_t(so) + size_t(m / 4) * kWarp + size_t(l);
+            swd[w] |= uint32_t(l) << (8 * (m % 4));
+          }
+          size_t j = 0;
+          for (const auto &pr : sched[size_t(l)]) {
+            const int32_t m = pr.first, x = pr.second;
+            mask |= 1u << m;
+            mp[size_t(co) + j * kWarp + size_t(l)] = tmap[size_t(l)][size_t(x)];
+            sr[size_t(co) + j * kWarp + size_t(l)] = trow[size_t(l)][size_t(x)];
+            ++j;
+            const size_t w = size_t(so) + size_t(m / 4) * kWarp + size_t(l);
+            swd[w] = (swd[w] & ~(0xffu << (8 * (m % 4)))) | (uint32_t(tsrc[size_t(l)][size_t(x)]) << (8 * (m % 4)));
+          }
+          mk.push_back(mask);
+        }
+        if (pass == 0) { u.li = co; u.lm = M; u.ls = so; u.lt = int32_t(T); }
+        else { u.ui = co; u.um = M; u.us = so; u.ut = int32_t(T); }
+      }
+      o.units.push_back(u);
+      return -1;
+    };
+    const int64_t nu = int64_t(list.size()), nrun = std::min<int64_t>(nu, 64);
+    std::vector<UnitRun> runs(static_cast<size_t>(nrun));
+#pragma omp parallel for schedule(dynamic, 1)
+    for (int64_t r = 0; r < nrun; ++r) {
+      std::vector<std::vector<int32_t>> se(kWarp), sw(kWarp);
+      UnitRun &o = runs[size_t(r)];
+      for (int64_t k = nu * r / nrun; k < nu * (r + 1) / nrun && o.bad < 0; ++k)
+        o.bad = add_unit(o, se, sw, list[size_t(k)].first, list[size_t(k)].second);
     }
-    H.color_unit[n_c] = int32_t(H.units.size());
+    auto join = [](auto &to, const auto &from) {
+      const int32_t base = int32_t(to.size());
+      to.insert(to.end(), from.begin(), from.end());
+      return base;
+    };
+    for (UnitRun &o : runs) {
+      if (o.bad >= 0) return fail(ICCG_ERR_ARG, o.bad, "warp-unit chain longer than 32 steps", bad, msg);
+      const int32_t lo = join(H.sl_col, o.sl_col), uo = join(H.su_col, o.su_col), li = join(H.wl_map, o.wl_map);
+      const int32_t ui = join(H.wu_map, o.wu_map), lsw = join(H.wl_src, o.wl_src), usw = join(H.wu_src, o.wu_src);
+      join(H.sl_map, o.sl_map);
+      join(H.su_map, o.su_map);
+      join(H.wl_srow, o.wl_srow);
+      join(H.wu_srow, o.wu_srow);
+      join(H.wl_mask, o.wl_mask);
+      join(H.wu_mask, o.wu_mask);
+      for (WarpUnit &u : o.units) {
+        u.lo += lo; u.uo += uo; u.li += li; u.ui += ui; u.ls += lsw; u.us += usw;
+      }
+      join(H.units, o.units);
+      o = UnitRun{};
+    }
   }
   const size_t lim = size_t(1) << 31;
   if (H.wl_map.size() >= lim || H.wu_map.size() >= lim) return fail(ICCG_ERR_ARG, -1, "warp-unit layout exceeds 2^31 entries", bad, msg);
@@ -740,7 +785,8 @@ extern "C" iccg_status iccg_check_layout(int32_t n, int64_t nnz, const int64_t *
   int64_t bad = -1;
   std::string msg;
   const iccg_status st = build_layout(n, nnz, rowptr, colind, val, perm, block_ptr, color_ptr, n_b, n_c,
-                                      std::max(group_rows, 1), lane_max, use_units ? 1 : 0, H, bad, msg);
+                                      std::max(group_rows, 1), lane_max, UnitRule{use_units ? 1 : 0, false, false}, H,
+                                      bad, msg);
   report[0] = report[1] = report[2] = report[3] = 0;
   if (st != ICCG_OK) {
     report[3] = bad;

@@ -310,16 +310,22 @@ struct HostLayout {
   int32_t seg_l = 0, seg_u = 0, seg_a = 0;      // largest segments (entries)
 };
 
+// The colors run as warp units: largest block of min_rows..32 rows (0: none at
+// all); also those of one-row blocks only, and those of one- and two-row blocks.
+struct UnitRule {
+  int32_t min_rows;
+  bool one, mixed;
+};
+
 // Validates inputs and builds the layout (groups of at most group_rows rows);
 // returns ICCG_OK or an error with (bad_index, message) filled in.
 // Colors whose blocks all have at most lane_max rows (<= 32; 0 = none) use
 // lane tiles.
-// Colors whose largest block has unit_min..32 rows use warp units instead
-// of lane tiles (unit_min = 0: no warp units).
+// Colors named by `units` use warp units instead of lane tiles.
 iccg_status build_layout(int32_t n, int64_t nnz, const int64_t *rowptr, const int32_t *colind,
                          const double *val, const int32_t *perm, const int32_t *block_ptr,
                          const int32_t *color_ptr, int32_t n_b, int32_t n_c, int32_t group_rows,
-                         int32_t lane_max, int32_t unit_min, HostLayout &out, int64_t &bad_index,
+                         int32_t lane_max, UnitRule units, HostLayout &out, int64_t &bad_index,
                          std::string &msg);
 
 // ---- launch plan (host side) ---------------------------------------------
