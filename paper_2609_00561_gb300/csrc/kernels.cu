@@ -601,10 +601,12 @@ struct SlotArgs {
 // last launch sums them).  In the last launch every CTA adds a fixed chunk of
 // the earlier launches' slots (complete: griddepcontrol.wait before) to its own
 // partials; then groups of CTAs, then the last group runs the epilogue.
+// (COOP: the cooperative sweep has decided at its start whether the solve goes on)
+template <bool COOP = false>
 __device__ __forceinline__ void launch_epilogue(const Params &P, int fin, const SlotArgs &sa, double rr_acc,
                                                 double rz_acc, double *red, int *flag) {
   if (sa.off < 0) return;
-  if (fin == FIN_ITER && __ldcg(&P.sc->done)) return;   // an iteration after the last one
+  if (!COOP && fin == FIN_ITER && __ldcg(&P.sc->done)) return;   // an iteration after the last one
   if (fin == FIN_NONE) {
     const double v = cta_sum2(rr_acc, rz_acc, red);
     if (threadIdx.x == 0) P.slot_rr[sa.off + blockIdx.x] = v;
@@ -2833,8 +2835,18 @@ coop_sweep_kernel(Params P, int c_lo, int fin, int rr0, int ntail) {
   const int NW = int(gridDim.x) * nw, nc = P.n_c;
   double rr_acc = 0.0, rz_acc = 0.0;
   pdl_wait();
-  double alpha = 0.0;
-  if (UPDATE && !load_alpha(P, alpha)) return;
+  // one decision per CTA: a CTA of this launch whose wait runs out may end the
+  // solve at any time
+  __shared__ double alpha_s;
+  if (threadIdx.x == 0) {
+    double a = 0.0;
+    flag = UPDATE ? int(load_alpha(P, a)) : 1;
+    alpha_s = a;
+  }
+  __syncthreads();
+  const double alpha = alpha_s;
+  if (!flag) return;
+  __syncthreads();   // flag is reused by the barriers
   GridSync gs{P.bar, 0u, &flag, nullptr, 0, 0, P.wait_ns};
   bool ok = true;
   for (int c = c_lo; c < nc - 1 && ok; ++c) {
@@ -2863,7 +2875,7 @@ coop_sweep_kernel(Params P, int c_lo, int fin, int rr0, int ntail) {
     return;
   }
   if (rr0 < 0) return;   // no sums wanted
-  launch_epilogue(P, fin, SlotArgs{rr0, 0}, rr_acc, rz_acc, red, &flag);
+  launch_epilogue<true>(P, fin, SlotArgs{rr0, 0}, rr_acc, rz_acc, red, &flag);
   const int G = int(gridDim.x), b = int(blockIdx.x);
   if (threadIdx.x == 0)
     for (int k = 1; k < ntail; ++k) P.slot_rr[rr0 + k * G + b] = P.slot_rz[rr0 + k * G + b] = 0.0;
