@@ -323,29 +323,56 @@ __device__ __forceinline__ void block_chain(const BatchRows<PT> &b, PT *w, const
   }
 }
 
-// the block's results from w: y (stored when `store`) and its share of <y, y>
-// forward, z backward
-template <typename PT, bool UPPER>
-__device__ __forceinline__ void block_store(const BatchSys &S, const BatchRows<PT> &b, const PT *w, int kp, int j,
-                                            int ch, int NC, bool store, double &yy) {
-  PT *res = reinterpret_cast<PT *>(UPPER ? S.z : S.y);
-  for (int k = ch; k < b.nr; k += NC) {
-    const PT v = w[k * kp + j];
-    if (store) res[size_t(b.r0 + k) * kp + j] = v;
-    if (!UPPER) {
-      const double d = widen(v);
-      yy += d * d;
+// r of kBatchRowsU rows of a chain, from row k0 (0 past the block)
+template <typename PT>
+__device__ __forceinline__ void block_r(const BatchSys &S, const BatchRows<PT> &b, int kp, int j, int k0, int NC,
+                                        double (&r)[kBatchRowsU]) {
+#pragma unroll
+  for (int u = 0; u < kBatchRowsU; ++u) {
+    const int k = k0 + u * NC;
+    r[u] = k < b.nr ? __ldcg(S.r + size_t(b.r0 + k) * kp + j) : 0.0;
+  }
+}
+
+// the block's y from w
+template <typename PT>
+__device__ __forceinline__ void block_store_y(const BatchSys &S, const BatchRows<PT> &b, const PT *w, int kp, int j,
+                                              int ch, int NC) {
+  PT *y = reinterpret_cast<PT *>(S.y);
+  for (int k = ch; k < b.nr; k += NC) y[size_t(b.r0 + k) * kp + j] = w[k * kp + j];
+}
+
+// the block's z from w and its share of <r, z>; r: that of the chain's first
+// rows, the following ones loaded a step ahead
+template <typename PT>
+__device__ __forceinline__ void block_store_z(const BatchSys &S, const BatchRows<PT> &b, const PT *w, int kp, int j,
+                                              int ch, int NC, double (&r)[kBatchRowsU], double &rz) {
+  PT *z = reinterpret_cast<PT *>(S.z);
+  for (int k0 = ch; k0 < b.nr; k0 += NC * kBatchRowsU) {
+    double next[kBatchRowsU];
+    block_r<PT>(S, b, kp, j, k0 + NC * kBatchRowsU, NC, next);
+#pragma unroll
+    for (int u = 0; u < kBatchRowsU; ++u) {
+      const int k = k0 + u * NC;
+      if (k < b.nr) {
+        const PT v = w[k * kp + j];
+        z[size_t(b.r0 + k) * kp + j] = v;
+        rz += r[u] * widen(v);
+      }
+      r[u] = next[u];
     }
   }
 }
 
-// One substitution pass of a system; yy receives the warp's share of <y, y>,
-// y = L^-1 r, which is <r, z> (z = L^-T y): the backward sweep need not read r.
-// A warp owns a block at a time and works in three parts: every row minus its entries to other colors (block_other: all chains
-// of the warp, several rows each in flight), the in-block recurrence
-// (block_chain: shared memory only), the results (block_store).  The block's
-// static data is staged ahead; the first block of the next color before the
-// barrier that ends the current one.
+// One substitution pass of a system; rz receives the lane's share of <r, z>, r
+// in 64 bits times the z that is stored (with an FP32 preconditioner <y, y>,
+// y = L^-1 r, differs from it by 1e-8, and an overflow of z would not show).
+// A warp owns a block at a time and works in three parts: every row minus its
+// entries to other colors (block_other: all chains of the warp, several rows
+// each in flight), the in-block recurrence (block_chain: shared memory only;
+// the rows' r is loaded meanwhile), the results (block_store_y / _z).  The
+// block's static data is staged ahead; the first block of the next color before
+// the barrier that ends the current one.
 //
 // Bound by latency: a chain that walked its block row by row paid two to three
 // dependent L2 loads for each of 32 rows, 60-120 us for a color phase; split
@@ -355,7 +382,7 @@ __device__ __forceinline__ void block_store(const BatchSys &S, const BatchRows<P
 // color of one system has fewer blocks than its CTAs have warps.
 template <typename PT>
 __device__ __forceinline__ bool batch_precond(const BatchSys &S, unsigned char *sm, const BatchSmem &m, int cap, int kp,
-                                              int gw, int total, double &yy, unsigned nct, unsigned &gen, int *flag) {
+                                              int gw, int total, double &rz, unsigned nct, unsigned &gen, int *flag) {
   const int lane = threadIdx.x & 31, j = lane % kp, ch = lane / kp, NC = kWarp / kp;
   PT *w = reinterpret_cast<PT *>(sm);
   const PT *sdv = reinterpret_cast<const PT *>(sm + m.o_dv);
@@ -373,14 +400,17 @@ __device__ __forceinline__ bool batch_precond(const BatchSys &S, unsigned char *
       __syncwarp();
       if (ch == 0) block_chain<PT, false>(b, w, sdv, ssp, kp, j);
       __syncwarp();
-      block_store<PT, false>(S, b, w, kp, j, ch, NC, !last, yy);
-      if (last) {
+      if (!last) {
+        block_store_y<PT>(S, b, w, kp, j, ch, NC);
+      } else {
         // the last color: backward sweep of the same block at once (no
         // later colors), y in w
         b = stage_block<PT, true>(S, blk, sm, m, cap, lane);
+        double r[kBatchRowsU];
+        block_r<PT>(S, b, kp, j, ch, NC, r);
         if (ch == 0) block_chain<PT, true>(b, w, sdv, ssp, kp, j);
         __syncwarp();
-        block_store<PT, true>(S, b, w, kp, j, ch, NC, true, yy);
+        block_store_z<PT>(S, b, w, kp, j, ch, NC, r, rz);
       }
       blk += total;
       have = blk < b1;
@@ -400,10 +430,12 @@ __device__ __forceinline__ bool batch_precond(const BatchSys &S, unsigned char *
     const int b1 = __ldg(S.cblk + c + 1);
     while (have) {
       block_other<PT, true>(S, b, w, ssp, kp, j, ch, NC);
+      double r[kBatchRowsU];
+      block_r<PT>(S, b, kp, j, ch, NC, r);
       __syncwarp();
       if (ch == 0) block_chain<PT, true>(b, w, sdv, ssp, kp, j);
       __syncwarp();
-      block_store<PT, true>(S, b, w, kp, j, ch, NC, true, yy);
+      block_store_z<PT>(S, b, w, kp, j, ch, NC, r, rz);
       blk += total;
       have = blk < b1;
       if (have) b = stage_block<PT, true>(S, blk, sm, m, cap, lane);
