@@ -515,8 +515,143 @@ __device__ __forceinline__ double batch_spmv(const BatchSys &S, unsigned char *s
   return acc;
 }
 
-// R: rows of a chain in flight in the SpMV (1, 2 or 4)
-template <typename PT, int R>
+// The same by walking (UPDATE: with the x / r update in front of the forward
+// sweep): a chain owns a block at a time and resolves it row by row; w is the
+// chain's scratch (block rows x kp).  A warp serves 32 / kp blocks at once, so
+// that it has more blocks in flight than batch_precond and, one latency after
+// another, needs longer for each.
+template <typename PT, bool UPDATE>
+__device__ __forceinline__ bool batch_precond_walk(const BatchSys &S, PT *w, int kp, int j, int gc, int total,
+                                              double alpha, bool act, double &rr, double &rz, unsigned nct,
+                                              unsigned &gen, int *flag) {
+  const PT *lv = b_lv<PT>(S), *uv = b_uv<PT>(S), *dv = b_dv<PT>(S);
+  PT *y = reinterpret_cast<PT *>(S.y);
+  PT *z = reinterpret_cast<PT *>(S.z);
+  const int nc = S.nc;
+  for (int c = 0; c < nc; ++c) {
+    const bool last = c == nc - 1;
+    const int b1 = __ldg(S.cblk + c + 1);
+    for (int blk = __ldg(S.cblk + c) + gc; blk < b1; blk += total) {
+      const int r0 = __ldg(S.bptr + blk), r1 = __ldg(S.bptr + blk + 1);
+      for (int i = r0; i < r1; ++i) {
+        double ri = __ldcg(S.r + size_t(i) * kp + j);
+        if (UPDATE && act) {
+          ri -= alpha * __ldcg(S.q + size_t(i) * kp + j);
+          S.r[size_t(i) * kp + j] = ri;
+          S.x[size_t(i) * kp + j] = __ldcg(S.x + size_t(i) * kp + j) + alpha * __ldcg(S.p + size_t(i) * kp + j);
+          rr += ri * ri;
+        }
+        PT acc = PT(ri);
+        const int e1 = __ldg(S.lrp + i + 1);
+        for (int e = __ldg(S.lrp + i); e < e1; ++e) {
+          const int col = __ldg(S.lcol + e);
+          const PT v = __ldg(lv + e);
+          const PT yc = col >= r0 ? w[(col - r0) * kp + j] : __ldcg(y + size_t(col) * kp + j);
+          acc -= v * yc;
+        }
+        const PT yi = acc * __ldg(dv + i);
+        w[(i - r0) * kp + j] = yi;
+        if (!last) y[size_t(i) * kp + j] = yi;
+      }
+      if (last) {
+        // the last color: backward sweep of the same block at once (no
+        // later colors), y in the scratch
+        for (int i = r1 - 1; i >= r0; --i) {
+          PT acc = w[(i - r0) * kp + j];
+          const int e1 = __ldg(S.urp + i + 1);
+          for (int e = __ldg(S.urp + i); e < e1; ++e) acc -= __ldg(uv + e) * w[(__ldg(S.ucol + e) - r0) * kp + j];
+          const PT zi = acc * __ldg(dv + i);
+          w[(i - r0) * kp + j] = zi;
+          z[size_t(i) * kp + j] = zi;
+          rz += __ldcg(S.r + size_t(i) * kp + j) * widen(zi);
+        }
+      }
+    }
+    // every color's results (for the last color: its z) complete before the
+    // next color reads them
+    if (!sys_sync(S.bar, nct, gen, flag, S.wait_ns)) return false;
+  }
+  for (int c = nc - 2; c >= 0; --c) {
+    const int b1 = __ldg(S.cblk + c + 1);
+    for (int blk = __ldg(S.cblk + c) + gc; blk < b1; blk += total) {
+      const int r0 = __ldg(S.bptr + blk), r1 = __ldg(S.bptr + blk + 1);
+      for (int i = r1 - 1; i >= r0; --i) {
+        PT acc = __ldcg(y + size_t(i) * kp + j);
+        const int e1 = __ldg(S.urp + i + 1);
+        for (int e = __ldg(S.urp + i); e < e1; ++e) {
+          const int col = __ldg(S.ucol + e);
+          const PT zc = col < r1 ? w[(col - r0) * kp + j] : __ldcg(z + size_t(col) * kp + j);
+          acc -= __ldg(uv + e) * zc;
+        }
+        const PT zi = acc * __ldg(dv + i);
+        w[(i - r0) * kp + j] = zi;
+        z[size_t(i) * kp + j] = zi;
+        rz += __ldcg(S.r + size_t(i) * kp + j) * widen(zi);
+      }
+    }
+    if (c > 0 && !sys_sync(S.bar, nct, gen, flag, S.wait_ns)) return false;
+  }
+  return true;
+}
+
+// A times a [n][kp] vector by walking: a chain per row (INIT or R = 1) or R
+// consecutive rows of a chain together.  INIT and results as in batch_spmv.
+template <int R, bool INIT>
+__device__ __forceinline__ double batch_spmv_walk(const BatchSys &S, int kp, int j, int gc, int total, bool act) {
+  const double *v = INIT ? S.x : S.p;
+  const int n = S.n;
+  double acc = 0.0;
+  if (!act) return acc;
+  if constexpr (INIT || R == 1) {
+    for (int i = gc; i < n; i += total) {
+      const size_t at = size_t(i) * kp + j;
+      double s = 0.0;
+      const int e1 = __ldg(S.arp + i + 1);
+      for (int e = __ldg(S.arp + i); e < e1; ++e)
+        s += __ldg(S.aval + e) * __ldcg(v + size_t(__ldg(S.acol + e)) * kp + j);
+      if (INIT) {
+        const double ri = __ldcg(S.r + at) - s;
+        S.r[at] = ri;
+        acc += ri * ri;
+      } else {
+        S.q[at] = s;
+        acc += __ldcg(v + at) * s;
+      }
+    }
+  } else {
+    for (int i0 = gc * R; i0 < n; i0 += total * R) {
+      int e0[R], e1[R];
+      double s[R];
+      int len = 0;
+#pragma unroll
+      for (int u = 0; u < R; ++u) {
+        const bool in = i0 + u < n;
+        e0[u] = in ? __ldg(S.arp + i0 + u) : 0;
+        e1[u] = in ? __ldg(S.arp + i0 + u + 1) : 0;
+        s[u] = 0.0;
+        len = max(len, e1[u] - e0[u]);
+      }
+      // the rows' t-th entries together (each row's sum in entry order)
+      for (int t = 0; t < len; ++t) {
+#pragma unroll
+        for (int u = 0; u < R; ++u)
+          if (e0[u] + t < e1[u])
+            s[u] += __ldg(S.aval + e0[u] + t) * __ldcg(v + size_t(__ldg(S.acol + e0[u] + t)) * kp + j);
+      }
+#pragma unroll
+      for (int u = 0; u < R; ++u)
+        if (i0 + u < n) {
+          S.q[size_t(i0 + u) * kp + j] = s[u];
+          acc += __ldcg(v + size_t(i0 + u) * kp + j) * s[u];
+        }
+    }
+  }
+  return acc;
+}
+
+// R: rows of a chain in flight in the SpMV (1, 2 or 4); WALK: the walking
+// forms, with a chain's row scratch as its only shared memory
+template <typename PT, int R, bool WALK>
 __global__ void __launch_bounds__(kMaxWarpsPerCta * kWarp, 1)
 batch_kernel(const BatchSys *sys, const int32_t *cta_sys, int k, int kp, BatchSmem plan, int cap, int maxit,
              double tol) {
@@ -537,6 +672,7 @@ batch_kernel(const BatchSys *sys, const int32_t *cta_sys, int k, int kp, BatchSm
   const int W = blockDim.x / kWarp, warp = threadIdx.x / kWarp;
   const int gw = lc * W + warp, totalw = int(nct) * W;
   unsigned char *wsm = smem + size_t(warp) * plan.bytes;
+  PT *wch = reinterpret_cast<PT *>(wsm) + size_t(ch % (kWarp / kp)) * (plan.bytes / int(sizeof(PT)) / (kWarp / kp));
   double *red = reinterpret_cast<double *>(smem + size_t(W) * plan.bytes);
   double *mypart = S.part + size_t(lc) * 4 * kp;
   const int n = S.n;
@@ -558,13 +694,17 @@ batch_kernel(const BatchSys *sys, const int32_t *cta_sys, int k, int kp, BatchSm
   ok = sys_sync(S.bar, nct, gen, &flag, S.wait_ns);
   // r0 = b - A x0, <r0, r0> (a row's b is read and r written by its own lane)
   if (ok) {
-    acc = batch_spmv<R, true>(S, wsm, plan, cap, kp, gw, totalw, true);
+    if constexpr (WALK) acc = batch_spmv_walk<R, true>(S, kp, j, gc, total, true);
+    else acc = batch_spmv<R, true>(S, wsm, plan, cap, kp, gw, totalw, true);
     cta_rhs_sum(acc, red, kp, mypart + 1 * kp);
     ok = sys_sync(S.bar, nct, gen, &flag, S.wait_ns);
   }
   // z0 = M^-1 r0, <r0, z0>
   double rr = 0.0, rz = 0.0;
-  if (ok) ok = batch_precond<PT>(S, wsm, plan, cap, kp, gw, totalw, rz, nct, gen, &flag);
+  if (ok) {
+    if constexpr (WALK) ok = batch_precond_walk<PT, false>(S, wch, kp, j, gc, total, 0.0, false, rr, rz, nct, gen, &flag);
+    else ok = batch_precond<PT>(S, wsm, plan, cap, kp, gw, totalw, rz, nct, gen, &flag);
+  }
   if (ok) {
     cta_rhs_sum(rz, red, kp, mypart + 3 * kp);
     ok = sys_sync(S.bar, nct, gen, &flag, S.wait_ns);
@@ -625,43 +765,49 @@ batch_kernel(const BatchSys *sys, const int32_t *cta_sys, int k, int kp, BatchSm
     }
     if (!(ok = sys_sync(S.bar, nct, gen, &flag, S.wait_ns))) break;
     // q = A p, <p, q>
-    acc = batch_spmv<R, false>(S, wsm, plan, cap, kp, gw, totalw, act);
+    if constexpr (WALK) acc = batch_spmv_walk<R, false>(S, kp, j, gc, total, act);
+    else acc = batch_spmv<R, false>(S, wsm, plan, cap, kp, gw, totalw, act);
     cta_rhs_sum(acc, red, kp, mypart + 2 * kp);
     if (!(ok = sys_sync(S.bar, nct, gen, &flag, S.wait_ns))) break;
     sys_rhs_sum(S.part, int(nct), kp, 2, sv[2], red);
     const double alpha = act ? st_rz[j] / sv[2][j] : 0.0;
-    // x / r update and <r,r> over all rows at once (in front of each color's
-    // forward sweep, where only that color's blocks are at work, it took twice
-    // as long), then z = M^-1 r and <r,z>
     rr = 0.0;
-    if (act) {
-      for (int i0 = gc; i0 < n; i0 += total * kBatchRowsU) {
-        double ri[kBatchRowsU], qi[kBatchRowsU], xi[kBatchRowsU], pi[kBatchRowsU];
+    rz = 0.0;
+    if constexpr (WALK) {
+      // x / r update, z = M^-1 r, <r,r>, <r,z>
+      if (!(ok = batch_precond_walk<PT, true>(S, wch, kp, j, gc, total, alpha, act, rr, rz, nct, gen, &flag))) break;
+    } else {
+      // x / r update and <r,r> over all rows at once (in front of each color's
+      // forward sweep, where only that color's blocks are at work, it took twice
+      // as long), then z = M^-1 r and <r,z>
+      if (act) {
+        for (int i0 = gc; i0 < n; i0 += total * kBatchRowsU) {
+          double ri[kBatchRowsU], qi[kBatchRowsU], xi[kBatchRowsU], pi[kBatchRowsU];
 #pragma unroll
-        for (int u = 0; u < kBatchRowsU; ++u) {
-          const int i = i0 + u * total;
-          const size_t at = size_t(i) * kp + j;
-          ri[u] = i < n ? __ldcg(S.r + at) : 0.0;
-          qi[u] = i < n ? __ldcg(S.q + at) : 0.0;
-          xi[u] = i < n ? __ldcg(S.x + at) : 0.0;
-          pi[u] = i < n ? __ldcg(S.p + at) : 0.0;
-        }
-#pragma unroll
-        for (int u = 0; u < kBatchRowsU; ++u) {
-          const int i = i0 + u * total;
-          if (i < n) {
+          for (int u = 0; u < kBatchRowsU; ++u) {
+            const int i = i0 + u * total;
             const size_t at = size_t(i) * kp + j;
-            ri[u] -= alpha * qi[u];
-            S.r[at] = ri[u];
-            S.x[at] = xi[u] + alpha * pi[u];
-            rr += ri[u] * ri[u];
+            ri[u] = i < n ? __ldcg(S.r + at) : 0.0;
+            qi[u] = i < n ? __ldcg(S.q + at) : 0.0;
+            xi[u] = i < n ? __ldcg(S.x + at) : 0.0;
+            pi[u] = i < n ? __ldcg(S.p + at) : 0.0;
+          }
+#pragma unroll
+          for (int u = 0; u < kBatchRowsU; ++u) {
+            const int i = i0 + u * total;
+            if (i < n) {
+              const size_t at = size_t(i) * kp + j;
+              ri[u] -= alpha * qi[u];
+              S.r[at] = ri[u];
+              S.x[at] = xi[u] + alpha * pi[u];
+              rr += ri[u] * ri[u];
+            }
           }
         }
       }
+      if (!(ok = sys_sync(S.bar, nct, gen, &flag, S.wait_ns))) break;
+      if (!(ok = batch_precond<PT>(S, wsm, plan, cap, kp, gw, totalw, rz, nct, gen, &flag))) break;
     }
-    if (!(ok = sys_sync(S.bar, nct, gen, &flag, S.wait_ns))) break;
-    rz = 0.0;
-    if (!(ok = batch_precond<PT>(S, wsm, plan, cap, kp, gw, totalw, rz, nct, gen, &flag))) break;
     cta_rhs_sum(rr, red, kp, mypart + 1 * kp);
     cta_rhs_sum(rz, red, kp, mypart + 3 * kp);
     if (!(ok = sys_sync(S.bar, nct, gen, &flag, S.wait_ns))) break;
@@ -727,8 +873,13 @@ cudaError_t allow_smem_b(K kernel) {
 using BatchKernel = void (*)(const BatchSys *, const int32_t *, int, int, BatchSmem, int, int, double);
 
 template <typename PT>
-BatchKernel batch_kernel_of(int R) {
-  return R == 4 ? batch_kernel<PT, 4> : (R == 2 ? batch_kernel<PT, 2> : batch_kernel<PT, 1>);
+BatchKernel batch_kernel_of(int R, bool walk) {
+  if (walk) return R == 4 ? batch_kernel<PT, 4, true> : (R == 2 ? batch_kernel<PT, 2, true> : batch_kernel<PT, 1, true>);
+  return R == 4 ? batch_kernel<PT, 4, false> : (R == 2 ? batch_kernel<PT, 2, false> : batch_kernel<PT, 1, false>);
+}
+
+BatchKernel batch_kernel_of(bool fp32, int R, bool walk) {
+  return fp32 ? batch_kernel_of<float>(R, walk) : batch_kernel_of<double>(R, walk);
 }
 
 }  // namespace
@@ -741,6 +892,7 @@ struct iccg_batch {
   cudaStream_t stream = nullptr;
   int nsys = 0, k = 0, kp = 0, smax = 1;
   int cap = 0;           // entries of a block or SpMV tile staged per warp
+  bool walk = false;          // the launch shape's kernel walks
   bool fp32 = false;
   std::vector<iccg_ctx *> ctxs;
   std::vector<int32_t> n;
@@ -777,15 +929,21 @@ cudaError_t b_alloc(iccg_batch *b, void **p, size_t bytes) {
   return cudaMemsetAsync(*p, 0, bytes + 64, b->stream);
 }
 
-BatchSmem batch_plan(const iccg_batch *b) { return batch_smem_plan(b->smax, b->kp, b->cap, b->fp32 ? 4 : 8); }
+// a warp's shared memory: the block buffers, or (walk) the rows of its chains' blocks
+BatchSmem batch_plan(const iccg_batch *b, bool walk) {
+  const int elem = b->fp32 ? 4 : 8;
+  if (!walk) return batch_smem_plan(b->smax, b->kp, b->cap, elem);
+  BatchSmem m{};
+  m.bytes = kWarp * b->smax * elem;
+  return m;
+}
 
-int batch_smem(const iccg_batch *b, int W) { return W * batch_plan(b).bytes + W * kWarp * 8; }
+int batch_smem(const iccg_batch *b, int W, bool walk) { return W * batch_plan(b, walk).bytes + W * kWarp * 8; }
 
-int batch_occupancy(const iccg_batch *b, int W, int smem) {
+int batch_occupancy(const iccg_batch *b, int W, bool walk) {
   int nb = 0;
-  const cudaError_t e =
-      b->fp32 ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, batch_kernel_of<float>(b->R), W * kWarp, size_t(smem))
-              : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, batch_kernel_of<double>(b->R), W * kWarp, size_t(smem));
+  const cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, batch_kernel_of(b->fp32, b->R, walk),
+                                                                      W * kWarp, size_t(batch_smem(b, W, walk)));
   if (e != cudaSuccess) {
     cudaGetLastError();
     return 0;
@@ -922,13 +1080,17 @@ cudaError_t batch_launch(iccg_batch *b, cudaStream_t s, int maxit, double tol) {
   cfg.numAttrs = 1;
   const BatchSys *sys = b->d_sys;
   const int32_t *cts = b->d_cta_sys;
-  if (b->fp32) return cudaLaunchKernelEx(&cfg, batch_kernel_of<float>(b->R), sys, cts, b->k, b->kp, batch_plan(b), b->cap, maxit, tol);
-  return cudaLaunchKernelEx(&cfg, batch_kernel_of<double>(b->R), sys, cts, b->k, b->kp, batch_plan(b), b->cap, maxit, tol);
+  return cudaLaunchKernelEx(&cfg, batch_kernel_of(b->fp32, b->R, b->walk), sys, cts, b->k, b->kp,
+                            batch_plan(b, b->walk), b->cap, maxit, tol);
 }
 
+// The form a shape runs: the walk where the block buffers do not fit beside one
+// another (64-row blocks, 32 right-hand sides, FP64: above 9 warps a CTA).
+bool shape_walks(const iccg_batch *b, int W) { return batch_occupancy(b, W, false) <= 0; }
+
 iccg_status set_shape(iccg_batch *b, int W, int cps, int sms) {
-  const int smem = batch_smem(b, W);
-  const int occ = batch_occupancy(b, W, smem);
+  const bool walk = shape_walks(b, W);
+  const int occ = batch_occupancy(b, W, walk);
   if (occ <= 0) {
     b->err_msg = "batched kernel does not fit an SM with this shape";
     return ICCG_ERR_ARG;
@@ -944,7 +1106,8 @@ iccg_status set_shape(iccg_batch *b, int W, int cps, int sms) {
   }
   b->W = W;
   b->cps = c;
-  b->smem = smem;
+  b->walk = walk;
+  b->smem = batch_smem(b, W, walk);
   destroy_batch_graph(b);
   return ICCG_OK;
 }
@@ -1050,9 +1213,9 @@ iccg_status iccg_batch_create(iccg_batch **out, iccg_ctx *const *ctxs, int32_t n
   cudaGetDevice(&prev);
   if (prev != b->device) cudaSetDevice(b->device);
   cudaError_t e = cudaSuccess;
-  for (int R : {1, 2, 4}) {
-    if (e == cudaSuccess) e = b->fp32 ? allow_smem_b(batch_kernel_of<float>(R)) : allow_smem_b(batch_kernel_of<double>(R));
-  }
+  for (int R : {1, 2, 4})
+    for (bool walk : {false, true})
+      if (e == cudaSuccess) e = allow_smem_b(batch_kernel_of(b->fp32, R, walk));
   const size_t pe = b->fp32 ? 4 : 8;
   int sms = 152;
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, b->device);
@@ -1221,7 +1384,7 @@ iccg_status iccg_batch_tune(iccg_batch *b, const double *const *B, double tol, i
   int bW = b->W, bC = b->cps;
   for (double E : Es)
   for (int W : Ws) {
-    const int occ = batch_occupancy(b, W, batch_smem(b, W));
+    const int occ = batch_occupancy(b, W, shape_walks(b, W));
     for (int cps = 1; cps <= std::min(occ, 4); cps *= 2) {
       b->wexp = E;
       if (set_shape(b, W, cps, sms) != ICCG_OK) continue;
