@@ -149,13 +149,16 @@ __device__ __forceinline__ void cta_rhs_sum(double v, double *red, int kp, doubl
 // j < kp; every CTA computes the same values.  The CTA's chains take the CTAs
 // in turn (their loads in flight together: one thread per j walking them took
 // 10 us for 100 CTAs), then one thread per j adds the chains' sums.
+// (The walk's kernel without unrolling: the registers of eight loads cost it 8%
+// with 32 right-hand sides in FP64.)
+template <bool WALK>
 __device__ __forceinline__ void sys_rhs_sum(const double *part, int nct, int kp, int slot, double *out, double *red) {
   const int ch = threadIdx.x / kp, j = threadIdx.x % kp, nchain = blockDim.x / kp;
   const int used = min(nchain, 16);
   __syncthreads();
   if (ch < used) {
     double s = 0.0;
-#pragma unroll 8
+#pragma unroll (WALK ? 1 : 8)
     for (int c = ch; c < nct; c += used) s += __ldcg(part + (size_t(c) * 4 + slot) * kp + j);
     red[ch * kp + j] = s;
   }
@@ -176,10 +179,11 @@ __device__ __forceinline__ void sys_rhs_sum(const double *part, int nct, int kp,
 constexpr int kSpmvRows = 16;   // rows of a warp's SpMV tile
 struct BatchSmem {
   int o_dv, o_val, o_col, o_rp, o_sp, bytes;
+  int chain;   // the walk: values of a chain's row scratch
 };
 __host__ __device__ inline BatchSmem batch_smem_plan(int smax, int kp, int cap, int elem) {
   const int rows = smax > kSpmvRows ? smax : kSpmvRows;
-  BatchSmem m;
+  BatchSmem m{};
   int o = r16b(smax * kp * elem);
   m.o_dv = o; o += r16b(smax * elem);
   m.o_val = o; o += r16b(cap * 8);
@@ -519,7 +523,7 @@ __device__ __forceinline__ double batch_spmv(const BatchSys &S, unsigned char *s
 // sweep): a chain owns a block at a time and resolves it row by row; w is the
 // chain's scratch (block rows x kp).  A warp serves 32 / kp blocks at once, so
 // that it has more blocks in flight than batch_precond and, one latency after
-// another, needs longer for each.
+// another, needs longer for each (batch_walks: which is the better one when).
 template <typename PT, bool UPDATE>
 __device__ __forceinline__ bool batch_precond_walk(const BatchSys &S, PT *w, int kp, int j, int gc, int total,
                                               double alpha, bool act, double &rr, double &rz, unsigned nct,
@@ -672,7 +676,7 @@ batch_kernel(const BatchSys *sys, const int32_t *cta_sys, int k, int kp, BatchSm
   const int W = blockDim.x / kWarp, warp = threadIdx.x / kWarp;
   const int gw = lc * W + warp, totalw = int(nct) * W;
   unsigned char *wsm = smem + size_t(warp) * plan.bytes;
-  PT *wch = reinterpret_cast<PT *>(wsm) + size_t(ch % (kWarp / kp)) * (plan.bytes / int(sizeof(PT)) / (kWarp / kp));
+  PT *wch = reinterpret_cast<PT *>(smem) + size_t(ch) * plan.chain;
   double *red = reinterpret_cast<double *>(smem + size_t(W) * plan.bytes);
   double *mypart = S.part + size_t(lc) * 4 * kp;
   const int n = S.n;
@@ -711,9 +715,9 @@ batch_kernel(const BatchSys *sys, const int32_t *cta_sys, int k, int kp, BatchSm
   }
   int it = 0;
   if (ok) {
-    sys_rhs_sum(S.part, int(nct), kp, 0, sv[0], red);
-    sys_rhs_sum(S.part, int(nct), kp, 1, sv[1], red);
-    sys_rhs_sum(S.part, int(nct), kp, 3, sv[3], red);
+    sys_rhs_sum<WALK>(S.part, int(nct), kp, 0, sv[0], red);
+    sys_rhs_sum<WALK>(S.part, int(nct), kp, 1, sv[1], red);
+    sys_rhs_sum<WALK>(S.part, int(nct), kp, 3, sv[3], red);
     if (threadIdx.x < kp) {
       const int t = threadIdx.x;
       const double bn = sqrt(sv[0][t]);
@@ -746,20 +750,20 @@ batch_kernel(const BatchSys *sys, const int32_t *cta_sys, int k, int kp, BatchSm
   while (ok && any_act) {
     const bool act = st_act[j] != 0;
     const double beta = st_beta[j];
-    // p = z + beta p
+    // p = z + beta p (U rows of a chain in flight)
     const PT *z = reinterpret_cast<const PT *>(S.z);
-    // (kBatchRowsU rows of a chain in flight)
+    constexpr int U = WALK ? R : kBatchRowsU;
     if (act) {
-      for (int i0 = gc; i0 < n; i0 += total * kBatchRowsU) {
-        double zz[kBatchRowsU], pp[kBatchRowsU];
+      for (int i0 = gc; i0 < n; i0 += total * U) {
+        double zz[U], pp[U];
 #pragma unroll
-        for (int u = 0; u < kBatchRowsU; ++u) {
+        for (int u = 0; u < U; ++u) {
           const int i = i0 + u * total;
           zz[u] = i < n ? widen(__ldcg(z + size_t(i) * kp + j)) : 0.0;
           pp[u] = i < n ? __ldcg(S.p + size_t(i) * kp + j) : 0.0;
         }
 #pragma unroll
-        for (int u = 0; u < kBatchRowsU; ++u)
+        for (int u = 0; u < U; ++u)
           if (i0 + u * total < n) S.p[size_t(i0 + u * total) * kp + j] = zz[u] + beta * pp[u];
       }
     }
@@ -769,7 +773,7 @@ batch_kernel(const BatchSys *sys, const int32_t *cta_sys, int k, int kp, BatchSm
     else acc = batch_spmv<R, false>(S, wsm, plan, cap, kp, gw, totalw, act);
     cta_rhs_sum(acc, red, kp, mypart + 2 * kp);
     if (!(ok = sys_sync(S.bar, nct, gen, &flag, S.wait_ns))) break;
-    sys_rhs_sum(S.part, int(nct), kp, 2, sv[2], red);
+    sys_rhs_sum<WALK>(S.part, int(nct), kp, 2, sv[2], red);
     const double alpha = act ? st_rz[j] / sv[2][j] : 0.0;
     rr = 0.0;
     rz = 0.0;
@@ -811,8 +815,8 @@ batch_kernel(const BatchSys *sys, const int32_t *cta_sys, int k, int kp, BatchSm
     cta_rhs_sum(rr, red, kp, mypart + 1 * kp);
     cta_rhs_sum(rz, red, kp, mypart + 3 * kp);
     if (!(ok = sys_sync(S.bar, nct, gen, &flag, S.wait_ns))) break;
-    sys_rhs_sum(S.part, int(nct), kp, 1, sv[1], red);
-    sys_rhs_sum(S.part, int(nct), kp, 3, sv[3], red);
+    sys_rhs_sum<WALK>(S.part, int(nct), kp, 1, sv[1], red);
+    sys_rhs_sum<WALK>(S.part, int(nct), kp, 3, sv[3], red);
     ++it;
     if (threadIdx.x < kp) {
       const int t = threadIdx.x;
@@ -892,7 +896,8 @@ struct iccg_batch {
   cudaStream_t stream = nullptr;
   int nsys = 0, k = 0, kp = 0, smax = 1;
   int cap = 0;           // entries of a block or SpMV tile staged per warp
-  bool walk = false;          // the launch shape's kernel walks
+  bool walk_better = false;   // the walk is the better form for these systems
+  bool walk = false;          // the launch shape's form
   bool fp32 = false;
   std::vector<iccg_ctx *> ctxs;
   std::vector<int32_t> n;
@@ -935,6 +940,7 @@ BatchSmem batch_plan(const iccg_batch *b, bool walk) {
   if (!walk) return batch_smem_plan(b->smax, b->kp, b->cap, elem);
   BatchSmem m{};
   m.bytes = kWarp * b->smax * elem;
+  m.chain = b->smax * b->kp;
   return m;
 }
 
@@ -1084,9 +1090,43 @@ cudaError_t batch_launch(iccg_batch *b, cudaStream_t s, int maxit, double tol) {
                             batch_plan(b, b->walk), b->cap, maxit, tol);
 }
 
-// The form a shape runs: the walk where the block buffers do not fit beside one
-// another (64-row blocks, 32 right-hand sides, FP64: above 9 warps a CTA).
-bool shape_walks(const iccg_batch *b, int W) { return batch_occupancy(b, W, false) <= 0; }
+// Where the walk is the better form (400 combinations of 8 batches, blocks of 1
+// to 64 rows, 1 to 32 right-hand sides and both precisions, ten iterations;
+// taking the better one everywhere would gain 0.4% more on average).  A warp per
+// block pays where a block fills its chains and the blocks of a color do not
+// outnumber the warps; the walk is better
+//  - for blocks of one and two rows (4 systems of sides 16..48, one-row blocks:
+//    0.65 against 8.1 ms with one right-hand side, 4.7 against 10.7 with 16; at
+//    worst 1.2 times the warp form's time: 20,000-row graph, two rows, one
+//    right-hand side);
+//  - for blocks of three to five rows with 16 or 32 right-hand sides (two chains
+//    or one to a warp: 27-point, 4-row blocks, 32: 0.74 of the time) or with
+//    more blocks a color than `warps` (sides 16..48, 4-row blocks, 4 right-hand
+//    sides: 0.70; with half as many blocks, one side of 40: 1.15);
+//  - for a single chain to a warp on wide rows (32 right-hand sides; 17 entries a
+//    row 0.72 to 1.15, 27-point 0.67 to 1.0, spring network 0.43 to 0.8; at 9
+//    entries and below the warp form is better from 8-row blocks on);
+//  - in FP32 for two chains on rows above 32 entries whose blocks are not staged
+//    (spring network, 16 right-hand sides, blocks of 32 rows: 0.87; FP64 1.07).
+bool batch_walks(const iccg_batch *b, int warps) {
+  double rows = 0.0, blocks = 0.0, entries = 0.0, per_color = 0.0;
+  for (const iccg_ctx *c : b->ctxs) {
+    rows += c->H.n;
+    blocks += c->H.n_b;
+    entries += double(c->H.acol.size());
+    per_color += double(c->H.n_b) / c->H.n_c;
+  }
+  const double mean = rows / blocks, wide = entries / rows;
+  if (mean < 3.0) return true;
+  if (mean < 6.0 && (b->kp >= 16 || per_color > warps)) return true;
+  if (b->kp >= 32 && wide > 12.0) return true;
+  return b->fp32 && b->kp >= 16 && wide > 32.0 && mean * wide > 2.0 * kBatchCap;
+}
+
+// The form a shape runs: the better one, or the walk where the block buffers do
+// not fit beside one another (64-row blocks, 32 right-hand sides, FP64: above 9
+// warps a CTA).
+bool shape_walks(const iccg_batch *b, int W) { return b->walk_better || batch_occupancy(b, W, false) <= 0; }
 
 iccg_status set_shape(iccg_batch *b, int W, int cps, int sms) {
   const bool walk = shape_walks(b, W);
@@ -1280,6 +1320,7 @@ iccg_status iccg_batch_create(iccg_batch **out, iccg_ctx *const *ctxs, int32_t n
     return ICCG_ERR_CUDA;
   }
   b->R = o.rows_per_thread > 0 ? o.rows_per_thread : 1;
+  b->walk_better = batch_walks(b, 16 * sms);   // 2 CTAs of 8 warps an SM: the usual shape
   iccg_status st = set_shape(b, o.warps_per_cta > 0 ? o.warps_per_cta : 8, o.ctas_per_sm, sms);
   if (st != ICCG_OK) return st;
   if (o.autotune) {

@@ -1,7 +1,9 @@
 """Launch shapes of the batched solve at the limit of an SM's shared memory: the
 warps of a CTA with the largest blocks and a full warp of right-hand sides, each
 as many as fit with one row scratch per right-hand side alone; against the
-oracle (bars of test_gpu_batched.py).  One warp more than that is refused."""
+oracle (bars of test_gpu_batched.py).  One warp more than that is refused.
+Then the block sizes and right-hand-side counts between which the kernel's form
+changes."""
 import numpy as np
 import pytest
 
@@ -52,4 +54,24 @@ def test_one_warp_more_is_refused():
     with pytest.raises(iccg.IccgError) as ei:
         iccg.BatchSolver([S], 32, warps_per_cta=14)
     assert ei.value.status == iccg.ICCG_ERR_ARG
+    S.close()
+
+
+@pytest.mark.parametrize("nrhs", [1, 8, 9, 16, 17])
+@pytest.mark.parametrize("block", [2, 3, 5, 6])
+@pytest.mark.parametrize("wide", [False, True])
+def test_small_blocks_match_oracle(wide, block, nrhs):
+    libbuild.build()
+    a, bl, S = _systems(False, block, wide)
+    B = np.random.default_rng(8).uniform(-1.0, 1.0, (nrhs, a.n))
+    batch = iccg.BatchSolver([S, S], nrhs)
+    X = [np.zeros_like(B), np.zeros_like(B)]
+    st, it, _, _ = batch.solve([B, B], X, 1e-8, 3000)
+    assert st == iccg.ICCG_OK
+    for j in range(0, nrhs, 8):
+        ref = oracle.iccg(a, B[j], bl["perm"], tol=1e-8, maxit=3000)
+        for x in X:
+            assert np.linalg.norm(x[j] - ref["x"]) <= 1e-10 * np.linalg.norm(ref["x"])
+        assert abs(int(it[0, j]) - ref["iterations"]) <= 1
+    batch.close()
     S.close()
