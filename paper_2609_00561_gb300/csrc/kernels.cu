@@ -1464,8 +1464,20 @@ __device__ __forceinline__ void pair_tile_staged(const Params &P, const PairPre<
 template <typename PT>
 constexpr int pair_stage_bytes() { return int(sizeof(PairStage<PT>)); }
 
+// Registers a thread: the kernel is bound by the loads in flight, i.e. by the CTAs
+// that fit beside one another with the gathers' registers: 9 CTAs of 4 warps an SM
+// in FP32 (56 registers), 8 in FP64, fewer for the staged forms with the x / r
+// update, which need more.  Left to itself the compiler takes 58 to 64 for some
+// FP32 forms (8 CTAs) and 40 for others (fewer loads in flight).  40 iterations in
+// FP32, two-row blocks: 27-point 66^3 10.0 ms, so 7.3; graph of degree 16, 200,000
+// rows 20.8 and 13.1; FP64 27-point 66^3 8.6 and 8.3.
+constexpr int pair_regs(int elem, int mode, bool update, bool stage) {
+  if (update && stage) return elem == 8 && mode == M_FUSED ? 96 : 64;
+  return elem == 4 ? 56 : 64;
+}
+
 template <typename PT, int MODE, bool UPDATE, bool STAGE>
-__global__ void __launch_bounds__(kMaxWarpsPerCta * kWarp)
+__global__ void __maxnreg__(pair_regs(int(sizeof(PT)), MODE, UPDATE, STAGE))
 pair_kernel(Params P, int t0, int t1, int fin, SlotArgs sa) {
   extern __shared__ __align__(16) unsigned char smem[];
   __shared__ double red[kRed];
