@@ -301,7 +301,7 @@ iccg_status iccg_setup(iccg_ctx **out, int32_t n, int64_t nnz, const int64_t *ro
   L.unit_T.assign(n_c, 0);
   L.Wu = 8;
   int32_t gbig = 1;
-  bool lane_tiles = false;
+  bool lane_tiles = false, one_row_tiles = false;   // colors run one CTA per lane tile
   for (int c = 0; c < n_c; ++c) {
     L.task0[c] = H.color_group[c];
     L.task1[c] = H.color_group[c + 1];
@@ -363,18 +363,25 @@ iccg_status iccg_setup(iccg_ctx **out, int32_t n, int64_t nnz, const int64_t *ro
       L.grid_c[c] = std::max(1, L.task1[c] - L.task0[c]);
     }
     gbig = std::max(gbig, L.grid_c[c]);
-    lane_tiles = lane_tiles || (nt > 0 && L.wtile[c] == 0);
+    if (nt > 0 && nu == 0 && L.wtile[c] == 0) {
+      lane_tiles = true;
+      one_row_tiles = one_row_tiles || steps == 1;
+    }
   }
   // Lane-tile kernels take more shared memory than the others, and launches
-  // with different L1 / shared-memory splits cannot share an SM.  Colors of few
-  // rows are launch bound: one split for all launches lets each start beside the
-  // previous one (18 colors of 9,000 rows: 223 against 252 us an iteration; 8
-  // colors of 7,500: 99 against 103).  Colors of many rows need the larger L1
-  // more (2 colors of 485,000 rows: 118 against 124 us), and then several
-  // iterations per pass lose what they save (118 us with four, 117 with one).  Other layouts: default
-  // splits, four iterations (n = 4096 46 against 48.5 us, 128^3 170 against 174).
-  if (lane_tiles && n / n_c < 100000) L.carve = 60;
-  else if (lane_tiles) L.body = 1;
+  // with different L1 / shared-memory splits cannot share an SM: one split for
+  // all launches lets each start beside the previous one.  It also takes L1 from
+  // the product and the gathers, which one-row blocks of many rows need more, and
+  // with their default splits several iterations per pass lose what they save.
+  // 40 iterations, one split and four iterations a pass / default splits and one:
+  // one-row blocks, 27-point 56^3 4.5 / 4.7 ms, 62^3 7.3 / 5.1, 90^3 14.1 / 11.6;
+  // graph of degree 16, 100,000 rows 7.8 / 7.7 (FP32 6.3 / 6.6), 200,000 10.0 / 9.9
+  // (8.1 / 8.7), 300,000 12.9 / 11.6 (10.0 / 10.1), a million 26.7 / 20.6; blocks of
+  // four rows, 27-point 56^3 6.9 / 7.0, 90^3 9.9 / 10.1, 110^3 16.1 / 16.3.
+  // Other layouts: default splits, four iterations (n = 4096 46 against 48.5 us an
+  // iteration, 128^3 170 against 174).
+  if (one_row_tiles && n >= 220000) L.body = 1;
+  else if (lane_tiles) L.carve = 60;
   // one cooperative launch per sweep when every color is pair tiles (blocks
   // of one or two rows) and every CTA of that launch can be resident
   {
