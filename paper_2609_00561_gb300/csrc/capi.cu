@@ -711,13 +711,18 @@ static iccg_status ensure_hist(iccg_ctx *ctx, int32_t maxit) {
   return ICCG_OK;
 }
 
+// init, the first iterations one a pass, the others several a pass (when the
+// layout has them so), final
 static iccg_status build_graph(iccg_ctx *ctx) {
   cudaGraph_t g = nullptr;
   CK(cudaGraphCreate(&g, 0), "graph");
   ctx->graph = g;
-  cudaGraphConditionalHandle h;
-  CK(cudaGraphConditionalHandleCreate(&h, g, 0, cudaGraphCondAssignDefault), "graph cond");
-  ctx->cond_handle = (unsigned long long)h;
+  const int U = solve_body_iterations(ctx->plan), nloop = U > 1 ? 2 : 1;
+  const int iters[2] = {1, U};
+  cudaGraphConditionalHandle h[2];
+  for (int k = 0; k < nloop; ++k) CK(cudaGraphConditionalHandleCreate(&h[k], g, 0, cudaGraphCondAssignDefault), "graph cond");
+  ctx->cond_handle = (unsigned long long)h[0];
+  ctx->cond_rest = nloop > 1 ? (unsigned long long)h[1] : 0ull;
   // capture on a private stream (the legacy default stream cannot capture);
   // the instantiated graph is launched on the context's stream
   cudaStream_t s = nullptr;
@@ -727,34 +732,35 @@ static iccg_status build_graph(iccg_ctx *ctx) {
   Lc.stream = s;
   CK(cudaStreamBeginCaptureToGraph(s, g, nullptr, nullptr, 0, cudaStreamCaptureModeThreadLocal), "capture");
   cudaError_t e = launch_solve_init(ctx->P, Lc, ctx->fp32, nullptr, nullptr);
-  cudaGraphNodeParams cp = {};
-  cudaGraphNode_t cnode = nullptr;
-  if (e == cudaSuccess) {
+  cudaGraphNodeParams cp[2] = {};
+  for (int k = 0; k < nloop && e == cudaSuccess; ++k) {
     cudaStreamCaptureStatus cst;
     const cudaGraphNode_t *deps = nullptr;
     size_t ndeps = 0;
+    cudaGraphNode_t cnode = nullptr;
     e = cudaStreamGetCaptureInfo(s, &cst, nullptr, nullptr, &deps, nullptr, &ndeps);
     if (e == cudaSuccess) {
-      cp.type = cudaGraphNodeTypeConditional;
-      cp.conditional.handle = h;
-      cp.conditional.type = cudaGraphCondTypeWhile;
-      cp.conditional.size = 1;
-      e = cudaGraphAddNode(&cnode, g, deps, nullptr, ndeps, &cp);
+      cp[k].type = cudaGraphNodeTypeConditional;
+      cp[k].conditional.handle = h[k];
+      cp[k].conditional.type = cudaGraphCondTypeWhile;
+      cp[k].conditional.size = 1;
+      e = cudaGraphAddNode(&cnode, g, deps, nullptr, ndeps, &cp[k]);
     }
     if (e == cudaSuccess) e = cudaStreamUpdateCaptureDependencies(s, &cnode, nullptr, 1, cudaStreamSetCaptureDependencies);
-    if (e == cudaSuccess) e = launch_solve_final(ctx->P, Lc);
   }
+  if (e == cudaSuccess) e = launch_solve_final(ctx->P, Lc);
   cudaGraph_t g2 = nullptr;
   cudaError_t e2 = cudaStreamEndCapture(s, &g2);
   if (e != cudaSuccess) return cuda_fail(ctx, e, "capture init");
   if (e2 != cudaSuccess) return cuda_fail(ctx, e2, "end capture");
-  cudaGraph_t body = cp.conditional.phGraph_out[0];
-  CK(cudaStreamBeginCaptureToGraph(s, body, nullptr, nullptr, 0, cudaStreamCaptureModeThreadLocal), "capture body");
-  for (int k = solve_body_iterations(Lc); k > 0 && e == cudaSuccess; --k)
-    e = launch_solve_body(ctx->P, Lc, ctx->fp32, nullptr, nullptr);
-  e2 = cudaStreamEndCapture(s, &body);
-  if (e != cudaSuccess) return cuda_fail(ctx, e, "capture body");
-  if (e2 != cudaSuccess) return cuda_fail(ctx, e2, "end capture body");
+  for (int k = 0; k < nloop; ++k) {
+    cudaGraph_t body = cp[k].conditional.phGraph_out[0];
+    CK(cudaStreamBeginCaptureToGraph(s, body, nullptr, nullptr, 0, cudaStreamCaptureModeThreadLocal), "capture body");
+    for (int i = 0; i < iters[k] && e == cudaSuccess; ++i) e = launch_solve_body(ctx->P, Lc, ctx->fp32, nullptr, nullptr);
+    e2 = cudaStreamEndCapture(s, &body);
+    if (e != cudaSuccess) return cuda_fail(ctx, e, "capture body");
+    if (e2 != cudaSuccess) return cuda_fail(ctx, e2, "end capture body");
+  }
   CK(cudaGraphInstantiate(&ctx->gexec, g, 0), "instantiate");
   return ICCG_OK;
 }
@@ -825,6 +831,7 @@ static iccg_status solve_impl(iccg_ctx *ctx, const double *b, double *x, double 
   sh->maxit = maxit;
   sh->use_cond = use_graph ? 1 : 0;
   sh->cond_handle = ctx->cond_handle;
+  sh->cond_rest = ctx->cond_rest;
   sh->status = ICCG_NOT_CONVERGED;
   CK(cudaMemcpyAsync(ctx->P.sc, sh, sizeof(Scalars), cudaMemcpyHostToDevice, s), "scalars");
   if (persistent) {

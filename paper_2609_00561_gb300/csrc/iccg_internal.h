@@ -169,6 +169,7 @@ struct __align__(16) Scalars {
   uint32_t ticket;       // arrival counter for "last CTA reduces" epilogues
   int32_t use_cond;      // 1 when a graph conditional handle is live
   unsigned long long cond_handle;
+  unsigned long long cond_rest;     // the loop of the later iterations (0: none)
 };
 
 // Everything a kernel needs; passed by value.
@@ -389,10 +390,15 @@ bool fac_unit_color(const Plan &L, int c);                   // color c's IC(0) 
 cudaError_t launch_factor(const Params &P, const Plan &L, int nL);
 cudaError_t launch_solve_init(const Params &P, const Plan &L, bool fp32, PhaseHook h, void *u);
 cudaError_t launch_solve_body(const Params &P, const Plan &L, bool fp32, PhaseHook h, void *u);
-// Iterations per pass of the graph's WHILE loop: the way from a pass's last
-// kernel to the next pass's first costs 3 to 4 us more than a launch, so up to
-// Plan::body iterations share one, within 160 launches (graph instantiation);
-// the launches after the last iteration return at once (Scalars::skip, done)
+// Iterations per pass of the graph's loop: the way from a pass's last kernel to
+// the next pass's first costs 3 to 4 us more than a launch, so up to Plan::body
+// iterations share one, within 160 launches (graph instantiation).  The launches
+// after the last iteration change nothing and do no work (Scalars::skip, done),
+// but each takes its 1 to 2 us: the first kFirstIterations go one a pass, so that
+// a short solve has none of them (one iteration, FP64: 128^3 CPM 631 us with all
+// iterations four a pass, so 450; 99x90x85 in blocks of 32 827 and 516; five: 1312
+// and 1143, 1611 and 1350).
+constexpr int kFirstIterations = 16;
 int solve_body_iterations(const Plan &L);
 // the SpMV phase of a PCG iteration: p = z + beta p, then q = A p and <p,q>
 cudaError_t launch_spmv_phase(const Params &P, const Plan &L, bool fp32);
@@ -434,7 +440,7 @@ struct iccg_ctx {
   cudaGraphExec_t gexec = nullptr;
   cudaGraphExec_t fexec = nullptr;      // IC(0): its launch sequence as one graph
   bool fgraph_failed = false;
-  unsigned long long cond_handle = 0;
+  unsigned long long cond_handle = 0, cond_rest = 0;
   // error record
   int64_t err_index = -1;
   std::string err_msg;

@@ -499,8 +499,11 @@ __device__ __forceinline__ void group_sweep(const Params &P, const GroupDesc &d,
 // ---------------------------------------------------------------------------
 // epilogues run by the last group of a launch
 // ---------------------------------------------------------------------------
-__device__ void set_condition(const Scalars *s, int keep_going) {
-  if (s->use_cond) cudaGraphSetConditional((cudaGraphConditionalHandle)s->cond_handle, keep_going ? 1u : 0u);
+__device__ void set_condition(const Scalars *s, bool go, int iter) {
+  if (!s->use_cond) return;
+  cudaGraphSetConditional((cudaGraphConditionalHandle)s->cond_handle,
+                          go && (s->cond_rest == 0 || iter < kFirstIterations) ? 1u : 0u);
+  if (s->cond_rest) cudaGraphSetConditional((cudaGraphConditionalHandle)s->cond_rest, go ? 1u : 0u);
 }
 
 // What finish_iteration reads, loaded while the sums are still being formed.
@@ -544,7 +547,7 @@ __device__ void finish_iteration(const Params &P, double sum, const IterScalars 
     s->rr = sum;
     s->done = done;
     if (done) s->skip = 1.0;
-    set_condition(s, !done);
+    set_condition(s, !done, k + 1);
   }
 }
 
@@ -576,7 +579,7 @@ __device__ void finish_init(const Params &P, double rz, double *red) {
     }
     s->done = done;
     s->skip = done ? 1.0 : 0.0;
-    set_condition(s, !done);
+    set_condition(s, !done, 0);
   }
 }
 
@@ -594,7 +597,18 @@ constexpr int kOneLevel = 2;
 struct SlotArgs {
   int off;      // this launch's first slot (-1: no sums wanted)
   int last;     // final launch: slots of the sweep's earlier launches
+  int iter;     // 1: a launch of an iteration, which the graph may run after the last one
 };
+
+// A backward launch's own look at the end of the solve (forward launches read it
+// with alpha).  Read before griddepcontrol.wait, where it costs nothing (after
+// it, the sweep's loads would wait for it): when a launch starts, everything up
+// to two launches before it is complete, the last iteration's end included.
+// A value set by the launch just before (a wait that ran out) may be seen or
+// not; the launch's sums are dropped then in any case (launch_epilogue).
+__device__ __forceinline__ bool sweep_ended(const Params &P, const SlotArgs &sa) {
+  return sa.iter != 0 && __ldcg(&P.sc->skip) != 0.0;
+}
 
 // End of a launch with a backward sweep: this CTA's <r,r> / <r,z> partials.  A
 // non-final launch stores them in its slot region (plain stores: the sweep's
@@ -676,14 +690,15 @@ color_kernel(Params P, int g0, int g1, GroupSmemPlan plan, int fin, SlotArgs sa)
   const GroupSmem<PT> m = group_smem<PT>(smem, plan);
   double rr_acc = 0.0, rz_acc = 0.0;
   const int g = g0 + blockIdx.x;
+  const bool end = MODE == M_BWD && sweep_ended(P, sa);
   if (g < g1) {
     const GroupDesc d = load_group(P.groups + g);
     const Sweep<PT> sw = sweep_static<PT>(P, d, MODE == M_BWD, m, tid, nthr);
     cp_wait_all();
-    __syncthreads();
+    const bool ended = __syncthreads_or(end) != 0;
     pdl_wait();
     if (MODE == M_BWD) {
-      group_sweep<PT, true, false>(P, d, sw, m, tid, nthr, 0.0, nullptr, false, true, rr_acc, rz_acc);
+      if (!ended) group_sweep<PT, true, false>(P, d, sw, m, tid, nthr, 0.0, nullptr, false, true, rr_acc, rz_acc);
     } else {
       double alpha = 0.0;
       const double *pn = P.p0;
@@ -999,7 +1014,9 @@ tile_kernel(Params P, int t0, int t1, TilePlan pl, int fin, SlotArgs sa) {
   int t = t0 + int(blockIdx.x), buf = 0;
   const int wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
   TileDesc td = load_tile(P.tiles + min(t, t1 - 1));
+  const bool end = MODE == M_BWD && sweep_ended(P, sa);
   if (t < t1) tile_stage<PT, FU, TWO>(P, td, tile_buf<PT>(smem, pl, bsize, 0), pl, threadIdx.x, blockDim.x);
+  if (MODE == M_BWD && __syncthreads_or(end)) t = t1;
   pdl_wait();
   if (t < t1) tile_stage_vec<PT, FU, UPDATE>(P, td, tile_buf<PT>(smem, pl, bsize, 0), pl, threadIdx.x, blockDim.x);
   cp_commit();
@@ -1157,7 +1174,9 @@ wtile_kernel(Params P, int t0, int t1, int cap_s, int fin, SlotArgs sa) {
   PT *wv = reinterpret_cast<PT *>(smem) + size_t(wid) * cap_s * kWarp;
   double rr_acc = 0.0, rz_acc = 0.0;
   int t = t0 + int(blockIdx.x) * nw + wid;
+  const bool end = MODE == M_BWD && sweep_ended(P, sa);
   TileDesc td = load_tile(P.tiles + min(t, t1 - 1));
+  if (MODE == M_BWD && __any_sync(0xffffffffu, end)) t = t1;
   pdl_wait();
   double alpha = 0.0;
   if (UPDATE && !load_alpha(P, alpha)) return;
@@ -1483,6 +1502,7 @@ pair_kernel(Params P, int t0, int t1, int fin, SlotArgs sa) {
   __shared__ double red[kRed];
   __shared__ int flag;
   const int lane = threadIdx.x & 31, wid = int(threadIdx.x >> 5);
+  const bool end = MODE == M_BWD && sweep_ended(P, sa);
   const int nw = int(blockDim.x >> 5), stride = int(gridDim.x) * nw;
   double rr_acc = 0.0, rz_acc = 0.0;
   int t = t0 + int(blockIdx.x) * nw + wid;
@@ -1490,6 +1510,10 @@ pair_kernel(Params P, int t0, int t1, int fin, SlotArgs sa) {
     PairStage<PT> &st = reinterpret_cast<PairStage<PT> *>(smem)[wid];
     PairPre<PT> q;
     if (t < t1) q = pair_stage<PT, MODE == M_BWD>(P, t, lane, st);
+    if (MODE == M_BWD && __any_sync(0xffffffffu, end)) {
+      cp_wait_all();
+      t = t1;
+    }
     pdl_wait();
     double alpha = 0.0;
     if (UPDATE && !load_alpha(P, alpha)) {
@@ -1507,6 +1531,7 @@ pair_kernel(Params P, int t0, int t1, int fin, SlotArgs sa) {
     // current tile runs, the first tile's before the wait
     int4 hn = make_int4(0, 0, 0, 0);
     if (t < t1) hn = pair_head(P.pairs + t);
+    if (MODE == M_BWD && __any_sync(0xffffffffu, end)) t = t1;
     pdl_wait();
     double alpha = 0.0;
     if (UPDATE && !load_alpha(P, alpha)) return;
@@ -1662,6 +1687,7 @@ unit_kernel(Params P, int u0, int u1, int T, int fin, SlotArgs sa) {
   PT *zv = reinterpret_cast<PT *>(P.z);
   const PT *dvg = invds<PT>(P);
   double rr_acc = 0.0, rz_acc = 0.0;
+  const bool end = MODE == M_BWD && sweep_ended(P, sa);
   bool waited = false, live = true;
   double alpha = 0.0;
   for (int u = u0 + int(blockIdx.x) * nw + wid; u < u1; u += int(gridDim.x) * nw) {
@@ -1689,6 +1715,7 @@ unit_kernel(Params P, int u0, int u1, int T, int fin, SlotArgs sa) {
       pdl_wait();
       waited = true;
       if (UPDATE && !(live = load_alpha(P, alpha))) break;
+      if (MODE == M_BWD && __any_sync(0xffffffffu, end)) break;
     }
     PT t = PT(0), x[kUnitChunk];
     double ri = 0.0;
@@ -2882,12 +2909,12 @@ coop_sweep_kernel(Params P, int c_lo, int fin, int rr0, int ntail) {
       P.sc->status = ICCG_ERR_TIMEOUT;
       P.sc->done = 1;
       P.sc->skip = 1.0;
-      set_condition(P.sc, 0);
+      set_condition(P.sc, false, 0);
     }
     return;
   }
   if (rr0 < 0) return;   // no sums wanted
-  launch_epilogue<true>(P, fin, SlotArgs{rr0, 0}, rr_acc, rz_acc, red, &flag);
+  launch_epilogue<true>(P, fin, SlotArgs{rr0, 0, 0}, rr_acc, rz_acc, red, &flag);
   const int G = int(gridDim.x), b = int(blockIdx.x);
   if (threadIdx.x == 0)
     for (int k = 1; k < ntail; ++k) P.slot_rr[rr0 + k * G + b] = P.slot_rz[rr0 + k * G + b] = 0.0;
@@ -3028,7 +3055,7 @@ cudaError_t launch_unit(const Params &P, const Plan &L, int c, int mode, bool up
 // <r,z> are wanted.
 template <typename PT>
 cudaError_t launch_fwd(const Params &P, const Plan &L, int c, bool update, bool fused, bool sums, int fin) {
-  const SlotArgs sa{sums ? L.off[c] : -1, 0};   // a final fused launch (one color) has no earlier slots
+  const SlotArgs sa{sums ? L.off[c] : -1, 0, update};   // a final fused launch (one color) has no earlier slots
   const int mode = fused ? M_FUSED : M_FWD;
   if (L.unit1[c] > L.unit0[c]) return launch_unit<PT>(P, L, c, mode, update, fin, sa);
   if (L.tile1[c] > L.tile0[c] && L.wtile[c] == 2) return launch_pair<PT>(P, L, c, mode, update, fin, sa);
@@ -3047,9 +3074,9 @@ cudaError_t launch_fwd(const Params &P, const Plan &L, int c, bool update, bool 
 }
 
 template <typename PT>
-cudaError_t launch_bwd(const Params &P, const Plan &L, int c, bool sums, int fin) {
+cudaError_t launch_bwd(const Params &P, const Plan &L, int c, bool update, bool sums, int fin) {
   const GroupSmemPlan pl = plan_of<PT>(P, false, true);
-  const SlotArgs sa{sums ? L.off[c] : -1, L.off[c]};
+  const SlotArgs sa{sums ? L.off[c] : -1, L.off[c], update};
   if (L.unit1[c] > L.unit0[c]) return launch_unit<PT>(P, L, c, M_BWD, false, fin, sa);
   if (L.tile1[c] > L.tile0[c] && L.wtile[c] == 2) return launch_pair<PT>(P, L, c, M_BWD, false, fin, sa);
   if (L.tile1[c] > L.tile0[c] && L.wtile[c]) return launch_wtile<PT>(P, L, c, M_BWD, false, fin, sa);
@@ -3103,7 +3130,7 @@ cudaError_t sweep(const Params &P, const Plan &L, bool update, int fin_last, Pha
   if (h) h(u, PH_FUSED, 0);
   for (int c = ct - 1; c >= 0 && e == cudaSuccess; --c) {
     if (h) h(u, PH_BWD, 1);
-    e = launch_bwd<PT>(P, L, c, sums, c == 0 ? fin_last : FIN_NONE);
+    e = launch_bwd<PT>(P, L, c, update, sums, c == 0 ? fin_last : FIN_NONE);
     if (h) h(u, PH_BWD, 0);
   }
   return e;
