@@ -77,14 +77,26 @@ __device__ __forceinline__ bool na_last(unsigned int *ticket, unsigned int expec
   return *flag != 0;
 }
 
-// A warp takes slices of 32 rows, whose CSR entries are one range: it copies
-// their columns and values into shared memory coalesced, kNaChunk at a time, and
-// a lane then sums its own row from there, the gathers of kNaBatch entries in
-// flight (consecutive rows gather neighbouring elements of p).  The next
-// slice's row pointers and first chunk are loaded while the current slice is
-// summed.  Bound by memory traffic and, equally, by the FP64 rate: an FP64
-// instruction costs a warp the same for 1 lane as for 32, so the <p, q> sum
-// runs once per CTA over all its slices, not once per 256 rows.
+// Two forms, by the number of rows.
+//
+// More rows than kNaGrid CTAs hold: a persistent grid.  A warp takes slices of 32
+// rows, whose CSR entries are one range.  A slice of at most kNaChunk entries (8 a
+// row: 5- and 7-point) is copied into shared memory coalesced, and a lane then
+// sums its own row from there, the gathers of kNaBatch entries in flight
+// (consecutive rows gather neighbouring elements of p); the next slice's row
+// pointers and entries are loaded while the current one is summed.  A slice with
+// more entries is read a lane per row from global memory (na_row): staged in
+// chunks, only the few lanes whose rows lie in the chunk would work at a time,
+// and an FP64 instruction costs a warp the same for 1 lane as for 32.  Bound by
+// memory traffic and, equally, by the FP64 rate, which is why the <p, q> sum
+// runs once per CTA over all its slices, not once per 256 rows.  7-point 160^3
+// 130 us with a CTA per 256 rows, 87 so; 27-point 155^3 377 and 352 (in chunks
+// 877).
+//
+// Fewer rows: a CTA per 256 rows, a lane per row, with the registers and the L1
+// that 64 warps an SM leave (latency bound; there is no next slice to load
+// meanwhile: 27-point 50^3 24 us, graph of degree 16, 100,000 rows 23 us, both
+// forms at 7-point 50^3 15 us).
 constexpr int kNaChunk = 256;
 constexpr int kNaBatch = 8;
 
@@ -105,9 +117,61 @@ __device__ __forceinline__ void na_load(NaChunk &k, const int32_t *colind, const
   }
 }
 
-__device__ __forceinline__ int na_count(int64_t b, int64_t e1) { return int(e1 - b < kNaChunk ? e1 - b : kNaChunk); }
+// <p, q> from the lanes' shares: over the CTA, groups of CTAs, the groups
+__device__ __forceinline__ void na_finish(double acc, double *red, int *flag, NaScratch *s, double *pq) {
+  const double cta = na_cta_sum(acc, red);
+  const int g = blockIdx.x / kNaGroup;
+  const int g0 = g * kNaGroup;
+  const int gs = min(kNaGroup, int(gridDim.x) - g0);
+  if (threadIdx.x == 0) s->part[blockIdx.x] = cta;
+  if (!na_last(&s->gticket[g], unsigned(gs), flag)) return;
+  const double gv = na_cta_sum(threadIdx.x < gs ? __ldcg(&s->part[g0 + threadIdx.x]) : 0.0, red);
+  if (threadIdx.x == 0) s->gsum[g] = gv;
+  const unsigned ng = (gridDim.x + kNaGroup - 1) / kNaGroup;
+  if (!na_last(&s->ticket, ng, flag)) return;
+  double t = 0.0;
+  for (unsigned k = threadIdx.x; k < ng; k += blockDim.x) t += __ldcg(&s->gsum[k]);
+  const double total = na_cta_sum(t, red);
+  if (threadIdx.x == 0) *pq = total;
+}
 
-__global__ void __launch_bounds__(kNaRowsPerCta)
+// A lane's row [b, e): the gathers of kNaWalk entries in flight while the next
+// ones' columns and values are loaded
+constexpr int kNaWalk = 4;
+__device__ __forceinline__ double na_row(const int32_t *colind, const double *val, const double *p, int64_t b,
+                                         int64_t e) {
+  colind += b;
+  val += b;
+  const int len = int(e - b);
+  double sum = 0.0;
+  int32_t c[kNaWalk];
+  double v[kNaWalk];
+#pragma unroll
+  for (int u = 0; u < kNaWalk; ++u) {
+    c[u] = u < len ? __ldg(colind + u) : 0;
+    v[u] = u < len ? __ldg(val + u) : 0.0;
+  }
+  for (int k0 = 0; k0 < len; k0 += kNaWalk) {
+    double x[kNaWalk], w[kNaWalk];
+#pragma unroll
+    for (int u = 0; u < kNaWalk; ++u) {
+      x[u] = k0 + u < len ? __ldg(p + c[u]) : 0.0;
+      w[u] = v[u];
+    }
+    const int n0 = k0 + kNaWalk;
+#pragma unroll
+    for (int u = 0; u < kNaWalk; ++u) {
+      c[u] = n0 + u < len ? __ldg(colind + n0 + u) : 0;
+      v[u] = n0 + u < len ? __ldg(val + n0 + u) : 0.0;
+    }
+#pragma unroll
+    for (int u = 0; u < kNaWalk; ++u)
+      if (k0 + u < len) sum += w[u] * x[u];
+  }
+  return sum;
+}
+
+__global__ void __launch_bounds__(kNaRowsPerCta, 4)
 spmv_dot_noalloc_kernel(int n, const int64_t *__restrict__ rowptr, const int32_t *__restrict__ colind,
                         const double *__restrict__ val, const double *__restrict__ p, double *__restrict__ q,
                         double *__restrict__ pq, NaScratch *s) {
@@ -122,37 +186,39 @@ spmv_dot_noalloc_kernel(int n, const int64_t *__restrict__ rowptr, const int32_t
   const int stride = int(gridDim.x) * kNaRowsPerCta;
   int i = blockIdx.x * kNaRowsPerCta + threadIdx.x;
   int64_t rs = 0, re = 0;
-  NaChunk nx;
   if (i - lane < n) {
     rs = rowptr[min(i, n)];
     re = rowptr[min(i + 1, n)];
+  }
+  NaChunk nx;
+  {
     const int64_t e0 = __shfl_sync(0xffffffffu, rs, 0), e1 = __shfl_sync(0xffffffffu, re, 31);
-    na_load(nx, colind, val, e0, na_count(e0, e1), lane);
+    na_load(nx, colind, val, e0, e1 - e0 <= kNaChunk ? int(e1 - e0) : 0, lane);
   }
   while (i - lane < n) {
     const int in = i + stride;   // at most 2 * ICCG_NOALLOC_MAX_ROWS
     const bool more = in - lane < n;
     const int64_t rsn = more ? rowptr[min(in, n)] : 0, ren = more ? rowptr[min(in + 1, n)] : 0;
     const int64_t e0 = __shfl_sync(0xffffffffu, rs, 0), e1 = __shfl_sync(0xffffffffu, re, 31);
+    const bool staged = e1 - e0 <= kNaChunk;
     const double pi = i < n ? p[i] : 0.0;
     double sum = 0.0;
-    for (int64_t b = e0;; b += kNaChunk) {
-      const int cnt = na_count(b, e1);
-      if (b > e0) na_load(nx, colind, val, b, cnt, lane);
-      __syncwarp();   // every lane is done with the previous chunk
+    if (staged) {
+      __syncwarp();   // every lane is done with the previous slice
 #pragma unroll
       for (int u = 0; u < kNaChunk / 32; ++u) {
         sc[u * 32 + lane] = nx.c[u];
         sv[u * 32 + lane] = nx.v[u];
       }
       __syncwarp();
-      if (b + kNaChunk >= e1 && more) {
-        const int64_t f0 = __shfl_sync(0xffffffffu, rsn, 0), f1 = __shfl_sync(0xffffffffu, ren, 31);
-        na_load(nx, colind, val, f0, na_count(f0, f1), lane);
-      }
-      const int lo = int(rs > b ? (rs - b < cnt ? rs - b : cnt) : 0);
-      const int hi = int(re > b ? (re - b < cnt ? re - b : cnt) : 0);
-      for (int k0 = lo; k0 < hi; k0 += kNaBatch) {
+    }
+    // (the walk before the next slice's loads: their registers in turn)
+    if (!staged) sum = na_row(colind, val, p, rs, re);
+    const int64_t f0 = __shfl_sync(0xffffffffu, rsn, 0), f1 = __shfl_sync(0xffffffffu, ren, 31);
+    na_load(nx, colind, val, f0, f1 - f0 <= kNaChunk ? int(f1 - f0) : 0, lane);
+    if (staged) {
+      const int hi = int(re - e0);
+      for (int k0 = int(rs - e0); k0 < hi; k0 += kNaBatch) {
         double x[kNaBatch];
 #pragma unroll
         for (int u = 0; u < kNaBatch; ++u) x[u] = k0 + u < hi ? p[sc[k0 + u]] : 0.0;
@@ -160,7 +226,6 @@ spmv_dot_noalloc_kernel(int n, const int64_t *__restrict__ rowptr, const int32_t
         for (int u = 0; u < kNaBatch; ++u)
           if (k0 + u < hi) sum += sv[k0 + u] * x[u];
       }
-      if (b + kNaChunk >= e1) break;
     }
     if (i < n) {
       q[i] = sum;
@@ -170,20 +235,25 @@ spmv_dot_noalloc_kernel(int n, const int64_t *__restrict__ rowptr, const int32_t
     re = ren;
     i = in;
   }
-  const double cta = na_cta_sum(acc, red);
-  const int g = blockIdx.x / kNaGroup;
-  const int g0 = g * kNaGroup;
-  const int gs = min(kNaGroup, int(gridDim.x) - g0);
-  if (threadIdx.x == 0) s->part[blockIdx.x] = cta;
-  if (!na_last(&s->gticket[g], unsigned(gs), &flag)) return;
-  const double gv = na_cta_sum(threadIdx.x < gs ? __ldcg(&s->part[g0 + threadIdx.x]) : 0.0, red);
-  if (threadIdx.x == 0) s->gsum[g] = gv;
-  const unsigned ng = (gridDim.x + kNaGroup - 1) / kNaGroup;
-  if (!na_last(&s->ticket, ng, &flag)) return;
-  double t = 0.0;
-  for (unsigned k = threadIdx.x; k < ng; k += blockDim.x) t += __ldcg(&s->gsum[k]);
-  const double total = na_cta_sum(t, red);
-  if (threadIdx.x == 0) *pq = total;
+  na_finish(acc, red, &flag, s, pq);
+}
+
+// a CTA per 256 rows
+__global__ void __launch_bounds__(kNaRowsPerCta)
+spmv_dot_noalloc_small(int n, const int64_t *__restrict__ rowptr, const int32_t *__restrict__ colind,
+                       const double *__restrict__ val, const double *__restrict__ p, double *__restrict__ q,
+                       double *__restrict__ pq, NaScratch *s) {
+  __shared__ double red[kNaWarps];
+  __shared__ int flag;
+  const int i = blockIdx.x * kNaRowsPerCta + threadIdx.x;
+  double acc = 0.0;
+  if (i < n) {
+    double sum = 0.0;
+    for (int64_t e = rowptr[i]; e < rowptr[i + 1]; ++e) sum += val[e] * p[colind[e]];
+    q[i] = sum;
+    acc = p[i] * sum;
+  }
+  na_finish(acc, red, &flag, s, pq);
 }
 
 std::mutex g_na_mutex;
@@ -215,7 +285,7 @@ extern "C" iccg_status iccg_spmv_dot_noalloc(int32_t n, const int64_t *rowptr, c
     s = g_na_ptr[dev];
   }
   if (n == 0) return cudaMemsetAsync(pq, 0, sizeof(double), st) == cudaSuccess ? ICCG_OK : ICCG_ERR_CUDA;
-  const int grid = std::min((n + kNaRowsPerCta - 1) / kNaRowsPerCta, kNaGrid);
+  const int ctas = (n + kNaRowsPerCta - 1) / kNaRowsPerCta;
   // the arrival counters must start at zero; the previous call left them at
   // their final counts
   // (one memset over both, adjacent: a second one cost 2 us per call)
@@ -223,10 +293,11 @@ extern "C" iccg_status iccg_spmv_dot_noalloc(int32_t n, const int64_t *rowptr, c
   // the launch's own status (cudaGetLastError would also report, and clear,
   // an error that earlier unrelated work of the caller left pending)
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(unsigned(grid));
+  cfg.gridDim = dim3(unsigned(std::min(ctas, kNaGrid)));
   cfg.blockDim = dim3(unsigned(kNaRowsPerCta));
   cfg.stream = st;
-  return cudaLaunchKernelEx(&cfg, spmv_dot_noalloc_kernel, n, rowptr, colind, val, p, q, pq, s) == cudaSuccess
+  return cudaLaunchKernelEx(&cfg, ctas <= kNaGrid ? spmv_dot_noalloc_small : spmv_dot_noalloc_kernel, n, rowptr, colind,
+                            val, p, q, pq, s) == cudaSuccess
              ? ICCG_OK
              : ICCG_ERR_CUDA;
 }
