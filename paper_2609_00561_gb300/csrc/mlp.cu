@@ -279,6 +279,17 @@ cudaError_t launch_pdl(void (*kernel)(KArgs...), int grid, int threads, size_t s
 // (gradient and Adam) took 73 us with a launch per layer.
 bool mlp_small(int nf, int h, int c) { return mlp_fused_floats(nf, h, c) * 4 <= 48 * 1024; }
 
+// The forward pass alone is fused for small batches only: its CTAs each stage the
+// weights for one sample or a few, one barrier-separated layer after another,
+// while the launches per layer have a thread per output.  us a call, per layer /
+// fused: 20-64-64-6 16.6 / 14.3 at batch 1216 (29 MB of weights staged), 16.6 / 17.3
+// at 2000 (47 MB); 20-95-95-6 18.7 / 14.9 at 608 (28 MB), 18.7 / 24.6 at 1000 (46
+// MB); 20-8-8-3 12.5 / 9.3 at 5000, 12.5 / 14.5 at 10000.  (The gradient's fused
+// kernel saves five launches and stays ahead at every batch up to 1,000,000.)
+bool mlp_forward_fused(int nf, int h, int c, int batch) {
+  return mlp_small(nf, h, c) && batch <= 5000 && mlp_fused_floats(nf, h, c) * 4 * batch <= 30000000;
+}
+
 template <bool GRAD>
 cudaError_t launch_fused(const MlpFused &a, cudaStream_t s) {
   const int threads = std::min(256, std::max(64, (a.h + 31) / 32 * 32));
@@ -313,7 +324,7 @@ iccg_status iccg_mlp_forward(const float *params, int32_t nf, int32_t hidden, in
                              int32_t batch, float *out, float *act, iccg_stream_t stream) {
   if (!params || !X || !out || !shape_ok(nf, hidden, ncls, batch)) return ICCG_ERR_ARG;
   cudaStream_t s = static_cast<cudaStream_t>(stream);
-  if (mlp_small(nf, hidden, ncls)) {
+  if (mlp_forward_fused(nf, hidden, ncls, batch)) {
     MlpFused a{};
     a.P = params; a.X = X; a.nf = nf; a.h = hidden; a.c = ncls; a.batch = batch; a.z = out;
     a.h1 = act;
