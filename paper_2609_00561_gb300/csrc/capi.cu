@@ -632,7 +632,7 @@ iccg_status iccg_setup(iccg_ctx **out, int32_t n, int64_t nnz, const int64_t *ro
   CK(dev_alloc(ctx, &P.part_a, size_t(P.npart_a)), "alloc reductions");
   CK(dev_alloc(ctx, &P.init_bb, size_t(P.nbb)), "alloc reductions");
   CK(dev_alloc(ctx, &P.sc, 1), "alloc scalars");
-  CK(dev_alloc(ctx, &P.err_row, 1), "alloc scalars");
+  CK(dev_alloc(ctx, &P.err_row, 2), "alloc scalars");
   CK(cudaMallocHost(&ctx->sc_host, sizeof(Scalars)), "pinned");
   std::memset(ctx->sc_host, 0, sizeof(Scalars));
   CK(cudaStreamSynchronize(ctx->stream), "setup sync");
@@ -657,7 +657,7 @@ iccg_status iccg_factor(iccg_ctx *ctx) {
     if (e == cudaSuccess) e = cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal);
     if (e == cudaSuccess) {
       Lc.stream = cs;
-      cudaError_t e1 = cudaMemsetAsync(ctx->P.err_row, 0xff, sizeof(unsigned long long), cs);
+      cudaError_t e1 = cudaMemsetAsync(ctx->P.err_row, 0xff, 2 * sizeof(unsigned long long), cs);
       if (e1 == cudaSuccess) e1 = launch_factor(ctx->P, Lc, int(ctx->H.nL));
       e = cudaStreamEndCapture(cs, &fg);
       if (e == cudaSuccess) e = e1;
@@ -676,14 +676,19 @@ iccg_status iccg_factor(iccg_ctx *ctx) {
   if (ctx->fexec) {
     CK(cudaGraphLaunch(ctx->fexec, ctx->stream), "factor graph launch");
   } else {
-    CK(cudaMemsetAsync(ctx->P.err_row, 0xff, sizeof(unsigned long long), ctx->stream), "factor");
+    CK(cudaMemsetAsync(ctx->P.err_row, 0xff, 2 * sizeof(unsigned long long), ctx->stream), "factor");
     CK(launch_factor(ctx->P, Lc, int(ctx->H.nL)), "factor launch");
   }
-  unsigned long long row = 0;
-  CK(cudaMemcpyAsync(&row, ctx->P.err_row, sizeof(row), cudaMemcpyDeviceToHost, ctx->stream), "factor");
+  unsigned long long row[2] = {0, 0};
+  CK(cudaMemcpyAsync(row, ctx->P.err_row, sizeof(row), cudaMemcpyDeviceToHost, ctx->stream), "factor");
   CK(cudaStreamSynchronize(ctx->stream), "factor sync");
-  if (row != ~0ULL) {
-    ctx->err_index = ctx->H.perm[size_t(row)];
+  if (row[1] != ~0ULL) {
+    ctx->err_index = ctx->H.perm[size_t(row[1])];
+    ctx->err_msg = "a row's wait for its block's earlier rows gave up (iccg_set_wait_limit)";
+    return ICCG_ERR_TIMEOUT;
+  }
+  if (row[0] != ~0ULL) {
+    ctx->err_index = ctx->H.perm[size_t(row[0])];
     ctx->err_msg = "IC(0) pivot not positive";
     return ICCG_ERR_BREAKDOWN;
   }
@@ -1104,7 +1109,10 @@ iccg_status iccg_set_wait_limit(iccg_ctx *ctx, uint64_t wait_ns) {
   if (!ctx) return ICCG_ERR_ARG;
   DeviceGuard guard(ctx->device);
   ctx->P.wait_ns = wait_ns ? wait_ns : kDefaultWaitNs;
-  destroy_graph(ctx);   // the captured launches hold the old limit
+  // the captured launches hold the old limit
+  destroy_graph(ctx);
+  if (ctx->fexec) cudaGraphExecDestroy(ctx->fexec);
+  ctx->fexec = nullptr;
   return ICCG_OK;
 }
 

@@ -234,14 +234,14 @@ struct Params {
   // persistent solve: first group of each color [n_c + 1], grid barrier
   const int32_t *color_group;
   GridBar *bar;
-  unsigned long long wait_ns;   // bounded grid-barrier wait (ns)
+  unsigned long long wait_ns;   // bounded wait of a grid barrier or of an IC(0) row for its block's rows (ns)
   // optional phase trace of the persistent solve: (ns << 4 | phase) per
   // barrier, written by CTA 0 (null: off); trace_len receives the count
   unsigned long long *trace;
   int32_t *trace_len;
   int32_t trace_cap;
   double *hist;
-  unsigned long long *err_row;  // IC(0) breakdown row (new numbering), ~0 = none
+  unsigned long long *err_row;  // [2] IC(0) breakdown row, row whose wait gave up (new numbering), ~0 = none
   const int32_t *fac_rows;      // IC(0) rows of the lane-tile colors, level by level
   const int4 *fac_rec;          // per fac_rows entry: row, first L entry, first pair, entries | pairs << 8
   const int32_t *fp_ptr, *fp_b;  // IC(0) update pairs (null: not built)

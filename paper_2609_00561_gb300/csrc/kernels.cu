@@ -73,6 +73,12 @@ __device__ __forceinline__ void pdl_wait() {
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
 
+__device__ __forceinline__ unsigned long long global_ns() {
+  unsigned long long t;
+  asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
+  return t;
+}
+
 __device__ __forceinline__ void cp_async16(void *smem, const void *gmem) {
   const unsigned s = static_cast<unsigned>(__cvta_generic_to_shared(smem));
   asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(s), "l"(gmem) : "memory");
@@ -2144,7 +2150,8 @@ __global__ void __launch_bounds__(kFacWarps * kWarp) factor_warp_kernel(Params P
 // the rows in turn (first rows of all blocks, second rows, ...), a warp per
 // row as above, and a finished row is announced through a flag in shared
 // memory, where its entries and 1/L_ii also stay for the rows that
-// follow.  A warp loads its next row's indices and its entries of other
+// follow.  A wait that lasts longer than P.wait_ns gives up: the CTA ends, and
+// the host reports ICCG_ERR_TIMEOUT (err_row[1]), not a pivot.  A warp loads its next row's indices and its entries of other
 // colors while the others work.
 //
 // Why: with a launch per level every level of a block cost a launch boundary
@@ -2155,7 +2162,7 @@ __global__ void __launch_bounds__(kFacWarps * kWarp) factor_warp_kernel(Params P
 // tree for the pivot's sum took 1.15 ms, but moved the factor's last bit; ill-
 // conditioned solves then differ by 1e-9.)
 constexpr int kFacUnitWarps = 4;
-constexpr int kFacSpin = 1 << 22;   // polls of a row's flags before giving up
+constexpr int kFacSpin = 1 << 22;   // polls of a row's flags before giving up, whatever the clock says
 
 inline int fac_unit_bytes(int cap) { return kFacUnitWarps * kFacWarpBytes + cap * 8; }
 
@@ -2163,6 +2170,7 @@ __global__ void __launch_bounds__(kFacUnitWarps * kWarp) factor_unit_kernel(Para
   extern __shared__ __align__(16) unsigned char fsm[];
   __shared__ double ivs[kWarp], ds[kWarp];
   __shared__ volatile int ready[kWarp];
+  __shared__ volatile int gave_up;
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   double *pv = reinterpret_cast<double *>(fsm + size_t(w) * kFacWarpBytes);
   uint8_t *ps = reinterpret_cast<uint8_t *>(pv + kFacPairs);
@@ -2171,6 +2179,7 @@ __global__ void __launch_bounds__(kFacUnitWarps * kWarp) factor_unit_kernel(Para
   const int row0 = d.row0, row1 = d.row0 + d.nrows;
   const int l0 = __ldg(P.lrp + row0), l1 = __ldg(P.lrp + row1);
   if (threadIdx.x < kWarp) ready[threadIdx.x] = 0;
+  if (threadIdx.x == 0) gave_up = 0;
   __syncthreads();
   bool waited = false;
   for (int t = w; t < S * d.nblk; t += kFacUnitWarps) {
@@ -2204,11 +2213,20 @@ __global__ void __launch_bounds__(kFacUnitWarps * kWarp) factor_unit_kernel(Para
       const int q = u * kWarp + lane;
       v[u] = q < np && (fb[u] < l0 || fb[u] >= l1) ? __ldcg(P.lval + fb[u]) : 0.0;
     }
-    for (int spin = 0; !__all_sync(0xffffffffu, !in || ready[col - row0] != 0); ++spin)
-      if (spin > kFacSpin) {
-        if (lane == 0) atomicMin(P.err_row, (unsigned long long)i);
-        break;
-      }
+    // (the clock is read at the first poll and every 32 polls)
+    bool ok = true;
+    unsigned long long t0 = 0;
+    for (int spin = 0; ok && !__all_sync(0xffffffffu, !in || ready[col - row0] != 0); ++spin) {
+      if ((spin & 31) != 0) continue;
+      const unsigned long long now = global_ns();
+      if (spin == 0) t0 = now;
+      ok = !__any_sync(0xffffffffu, now - t0 > P.wait_ns || spin > kFacSpin || gave_up != 0);
+    }
+    if (!ok) {
+      gave_up = 1;
+      if (lane == 0) atomicMin(P.err_row + 1, (unsigned long long)i);
+      break;
+    }
     __threadfence_block();
     if (in) iv = ivs[col - row0];
 #pragma unroll
@@ -2240,7 +2258,7 @@ __global__ void __launch_bounds__(kFacUnitWarps * kWarp) factor_unit_kernel(Para
   }
   if (!waited) pdl_wait();
   __syncthreads();
-  if (threadIdx.x < d.nrows) {
+  if (gave_up == 0 && threadIdx.x < d.nrows) {
     P.invd[row0 + threadIdx.x] = ivs[threadIdx.x];
     P.ldiag[row0 + threadIdx.x] = ds[threadIdx.x];
   }
@@ -2514,12 +2532,6 @@ __device__ __forceinline__ unsigned ld_acquire_u32(const unsigned *p) {
   unsigned v;
   asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
   return v;
-}
-
-__device__ __forceinline__ unsigned long long global_ns() {
-  unsigned long long t;
-  asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
-  return t;
 }
 
 // Sense-reversing grid barrier with a bounded wait.  Returns false (for the
