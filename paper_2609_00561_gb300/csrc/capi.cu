@@ -302,6 +302,7 @@ iccg_status iccg_setup(iccg_ctx **out, int32_t n, int64_t nnz, const int64_t *ro
   L.Wu = 8;
   int32_t gbig = 1;
   bool lane_tiles = false, one_row_tiles = false;   // colors run one CTA per lane tile
+  bool groups = false;                              // colors run one CTA per group
   for (int c = 0; c < n_c; ++c) {
     L.task0[c] = H.color_group[c];
     L.task1[c] = H.color_group[c + 1];
@@ -363,6 +364,7 @@ iccg_status iccg_setup(iccg_ctx **out, int32_t n, int64_t nnz, const int64_t *ro
       L.grid_c[c] = std::max(1, L.task1[c] - L.task0[c]);
     }
     gbig = std::max(gbig, L.grid_c[c]);
+    groups = groups || (nt == 0 && nu == 0);
     if (nt > 0 && nu == 0 && L.wtile[c] == 0) {
       lane_tiles = true;
       one_row_tiles = one_row_tiles || steps == 1;
@@ -382,6 +384,10 @@ iccg_status iccg_setup(iccg_ctx **out, int32_t n, int64_t nnz, const int64_t *ro
   // iteration, 128^3 170 against 174).
   if (one_row_tiles && n >= 220000) L.body = 1;
   else if (lane_tiles) L.carve = 60;
+  // Groups (blocks above 32 rows): an iteration takes a millisecond and more, so
+  // that several a pass gain nothing, and backward launches after the last one
+  // would do all their work again.
+  if (groups) L.body = 1;
   // one cooperative launch per sweep when every color is pair tiles (blocks
   // of one or two rows) and every CTA of that launch can be resident
   {

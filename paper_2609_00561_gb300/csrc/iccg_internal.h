@@ -393,11 +393,11 @@ cudaError_t launch_solve_body(const Params &P, const Plan &L, bool fp32, PhaseHo
 // Iterations per pass of the graph's loop: the way from a pass's last kernel to
 // the next pass's first costs 3 to 4 us more than a launch, so up to Plan::body
 // iterations share one, within 160 launches (graph instantiation).  The launches
-// after the last iteration change nothing and do no work (Scalars::skip, done),
-// but each takes its 1 to 2 us: the first kFirstIterations go one a pass, so that
-// a short solve has none of them (one iteration, FP64: 128^3 CPM 631 us with all
-// iterations four a pass, so 450; 99x90x85 in blocks of 32 827 and 516; five: 1312
-// and 1143, 1611 and 1350).
+// after the last iteration change nothing; most do no work either (Scalars::skip,
+// done; sweep_ended), but each takes its 1 to 2 us: the first kFirstIterations go
+// one a pass, so that a short solve has none of them (one iteration, FP64: 128^3
+// CPM 631 us with all iterations four a pass, so 450; 99x90x85 in blocks of 32 827
+// and 500; five: 1312 and 1143, 1611 and 1290).
 constexpr int kFirstIterations = 16;
 int solve_body_iterations(const Plan &L);
 // the SpMV phase of a PCG iteration: p = z + beta p, then q = A p and <p,q>

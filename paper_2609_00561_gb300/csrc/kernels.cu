@@ -607,11 +607,16 @@ struct SlotArgs {
 };
 
 // A backward launch's own look at the end of the solve (forward launches read it
-// with alpha).  Read before griddepcontrol.wait, where it costs nothing (after
-// it, the sweep's loads would wait for it): when a launch starts, everything up
-// to two launches before it is complete, the last iteration's end included.
-// A value set by the launch just before (a wait that ran out) may be seen or
-// not; the launch's sums are dropped then in any case (launch_epilogue).
+// with alpha), in the kernels of warps on their own.  The load goes out before
+// griddepcontrol.wait and is looked at after it: loaded after the wait, the
+// sweep's loads would have to wait for it; looked at before, the wait itself
+// would, with which the next launch may start.  When a launch starts, everything
+// up to two launches before it is complete, the last iteration's end included; a
+// value set by the launch just before (a wait that ran out) may be seen or not.
+// Either way the launch's sums are dropped (launch_epilogue).  Where a CTA would
+// have to agree on it (lane tiles, groups) every launch would pay more than the
+// solve's last ones save (27-point 56^3, 40 iterations: blocks of four rows in
+// FP32 7.0 against 6.6 ms, blocks of 64 32.4 against 31.6): those run once more.
 __device__ __forceinline__ bool sweep_ended(const Params &P, const SlotArgs &sa) {
   return sa.iter != 0 && __ldcg(&P.sc->skip) != 0.0;
 }
@@ -696,15 +701,14 @@ color_kernel(Params P, int g0, int g1, GroupSmemPlan plan, int fin, SlotArgs sa)
   const GroupSmem<PT> m = group_smem<PT>(smem, plan);
   double rr_acc = 0.0, rz_acc = 0.0;
   const int g = g0 + blockIdx.x;
-  const bool end = MODE == M_BWD && sweep_ended(P, sa);
   if (g < g1) {
     const GroupDesc d = load_group(P.groups + g);
     const Sweep<PT> sw = sweep_static<PT>(P, d, MODE == M_BWD, m, tid, nthr);
     cp_wait_all();
-    const bool ended = __syncthreads_or(end) != 0;
+    __syncthreads();
     pdl_wait();
     if (MODE == M_BWD) {
-      if (!ended) group_sweep<PT, true, false>(P, d, sw, m, tid, nthr, 0.0, nullptr, false, true, rr_acc, rz_acc);
+      group_sweep<PT, true, false>(P, d, sw, m, tid, nthr, 0.0, nullptr, false, true, rr_acc, rz_acc);
     } else {
       double alpha = 0.0;
       const double *pn = P.p0;
@@ -1020,9 +1024,7 @@ tile_kernel(Params P, int t0, int t1, TilePlan pl, int fin, SlotArgs sa) {
   int t = t0 + int(blockIdx.x), buf = 0;
   const int wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
   TileDesc td = load_tile(P.tiles + min(t, t1 - 1));
-  const bool end = MODE == M_BWD && sweep_ended(P, sa);
   if (t < t1) tile_stage<PT, FU, TWO>(P, td, tile_buf<PT>(smem, pl, bsize, 0), pl, threadIdx.x, blockDim.x);
-  if (MODE == M_BWD && __syncthreads_or(end)) t = t1;
   pdl_wait();
   if (t < t1) tile_stage_vec<PT, FU, UPDATE>(P, td, tile_buf<PT>(smem, pl, bsize, 0), pl, threadIdx.x, blockDim.x);
   cp_commit();
@@ -1182,8 +1184,8 @@ wtile_kernel(Params P, int t0, int t1, int cap_s, int fin, SlotArgs sa) {
   int t = t0 + int(blockIdx.x) * nw + wid;
   const bool end = MODE == M_BWD && sweep_ended(P, sa);
   TileDesc td = load_tile(P.tiles + min(t, t1 - 1));
-  if (MODE == M_BWD && __any_sync(0xffffffffu, end)) t = t1;
   pdl_wait();
+  if (MODE == M_BWD && __any_sync(0xffffffffu, end)) t = t1;
   double alpha = 0.0;
   if (UPDATE && !load_alpha(P, alpha)) return;
   for (; t < t1; t += int(gridDim.x) * nw) {
@@ -1516,11 +1518,11 @@ pair_kernel(Params P, int t0, int t1, int fin, SlotArgs sa) {
     PairStage<PT> &st = reinterpret_cast<PairStage<PT> *>(smem)[wid];
     PairPre<PT> q;
     if (t < t1) q = pair_stage<PT, MODE == M_BWD>(P, t, lane, st);
+    pdl_wait();
     if (MODE == M_BWD && __any_sync(0xffffffffu, end)) {
       cp_wait_all();
       t = t1;
     }
-    pdl_wait();
     double alpha = 0.0;
     if (UPDATE && !load_alpha(P, alpha)) {
       cp_wait_all();
@@ -1537,8 +1539,8 @@ pair_kernel(Params P, int t0, int t1, int fin, SlotArgs sa) {
     // current tile runs, the first tile's before the wait
     int4 hn = make_int4(0, 0, 0, 0);
     if (t < t1) hn = pair_head(P.pairs + t);
-    if (MODE == M_BWD && __any_sync(0xffffffffu, end)) t = t1;
     pdl_wait();
+    if (MODE == M_BWD && __any_sync(0xffffffffu, end)) t = t1;
     double alpha = 0.0;
     if (UPDATE && !load_alpha(P, alpha)) return;
     for (; t < t1; t += stride) {
