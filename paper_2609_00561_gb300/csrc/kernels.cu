@@ -60,7 +60,8 @@ namespace {
 
 constexpr int kVecThreads = 256;
 constexpr int kChunk = 4;    // row entries processed per predicated batch
-constexpr int kRed = 6 * kMaxWarpsPerCta;   // reduction scratch of a CTA (doubles)
+constexpr int kRedWarp = 6;                        // reduction scratch of a warp (doubles)
+constexpr int kRed = kRedWarp * kMaxWarpsPerCta;   // and of a CTA
 enum StepMode { M_FWD = 0, M_BWD = 1, M_FUSED = 2 };
 
 // Programmatic dependent launch: everything before this call runs while the
@@ -133,18 +134,17 @@ __device__ __forceinline__ double warp_sum(double v) {
   return v;
 }
 
-// Sums of a and b over the CTA in a fixed order (red: 2 kMaxWarpsPerCta
-// doubles): the warps' sums one after another.  In warp 0, lane 0 returns a's
+// Sums of a and b over the CTA in a fixed order (red: 2 doubles a warp): the warps' sums one after another.  In warp 0, lane 0 returns a's
 // and lane 16 b's (both in the same instructions).
 __device__ __forceinline__ double cta_sum2(double a, double b, double *red) {
   double v = warp_sum2(a, b);
   const int w = threadIdx.x >> 5, l = threadIdx.x & 31, nw = blockDim.x >> 5;
   if (nw == 1) return v;
   __syncthreads();
-  if ((l & 15) == 0) red[(l >> 4) * kMaxWarpsPerCta + w] = v;
+  if ((l & 15) == 0) red[(l >> 4) * nw + w] = v;
   __syncthreads();
   if (w == 0) {
-    const double *p = red + (l >> 4) * kMaxWarpsPerCta;
+    const double *p = red + (l >> 4) * nw;
     v = p[0];
     for (int k = 1; k < nw; ++k) v += p[k];
   }
@@ -657,15 +657,16 @@ __device__ __forceinline__ void launch_epilogue(const Params &P, int fin, const 
       __threadfence();
     }
     if (!arrive_last(&P.sc->ticket, uint32_t(nb), flag)) return;
-    double *gs = red + 2 * kMaxWarpsPerCta;
+    const int nw = int(blockDim.x >> 5);
+    double *gs = red + 2 * nw;
     for (int g = threadIdx.x >> 5; g < ng; g += int(blockDim.x >> 5)) {
       const int k = g * kGroup + int(threadIdx.x & 31);
       v = warp_sum2(k < nb ? __ldcg(P.part0 + k) : 0.0, k < nb ? __ldcg(P.part1 + k) : 0.0);
-      if ((threadIdx.x & 15) == 0) gs[((threadIdx.x >> 4) & 1) * 2 * kMaxWarpsPerCta + g] = v;
+      if ((threadIdx.x & 15) == 0) gs[((threadIdx.x >> 4) & 1) * 2 * nw + g] = v;
     }
     __syncthreads();
     p0 = gs;
-    p1 = gs + 2 * kMaxWarpsPerCta;
+    p1 = gs + 2 * nw;
   } else {
     double gv;
     if (!group_reduce(P, v, red, flag, gv)) return;
@@ -1006,15 +1007,24 @@ __device__ __forceinline__ void tile_phase_c(const Params &P, const TileDesc &t,
   }
 }
 
+// Static shared memory of a lane-tile launch that reduces (red and flag).  CTAs of
+// one warp (ONE; one-row blocks) have only what one warp needs: with 784 bytes they
+// lost a place on an SM to it (27-point 124^3, FP32, 40 iterations 17.3 ms, so
+// 15.7).  Forward launches reduce nothing; they get the same bytes as dynamic
+// shared memory.  The grid is one CTA for every place on the SMs: with room left
+// beside a full grid the next launch's first CTAs start there, and some SMs end up
+// with more of them than others (110^3, FP64 18.7 ms; so 15.9).
+constexpr int tile_red_bytes(bool one) { return (one ? kRedWarp : kRed) * 8 + 16; }
+
 // A lane-tile launch: CTAs walk the color's tiles grid-stride; the static
 // data of the next tile is copied into the other buffer while the current one
 // is computed (the first tile's before griddepcontrol.wait); one <r,r> /
 // <r,z> reduction per CTA at the end.
-template <typename PT, int MODE, bool UPDATE>
+template <typename PT, int MODE, bool UPDATE, bool ONE>
 __global__ void __launch_bounds__(kMaxWarpsPerCta * kWarp)
 tile_kernel(Params P, int t0, int t1, TilePlan pl, int fin, SlotArgs sa) {
   extern __shared__ __align__(16) unsigned char smem[];
-  __shared__ double red[kRed];
+  __shared__ double red[ONE ? kRedWarp : kRed];
   __shared__ int flag;
   constexpr bool FU = MODE == M_BWD, TWO = MODE == M_FUSED;
   const int bsize = TWO && pl.cap_i2 > 0 ? pl.buf2 : pl.buf1;
@@ -2988,23 +2998,24 @@ TilePlan tile_plan_of(const Params &P, bool stage_ext = true) {
   return p;
 }
 
-template <typename PT>
-cudaError_t launch_tile(const Params &P, const Plan &L, int c, int mode, bool update, int fin, const SlotArgs &sa) {
+template <typename PT, bool ONE>
+cudaError_t launch_tile_w(const Params &P, const Plan &L, int c, int mode, bool update, int fin, const SlotArgs &sa) {
   const TilePlan pl = tile_plan_of<PT>(P, L.stage_ext[c] != 0);
   const int g = L.grid_c[c], t0 = L.tile0[c], t1 = L.tile1[c], th = L.Wt * kWarp;
-  // Forward launches reduce nothing and have none of the other launches' static
-  // shared memory (red and flag): it is added to theirs.  With room left on an SM
-  // the next launch's first CTAs start there beside a full grid, and as the grid
-  // is one CTA for every place, some SMs end up with more of them than others
-  // (one-row blocks, 27-point, 110^3, 40 iterations: 18.7 ms; so 15.9).
-  const int sm = tile_launch_bytes(pl, mode == M_FUSED) + (mode == M_FWD ? kRed * int(sizeof(double)) + 16 : 0);
-  if (mode == M_BWD) return launch(tile_kernel<PT, M_BWD, false>, g, th, sm, L, P, t0, t1, pl, fin, sa);
+  const int sm = tile_launch_bytes(pl, mode == M_FUSED) + (mode == M_FWD ? tile_red_bytes(ONE) : 0);
+  if (mode == M_BWD) return launch(tile_kernel<PT, M_BWD, false, ONE>, g, th, sm, L, P, t0, t1, pl, fin, sa);
   if (update) {
-    if (mode == M_FUSED) return launch(tile_kernel<PT, M_FUSED, true>, g, th, sm, L, P, t0, t1, pl, fin, sa);
-    return launch(tile_kernel<PT, M_FWD, true>, g, th, sm, L, P, t0, t1, pl, fin, sa);
+    if (mode == M_FUSED) return launch(tile_kernel<PT, M_FUSED, true, ONE>, g, th, sm, L, P, t0, t1, pl, fin, sa);
+    return launch(tile_kernel<PT, M_FWD, true, ONE>, g, th, sm, L, P, t0, t1, pl, fin, sa);
   }
-  if (mode == M_FUSED) return launch(tile_kernel<PT, M_FUSED, false>, g, th, sm, L, P, t0, t1, pl, fin, sa);
-  return launch(tile_kernel<PT, M_FWD, false>, g, th, sm, L, P, t0, t1, pl, fin, sa);
+  if (mode == M_FUSED) return launch(tile_kernel<PT, M_FUSED, false, ONE>, g, th, sm, L, P, t0, t1, pl, fin, sa);
+  return launch(tile_kernel<PT, M_FWD, false, ONE>, g, th, sm, L, P, t0, t1, pl, fin, sa);
+}
+
+template <typename PT>
+cudaError_t launch_tile(const Params &P, const Plan &L, int c, int mode, bool update, int fin, const SlotArgs &sa) {
+  return L.Wt == 1 ? launch_tile_w<PT, true>(P, L, c, mode, update, fin, sa)
+                   : launch_tile_w<PT, false>(P, L, c, mode, update, fin, sa);
 }
 
 template <typename PT>
@@ -3182,11 +3193,16 @@ cudaError_t configure_pt() {
   if (e == cudaSuccess) e = allow_smem(color_kernel<PT, M_FWD, false>);
   if (e == cudaSuccess) e = allow_smem(color_kernel<PT, M_BWD, false>);
   if (e == cudaSuccess) e = allow_smem(persistent_kernel<PT>);
-  if (e == cudaSuccess) e = allow_smem(tile_kernel<PT, M_FUSED, true>);
-  if (e == cudaSuccess) e = allow_smem(tile_kernel<PT, M_FWD, true>);
-  if (e == cudaSuccess) e = allow_smem(tile_kernel<PT, M_FUSED, false>);
-  if (e == cudaSuccess) e = allow_smem(tile_kernel<PT, M_FWD, false>);
-  if (e == cudaSuccess) e = allow_smem(tile_kernel<PT, M_BWD, false>);
+  if (e == cudaSuccess) e = allow_smem(tile_kernel<PT, M_FUSED, true, false>);
+  if (e == cudaSuccess) e = allow_smem(tile_kernel<PT, M_FUSED, true, true>);
+  if (e == cudaSuccess) e = allow_smem(tile_kernel<PT, M_FWD, true, false>);
+  if (e == cudaSuccess) e = allow_smem(tile_kernel<PT, M_FWD, true, true>);
+  if (e == cudaSuccess) e = allow_smem(tile_kernel<PT, M_FUSED, false, false>);
+  if (e == cudaSuccess) e = allow_smem(tile_kernel<PT, M_FUSED, false, true>);
+  if (e == cudaSuccess) e = allow_smem(tile_kernel<PT, M_FWD, false, false>);
+  if (e == cudaSuccess) e = allow_smem(tile_kernel<PT, M_FWD, false, true>);
+  if (e == cudaSuccess) e = allow_smem(tile_kernel<PT, M_BWD, false, false>);
+  if (e == cudaSuccess) e = allow_smem(tile_kernel<PT, M_BWD, false, true>);
   if (e == cudaSuccess) e = allow_smem(pair_kernel<PT, M_FUSED, true, true>);
   if (e == cudaSuccess) e = allow_smem(pair_kernel<PT, M_FWD, true, true>);
   if (e == cudaSuccess) e = allow_smem(pair_kernel<PT, M_FUSED, false, true>);
@@ -3213,10 +3229,10 @@ int spmv_smem_bytes(int cap) { return r16((cap + 8) * 8) + r16((cap + 8) * 4); }
 
 int tile_resident_ctas(bool fp32, int threads, int smem) {
   int nb = 0;
-  const cudaError_t e =
-      fp32 ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, tile_kernel<float, M_FUSED, true>, threads, size_t(smem))
-           : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, tile_kernel<double, M_FUSED, true>, threads, size_t(smem));
-  if (e != cudaSuccess) {
+  const auto kernel = threads == kWarp
+                          ? (fp32 ? tile_kernel<float, M_FUSED, true, true> : tile_kernel<double, M_FUSED, true, true>)
+                          : (fp32 ? tile_kernel<float, M_FUSED, true, false> : tile_kernel<double, M_FUSED, true, false>);
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, kernel, threads, size_t(smem)) != cudaSuccess) {
     cudaGetLastError();
     return 1;
   }
