@@ -1691,8 +1691,18 @@ __device__ __forceinline__ PT unit_chain(PT t, int M, uint32_t mask, uint32_t wm
 // shared memory of a warp-unit CTA, coefficients at most T terms deep
 inline int unit_smem_bytes(int T, int elem) { return kUnitWarps * (T + 1) * kWarp * elem; }
 
+// CTAs an SM that a form's registers have to leave room for: those that its loads
+// and chain need (72 to 80 registers in FP64 with 32-step chains and in the fused
+// forms, 64 otherwise; 48 or 64 in FP32).  Left to itself the compiler takes 64 for
+// the FP64 backward form of 32 steps, which has fewer loads in flight then (27-point
+// 96^3, blocks of 32 rows, one application with a product: 433 us; so 404).
+constexpr int unit_ctas(int elem, int mode, int S) {
+  if (elem == 8) return mode == M_FUSED || S == kWarp ? 3 : 4;
+  return mode == M_FUSED || (mode == M_BWD && (S == 1 || S == kWarp)) ? 4 : 5;
+}
+
 template <typename PT, int MODE, bool UPDATE, int S>
-__global__ void __launch_bounds__(kUnitWarps * kWarp)
+__global__ void __launch_bounds__(kUnitWarps * kWarp, unit_ctas(int(sizeof(PT)), MODE, S))
 unit_kernel(Params P, int u0, int u1, int T, int fin, SlotArgs sa) {
   __shared__ double red[kRed];
   extern __shared__ __align__(16) unsigned char usm[];
