@@ -398,7 +398,7 @@ cudaError_t launch_solve_body(const Params &P, const Plan &L, bool fp32, PhaseHo
 // one a pass, so that a short solve has none of them (one iteration, FP64: 128^3
 // CPM 631 us with all iterations four a pass, so 450; 99x90x85 in blocks of 32 827
 // and 500; five: 1312 and 1143, 1611 and 1290).
-constexpr int kFirstIterations = 16;
+constexpr int kFirstIterations = 8;
 int solve_body_iterations(const Plan &L);
 // the SpMV phase of a PCG iteration: p = z + beta p, then q = A p and <p,q>
 cudaError_t launch_spmv_phase(const Params &P, const Plan &L, bool fp32);
