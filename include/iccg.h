@@ -225,9 +225,11 @@ iccg_status iccg_info(const iccg_ctx *ctx, int64_t out[18]);
 /* Wall-time limit (ns) of every device-side wait of this context: the grid
  * barriers of the persistent solver and of the cooperative sweep
  * (opts.fuse_sweep; Alg. 1's colors are separated by one barrier each
- * there).  A wait that runs past it makes the kernel stop at once and
- * iccg_solve return ICCG_ERR_TIMEOUT; the context stays usable.  0 restores
- * the default (4 s).  Per-color launches have no device-side waits. */
+ * there), and in iccg_factor a row's wait for earlier rows of its block (warp
+ * units, one launch a color).  A wait that runs past it makes the kernel stop at
+ * once and iccg_solve (iccg_factor) return ICCG_ERR_TIMEOUT; the context stays
+ * usable.  0 restores the default (4 s).  The solve's per-color launches have no
+ * device-side waits. */
 iccg_status iccg_set_wait_limit(iccg_ctx *ctx, uint64_t wait_ns);
 
 iccg_status iccg_last_error(const iccg_ctx *ctx, int64_t *row_or_block, const char **msg);

@@ -12,14 +12,16 @@
 // its lanes, and every vector access of the chain is one coalesced line.
 //
 // Schedule.  The grid is split into per-system CTA ranges (assign_ctas, at
-// least one CTA each); a system's CTAs synchronise
-// only among themselves (a bounded-wait barrier per system), so systems
-// progress independently.  Per iteration and system: p update | SpMV and
-// <p,q> | x / r update | forward colors (the last color's backward sweep
-// fused) | backward colors | reduction, with a barrier after each
-// phase (2 n_c + 3).  A warp owns a whole block at a time (batch_precond):
-// everything but the in-block recurrence is done for all rows at once, the
-// recurrence itself (rows in order, Alg. 1) on shared memory only.  Reductions
+// least one CTA each); a system's CTAs synchronise only among themselves (a
+// bounded-wait barrier per system), so systems progress independently.  Per
+// iteration and system: p update | SpMV and <p,q> | x / r update | forward colors
+// (the last color's backward sweep fused) | backward colors and the sums, with a
+// barrier after each phase (2 n_c + 2 for two colors or more).  A warp owns a
+// whole block at a time (batch_precond): everything but the in-block recurrence
+// is done for all rows at once, the recurrence itself (rows in order, Alg. 1) on
+// shared memory only.  For small blocks, and for wide rows with many right-hand
+// sides, a chain owns a block instead and walks its rows, the x / r update of a
+// color in front of them (batch_precond_walk; batch_walks says when).  Reductions
 // are per right-hand side, per CTA, summed in a fixed order by every CTA of the
 // system after a barrier.
 // A right-hand side that converged (or met a non-finite value) is frozen.
@@ -35,7 +37,7 @@
 namespace iccg {
 namespace {
 
-constexpr int kBatchMaxBlock = 64;   // rows of a block (a chain's scratch in shared memory)
+constexpr int kBatchMaxBlock = 64;   // rows of a block (its row values in shared memory)
 constexpr int kBatchCap = 512;       // most entries a warp stages (6 KB)
 constexpr long long kBatchSpinLimit = 1ll << 27;
 
@@ -378,11 +380,11 @@ __device__ __forceinline__ void block_store_z(const BatchSys &S, const BatchRows
 // block's static data is staged ahead; the first block of the next color before
 // the barrier that ends the current one.
 //
-// Bound by latency: a chain that walked its block row by row paid two to three
+// Bound by latency: a chain that walks its block row by row pays two to three
 // dependent L2 loads for each of 32 rows, 60-120 us for a color phase; split
 // so, a phase costs a few such trips (8 systems of sides 16..64, 16 right-hand
-// sides, FP32: 155 ms with the walk, 85 ms so; 3 systems of sides 21..57, 4
-// right-hand sides, FP64: 102 against 19 ms).  What remains is still latency: a
+// sides, FP32, blocks of 32 rows: 143 ms with the walk, 82 ms so; 4 systems of
+// sides 16..48, 4 right-hand sides, FP64, ten iterations: 20.1 and 4.8 ms).  What remains is still latency: a
 // color of one system has fewer blocks than its CTAs have warps.
 template <typename PT>
 __device__ __forceinline__ bool batch_precond(const BatchSys &S, unsigned char *sm, const BatchSmem &m, int cap, int kp,
@@ -913,7 +915,7 @@ struct iccg_batch {
   // launch shape
   int W = 8, cps = 1, grid = 0, smem = 0, max_part_ctas = 0;
   int R = 1;             // rows per chain and pass (SpMV, p update)
-  double wexp = 4.0 / 3.0;     // CTAs per system: 1 by rows, 4/3 by rows x estimated iterations
+  bool by_work = true;         // CTAs per system by rows x estimated iterations, else by rows
   std::vector<double> work;    // rows x estimated iterations of each system
   std::vector<int32_t> cta0;
   cudaGraph_t graph = nullptr;
@@ -985,16 +987,16 @@ double system_work(const HostLayout &H) {
   return n / std::sqrt(std::pow(n, -2.0 / 3.0) + 0.2 * std::max(delta, 0.0));
 }
 
-// CTA ranges per system (>= 1 each) for a grid of G CTAs: wexp = 1 in
-// proportion to the rows, wexp = 4/3 to rows x estimated iterations (rows^(4/3)
-// without diagonal dominance); returns false when G < nsys.  8 systems of sides
-// 16..64 with shifts in [1e-4, 1e-1] need 24 to 79 iterations.
+// CTA ranges per system (>= 1 each) for a grid of G CTAs, in proportion to the
+// systems' rows or (by_work) to rows x estimated iterations; returns false when
+// G < nsys.  8 systems of sides 16..64 with shifts in [1e-4, 1e-1] need 24 to 79
+// iterations.
 bool assign_ctas(iccg_batch *b, int G) {
   if (G < b->nsys) return false;
   double tot = 0.0;
   std::vector<double> wt(b->nsys);
   for (int s = 0; s < b->nsys; ++s) {
-    wt[s] = b->wexp > 1.0 ? b->work[s] : double(b->n[s]);
+    wt[s] = b->by_work ? b->work[s] : double(b->n[s]);
     tot += wt[s];
   }
   std::vector<int32_t> c(b->nsys, 1);
@@ -1420,14 +1422,14 @@ iccg_status iccg_batch_tune(iccg_batch *b, const double *const *B, double tol, i
   const double ttol = B ? tol : 0.0;
   const int tmax = B ? maxit : 20;
   const int Ws[3] = {4, 8, 16};
-  const double Es[2] = {1.0, 4.0 / 3.0};
-  double best = 1e300, bE = b->wexp;
+  double best = 1e300;
+  bool bE = b->by_work;
   int bW = b->W, bC = b->cps;
-  for (double E : Es)
+  for (bool E : {false, true})
   for (int W : Ws) {
     const int occ = batch_occupancy(b, W, shape_walks(b, W));
     for (int cps = 1; cps <= std::min(occ, 4); cps *= 2) {
-      b->wexp = E;
+      b->by_work = E;
       if (set_shape(b, W, cps, sms) != ICCG_OK) continue;
       for (auto &x : hx) std::fill(x.begin(), x.end(), 0.0);
       // the first call captures the graph; the second is timed
@@ -1441,7 +1443,7 @@ iccg_status iccg_batch_tune(iccg_batch *b, const double *const *B, double tol, i
     }
   }
   // rows per thread at the best shape
-  b->wexp = bE;
+  b->by_work = bE;
   int bR = b->R;
   const int R0 = b->R;
   for (int R : {1, 2, 4}) {
@@ -1476,7 +1478,7 @@ iccg_status iccg_batch_info(const iccg_batch *b, int32_t out[7]) {
   out[2] = b->grid;
   out[3] = b->kp;
   out[4] = b->smax;
-  out[5] = int32_t(b->wexp * 3.0 + 0.5);   // 3 x the CTA-split exponent (3: rows, 4: rows^(4/3))
+  out[5] = b->by_work ? 4 : 3;   // the CTA split: 4 by rows x estimated iterations, 3 by rows
   out[6] = b->R;
   return ICCG_OK;
 }

@@ -318,9 +318,10 @@ iccg_status iccg_setup(iccg_ctx **out, int32_t n, int64_t nnz, const int64_t *ro
       if (td.nsteps != 2 || H.steps[size_t(td.step0) + 1].cnt != H.steps[size_t(td.step0)].cnt) pairs = false;
     }
     // automatic: colors of two-row blocks only as pair kernels, one-row blocks
-    // of narrow rows as warp tiles, one CTA per tile otherwise (on a GB300 the pair kernels measured 7% faster for
-    // ABMC with blocks of 2 rows, slower where one-row blocks share a tile
-    // with two-row ones, and no better for one-row blocks alone)
+    // of narrow rows as warp tiles, one CTA per tile otherwise (on a GB300 the
+    // pair kernels measured 7% faster for ABMC with blocks of 2 rows, slower where
+    // one-row blocks share a tile with two-row ones, and no better for one-row
+    // blocks alone)
     L.wtile[c] = 0;
     if (nt > 0 && (o.tile_mapping == ICCG_TILES_WARP || (autom && narrow && steps == 1))) L.wtile[c] = 1;
     if (nt > 0 && steps <= 2 && ((pairs && o.tile_mapping == ICCG_TILES_AUTO) || o.tile_mapping == ICCG_TILES_PAIR))

@@ -588,11 +588,6 @@ __global__ void to_i32(int64_t n, const int64_t *a, int32_t *b) {
     b[i] = int32_t(a[i]);
 }
 
-__global__ void i32_to_i64(int64_t n, const int32_t *a, int64_t *b) {
-  for (int64_t i = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; i < n; i += int64_t(gridDim.x) * blockDim.x)
-    b[i] = a[i];
-}
-
 // ---------------------------------------------------------------------------
 // Leiden block order: size descending, ties by smallest row
 // ---------------------------------------------------------------------------

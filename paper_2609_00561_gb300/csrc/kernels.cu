@@ -127,13 +127,6 @@ __device__ __forceinline__ double widen(float f) {
   return __hiloint2double(int((b & 0x80000000u) | (m ? (m >> 3) + 0x38000000u : 0u)), int(b << 29));
 }
 
-// sum over the warp, valid in lane 0
-__device__ __forceinline__ double warp_sum(double v) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-  return v;
-}
-
 // Sums of a and b over the CTA in a fixed order (red: 2 doubles a warp): the warps' sums one after another.  In warp 0, lane 0 returns a's
 // and lane 16 b's (both in the same instructions).
 __device__ __forceinline__ double cta_sum2(double a, double b, double *red) {
@@ -180,8 +173,8 @@ __device__ __forceinline__ bool arrive_last(uint32_t *ticket, uint32_t expected,
   return *flag != 0;
 }
 
-// First level: each CTA publishes (a, b), valid in lanes 0 and 16 of its first
-// warp; the last CTA of the group returns true with the group's sums there.
+// First level: each CTA publishes its two sums (v of lanes 0 and 16 of its first
+// warp); the last CTA of the group returns true with the group's in gv there.
 __device__ __forceinline__ bool group_reduce(const Params &P, double v, double *red, int *flag, double &gv) {
   const int g = blockIdx.x / kGroup;
   const int g0 = g * kGroup;
@@ -1983,7 +1976,6 @@ __device__ __forceinline__ void factor_row_merge(const Params &P, int i) {
 // compare-and-select, so no load waits on another.  The terms are
 // subtracted in ascending k, as in the general form.
 constexpr int kFacRow = 32;
-constexpr int kFacThreads = 64;    // small CTAs: a level's rows spread over many SMs' FP64 units
 
 __device__ __forceinline__ void factor_row(const Params &P, int i, int32_t *sc, double *sv) {
   const int rb = P.lrp[i], ni = P.lrp[i + 1] - rb;

@@ -1,7 +1,9 @@
 // MLP of the learned blocking: forward pass, loss gradient and Adam step as
 // plain CUDA kernels (FP32; the network has ~6k parameters and batches of a
-// few hundred matrices, so one thread per output element is the whole
-// mapping; no tensor cores).  Layout of the flat parameter array:
+// few hundred matrices: bound by launches and latency, no tensor cores).  Weights
+// that fit a CTA's shared memory: a CTA per sample through all layers (mlp_fused);
+// wider networks, and the forward pass of large batches: a launch per layer, a
+// thread per output element.  Layout of the flat parameter array:
 //   W1 [nf][h], b1 [h], W2 [h][h], b2 [h], W3 [h][c+1], b3 [c+1]
 // (c = ncls; the last output is the regression head).  Every sum runs in a
 // fixed order, so results do not depend on the launch shape.
@@ -129,7 +131,8 @@ __global__ void mlp_wgrad(MlpLayers L, int batch, int64_t np, const float *lb, f
 // step ran 8 dependent launches of 3-6 us each on a few thousand threads
 // reading their weights from L2; here the layers follow one another inside a
 // CTA behind barriers.  What an earlier kernel of the step writes is read from
-// L2 (this kernel may have started before that one ended).  Every sum keeps its order (results are the same bits).
+// L2 (this kernel may have started before that one ended).  Every sum has the
+// order of the launches per layer (the same bits).
 struct MlpFused {
   const float *P, *X;
   int nf, h, c, batch;

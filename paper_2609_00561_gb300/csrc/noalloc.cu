@@ -31,18 +31,19 @@ namespace {
 
 constexpr int kNaWarps = 8;                       // warps per CTA
 constexpr int kNaRowsPerCta = kNaWarps * 32;      // one row per lane
-constexpr int kNaMaxCtas = ICCG_NOALLOC_MAX_ROWS / kNaRowsPerCta;
+constexpr int kNaGrid = 4 * 152;                  // CTAs of a launch at most: those a GB300 holds at once
 constexpr int kNaGroup = 32;                      // CTAs per first-level group
-constexpr int kNaMaxGroups = kNaMaxCtas / kNaGroup;
+constexpr int kNaGroups = kNaGrid / kNaGroup;
 
 struct NaScratch {
-  double part[kNaMaxCtas];        // per-CTA partial of <p, q>
-  double gsum[kNaMaxGroups];      // per-group sums
-  unsigned int gticket[kNaMaxGroups];
+  double part[kNaGrid];           // per-CTA partial of <p, q>
+  double gsum[kNaGroups];         // per-group sums
+  unsigned int gticket[kNaGroups];
   unsigned int ticket;            // groups finished
 };
 
-static_assert(kNaMaxCtas * kNaRowsPerCta == ICCG_NOALLOC_MAX_ROWS, "row limit must split into CTAs");
+static_assert(kNaGroups * kNaGroup == kNaGrid, "the CTAs must split into whole groups");
+static_assert(int64_t(ICCG_NOALLOC_MAX_ROWS) + int64_t(kNaGrid) * kNaRowsPerCta <= INT32_MAX, "a row index past the last");
 static_assert(offsetof(NaScratch, ticket) == offsetof(NaScratch, gticket) + sizeof(NaScratch::gticket), "cleared together");
 
 static __device__ __align__(256) unsigned char g_noalloc_scratch[sizeof(NaScratch)];
@@ -99,8 +100,6 @@ __device__ __forceinline__ bool na_last(unsigned int *ticket, unsigned int expec
 // forms at 7-point 50^3 15 us).
 constexpr int kNaChunk = 256;
 constexpr int kNaBatch = 8;
-
-constexpr int kNaGrid = 4 * 152;   // CTAs of a launch at most: those a GB300 holds at once
 
 struct NaChunk {
   int32_t c[kNaChunk / 32];
@@ -196,7 +195,7 @@ spmv_dot_noalloc_kernel(int n, const int64_t *__restrict__ rowptr, const int32_t
     na_load(nx, colind, val, e0, e1 - e0 <= kNaChunk ? int(e1 - e0) : 0, lane);
   }
   while (i - lane < n) {
-    const int in = i + stride;   // at most 2 * ICCG_NOALLOC_MAX_ROWS
+    const int in = i + stride;   // below ICCG_NOALLOC_MAX_ROWS + kNaGrid * kNaRowsPerCta
     const bool more = in - lane < n;
     const int64_t rsn = more ? rowptr[min(in, n)] : 0, ren = more ? rowptr[min(in + 1, n)] : 0;
     const int64_t e0 = __shfl_sync(0xffffffffu, rs, 0), e1 = __shfl_sync(0xffffffffu, re, 31);
