@@ -1,6 +1,6 @@
-"""Device graph of patterns with one very long row among short ones (a hub linked
-with every row) and of rows all above what a warp sorts: equal to the host's graph
-and coloring, and no more scratch than the sort itself needs is held."""
+"""Device graph and coloring of patterns with one very long row among short ones (a
+hub linked with every row, at the start, the end and in between): equal to the
+host's."""
 import numpy as np
 import pytest
 
